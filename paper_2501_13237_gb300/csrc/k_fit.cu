@@ -1,5 +1,6 @@
-// a8 -- noise-strength extrapolation to lambda* in float64, one thread per
-// observable (Sec. 2.2.3 (B); App. B.2).
+// a8 -- noise-strength extrapolation to lambda* in float64 (Sec. 2.2.3 (B);
+// App. B.2): one thread per observable for POLY and EXP_LOGLIN (fit_kernel),
+// one cluster per observable that needs EXP3 (exp3_kernel).
 //   POLY(m):     least squares in t = (lambda - lambda*)/max|lambda - lambda*| by
 //                Householder QR; estimate = constant coefficient.
 //   EXP_LOGLIN:  criterion 2 (|y| >= 1e-10), criterion 3 (sign of the
@@ -22,11 +23,16 @@
 //   (F_k = 1: left side 0; F_k = F_{k-1}: 0 if O_k = O_{k-1}, else infinite).
 // The fit then sees only the levels passing criterion 1 (mask), keeps the dip
 // size of all levels, and falls back to the D_k emulation at lambda*.
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace nne {
 
 constexpr int FIT_MAXL = 64;
+constexpr int FIT_NEEDS_EXP3 = 1 << 20;   // status between fit_kernel and exp3_kernel
 constexpr double DELTA_F = 2.0, DELTA_D = 20.0, SMALL = 1e-10, DIP_FID = 0.99;
 
 __device__ void nofit(int nl, const double* lam, const double* y, double ls, double* est, int* st) {
@@ -102,48 +108,19 @@ __device__ double exp3_profile(double b, int nl, const double* lam, const double
   return loss;
 }
 
-__device__ void exp3_fit(int nl, const double* lam, const double* y, double ls, double* est, int* st) {
+// EXP3 needs at least three levels that are not all equal; 50 / span otherwise.
+__device__ bool exp3_range(int nl, const double* lam, double* B) {
   double lmin = 1e300, lmax = -1e300;
   for (int j = 0; j < nl; ++j) { lmin = fmin(lmin, lam[j]); lmax = fmax(lmax, lam[j]); }
   const double span = nl > 0 ? lmax - lmin : 0;
-  if (nl < 3 || !(span > 0)) { nofit(nl, lam, y, ls, est, st); return; }
-  const double B = 50.0 / span;
-  const int NG = 4001;
-  const double step = (2 * B) / (NG - 1);
-  double a, c, best = 1e300;
-  int bi = 0;
-  for (int i = 0; i < NG; ++i) {
-    const double b = (i == NG - 1) ? B : i * step - B;
-    const double l = (b == 0.0) ? 1e300 : exp3_profile(b, nl, lam, y, &a, &c);
-    if (l < best) { best = l; bi = i; }
-  }
-  auto gridb = [&](int i) { return (i == NG - 1) ? B : i * step - B; };
-  double lo = gridb(max(bi - 1, 0)), hi = gridb(min(bi + 1, NG - 1));
-  const double g = (sqrt(5.0) - 1.0) / 2.0;
-  double x1 = hi - g * (hi - lo), x2 = lo + g * (hi - lo);
-  auto f = [&](double b) { return b == 0.0 ? 1e300 : exp3_profile(b, nl, lam, y, &a, &c); };
-  double f1 = f(x1), f2 = f(x2);
-  const double tol = 1e-12 * B;
-  for (int it = 0; it < 200 && hi - lo > tol; ++it) {
-    if (f1 <= f2) {
-      hi = x2; x2 = x1; f2 = f1;
-      x1 = hi - g * (hi - lo);
-      f1 = f(x1);
-    } else {
-      lo = x1; x1 = x2; f1 = f2;
-      x2 = lo + g * (hi - lo);
-      f2 = f(x2);
-    }
-  }
-  double b = 0.5 * (lo + hi);
-  if (b == 0.0) b = lo;
-  exp3_profile(b, nl, lam, y, &a, &c);
-  *est = a * exp(-b * ls) + c;
-  *st = NNE_OK;
+  if (nl < 3 || !(span > 0)) return false;
+  *B = 50.0 / span;
+  return true;
 }
 
 __device__ void loglin_fit(int nl, const double* lam, const double* y, const double* logf, double ls,
                            const double* yzero, int o, double dgiven, double* est, int* st) {
+  // (*st = FIT_NEEDS_EXP3: fewer than two levels survive, or all survivors share one lambda)
   int jmin = 0;
   for (int j = 1; j < nl; ++j)
     if (lam[j] < lam[jmin]) jmin = j;
@@ -155,7 +132,7 @@ __device__ void loglin_fit(int nl, const double* lam, const double* y, const dou
     keep[j] = fabs(y[j]) >= SMALL && sg == ref;
     nk += keep[j];
   }
-  if (nk < 2) { exp3_fit(nl, lam, y, ls, est, st); return; }
+  if (nk < 2) { *st = FIT_NEEDS_EXP3; return; }
   // dip size over all supplied levels (given by the caller when the fit sees a subset)
   double d = dgiven > 0 ? dgiven : 1e300;
   bool found = dgiven > 0;
@@ -183,7 +160,7 @@ __device__ void loglin_fit(int nl, const double* lam, const double* y, const dou
   for (int i = 0; i < m; ++i)
     for (int j = i + 1; j < m; ++j)
       if (x[i] != x[j]) { lpmax = fmax(lpmax, lw2[i] + lw2[j] + 2.0 * log(fabs(x[i] - x[j]))); any = true; }
-  if (!any) { exp3_fit(nl, lam, y, ls, est, st); return; }
+  if (!any) { *st = FIT_NEEDS_EXP3; return; }
   double num = 0, den = 0;
   for (int i = 0; i < m; ++i)
     for (int j = i + 1; j < m; ++j)
@@ -219,23 +196,43 @@ __device__ double dip_all(int nl, const double* lam, const double* logf) {
   return lmax - lmin > 0 ? lmax - lmin : 1.0;
 }
 
+// The levels of observable o that the fit may use (mask null: all): count.
+__device__ int gather_levels(int nl, const double* lam, const double* vals, const double* logf, int n_obs, int o,
+                             const uint8_t* mask, double* y, double* lc, double* fc) {
+  int m = 0;
+  for (int j = 0; j < nl; ++j) {
+    if (mask && !mask[(long long)j * n_obs + o]) continue;
+    y[m] = vals[(long long)j * n_obs + o];
+    lc[m] = lam[j];
+    if (fc) fc[m] = logf ? logf[j] : 0.0;
+    ++m;
+  }
+  return m;
+}
+
+// NOFIT of a masked fit: the value at lambda* over all levels.
+__device__ void store_fit(int nl, const double* lam, const double* vals, int n_obs, int o, double ls,
+                          const uint8_t* mask, const double* fb, double est, int st, double* out, int* status) {
+  if (st == NNE_ERR_NOFIT && (fb || mask)) {
+    const double* src = fb ? fb : vals;
+    est = nan("");
+    for (int j = 0; j < nl; ++j)
+      if (lam[j] == ls) { est = src[(long long)j * n_obs + o]; break; }
+  }
+  out[o] = est;
+  status[o] = st;
+}
+
 // mask (nl x n_obs, lambda-major; null: every level): levels the fit may use;
 // fb (nl x n_obs; null: the fitted values): where the NOFIT fallback reads the
-// value at lambda*.
+// value at lambda*.  Observables that need EXP3 get status FIT_NEEDS_EXP3.
 __global__ void fit_kernel(int nl, const double* lam, const double* vals, const double* logf, int n_obs, int method,
                            int degree, double ls, const double* yzero, const uint8_t* mask, const double* fb,
                            double* out, int* status) {
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= n_obs) return;
   double y[FIT_MAXL], lc[FIT_MAXL], fc[FIT_MAXL];
-  int m = 0;
-  for (int j = 0; j < nl; ++j) {
-    if (mask && !mask[(long long)j * n_obs + o]) continue;
-    y[m] = vals[(long long)j * n_obs + o];
-    lc[m] = lam[j];
-    fc[m] = logf ? logf[j] : 0.0;
-    ++m;
-  }
+  const int m = gather_levels(nl, lam, vals, logf, n_obs, o, mask, y, lc, fc);
   const double dgiven = mask ? dip_all(nl, lam, logf) : -1.0;
   double est = nan("");
   int st = NNE_ERR_NOFIT;
@@ -246,16 +243,150 @@ __global__ void fit_kernel(int nl, const double* lam, const double* vals, const 
   } else if (method == NNE_FIT_EXP_LOGLIN) {
     loglin_fit(m, lc, y, logf ? fc : nullptr, ls, yzero, o, dgiven, &est, &st);
   } else {
-    exp3_fit(m, lc, y, ls, &est, &st);
+    st = FIT_NEEDS_EXP3;
   }
-  if (st == NNE_ERR_NOFIT && (fb || mask)) {
-    const double* src = fb ? fb : vals;
-    est = nan("");
-    for (int j = 0; j < nl; ++j)
-      if (lam[j] == ls) { est = src[(long long)j * n_obs + o]; break; }
+  if (st == FIT_NEEDS_EXP3) {
+    status[o] = st;
+    return;
   }
-  out[o] = est;
-  status[o] = st;
+  store_fit(nl, lam, vals, n_obs, o, ls, mask, fb, est, st, out, status);
+}
+
+// EXP3 of the observables fit_kernel marked: one cluster of EXP3_CS CTAs each
+// (the other clusters leave at once).
+//
+// Bound by float64 arithmetic, which runs at 1/64 of the float32 rate: a
+// profile at one b costs about 40 operations per level (the exponential most
+// of all), and the grid has 4001 points.  One thread per observable took the
+// 4061 profiles one after the other: 22.7 ms for 199 observables at 5 levels
+// of which a handful need EXP3.  The grid's points are independent, so they
+// are dealt to the EXP3_CS x 128 threads (the best is the smallest loss, the
+// lowest index among equal ones, as a scan in order finds it); the golden
+// section that follows is a serial chain of about 60 profiles, each formed by
+// one warp with a level per lane and the sums in level order (whole call of
+// that table: 22.8 ms -> 0.33 ms).
+constexpr int EXP3_CS = 8, EXP3_THREADS = 128, EXP3_GRID = 4001;
+
+__global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS)
+    exp3_kernel(int nl, const double* lam, const double* vals, int n_obs, double ls, const uint8_t* mask,
+                const double* fb, double* out, int* status, int o0) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int o = o0 + (int)(blockIdx.x / EXP3_CS);
+  if (status[o] != FIT_NEEDS_EXP3) return;   // the same for every CTA of the cluster
+  __shared__ double y[FIT_MAXL], lc[FIT_MAXL];
+  __shared__ double wbest[EXP3_THREADS / 32];
+  __shared__ int widx[EXP3_THREADS / 32];
+  __shared__ double cbest[EXP3_CS];
+  __shared__ int cidx[EXP3_CS];
+  __shared__ int m_s, ok_s;
+  __shared__ double B_s;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) {
+    m_s = gather_levels(nl, lam, vals, nullptr, n_obs, o, mask, y, lc, nullptr);
+    double B = 0;
+    ok_s = exp3_range(m_s, lc, &B) ? 1 : 0;
+    B_s = B;
+  }
+  cluster.sync();   // also: every CTA has read status[o], and runs, before rank 0 is written to
+  const int m = m_s;
+  if (!ok_s) {
+    if (rank == 0 && tid == 0) {
+      double est;
+      int st;
+      nofit(m, lc, y, ls, &est, &st);
+      store_fit(nl, lam, vals, n_obs, o, ls, mask, fb, est, st, out, status);
+    }
+    return;
+  }
+  const double B = B_s, step = (2 * B) / (EXP3_GRID - 1);
+  auto gridb = [&](int i) { return (i == EXP3_GRID - 1) ? B : i * step - B; };
+  double best = 1e300, a, c;
+  int bi = 0;
+  for (int i = rank * EXP3_THREADS + tid; i < EXP3_GRID; i += EXP3_CS * EXP3_THREADS) {
+    const double b = gridb(i);
+    const double l = (b == 0.0) ? 1e300 : exp3_profile(b, m, lc, y, &a, &c);
+    if (l < best) { best = l; bi = i; }
+  }
+  for (int d = 16; d > 0; d >>= 1) {
+    const double l2 = __shfl_xor_sync(0xffffffffu, best, d);
+    const int i2 = __shfl_xor_sync(0xffffffffu, bi, d);
+    if (l2 < best || (l2 == best && i2 < bi)) { best = l2; bi = i2; }
+  }
+  if (lane == 0) {
+    wbest[tid >> 5] = best;
+    widx[tid >> 5] = bi;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < EXP3_THREADS / 32; ++w)
+      if (wbest[w] < best || (wbest[w] == best && widx[w] < bi)) { best = wbest[w]; bi = widx[w]; }
+    *cluster.map_shared_rank(&cbest[rank], 0) = best;
+    *cluster.map_shared_rank(&cidx[rank], 0) = bi;
+  }
+  cluster.sync();
+  if (rank != 0 || tid >= 32) return;
+  best = cbest[0];
+  bi = cidx[0];
+  for (int r = 1; r < EXP3_CS; ++r)
+    if (cbest[r] < best || (cbest[r] == best && cidx[r] < bi)) { best = cbest[r]; bi = cidx[r]; }
+  // one profile by the warp: lane j forms the exponentials of levels j and j + 32
+  auto profile = [&](double b) {
+    double e0 = lane < m ? exp(-b * lc[lane]) : 0.0, e1 = lane + 32 < m ? exp(-b * lc[lane + 32]) : 0.0;
+    auto e = [&](int j) { return __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31); };
+    double em = 0, ym = 0;
+    for (int j = 0; j < m; ++j) { em += e(j); ym += y[j]; }
+    em /= m;
+    ym /= m;
+    double see = 0, sey = 0;
+    for (int j = 0; j < m; ++j) { const double ej = e(j); see += (ej - em) * (ej - em); sey += (ej - em) * (y[j] - ym); }
+    a = see > 0 ? sey / see : 0.0;
+    c = ym - a * em;
+    double loss = 0;
+    for (int j = 0; j < m; ++j) { const double r = a * e(j) + c - y[j]; loss += r * r; }
+    return loss;
+  };
+  double lo = gridb(max(bi - 1, 0)), hi = gridb(min(bi + 1, EXP3_GRID - 1));
+  const double g = (sqrt(5.0) - 1.0) / 2.0;
+  double x1 = hi - g * (hi - lo), x2 = lo + g * (hi - lo);
+  auto f = [&](double b) { return b == 0.0 ? 1e300 : profile(b); };
+  double f1 = f(x1), f2 = f(x2);
+  const double tol = 1e-12 * B;
+  for (int it = 0; it < 200 && hi - lo > tol; ++it) {
+    if (f1 <= f2) {
+      hi = x2; x2 = x1; f2 = f1;
+      x1 = hi - g * (hi - lo);
+      f1 = f(x1);
+    } else {
+      lo = x1; x1 = x2; f1 = f2;
+      x2 = lo + g * (hi - lo);
+      f2 = f(x2);
+    }
+  }
+  double b = 0.5 * (lo + hi);
+  if (b == 0.0) b = lo;
+  profile(b);
+  if (lane == 0) {
+    out[o] = a * exp(-b * ls) + c;
+    status[o] = NNE_OK;
+  }
+}
+
+// Both kernels; the EXP3 pass only where the method can reach it.
+static cudaError_t launch_fit(cudaStream_t st, int nl, const double* lam, const double* vals, const double* logf,
+                              int n_obs, int method, int degree, double ls, const double* yzero, const uint8_t* mask,
+                              const double* fb, double* out, int* status) {
+  fit_kernel<<<(n_obs + 63) / 64, 64, 0, st>>>(nl, lam, vals, logf, n_obs, method, degree, ls, yzero, mask, fb, out,
+                                              status);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || method == NNE_FIT_POLY) return e;
+  constexpr int PER_LAUNCH = 1 << 24;   // observables per launch: the grid stays below 2^31 CTAs
+  for (int o0 = 0; o0 < n_obs && e == cudaSuccess; o0 += std::min(PER_LAUNCH, n_obs - o0)) {
+    exp3_kernel<<<std::min(PER_LAUNCH, n_obs - o0) * EXP3_CS, EXP3_THREADS, 0, st>>>(nl, lam, vals, n_obs, ls, mask, fb,
+                                                                                  out, status, o0);
+    e = cudaGetLastError();
+  }
+  return e;
 }
 
 // (A) over k rungs: vals (k x nl x n_obs), logf (k x nl) -> obar (nl x n_obs), conv (nl x n_obs).
@@ -299,17 +430,16 @@ cudaError_t extrapolate_fit(cudaStream_t st, int n_lambda, const double* d_lam, 
                             const double* d_logfid, int n_obs, int method, int degree, double lambda_star,
                             const double* d_yzero, double* d_out, int* d_status) {
   if (n_obs <= 0) return cudaSuccess;
-  ProfScope ps(st, K_FIT);
-  fit_kernel<<<(n_obs + 63) / 64, 64, 0, st>>>(n_lambda, d_lam, d_vals, d_logfid, n_obs, method, degree, lambda_star,
-                                              d_yzero, nullptr, nullptr, d_out, d_status);
-  return cudaGetLastError();
+  ProfScope ps(st, K_FIT, method == NNE_FIT_POLY ? 1 : 2);
+  return launch_fit(st, n_lambda, d_lam, d_vals, d_logfid, n_obs, method, degree, lambda_star, d_yzero, nullptr,
+                    nullptr, d_out, d_status);
 }
 
 cudaError_t extrapolate_ladder(cudaStream_t st, int k, int n_lambda, const double* d_lam, const double* d_vals,
                                const double* d_logfid, int n_obs, int method, int degree, double lambda_star,
                                const double* d_yzero, double* d_obar, uint8_t* d_conv, double* d_out, int* d_status) {
   if (n_obs <= 0) return cudaSuccess;
-  ProfScope ps(st, K_FIT, 2);
+  ProfScope ps(st, K_FIT, method == NNE_FIT_POLY ? 2 : 3);
   const long long cells = (long long)n_lambda * n_obs;
   ladder_kernel<<<(unsigned)((cells + 127) / 128), 128, 0, st>>>(k, n_lambda, n_obs, d_vals, d_logfid, d_obar, d_conv);
   cudaError_t e = cudaGetLastError();
@@ -317,9 +447,8 @@ cudaError_t extrapolate_ladder(cudaStream_t st, int k, int n_lambda, const doubl
   // (B) on the fidelity-extrapolated values, F^max = the top rung, fallback to the top rung's values
   const double* top_logf = d_logfid + (long long)(k - 1) * n_lambda;
   const double* top_vals = d_vals + (long long)(k - 1) * cells;
-  fit_kernel<<<(n_obs + 63) / 64, 64, 0, st>>>(n_lambda, d_lam, d_obar, top_logf, n_obs, method, degree, lambda_star,
-                                              d_yzero, d_conv, top_vals, d_out, d_status);
-  return cudaGetLastError();
+  return launch_fit(st, n_lambda, d_lam, d_obar, top_logf, n_obs, method, degree, lambda_star, d_yzero, d_conv,
+                    top_vals, d_out, d_status);
 }
 
 }  // namespace nne
