@@ -273,9 +273,9 @@ nne_status nne_cgemm_c64(nne_ctx* ctx, int op_a, int op_b, int M, int N, int K, 
  * NNE_OPT_EIG_FP64 (default 1): complex64 states solve the truncation's
  * Hermitian eigenproblems (the Gram matrix of the exact truncation, the
  * Rayleigh-Ritz matrix of the subspace iteration, the centre compression)
- * with float64 quality: the Householder reduction in float64 (matrices that
- * fit a cluster's shared memory) or in double-float arithmetic on the
- * float32 pipes (larger ones; about 2^-46 relative), bisection and inverse
+ * with float64 quality: the Householder reduction in float64 (matrices of up to
+ * 160 rows) or in double-float arithmetic on the float32 pipes (larger ones;
+ * about 2^-46 relative, in one cluster's shared memory up to 384 rows), bisection and inverse
  * iteration in float64, the back-transformation in float32; 0 runs them in
  * float32 (about 1.5x the gate-step rate at chi = 512, with a float32
  * reduction's error of eps_32 times the largest eigenvalue, which turns the

@@ -421,283 +421,6 @@ __global__ void __launch_bounds__(256) entropy_kernel(const R* lamb, int n, int 
   if (threadIdx.x == 0) S[(long long)blockIdx.x * sS] = h;
 }
 
-// ---------------------------------------------------------------- double-float reduction
-// The complex64 path's float64-quality reduction with its O(n^3) arithmetic on
-// the float32 pipes.  Every entry of the trailing matrix is an unevaluated sum
-// hi + lo of two floats per component (a "double-float", Dekker 1971; about
-// 2^-46 relative): float4 {re_hi, re_lo, im_hi, im_lo}, 16 bytes like a
-// complex128.  Products take the exact rounding error of hi*hi from an FMA
-// (TwoProduct) plus the hi*lo cross terms; sums carry their exact rounding
-// error by Knuth's TwoSum into the lo part (the accumulation of Ogita, Rump
-// and Oishi's Dot2), renormalised once per stored entry.  A float64 complex
-// multiply-add (4 FMAs at GB300's 1/64 float64 rate) becomes 4 x 12 float32
-// operations.  The Householder vector, the norms, K and w are formed in
-// float64 (O(m) per column); d, e and the reflectors are written in float64.
-// Lower triangle only, as in the float64 kernel.
-__device__ __forceinline__ float4 df_from_cd(cx<double> a) {
-  const float rh = (float)a.re, ih = (float)a.im;
-  return make_float4(rh, (float)(a.re - (double)rh), ih, (float)(a.im - (double)ih));
-}
-__device__ __forceinline__ double df_to_d(float hi, float lo) { return (double)hi + (double)lo; }
-// (hi, lo) += x * y, x = xh + xl, y = yh + yl
-__device__ __forceinline__ void df_mac(float& hi, float& lo, float xh, float xl, float yh, float yl) {
-  const float ph = __fmul_rn(xh, yh);
-  const float pe = fmaf(xh, yl, fmaf(xl, yh, fmaf(xh, yh, -ph)));
-  const float s = __fadd_rn(hi, ph);
-  const float bb = __fsub_rn(s, hi);
-  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(ph, bb));
-  hi = s;
-  lo = __fadd_rn(lo, __fadd_rn(e, pe));
-}
-// (hi, lo) += (bh, bl)
-__device__ __forceinline__ void df_add(float& hi, float& lo, float bh, float bl) {
-  const float s = __fadd_rn(hi, bh);
-  const float bb = __fsub_rn(s, hi);
-  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(bh, bb));
-  hi = s;
-  lo = __fadd_rn(lo, __fadd_rn(e, bl));
-}
-__device__ __forceinline__ void df_norm(float& hi, float& lo) {
-  const float s = __fadd_rn(hi, lo);
-  lo = __fsub_rn(lo, __fsub_rn(s, hi));
-  hi = s;
-}
-// acc (re, im) += a * v (conj_a: conj(a) * v)
-template <bool CONJ_A>
-__device__ __forceinline__ void df_cmac(float4& acc, float4 a, float4 v) {
-  const float sa = CONJ_A ? -1.f : 1.f;
-  df_mac(acc.x, acc.y, a.x, a.y, v.x, v.y);                       // re: a.re v.re
-  df_mac(acc.x, acc.y, -sa * a.z, -sa * a.w, v.z, v.w);           //     -/+ a.im v.im
-  df_mac(acc.z, acc.w, a.x, a.y, v.z, v.w);                       // im: a.re v.im
-  df_mac(acc.z, acc.w, sa * a.z, sa * a.w, v.x, v.y);             //     +/- a.im v.re
-  // renormalised every two terms: the lo parts stay small (10x less error over long sums)
-  df_norm(acc.x, acc.y);
-  df_norm(acc.z, acc.w);
-}
-__device__ __forceinline__ float4 df_warp_sum(float4 a) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const float bh = __shfl_xor_sync(0xffffffffu, a.x, o), bl = __shfl_xor_sync(0xffffffffu, a.y, o);
-    const float ch = __shfl_xor_sync(0xffffffffu, a.z, o), cl = __shfl_xor_sync(0xffffffffu, a.w, o);
-    df_add(a.x, a.y, bh, bl);
-    df_add(a.z, a.w, ch, cl);
-  }
-  return a;
-}
-
-__global__ void cx_f2df_kernel(const cx<float>* X, long long sX, int n, float4* Y, long long sY) {
-  const long long count = (long long)n * n;
-  const int z = blockIdx.y;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
-    const cx<float> v = X[z * sX + i];
-    Y[z * sY + i] = make_float4(v.re, 0.f, v.im, 0.f);
-  }
-}
-
-// (ph, pl) = x * y for double-floats, renormalised
-__device__ __forceinline__ float2 df_mul(float xh, float xl, float yh, float yl) {
-  const float ph = __fmul_rn(xh, yh);
-  const float pl = fmaf(xh, yl, fmaf(xl, yh, fmaf(xh, yh, -ph)));
-  const float s = __fadd_rn(ph, pl);
-  return make_float2(s, __fsub_rn(pl, __fsub_rn(s, ph)));
-}
-// block-wide double-float sum (every thread gets it); red holds 2 x 32 floats
-__device__ __forceinline__ float2 df_block_sum(float hi, float lo, float* red) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
-    df_add(hi, lo, bh, bl);
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) {
-    red[2 * (threadIdx.x >> 5)] = hi;
-    red[2 * (threadIdx.x >> 5) + 1] = lo;
-  }
-  __syncthreads();
-  float th = 0.f, tl = 0.f;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) df_add(th, tl, red[2 * w], red[2 * w + 1]);
-  return make_float2(th, tl);
-}
-
-// Every O(m) step of a column is double-float as well (norms, the reflector,
-// K, w), so the float64 pipe only sees one thread's pivot per column; the
-// reflectors go out rounded to float32 for the float32 back-transformation,
-// d and e in float64.
-template <int U>
-__global__ void __launch_bounds__(512) tridiag_df_kernel(float4* Hb, long long sH, int n, double* db, cx<double>* eb,
-                                                          int ldde, float4* Pb, float2* Kb, cx<float>* Vhb,
-                                                          long long sVh) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const int CS = (int)cluster.num_blocks();
-  const int rank = (int)cluster.block_rank();
-  const int z = blockIdx.y;
-  float4* H = Hb + z * sH;
-  double* d = db + (long long)z * ldde;
-  cx<double>* e = eb + (long long)z * ldde;
-  float4* P = Pb + (long long)z * ldde;
-  float2* Kp = Kb + z * 32;
-  extern __shared__ __align__(16) unsigned char df_smem[];
-  float4* vdf = reinterpret_cast<float4*>(df_smem);   // n: the Householder vector
-  float4* wdf = vdf + n;                              // n: w = 2p - 2Kv
-  __shared__ float red[64];
-  __shared__ float4 alpha_s;
-  __shared__ float2 inv_s;
-  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
-  const int gw = rank * nw + warp, GW = CS * nw;
-
-  for (int j = 0; j + 2 < n; ++j) {
-    const int m = n - j - 1;
-    // column j below the diagonal, and its squared norm
-    float nh = 0.f, nl = 0.f;
-    {
-      const float4* colj = H + (long long)(j + 1) * n + j;
-      for (int t = tid; t < m; t += nth) {
-        const float4 a = colj[(long long)t * n];
-        vdf[t] = a;
-        df_mac(nh, nl, a.x, a.y, a.x, a.y);
-        df_mac(nh, nl, a.z, a.w, a.z, a.w);
-      }
-    }
-    const float2 xn2f = df_block_sum(nh, nl, red);
-    if (tid == 0) {
-      // pivot in float64 on one thread: alpha = -e^{i arg x0} ||x||, un = ||x - alpha e0||
-      const float4 x0 = vdf[0];
-      const cx<double> x0d = mk<double>(df_to_d(x0.x, x0.y), df_to_d(x0.z, x0.w));
-      double pr, pi, ax0;
-      unit_phase_of(x0d, &pr, &pi, &ax0);
-      const double xn2 = df_to_d(xn2f.x, xn2f.y), xn = sqrt(xn2);
-      cx<double> alpha = mk<double>(0, 0);
-      double un = 0;
-      if (xn > 0) {
-        alpha = mk<double>(-xn * pr, -xn * pi);
-        un = sqrt(2.0 * xn2 + 2.0 * xn * ax0);
-      }
-      const double inv = un > 0 ? 1.0 / un : 0.0;
-      alpha_s = df_from_cd(alpha);
-      const float ih = (float)inv;
-      inv_s = make_float2(ih, (float)(inv - (double)ih));
-      if (rank == 0) {
-        const float4 hjj = H[(long long)j * n + j];
-        d[j] = df_to_d(hjj.x, hjj.y);
-        e[j] = alpha;
-      }
-    }
-    __syncthreads();
-    {
-      const float4 al = alpha_s;
-      const float2 iv = inv_s;
-      cx<float>* rj = Vhb + z * sVh + (long long)j * n + (j + 1);
-      for (int t = tid; t < m; t += nth) {
-        float4 u = vdf[t];
-        if (t == 0) {
-          df_add(u.x, u.y, -al.x, -al.y);
-          df_add(u.z, u.w, -al.z, -al.w);
-        }
-        const float2 vr = df_mul(u.x, u.y, iv.x, iv.y), vi = df_mul(u.z, u.w, iv.x, iv.y);
-        vdf[t] = make_float4(vr.x, vr.y, vi.x, vi.y);
-        if (rank == 0) rj[t] = mk<float>(vr.x, -vi.x);   // reflector j, conjugated, for the back-transform
-      }
-    }
-    __syncthreads();
-    // p = A v on own rows (lower part of row t, then its upper part read down column t); K = v^H p
-    float kh = 0.f, kl = 0.f;
-    for (int t = gw; t < m; t += GW) {
-      const float4* row = H + (long long)(j + 1 + t) * n + (j + 1);
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), acc2 = acc;
-      int k = lane;
-      for (; k + 32 * (U - 1) <= t; k += 32 * U) {
-        float4 a[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) a[u] = row[k + 32 * u];
-#pragma unroll
-        for (int u = 0; u < U; ++u) df_cmac<false>((u & 1) ? acc2 : acc, a[u], vdf[k + 32 * u]);
-      }
-      for (; k <= t; k += 32) df_cmac<false>(acc, row[k], vdf[k]);
-      const float4* colt = H + (long long)(j + 1) * n + (j + 1 + t);
-      k = t + 1 + lane;
-      for (; k + 32 * (U - 1) < m; k += 32 * U) {
-        float4 a[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) a[u] = colt[(long long)(k + 32 * u) * n];
-#pragma unroll
-        for (int u = 0; u < U; ++u) df_cmac<true>((u & 1) ? acc2 : acc, a[u], vdf[k + 32 * u]);
-      }
-      for (; k < m; k += 32) df_cmac<true>(acc, colt[(long long)k * n], vdf[k]);
-      df_add(acc.x, acc.y, acc2.x, acc2.y);
-      df_add(acc.z, acc.w, acc2.z, acc2.w);
-      acc = df_warp_sum(acc);
-      if (lane == 0) {
-        P[t] = acc;
-        const float4 vt = vdf[t];
-        df_mac(kh, kl, vt.x, vt.y, acc.x, acc.y);
-        df_mac(kh, kl, vt.z, vt.w, acc.z, acc.w);
-      }
-    }
-    {
-      const float2 kp = df_block_sum(kh, kl, red);
-      if (tid == 0) Kp[rank] = kp;
-    }
-    __threadfence();
-    cluster.sync();
-    float Kh = 0.f, Kl = 0.f;
-    for (int c = 0; c < CS; ++c) df_add(Kh, Kl, Kp[c].x, Kp[c].y);
-    // w = 2p - 2 K v  (2K exact in double-float)
-    const float K2h = 2.f * Kh, K2l = 2.f * Kl;
-    for (int t = tid; t < m; t += nth) {
-      const float4 p = P[t], vt = vdf[t];
-      float rh = 2.f * p.x, rl = 2.f * p.y, ih = 2.f * p.z, il = 2.f * p.w;
-      df_mac(rh, rl, -K2h, -K2l, vt.x, vt.y);
-      df_mac(ih, il, -K2h, -K2l, vt.z, vt.w);
-      df_norm(rh, rl);
-      df_norm(ih, il);
-      wdf[t] = make_float4(rh, rl, ih, il);
-    }
-    __syncthreads();
-    // A <- A - v w^H - w v^H on the lower triangle of own rows (U entries in flight per lane)
-    for (int t = gw; t < m; t += GW) {
-      float4* row = H + (long long)(j + 1 + t) * n + (j + 1);
-      const float4 vt = vdf[t], wt = wdf[t];
-      for (int k0 = lane; k0 <= t; k0 += 32 * U) {
-        float4 a[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (k0 + 32 * u <= t) a[u] = row[k0 + 32 * u];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int k = k0 + 32 * u;
-          if (k > t) break;
-          const float4 wk = wdf[k], vk = vdf[k];
-          float4 b = a[u];
-          // re: - (vt.re wk.re + vt.im wk.im + wt.re vk.re + wt.im vk.im)
-          df_mac(b.x, b.y, -vt.x, -vt.y, wk.x, wk.y);
-          df_mac(b.x, b.y, -vt.z, -vt.w, wk.z, wk.w);
-          df_mac(b.x, b.y, -wt.x, -wt.y, vk.x, vk.y);
-          df_mac(b.x, b.y, -wt.z, -wt.w, vk.z, vk.w);
-          // im: - (vt.im wk.re - vt.re wk.im + wt.im vk.re - wt.re vk.im)
-          df_mac(b.z, b.w, -vt.z, -vt.w, wk.x, wk.y);
-          df_mac(b.z, b.w, vt.x, vt.y, wk.z, wk.w);
-          df_mac(b.z, b.w, -wt.z, -wt.w, vk.x, vk.y);
-          df_mac(b.z, b.w, wt.x, wt.y, vk.z, vk.w);
-          df_norm(b.x, b.y);
-          df_norm(b.z, b.w);
-          row[k] = b;
-        }
-      }
-    }
-    __threadfence();
-    cluster.sync();
-  }
-  if (rank == 0 && tid == 0) {
-    if (n >= 2) {
-      const float4 a = H[(long long)(n - 2) * n + (n - 2)], b = H[(long long)(n - 1) * n + (n - 1)];
-      const float4 c = H[(long long)(n - 1) * n + (n - 2)];
-      d[n - 2] = df_to_d(a.x, a.y);
-      d[n - 1] = df_to_d(b.x, b.y);
-      e[n - 2] = mk<double>(df_to_d(c.x, c.y), df_to_d(c.z, c.w));
-    } else {
-      d[0] = df_to_d(H[0].x, H[0].y);
-    }
-  }
-}
-
 // ---------------------------------------------------------------- launchers
 template <typename K, typename... Args>
 static cudaError_t launch_cluster_t(K kernel, int cs, int batch, int threads, size_t smem, cudaStream_t st,
@@ -734,13 +457,7 @@ static int cluster_size_for(int n) { return n >= 512 ? 8 : (n >= 128 ? 4 : (n >=
 // gives at least 8 active clusters (GB300's GPCs hold only 7 clusters of
 // 13-16 single-SM CTAs).  The size depends on nothing but the kernel, so
 // results do not depend on how instances are batched.
-constexpr size_t TRIDIAG64_SMEM = 120 * 1024;
-// double-float reduction launch: 256 threads, TRIDIAG_DF_UNROLL loads in flight per lane in the
-// product A v and the rank-2 update (its loads wait on L2: ncu shows long-scoreboard stalls and
-// 1.6 % L2 throughput with one load per lane)
-constexpr int TRIDIAG_DF_THREADS = 256;
-constexpr int TRIDIAG_DF_UNROLL = 4;
-static int tridiag64_cluster_size(const void* kernel) {
+int tridiag64_cluster_size(const void* kernel) {
   static std::mutex mu;
   static std::map<const void*, int> memo;
   std::lock_guard<std::mutex> lk(mu);
@@ -1013,12 +730,23 @@ __global__ void re_d2f_kernel(const double* X, float* Y, long long count) {
 
 static inline size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
+// Complex64 eigenproblems up to this size keep the float64 reduction, larger
+// ones take the double-float one (k_tridiag_df.cu).  The double-float kernel is
+// the faster at every size (n = 64: 174 against 514 us, 128: 431 against 1300),
+// but small bonds cut shallow circuits between near-degenerate pairs, where the
+// kept vector follows the last bits of the reduction: <P> of 5 in 45 bursts of
+// jobs with bonds of 12-40 moved by more than 2e-5 of their norm (up to 7.6e-5,
+// as far as the complex64 result itself is from an exact one), against 1 in 200
+// circuits with bonds of 41-72.  Up to bonds of 40 results stay as they were.
+constexpr int EIGH_F64_MAX = 160;
+
 MixedEighWork eigh_mixed_workspace(int n, int r) {
   // per matrix; every array is batch-major, so a batch of b matrices needs b times these bytes
   MixedEighWork w;
   const size_t nn = (size_t)n * n, nr = (size_t)n * r;
   const int nbw = (n + 31) / 32;
-  w.cx_bytes = al256(16 * nn) * 2 + al256(16 * (size_t)n) * 3 + al256(8 * nn) + al256(8 * (size_t)n) +
+  const size_t nf = (size_t)std::min(n, EIGH_F64_MAX);   // a state's smaller problems take the float64 path
+  w.cx_bytes = al256(std::max(16 * nn, 32 * nf * nf)) + al256(16 * (size_t)n) * 3 + al256(8 * nn) + al256(8 * (size_t)n) +
                al256(8 * (size_t)nbw * 1024) + al256(8 * (size_t)wy_workspace(r)) +
                al256(8 * (size_t)qr_workspace(n, r).cx_elems) + 1024;
   w.re_bytes = al256(8 * (size_t)n) * 2 + al256(8 * (size_t)r) + al256(8 * nr) * 5 + al256(4 * nr) + 512 +
@@ -1029,8 +757,9 @@ MixedEighWork eigh_mixed_workspace(int n, int r) {
 
 // Top-r eigenvectors of the complex64 Hermitian H[z] (n x n, ld n), written to
 // U[z] (n x r, ld r, columns by decreasing eigenvalue, orthonormal).  The
-// Householder reduction, the eigenvalues (bisection) and the eigenvectors of
-// the tridiagonal (inverse iteration) run in float64; the back-transformation
+// Householder reduction runs in float64 (n <= EIGH_F64_MAX) or double-float, the eigenvalues
+// (bisection) and the eigenvectors of the tridiagonal (inverse iteration) in
+// float64; the back-transformation
 // through the reflectors and the final orthonormalisation run in float32.  A
 // float32 reduction has a backward error of eps_32 ||H||, which turns the
 // eigenvectors next to the truncation cut by eps_32 ||H|| / gap there (about
@@ -1050,11 +779,10 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
     base += al256(bytes);
     return p;
   };
-  cx<double>* Hd = reinterpret_cast<cx<double>*>(take(c, 16 * nn * B));
-  cx<double>* Vhd = reinterpret_cast<cx<double>*>(take(c, 16 * nn * B));
+  cx<double>* Hd = reinterpret_cast<cx<double>*>(take(c, 16 * nn * B * (n <= EIGH_F64_MAX ? 2 : 1)));
   cx<double>* ed = reinterpret_cast<cx<double>*>(take(c, 16 * (size_t)n * B));
   cx<double>* phid = reinterpret_cast<cx<double>*>(take(c, 16 * (size_t)n * B));
-  cx<double>* Pd = reinterpret_cast<cx<double>*>(take(c, 16 * (size_t)n * B));
+  float4* P = reinterpret_cast<float4*>(take(c, 16 * (size_t)n * B));
   cx<float>* Vhf = reinterpret_cast<cx<float>*>(take(c, 8 * nn * B));
   cx<float>* phif = reinterpret_cast<cx<float>*>(take(c, 8 * (size_t)n * B));
   cx<float>* Tw = reinterpret_cast<cx<float>*>(take(c, 8 * (size_t)nbw * 1024 * B));
@@ -1070,40 +798,31 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
   double* U1 = reinterpret_cast<double*>(take(q, 8 * nr * B));
   double* U2 = reinterpret_cast<double*>(take(q, 8 * nr * B));
   float* Zf = reinterpret_cast<float*>(take(q, 4 * nr * B));
-  double* Kp = reinterpret_cast<double*>(take(q, 8 * 32 * B));
+  float2* Kp = reinterpret_cast<float2*>(take(q, 8 * 32 * B));
   float* df = reinterpret_cast<float*>(take(q, 4 * (size_t)n * B));
   float* ef = reinterpret_cast<float*>(take(q, 4 * (size_t)n * B));
   float* lamf = reinterpret_cast<float*>(take(q, 4 * (size_t)r * B));
   uint8_t* piv = reinterpret_cast<uint8_t*>(u8_ws);
   cudaError_t ce;
-  const bool in_smem = smem_cluster_size<double>(n) > 0;
-  {
-    ProfScope ps(st, K_ELEMWISE);
-    const dim3 grid((unsigned)std::min<size_t>((nn + 255) / 256, 1024), batch);
-    if (in_smem)
+  if (n <= EIGH_F64_MAX) {
+    cx<double>* Vhd = Hd + nn * B;
+    {
+      ProfScope ps(st, K_ELEMWISE);
+      const dim3 grid((unsigned)std::min<size_t>((nn + 255) / 256, 1024), batch);
       cx_f2d_kernel<<<grid, 256, 0, st>>>(H, sH, n, n, n, Hd, (long long)nn);
-    else
-      cx_f2df_kernel<<<grid, 256, 0, st>>>(H, sH, n, reinterpret_cast<float4*>(Hd), (long long)nn);
-  }
-  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  if (in_smem) {
+    }
+    if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
     if ((ce = cudaMemsetAsync(Vhd, 0, 16 * nn * B, st)) != cudaSuccess) return ce;
+    if ((ce = tridiag_smem<double>(st, Hd, (long long)nn, n, dd, ed, n, Vhd, (long long)nn, batch)) != cudaSuccess)
+      return ce;
+    ProfScope ps(st, K_ELEMWISE);
+    cx_d2f_kernel<<<1024, 256, 0, st>>>(Vhd, Vhf, (long long)(nn * B));
+    if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
   } else {
     if ((ce = cudaMemsetAsync(Vhf, 0, 8 * nn * B, st)) != cudaSuccess) return ce;
+    if ((ce = tridiag_df(st, H, sH, n, reinterpret_cast<float4*>(Hd), P, Kp, dd, ed, Vhf, batch)) != cudaSuccess)
+      return ce;
   }
-  if (in_smem) {
-    ce = tridiag_smem<double>(st, Hd, (long long)nn, n, dd, ed, n, Vhd, (long long)nn, batch);
-  } else {
-    // double-float reduction: float64 quality on the float32 pipes; writes the
-    // float32 reflectors directly
-    const int cs = tridiag64_cluster_size((const void*)tridiag_df_kernel<TRIDIAG_DF_UNROLL>);
-    const size_t smem = std::max<size_t>(32 * (size_t)n, TRIDIAG64_SMEM);
-    ProfScope ps(st, K_TRIDIAG, 1, 16.0 / 3.0 * (double)n * n * n * batch);
-    ce = launch_cluster_t(tridiag_df_kernel<TRIDIAG_DF_UNROLL>, cs, batch, TRIDIAG_DF_THREADS, smem, st,
-                          reinterpret_cast<float4*>(Hd), (long long)nn, n, dd, ed, n, reinterpret_cast<float4*>(Pd),
-                          reinterpret_cast<float2*>(Kp), Vhf, (long long)nn);
-  }
-  if (ce != cudaSuccess) return ce;
   {
     ProfScope ps(st, K_ELEMWISE);
     tridiag_phases_kernel<double><<<batch, 256, 0, st>>>(ed, n, n, eabs, phid);
@@ -1136,7 +855,6 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
   {
     ProfScope ps(st, K_ELEMWISE);
-    if (in_smem) cx_d2f_kernel<<<1024, 256, 0, st>>>(Vhd, Vhf, (long long)(nn * B));
     cx_d2f_kernel<<<64, 256, 0, st>>>(phid, phif, (long long)(n * B));
     re_d2f_kernel<<<1024, 256, 0, st>>>(Z, Zf, (long long)(nr * B));
   }

@@ -1,0 +1,597 @@
+// Householder reduction of complex Hermitian matrices to real tridiagonal form
+// in double-float arithmetic (complex64 states' eigenproblems): float64
+// quality on the float32 pipes.
+//
+// tridiag_df_kernel   the matrix in L2, lower triangle only: the first jend
+//                     columns of matrices that do not fit in shared memory;
+// tridiag_dfs_kernel  the (trailing) matrix in the shared memory of one
+//                     cluster: the whole reduction of the sizes that fit and
+//                     the rest of larger ones.
+#include <map>
+#include <mutex>
+#include <tuple>
+
+#include "df.cuh"
+#include "kernels.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace nne {
+
+__global__ void cx_f2df_kernel(const cx<float>* X, long long sX, int n, float4* Y, long long sY) {
+  const long long count = (long long)n * n;
+  const int z = blockIdx.y;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
+    const cx<float> v = X[z * sX + i];
+    Y[z * sY + i] = make_float4(v.re, 0.f, v.im, 0.f);
+  }
+}
+
+// Every O(m) step of a column is double-float as well (norms, the reflector,
+// K, w), so the float64 pipe only sees one thread's pivot per column; the
+// reflectors go out rounded to float32 for the float32 back-transformation,
+// d and e in float64.
+template <int U>
+__global__ void __launch_bounds__(512) tridiag_df_kernel(float4* Hb, long long sH, int n, double* db, cx<double>* eb,
+                                                          int ldde, float4* Pb, float2* Kb, cx<float>* Vhb,
+                                                          long long sVh, int jend) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CS = (int)cluster.num_blocks();
+  const int rank = (int)cluster.block_rank();
+  const int z = blockIdx.y;
+  float4* H = Hb + z * sH;
+  double* d = db + (long long)z * ldde;
+  cx<double>* e = eb + (long long)z * ldde;
+  float4* P = Pb + (long long)z * ldde;
+  float2* Kp = Kb + z * 32;
+  extern __shared__ __align__(16) unsigned char df_smem[];
+  float4* vdf = reinterpret_cast<float4*>(df_smem);   // n: the Householder vector
+  float4* wdf = vdf + n;                              // n: w = 2p - 2Kv
+  __shared__ float red[64];
+  __shared__ float4 alpha_s;
+  __shared__ float2 inv_s;
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
+  const int gw = rank * nw + warp, GW = CS * nw;
+
+  for (int j = 0; j < jend; ++j) {
+    const int m = n - j - 1;
+    // column j below the diagonal, and its squared norm
+    float nh = 0.f, nl = 0.f;
+    {
+      const float4* colj = H + (long long)(j + 1) * n + j;
+      for (int t = tid; t < m; t += nth) {
+        const float4 a = colj[(long long)t * n];
+        vdf[t] = a;
+        df_mac(nh, nl, a.x, a.y, a.x, a.y);
+        df_mac(nh, nl, a.z, a.w, a.z, a.w);
+      }
+    }
+    const float2 xn2f = df_block_sum(nh, nl, red);
+    if (tid == 0) {
+      // pivot in float64 on one thread: alpha = -e^{i arg x0} ||x||, un = ||x - alpha e0||
+      const float4 x0 = vdf[0];
+      const cx<double> x0d = mk<double>(df_to_d(x0.x, x0.y), df_to_d(x0.z, x0.w));
+      double pr, pi, ax0;
+      unit_phase_of(x0d, &pr, &pi, &ax0);
+      const double xn2 = df_to_d(xn2f.x, xn2f.y), xn = sqrt(xn2);
+      cx<double> alpha = mk<double>(0, 0);
+      double un = 0;
+      if (xn > 0) {
+        alpha = mk<double>(-xn * pr, -xn * pi);
+        un = sqrt(2.0 * xn2 + 2.0 * xn * ax0);
+      }
+      const double inv = un > 0 ? 1.0 / un : 0.0;
+      alpha_s = df_from_cd(alpha);
+      const float ih = (float)inv;
+      inv_s = make_float2(ih, (float)(inv - (double)ih));
+      if (rank == 0) {
+        const float4 hjj = H[(long long)j * n + j];
+        d[j] = df_to_d(hjj.x, hjj.y);
+        e[j] = alpha;
+      }
+    }
+    __syncthreads();
+    {
+      const float4 al = alpha_s;
+      const float2 iv = inv_s;
+      cx<float>* rj = Vhb + z * sVh + (long long)j * n + (j + 1);
+      for (int t = tid; t < m; t += nth) {
+        float4 u = vdf[t];
+        if (t == 0) {
+          df_add(u.x, u.y, -al.x, -al.y);
+          df_add(u.z, u.w, -al.z, -al.w);
+        }
+        const float2 vr = df_mul(u.x, u.y, iv.x, iv.y), vi = df_mul(u.z, u.w, iv.x, iv.y);
+        vdf[t] = make_float4(vr.x, vr.y, vi.x, vi.y);
+        if (rank == 0) rj[t] = mk<float>(vr.x, -vi.x);   // reflector j, conjugated, for the back-transform
+      }
+    }
+    __syncthreads();
+    // p = A v on own rows (lower part of row t, then its upper part read down column t); K = v^H p
+    float kh = 0.f, kl = 0.f;
+    for (int t = gw; t < m; t += GW) {
+      const float4* row = H + (long long)(j + 1 + t) * n + (j + 1);
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), acc2 = acc;
+      int k = lane;
+      for (; k + 32 * (U - 1) <= t; k += 32 * U) {
+        float4 a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] = row[k + 32 * u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) df_cmac<false>((u & 1) ? acc2 : acc, a[u], vdf[k + 32 * u]);
+      }
+      for (; k <= t; k += 32) df_cmac<false>(acc, row[k], vdf[k]);
+      const float4* colt = H + (long long)(j + 1) * n + (j + 1 + t);
+      k = t + 1 + lane;
+      for (; k + 32 * (U - 1) < m; k += 32 * U) {
+        float4 a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] = colt[(long long)(k + 32 * u) * n];
+#pragma unroll
+        for (int u = 0; u < U; ++u) df_cmac<true>((u & 1) ? acc2 : acc, a[u], vdf[k + 32 * u]);
+      }
+      for (; k < m; k += 32) df_cmac<true>(acc, colt[(long long)k * n], vdf[k]);
+      df_add(acc.x, acc.y, acc2.x, acc2.y);
+      df_add(acc.z, acc.w, acc2.z, acc2.w);
+      acc = df_warp_sum(acc);
+      if (lane == 0) {
+        P[t] = acc;
+        const float4 vt = vdf[t];
+        df_mac(kh, kl, vt.x, vt.y, acc.x, acc.y);
+        df_mac(kh, kl, vt.z, vt.w, acc.z, acc.w);
+      }
+    }
+    {
+      const float2 kp = df_block_sum(kh, kl, red);
+      if (tid == 0) Kp[rank] = kp;
+    }
+    __threadfence();
+    cluster.sync();
+    float Kh = 0.f, Kl = 0.f;
+    for (int c = 0; c < CS; ++c) df_add(Kh, Kl, Kp[c].x, Kp[c].y);
+    // w = 2p - 2 K v  (2K exact in double-float)
+    const float K2h = 2.f * Kh, K2l = 2.f * Kl;
+    for (int t = tid; t < m; t += nth) {
+      const float4 p = P[t], vt = vdf[t];
+      float rh = 2.f * p.x, rl = 2.f * p.y, ih = 2.f * p.z, il = 2.f * p.w;
+      df_mac(rh, rl, -K2h, -K2l, vt.x, vt.y);
+      df_mac(ih, il, -K2h, -K2l, vt.z, vt.w);
+      df_norm(rh, rl);
+      df_norm(ih, il);
+      wdf[t] = make_float4(rh, rl, ih, il);
+    }
+    __syncthreads();
+    // A <- A - v w^H - w v^H on the lower triangle of own rows (U entries in flight per lane)
+    for (int t = gw; t < m; t += GW) {
+      float4* row = H + (long long)(j + 1 + t) * n + (j + 1);
+      const float4 vt = vdf[t], wt = wdf[t];
+      for (int k0 = lane; k0 <= t; k0 += 32 * U) {
+        float4 a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (k0 + 32 * u <= t) a[u] = row[k0 + 32 * u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int k = k0 + 32 * u;
+          if (k > t) break;
+          const float4 wk = wdf[k], vk = vdf[k];
+          float4 b = a[u];
+          // re: - (vt.re wk.re + vt.im wk.im + wt.re vk.re + wt.im vk.im)
+          df_mac(b.x, b.y, -vt.x, -vt.y, wk.x, wk.y);
+          df_mac(b.x, b.y, -vt.z, -vt.w, wk.z, wk.w);
+          df_mac(b.x, b.y, -wt.x, -wt.y, vk.x, vk.y);
+          df_mac(b.x, b.y, -wt.z, -wt.w, vk.z, vk.w);
+          // im: - (vt.im wk.re - vt.re wk.im + wt.im vk.re - wt.re vk.im)
+          df_mac(b.z, b.w, -vt.z, -vt.w, wk.x, wk.y);
+          df_mac(b.z, b.w, vt.x, vt.y, wk.z, wk.w);
+          df_mac(b.z, b.w, -wt.z, -wt.w, vk.x, vk.y);
+          df_mac(b.z, b.w, wt.x, wt.y, vk.z, vk.w);
+          df_norm(b.x, b.y);
+          df_norm(b.z, b.w);
+          row[k] = b;
+        }
+      }
+    }
+    __threadfence();
+    cluster.sync();
+  }
+}
+
+// ---------------------------------------------------------------- shared-memory resident
+// One cluster per matrix; the rows, both triangles, are dealt cyclically to
+// its CTAs and stay in shared memory.  Thread t of every CTA owns entry t of
+// the current column, so n <= NT.
+//
+// What bounds it: per column a chain of one exchange and two block sums, and
+// 3 complex multiply-adds per entry of the trailing matrix on the float32
+// pipes.  Hence
+//   * one cluster barrier per column: the CTAs push their part of p = A v to
+//     all others before it; after it every CTA forms K = v^H p, w, the next
+//     column (the stored row j+1 of its owner, read through distributed shared
+//     memory, minus its part of the rank-2 update) and the next reflector
+//     itself, with the same operations in the same order, so no second
+//     exchange is needed;
+//   * one pass over the matrix per column: the rank-2 update of column j and
+//     the product with v_{j+1} read and write each entry once;
+//   * no float64: GB300 has two float64 lanes per SM.
+// The matrix is scaled by a power of two to a largest diagonal entry in
+// [1, 2); columns below norm 2^-50 then count as null (their squares would
+// leave float32's range, and an inaccurate norm makes a reflector that is not
+// unitary), a backward error below eps_64 ||H||.
+//
+// Source: complex64 (SRC_DF false) or the double-float trailing block of
+// tridiag_df_kernel (true), both n0 x n0 with the lower triangle valid; the
+// block starts at row and column `off` and has n = n0 - off rows.
+template <int NT, bool SRC_DF>
+__global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict__ Hsrc, long long sH, int n0, int off,
+                                                         double* db, cx<double>* eb, int ldde, cx<float>* Vhb,
+                                                         long long sVh, int maxloc) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CS = (int)cluster.num_blocks();
+  const int rank = (int)cluster.block_rank();
+  const int z = blockIdx.y, n = n0 - off;
+  double* d = db + (long long)z * ldde + off;
+  cx<double>* e = eb + (long long)z * ldde + off;
+  cx<float>* Vh = Vhb + z * sVh + (long long)off * n0 + off;
+  extern __shared__ __align__(16) unsigned char dfs_smem[];
+  float4* Hl = reinterpret_cast<float4*>(dfs_smem);     // [maxloc][n] own rows
+  float4* vb = Hl + (long long)maxloc * n;              // [2][n] reflectors of this and the last column
+  float4* wb = vb + 2 * n;                              // n: w of the last column
+  float4* pb = wb + n;                                  // [2][n] p of all rows, pushed by their owners
+  float2* kbuf = reinterpret_cast<float2*>(pb + 2 * n); // [2][CS][NW] shares of K, pushed by their warps
+  constexpr int NW = NT / 32;
+  __shared__ float2 redN[NW];
+  __shared__ float redM[NW];
+  __shared__ float4 x0_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nloc = n > rank ? (n - rank + CS - 1) / CS : 0;
+  auto source = [&](int i, int c) {   // entry (i, c), c <= i
+    if (SRC_DF)
+      return reinterpret_cast<const float4*>(Hsrc)[z * sH + (long long)(off + i) * n0 + off + c];
+    const cx<float> a = reinterpret_cast<const cx<float>*>(Hsrc)[z * sH + (long long)(off + i) * n0 + off + c];
+    return make_float4(a.re, 0.f, a.im, 0.f);
+  };
+  // power-of-two scale from the largest diagonal entry
+  float mx = tid < n ? fabsf(source(tid, tid).x) : 0.f;
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) redM[warp] = mx;
+  __syncthreads();
+  for (int w2 = 0; w2 < NW; ++w2) mx = fmaxf(mx, redM[w2]);
+  int ex = 0;
+  if (mx > 0.f && mx < INFINITY) ex = min(max(ilogbf(mx), -120), 120);
+  const float sc = ldexpf(1.f, -ex);
+  const double back = ldexp(1.0, ex);
+  for (long long q = tid; q < (long long)nloc * n; q += NT) {
+    const int li = (int)(q / n), c = (int)(q % n), i = rank + li * CS;
+    float4 a;
+    if (c <= i) {
+      a = source(i, c);
+    } else {
+      a = source(c, i);
+      a.z = -a.z;
+      a.w = -a.w;
+    }
+    if (c == i) a.z = a.w = 0.f;
+    Hl[q] = make_float4(a.x * sc, a.y * sc, a.z * sc, a.w * sc);
+  }
+  // sum over the block, in the same order in every CTA (s: NW shared partials)
+  auto block_df = [&](float hi, float lo, float2* s) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
+      df_add(hi, lo, bh, bl);
+    }
+    if (lane == 0) s[warp] = make_float2(hi, lo);
+    __syncthreads();
+    float2 t = s[lane % NW];
+    for (int o = NW / 2; o > 0; o >>= 1) {
+      const float bh = __shfl_xor_sync(0xffffffffu, t.x, o), bl = __shfl_xor_sync(0xffffffffu, t.y, o);
+      df_add(t.x, t.y, bh, bl);
+    }
+    t.x = __shfl_sync(0xffffffffu, t.x, 0);
+    t.y = __shfl_sync(0xffffffffu, t.y, 0);
+    df_norm(t.x, t.y);
+    return t;
+  };
+  // b -= v conj(wk) + w conj(vk)
+  auto rank2 = [](float4& b, float4 vt, float4 wt, float4 vk, float4 wk) {
+    df_mac(b.x, b.y, -vt.x, -vt.y, wk.x, wk.y);
+    df_mac(b.z, b.w, -vt.z, -vt.w, wk.x, wk.y);
+    df_mac(b.x, b.y, -vt.z, -vt.w, wk.z, wk.w);
+    df_mac(b.z, b.w, vt.x, vt.y, wk.z, wk.w);
+    df_mac(b.x, b.y, -wt.x, -wt.y, vk.x, vk.y);
+    df_mac(b.z, b.w, -wt.z, -wt.w, vk.x, vk.y);
+    df_mac(b.x, b.y, -wt.z, -wt.w, vk.z, vk.w);
+    df_mac(b.z, b.w, wt.x, wt.y, vk.z, vk.w);
+    df_norm(b.x, b.y);
+    df_norm(b.z, b.w);
+  };
+  // reflector r (column r below the diagonal: entry t of it is x, held by thread t < m) -> vout, Vh row r, e[r]
+  auto reflector = [&](int r, int m, float4 x, float4* vout) {
+    float nh = 0.f, nl = 0.f;
+    if (tid < m) {
+      df_mac(nh, nl, x.x, x.y, x.x, x.y);
+      df_mac(nh, nl, x.z, x.w, x.z, x.w);
+    }
+    if (tid == 0) x0_s = x;
+    const float2 xn2 = block_df(nh, nl, redN);
+    const float4 x0 = x0_s;
+    float2 ar = make_float2(0.f, 0.f), ai = ar, inv = ar;   // alpha, 1 / ||x - alpha e_0||
+    if (xn2.x >= 0x1p-100f) {
+      // alpha = -e^{i arg x_0} ||x||, the phase from x_0 scaled away from float32's denormal squares
+      const bool small = fmaxf(fabsf(x0.x), fabsf(x0.z)) < 0x1p-30f;
+      const float up = small ? 0x1p60f : 1.f, dn = small ? 0x1p-60f : 1.f;
+      const float2 a = make_float2(x0.x * up, x0.y * up), b = make_float2(x0.z * up, x0.w * up);
+      const float2 q2 = df_add2(df_mul2(a, a), df_mul2(b, b));
+      const float2 xn = df_mul2(xn2, df_rsqrt(xn2));
+      float2 pr = make_float2(1.f, 0.f), pi = make_float2(0.f, 0.f), ax0 = pi;
+      if (q2.x > 0x1p-100f) {
+        const float2 qi = df_rsqrt(q2);
+        pr = df_mul2(a, qi);
+        pi = df_mul2(b, qi);
+        ax0 = df_mul2(q2, qi);
+        ax0 = make_float2(ax0.x * dn, ax0.y * dn);
+      }
+      ar = df_mul(-pr.x, -pr.y, xn.x, xn.y);
+      ai = df_mul(-pi.x, -pi.y, xn.x, xn.y);
+      const float2 u2 = df_add2(xn2, df_mul2(xn, ax0));
+      inv = df_rsqrt(make_float2(2.f * u2.x, 2.f * u2.y));
+    }
+    if (tid < m) {
+      if (tid == 0) {
+        df_add(x.x, x.y, -ar.x, -ar.y);
+        df_add(x.z, x.w, -ai.x, -ai.y);
+      }
+      const float2 vr = df_mul(x.x, x.y, inv.x, inv.y), vi = df_mul(x.z, x.w, inv.x, inv.y);
+      vout[tid] = make_float4(vr.x, vr.y, vi.x, vi.y);
+      if (rank == r % CS) Vh[(long long)r * n0 + r + 1 + tid] = mk<float>(vr.x, -vi.x);
+    }
+    if (rank == 0 && tid == 0) e[r] = mk<double>(df_to_d(ar.x, ar.y) * back, df_to_d(ai.x, ai.y) * back);
+  };
+  {
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < n - 1) {
+      const float4 a = source(tid + 1, 0);
+      x = make_float4(a.x * sc, a.y * sc, a.z * sc, a.w * sc);
+    }
+    reflector(0, n - 1, x, vb);
+    if (rank == 0 && tid == 0) {
+      const float4 a = source(0, 0);
+      d[0] = df_to_d(a.x, a.y);
+    }
+  }
+  cluster.sync();   // every CTA of the cluster runs before anyone writes into its shared memory
+  for (int j = 0; j + 2 < n; ++j) {
+    const int m = n - j - 1;
+    const float4* v = vb + (j & 1) * n;              // v_j: entry t is row j + 1 + t
+    const float4* vo = vb + ((j & 1) ^ 1) * n + 1;   // v_{j-1} at row j + 1
+    const float4* wo = wb + 1;                       // w_{j-1} at row j + 1
+    float4* p = pb + (j & 1) * n;
+    // own rows i > j, two per warp at a time: A <- A - v_{j-1} w^H - w v_{j-1}^H
+    // on columns > j, p_i = row . v_j, and this warp's share of K = v_j^H p
+    const int l0 = j + 1 > rank ? (j + 1 - rank + CS - 1) / CS : 0;
+    float kh = 0.f, kl = 0.f;
+    for (int li = l0 + warp; li < nloc; li += 2 * NW) {
+      const bool two = li + NW < nloc;
+      const int t = rank + li * CS - j - 1, t2 = t + NW * CS;
+      float4* row = Hl + (long long)li * n + (j + 1);
+      float4* row2 = row + (long long)NW * n;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), acc2 = acc;
+      if (j == 0) {
+        for (int k = lane; k < m; k += 32) {
+          const float4 vn = v[k];
+          df_cmac<false>(acc, row[k], vn);
+          if (two) df_cmac<false>(acc2, row2[k], vn);
+        }
+      } else if (two) {
+        const float4 vt = vo[t], wt = wo[t], vt2 = vo[t2], wt2 = wo[t2];
+        for (int k = lane; k < m; k += 32) {
+          const float4 wk = wo[k], vk = vo[k], vn = v[k];
+          float4 b = row[k], b2 = row2[k];
+          rank2(b, vt, wt, vk, wk);
+          rank2(b2, vt2, wt2, vk, wk);
+          row[k] = b;
+          row2[k] = b2;
+          df_cmac<false>(acc, b, vn);
+          df_cmac<false>(acc2, b2, vn);
+        }
+      } else {
+        const float4 vt = vo[t], wt = wo[t];
+        for (int k = lane; k < m; k += 32) {
+          float4 b = row[k];
+          rank2(b, vt, wt, vo[k], wo[k]);
+          row[k] = b;
+          df_cmac<false>(acc, b, v[k]);
+        }
+      }
+      // both rows' sums in five steps: lanes 0-15 end with the first row's, 16-31 with the second's
+      const bool up = lane & 16;
+      {
+        const float4 give = up ? acc : acc2;
+        acc = up ? acc2 : acc;
+        const float bh = __shfl_xor_sync(0xffffffffu, give.x, 16), bl = __shfl_xor_sync(0xffffffffu, give.y, 16);
+        const float ch = __shfl_xor_sync(0xffffffffu, give.z, 16), cl = __shfl_xor_sync(0xffffffffu, give.w, 16);
+        df_add(acc.x, acc.y, bh, bl);
+        df_add(acc.z, acc.w, ch, cl);
+      }
+      for (int o = 8; o > 0; o >>= 1) {
+        const float bh = __shfl_xor_sync(0xffffffffu, acc.x, o), bl = __shfl_xor_sync(0xffffffffu, acc.y, o);
+        const float ch = __shfl_xor_sync(0xffffffffu, acc.z, o), cl = __shfl_xor_sync(0xffffffffu, acc.w, o);
+        df_add(acc.x, acc.y, bh, bl);
+        df_add(acc.z, acc.w, ch, cl);
+      }
+      // every CTA gets the same bits (the lanes' lo parts may differ by rounding)
+      const int src = lane & 16;
+      acc.x = __shfl_sync(0xffffffffu, acc.x, src);
+      acc.y = __shfl_sync(0xffffffffu, acc.y, src);
+      acc.z = __shfl_sync(0xffffffffu, acc.z, src);
+      acc.w = __shfl_sync(0xffffffffu, acc.w, src);
+      const int tr = up ? t2 : t;
+      if (!up || two) {
+        const float4 vt = v[tr];
+        df_mac(kh, kl, vt.x, vt.y, acc.x, acc.y);
+        df_mac(kh, kl, vt.z, vt.w, acc.z, acc.w);
+        if ((lane & 15) < CS) *cluster.map_shared_rank(p + tr, lane & 15) = acc;
+      }
+    }
+    {
+      float2* kb = kbuf + (j & 1) * CS * NW;
+      const float bh = __shfl_xor_sync(0xffffffffu, kh, 16), bl = __shfl_xor_sync(0xffffffffu, kl, 16);
+      df_add(kh, kl, bh, bl);
+      kh = __shfl_sync(0xffffffffu, kh, 0);
+      kl = __shfl_sync(0xffffffffu, kl, 0);
+      if (lane < CS) *cluster.map_shared_rank(kb + rank * NW + warp, lane) = make_float2(kh, kl);
+    }
+    cluster.sync();
+    // row j + 1 (its owner's last word on it), K = v^H p
+    const int own = (j + 1) % CS;
+    const float4* rj1 = cluster.map_shared_rank(Hl + (long long)((j + 1) / CS) * n + (j + 1), own);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid + 1 < m) {
+      a = rj1[tid + 1];
+      a.z = -a.z;   // entry (j + 2 + tid, j + 1) by symmetry
+      a.w = -a.w;
+    }
+    float2 K = make_float2(0.f, 0.f);
+    {
+      const float2* kb = kbuf + (j & 1) * CS * NW;
+      for (int q = lane; q < CS * NW; q += 32) df_add(K.x, K.y, kb[q].x, kb[q].y);
+      for (int o = 16; o > 0; o >>= 1) {
+        const float bh = __shfl_xor_sync(0xffffffffu, K.x, o), bl = __shfl_xor_sync(0xffffffffu, K.y, o);
+        df_add(K.x, K.y, bh, bl);
+      }
+      K.x = __shfl_sync(0xffffffffu, K.x, 0);
+      K.y = __shfl_sync(0xffffffffu, K.y, 0);
+    }
+    const float k2h = -2.f * K.x, k2l = -2.f * K.y;
+    auto wof = [&](float4 vt, float4 pt) {   // w = 2 p - 2 K v
+      float4 w = make_float4(2.f * pt.x, 2.f * pt.y, 2.f * pt.z, 2.f * pt.w);
+      df_mac(w.x, w.y, k2h, k2l, vt.x, vt.y);
+      df_mac(w.z, w.w, k2h, k2l, vt.z, vt.w);
+      df_norm(w.x, w.y);
+      df_norm(w.z, w.w);
+      return w;
+    };
+    const float4 v0 = v[0], w0 = wof(v0, p[0]);
+    if (tid + 1 < m) {
+      const float4 vt = v[tid + 1], wt = wof(vt, p[tid + 1]);
+      wb[tid + 1] = wt;
+      rank2(a, vt, wt, v0, w0);
+    }
+    if (rank == own && tid == 0) {
+      // d[j + 1] = A[j+1][j+1] - 2 Re(v_0 conj(w_0))
+      const float4 g = Hl[(long long)((j + 1) / CS) * n + (j + 1)];
+      float gh = g.x, gl = g.y;
+      df_mac(gh, gl, -2.f * v0.x, -2.f * v0.y, w0.x, w0.y);
+      df_mac(gh, gl, -2.f * v0.z, -2.f * v0.w, w0.z, w0.w);
+      d[j + 1] = df_to_d(gh, gl) * back;
+    }
+    if (j + 3 < n) {
+      reflector(j + 1, m - 1, a, vb + ((j & 1) ^ 1) * n);
+    } else if (tid == 0) {
+      // the last 2 x 2 block: subdiagonal, and the corner by its owner
+      if (rank == 0) e[n - 2] = mk<double>(df_to_d(a.x, a.y) * back, df_to_d(a.z, a.w) * back);
+      if (rank == (n - 1) % CS) {
+        const float4 g = Hl[(long long)((n - 1) / CS) * n + (n - 1)], v1 = v[1], w1 = wof(v1, p[1]);
+        float gh = g.x, gl = g.y;
+        df_mac(gh, gl, -2.f * v1.x, -2.f * v1.y, w1.x, w1.y);
+        df_mac(gh, gl, -2.f * v1.z, -2.f * v1.w, w1.z, w1.w);
+        d[n - 1] = df_to_d(gh, gl) * back;
+      }
+    }
+    __syncthreads();
+  }
+  cluster.sync();   // rows of this CTA may still be read by others
+}
+
+// ---------------------------------------------------------------- launchers
+namespace {
+
+// double-float reduction launch: 256 threads, TRIDIAG_DF_UNROLL loads in flight per lane in the
+// product A v and the rank-2 update (its loads wait on L2: ncu shows long-scoreboard stalls and
+// 1.6 % L2 throughput with one load per lane)
+constexpr int TRIDIAG_DF_THREADS = 256;
+constexpr int TRIDIAG_DF_UNROLL = 4;
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_df(void (*kernel)(KArgs...), int cs, int batch, int threads, size_t smem, cudaStream_t st, Args... args) {
+  cudaError_t e = ensure_kernel_smem((const void*)kernel, smem, cs > 8);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cs, batch, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+size_t dfs_bytes(int n, int cs) {
+  return 16 * ((size_t)((n + cs - 1) / cs) * n + 5 * (size_t)n) + 2 * sizeof(float2) * cs * (512 / 32);
+}
+constexpr size_t DFS_SMEM = 226 * 1024;   // dynamic shared memory per CTA (227 KB less the static part)
+
+template <int NT, bool SRC_DF>
+cudaError_t dfs_nt(cudaStream_t st, const void* H, long long sH, int n0, int off, double* d, cx<double>* e, int ldde,
+                   cx<float>* Vh, long long sVh, int batch, int cs) {
+  const int n = n0 - off, maxloc = (n + cs - 1) / cs;
+  return launch_df(tridiag_dfs_kernel<NT, SRC_DF>, cs, batch, NT, dfs_bytes(n, cs), st, H, sH, n0, off, d, e, ldde, Vh,
+                   sVh, maxloc);
+}
+
+}  // namespace
+
+// CTAs per matrix: more of them shorten a column's pass over the matrix until
+// the exchange (about 2.5 us per column) dominates.  Measured on batches of 5 (us
+// per launch on 4 / 8 / 12 CTAs; the float64 kernel in brackets): n = 180: 959 /
+// 740 / 670 (1866), 256: - / 1373 / 1239 (4175), 384: - / - / 2764.  Twelve is the
+// most that lets eight clusters run at once on the GPU's GPCs (sixteen: 2572 for
+// five matrices of 384, two waves for eight), and 384 rows of 12 CTAs fill their
+// shared memory.
+constexpr int DFS_CS = 12, DFS_MAX = 384;
+
+static cudaError_t tridiag_dfs(cudaStream_t st, bool src_df, const void* H, long long sH, int n0, int off, double* d,
+                               cx<double>* e, int ldde, cx<float>* Vh, long long sVh, int batch) {
+  const int n = n0 - off;
+  if (n < 3 || n > DFS_MAX || dfs_bytes(n, DFS_CS) > DFS_SMEM) return cudaErrorInvalidValue;
+  if (src_df) return dfs_nt<512, true>(st, H, sH, n0, off, d, e, ldde, Vh, sVh, batch, DFS_CS);
+  if (n <= 256) return dfs_nt<256, false>(st, H, sH, n0, off, d, e, ldde, Vh, sVh, batch, DFS_CS);
+  return dfs_nt<512, false>(st, H, sH, n0, off, d, e, ldde, Vh, sVh, batch, DFS_CS);
+}
+
+// d, e (T[k+1][k] = e[k]) and the float32 reflectors (row j of Vh, conjugated,
+// columns j + 1 on; the rest of Vh untouched) of the Hermitian H[z] (n x n,
+// lower triangle read).  Up to DFS_MAX rows the whole reduction runs in shared
+// memory; above, the L2-resident kernel takes the columns until the trailing
+// block fits.  work: batch x n x n float4 (n > DFS_MAX only), P: batch x n
+// float4, Kp: batch x 32 float2.
+cudaError_t tridiag_df(cudaStream_t st, const cx<float>* H, long long sH, int n, float4* work, float4* P, float2* Kp,
+                       double* d, cx<double>* e, cx<float>* Vh, int batch) {
+  const long long nn = (long long)n * n;
+  cudaError_t ce;
+  if (n <= DFS_MAX) {
+    ProfScope ps(st, K_TRIDIAG, 1, 16.0 / 3.0 * (double)n * n * n * batch);
+    return tridiag_dfs(st, false, H, sH, n, 0, d, e, n, Vh, nn, batch);
+  }
+  {
+    ProfScope ps(st, K_ELEMWISE);
+    const dim3 grid((unsigned)std::min<long long>((nn + 255) / 256, 1024), batch);
+    cx_f2df_kernel<<<grid, 256, 0, st>>>(H, sH, n, work, nn);
+    if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  }
+  ProfScope ps(st, K_TRIDIAG, 2, 16.0 / 3.0 * (double)n * n * n * batch);
+  const int cs = tridiag64_cluster_size((const void*)tridiag_df_kernel<TRIDIAG_DF_UNROLL>);
+  const size_t smem = std::max<size_t>(32 * (size_t)n, TRIDIAG64_SMEM);
+  const int jend = n - DFS_MAX;
+  if ((ce = launch_df(tridiag_df_kernel<TRIDIAG_DF_UNROLL>, cs, batch, TRIDIAG_DF_THREADS, smem, st, work, nn, n, d, e,
+                      n, P, Kp, Vh, nn, jend)) != cudaSuccess)
+    return ce;
+  return tridiag_dfs(st, true, work, nn, n, jend, d, e, n, Vh, nn, batch);
+}
+
+}  // namespace nne

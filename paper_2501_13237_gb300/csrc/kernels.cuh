@@ -106,6 +106,14 @@ template <typename R>
 cudaError_t gram_entropy(cudaStream_t st, cx<R>* H, long long sH, int n, void* cx_ws, void* re_ws, int batch,
                          double* S, long long sS);
 
+// ---- k_tridiag_df.cu (double-float reduction of complex64 eigenproblems)
+cudaError_t tridiag_df(cudaStream_t st, const cx<float>* H, long long sH, int n, float4* work, float4* P, float2* Kp,
+                       double* d, cx<double>* e, cx<float>* Vh, int batch);
+// Cluster size of the L2-resident float64-quality reductions (k_linalg.cu) and the
+// shared-memory request that gives each of their CTAs an SM of its own.
+int tridiag64_cluster_size(const void* kernel);
+constexpr size_t TRIDIAG64_SMEM = 120 * 1024;
+
 template <typename R>
 int smem_cluster_size(int n);
 template <typename R>
