@@ -8,12 +8,14 @@ namespace nne {
 
 // C[z] = alpha * op(A[z]) * op(B[z]) + beta * C[z], row-major, M x N x K.
 // op N: element (i, k) of A is A[i * lda + k]; op C: conj(A[k * lda + i]).
-template <typename R, int OPA, int OPB>
+// BM x BM outputs per CTA of 256 threads, (BM / 16)^2 per thread.  Every output is
+// the same sum in the same order whatever BM is.
+template <typename R, int OPA, int OPB, int BM>
 __global__ void __launch_bounds__(256) cgemm_kernel(int M, int N, int K, cx<R> alpha,
                                                      const cx<R>* __restrict__ A, long long sA, int lda,
                                                      const cx<R>* __restrict__ B, long long sB, int ldb,
                                                      cx<R> beta, cx<R>* __restrict__ C, long long sC, int ldc) {
-  constexpr int BM = 64, BN = 64, BK = 16;
+  constexpr int BN = BM, BK = 16, TM = BM / 16;
   __shared__ cx<R> As[BK][BM];
   __shared__ cx<R> Bs[BK][BN];
   const int z = blockIdx.z;
@@ -22,11 +24,11 @@ __global__ void __launch_bounds__(256) cgemm_kernel(int M, int N, int K, cx<R> a
   C += z * sC;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int row0 = blockIdx.y * BM, col0 = blockIdx.x * BN;
-  cx<R> acc[4][4];
+  cx<R> acc[TM][TM];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mk<R>(0, 0);
+    for (int j = 0; j < TM; ++j) acc[i][j] = mk<R>(0, 0);
   for (int k0 = 0; k0 < K; k0 += BK) {
     for (int e = tid; e < BM * BK; e += 256) {
       int i, k;
@@ -47,25 +49,25 @@ __global__ void __launch_bounds__(256) cgemm_kernel(int M, int N, int K, cx<R> a
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < BK; ++k) {
-      cx<R> a[4], b[4];
+      cx<R> a[TM], b[TM];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
+      for (int i = 0; i < TM; ++i) a[i] = As[k][ty + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx + 16 * j];
+      for (int j = 0; j < TM; ++j) b[j] = Bs[k][tx + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) fma_(acc[i][j], a[i], b[j]);
+        for (int j = 0; j < TM; ++j) fma_(acc[i][j], a[i], b[j]);
     }
     __syncthreads();
   }
   const bool use_beta = (beta.re != R(0) || beta.im != R(0));
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < TM; ++i) {
     const int gi = row0 + ty + 16 * i;
     if (gi >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < TM; ++j) {
       const int gj = col0 + tx + 16 * j;
       if (gj >= N) continue;
       cx<R> v = alpha * acc[i][j];
@@ -74,6 +76,20 @@ __global__ void __launch_bounds__(256) cgemm_kernel(int M, int N, int K, cx<R> a
       *c = v;
     }
   }
+}
+
+// Tile of the SIMT kernel: the largest that still gives every SM a CTA, else
+// the smallest.  The matrices that come here are small (complex64: an edge
+// below 64; complex128: all), and with 64 x 64 tiles a 256 x 256 product of 4
+// instances ran on 64 of 152 SMs: float64 runs at two lanes per SM, so idle SMs
+// cost their full share.  Float64 tiles also want several CTAs per SM, to even
+// out the last wave.  Circuit of 8 qubits in complex128, bonds up to 256: the
+// GEMM class of a run 99.6 -> 12.5 ms.
+template <typename R>
+static int simt_tile(int M, int N, int batch) {
+  auto tiles = [&](int b) { return (long long)((M + b - 1) / b) * ((N + b - 1) / b) * batch; };
+  const long long want = std::is_same<R, double>::value ? 4 * 152 : 152;
+  return tiles(64) >= want ? 64 : (tiles(32) >= want ? 32 : 16);
 }
 
 template <typename R>
@@ -91,15 +107,22 @@ cudaError_t cgemm(cudaStream_t st, int opA, int opB, int M, int N, int K, cx<R> 
                     reinterpret_cast<const cx<float>*>(A), sA, lda, reinterpret_cast<const cx<float>*>(B), sB, ldb,
                     *reinterpret_cast<const cx<float>*>(&beta), reinterpret_cast<cx<float>*>(C), sC, ldc, batch);
   ProfScope ps(st, K_GEMM, 1, 8.0 * M * N * (double)K * batch);
-  dim3 grid((N + 63) / 64, (M + 63) / 64, batch);
-  if (opA == OP_N && opB == OP_N)
-    cgemm_kernel<R, OP_N, OP_N><<<grid, 256, 0, st>>>(M, N, K, alpha, A, sA, lda, B, sB, ldb, beta, C, sC, ldc);
-  else if (opA == OP_N && opB == OP_C)
-    cgemm_kernel<R, OP_N, OP_C><<<grid, 256, 0, st>>>(M, N, K, alpha, A, sA, lda, B, sB, ldb, beta, C, sC, ldc);
-  else if (opA == OP_C && opB == OP_N)
-    cgemm_kernel<R, OP_C, OP_N><<<grid, 256, 0, st>>>(M, N, K, alpha, A, sA, lda, B, sB, ldb, beta, C, sC, ldc);
-  else
-    cgemm_kernel<R, OP_C, OP_C><<<grid, 256, 0, st>>>(M, N, K, alpha, A, sA, lda, B, sB, ldb, beta, C, sC, ldc);
+  const int bm = simt_tile<R>(M, N, batch);
+  dim3 grid((N + bm - 1) / bm, (M + bm - 1) / bm, batch);
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, 256, 0, st>>>(M, N, K, alpha, A, sA, lda, B, sB, ldb, beta, C, sC, ldc);
+  };
+#define NNE_SIMT(OA, OB)                                      \
+  do {                                                        \
+    if (bm == 64) launch(cgemm_kernel<R, OA, OB, 64>);        \
+    else if (bm == 32) launch(cgemm_kernel<R, OA, OB, 32>);   \
+    else launch(cgemm_kernel<R, OA, OB, 16>);                 \
+  } while (0)
+  if (opA == OP_N && opB == OP_N) NNE_SIMT(OP_N, OP_N);
+  else if (opA == OP_N && opB == OP_C) NNE_SIMT(OP_N, OP_C);
+  else if (opA == OP_C && opB == OP_N) NNE_SIMT(OP_C, OP_N);
+  else NNE_SIMT(OP_C, OP_C);
+#undef NNE_SIMT
   return cudaGetLastError();
 }
 

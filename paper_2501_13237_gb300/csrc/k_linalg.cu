@@ -502,86 +502,6 @@ static cudaError_t tridiag_global(cudaStream_t st, cx<R>* H, long long sH, int n
   return launch_cluster(tridiag_kernel<R, lower>, cs, batch, smem, st, H, sH, n, d, e, ldde, P, Kp, Vh, sVh);
 }
 
-EighWork eigh_workspace(int n, int r) {
-  EighWork w;
-  const long long qn = std::max(n, r);
-  // cx: e, phi, P (n each), Vh (n x n), WY factors (ceil(n/32) x 32 x 32), WY application workspace
-  //     (for r columns), QR workspace of an n x r matrix
-  w.cx_elems = 3LL * n + (long long)n * n + ((n + 31) / 32) * 1024LL + wy_workspace(r) + qr_workspace(n, r).cx_elems +
-               32;
-  // re: d, eabs (n each), lam (r), Z (n r), L/U0/U1/U2 (4 n r), Kpart (32 doubles = 64 floats)
-  w.re_elems = 2LL * n + r + 5LL * n * r + 64 + qn;
-  w.u8_elems = (long long)n * r;
-  return w;
-}
-
-template <typename R>
-cudaError_t eigh_top(cudaStream_t st, cx<R>* H, long long sH, int n, int r, cx<R>* U, long long sU, void* cx_ws,
-                     void* re_ws, void* u8_ws, int batch, int* err) {
-  (void)err;
-  if (batch <= 0) return cudaSuccess;
-  const EighWork w = eigh_workspace(n, r);
-  cx<R>* cxb = reinterpret_cast<cx<R>*>(cx_ws);
-  R* reb = reinterpret_cast<R*>(re_ws);
-  uint8_t* u8b = reinterpret_cast<uint8_t*>(u8_ws);
-  // per-batch-entry layouts are interleaved by "ld" strides below
-  const int ldde = n;
-  cx<R>* e = cxb;                                   // batch x n
-  cx<R>* phi = e + (long long)batch * n;            // batch x n
-  cx<R>* P = phi + (long long)batch * n;            // batch x n
-  cx<R>* Vh = P + (long long)batch * n;             // batch x n x n
-  cx<R>* Tw = Vh + (long long)batch * n * n;        // batch x nb x 1024
-  const int nbw = (n + 31) / 32;
-  cx<R>* wyws = Tw + (long long)batch * nbw * 1024;          // batch x wy_workspace(r)
-  cx<R>* qrws = wyws + (long long)batch * wy_workspace(r);   // QR workspace for batch n x r matrices
-  R* d = reb;                                       // batch x n
-  R* eabs = d + (long long)batch * n;               // batch x n
-  R* lam = eabs + (long long)batch * n;             // batch x r
-  R* Z = lam + (long long)batch * r;                // batch x n r
-  R* Ls = Z + (long long)batch * n * r;             // 4 arrays of batch x n r
-  R* U0 = Ls + (long long)batch * n * r;
-  R* U1 = U0 + (long long)batch * n * r;
-  R* U2 = U1 + (long long)batch * n * r;
-  double* Kp = reinterpret_cast<double*>(U2 + (long long)batch * n * r + 1);
-  Kp = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(Kp) + 15) & ~uintptr_t(15));
-  (void)w;
-  cudaError_t ce = cudaMemsetAsync(Vh, 0, sizeof(cx<R>) * (size_t)batch * n * n, st);
-  if (ce != cudaSuccess) return ce;
-  if (smem_cluster_size<R>(n) > 0) {
-    ce = tridiag_smem<R>(st, H, sH, n, d, e, ldde, Vh, (long long)n * n, batch);
-  } else {
-    ce = tridiag_global<R>(st, H, sH, n, d, e, ldde, P, Kp, Vh, (long long)n * n, batch);
-  }
-  if (ce != cudaSuccess) return ce;
-  {
-    ProfScope ps(st, K_ELEMWISE);
-    tridiag_phases_kernel<R><<<batch, 256, 0, st>>>(e, n, ldde, eabs, phi);
-  }
-  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  const int total = batch * r;
-  {
-    ProfScope ps(st, K_BISECT);
-    bisect_kernel<R><<<(total * 32 + 255) / 256, 256, 0, st>>>(d, eabs, n, r, ldde, lam, r, total);
-  }
-  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  const long long sS = (long long)n * r;
-  {
-    ProfScope ps(st, K_INVITER);
-    inviter_kernel<R><<<(total + 127) / 128, 128, 0, st>>>(d, eabs, n, r, ldde, lam, r, Z, sS, Ls, U0, U1, U2, u8b,
-                                                           sS, total, 32);
-  }
-  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  ce = backtransform_wy<R>(st, Vh, (long long)n * n, n, Z, sS, phi, ldde, r, U, sU, Tw, wyws, batch);
-  if (ce != cudaSuccess) return ce;
-  // orthonormalise the eigenvector block (QR; Q written over U)
-  return qr<R>(st, U, sU, n, r, U, sU, nullptr, 0, qrws, batch);
-}
-
-// Eigenvalues per warp of the float64 inverse iteration (measured at n = 640,
-// 2 x 512 eigenvalues: 32 per warp 2.87 ms, 8 per warp 2.52 ms, 2 per warp 2.78 ms).
-constexpr int INVITER64_PER_WARP = 8;
-
-// ---------------------------------------------------------------- mixed precision
 // Top r eigenvalues (descending) of the real tridiagonal (d, e) in float64.
 // Four lanes per eigenvalue, eight eigenvalues per warp: each round the four
 // lanes count at four interior points of the bracket (it shrinks five-fold)
@@ -708,6 +628,113 @@ __global__ void re_d2f_pair_kernel(const double* a, const double* b, float* fa, 
   }
 }
 
+// Top r eigenvalues of batch tridiagonals in float64: a float32 multisection of
+// the rounded tridiagonal brackets every eigenvalue to about eps_32 ||T||,
+// float64 bisection narrows the brackets.  scratch: batch x (2 n + r) floats.
+static cudaError_t bisect_f64(cudaStream_t st, const double* d, const double* e, int n, int r, float* scratch,
+                              double* lam, int batch) {
+  float* df = scratch;
+  float* ef = df + (size_t)n * batch;
+  float* lamf = ef + (size_t)n * batch;
+  const int total = batch * r;
+  cudaError_t ce;
+  {
+    ProfScope ps(st, K_BISECT);
+    re_d2f_pair_kernel<<<64, 256, 0, st>>>(d, e, df, ef, (long long)n * batch);
+    bisect_kernel<float><<<(total * 32 + 255) / 256, 256, 0, st>>>(df, ef, n, r, n, lamf, r, total);
+  }
+  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  ProfScope ps(st, K_BISECT64);
+  const dim3 grid((r + BIS64_THREADS / 4 - 1) / (BIS64_THREADS / 4), batch);
+  const size_t bsm = 2 * sizeof(double) * (size_t)n;
+  if ((ce = ensure_kernel_smem((const void*)bisect64_kernel, bsm, false)) != cudaSuccess) return ce;
+  bisect64_kernel<<<grid, BIS64_THREADS, bsm, st>>>(d, e, n, r, n, lamf, lam, r);
+  return cudaGetLastError();
+}
+
+EighWork eigh_workspace(int n, int r) {
+  EighWork w;
+  const long long qn = std::max(n, r);
+  // cx: e, phi, P (n each), Vh (n x n), WY factors (ceil(n/32) x 32 x 32), WY application workspace
+  //     (for r columns), QR workspace of an n x r matrix
+  w.cx_elems = 3LL * n + (long long)n * n + ((n + 31) / 32) * 1024LL + wy_workspace(r) + qr_workspace(n, r).cx_elems +
+               32;
+  // re: d, eabs (n each), lam (r), Z (n r), L/U0/U1/U2 (4 n r), Kpart (32 doubles = 64 floats)
+  w.re_elems = 2LL * n + r + 5LL * n * r + 64 + qn;
+  w.u8_elems = (long long)n * r;
+  return w;
+}
+
+template <typename R>
+cudaError_t eigh_top(cudaStream_t st, cx<R>* H, long long sH, int n, int r, cx<R>* U, long long sU, void* cx_ws,
+                     void* re_ws, void* u8_ws, int batch, int* err) {
+  (void)err;
+  if (batch <= 0) return cudaSuccess;
+  const EighWork w = eigh_workspace(n, r);
+  cx<R>* cxb = reinterpret_cast<cx<R>*>(cx_ws);
+  R* reb = reinterpret_cast<R*>(re_ws);
+  uint8_t* u8b = reinterpret_cast<uint8_t*>(u8_ws);
+  // per-batch-entry layouts are interleaved by "ld" strides below
+  const int ldde = n;
+  cx<R>* e = cxb;                                   // batch x n
+  cx<R>* phi = e + (long long)batch * n;            // batch x n
+  cx<R>* P = phi + (long long)batch * n;            // batch x n
+  cx<R>* Vh = P + (long long)batch * n;             // batch x n x n
+  cx<R>* Tw = Vh + (long long)batch * n * n;        // batch x nb x 1024
+  const int nbw = (n + 31) / 32;
+  cx<R>* wyws = Tw + (long long)batch * nbw * 1024;          // batch x wy_workspace(r)
+  cx<R>* qrws = wyws + (long long)batch * wy_workspace(r);   // QR workspace for batch n x r matrices
+  R* d = reb;                                       // batch x n
+  R* eabs = d + (long long)batch * n;               // batch x n
+  R* lam = eabs + (long long)batch * n;             // batch x r
+  R* Z = lam + (long long)batch * r;                // batch x n r
+  R* Ls = Z + (long long)batch * n * r;             // 4 arrays of batch x n r
+  R* U0 = Ls + (long long)batch * n * r;
+  R* U1 = U0 + (long long)batch * n * r;
+  R* U2 = U1 + (long long)batch * n * r;
+  double* Kp = reinterpret_cast<double*>(U2 + (long long)batch * n * r + 1);
+  Kp = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(Kp) + 15) & ~uintptr_t(15));
+  (void)w;
+  cudaError_t ce = cudaMemsetAsync(Vh, 0, sizeof(cx<R>) * (size_t)batch * n * n, st);
+  if (ce != cudaSuccess) return ce;
+  if (smem_cluster_size<R>(n) > 0) {
+    ce = tridiag_smem<R>(st, H, sH, n, d, e, ldde, Vh, (long long)n * n, batch);
+  } else {
+    ce = tridiag_global<R>(st, H, sH, n, d, e, ldde, P, Kp, Vh, (long long)n * n, batch);
+  }
+  if (ce != cudaSuccess) return ce;
+  {
+    ProfScope ps(st, K_ELEMWISE);
+    tridiag_phases_kernel<R><<<batch, 256, 0, st>>>(e, n, ldde, eabs, phi);
+  }
+  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  const int total = batch * r;
+  if constexpr (std::is_same<R, double>::value) {
+    // the division-free float64 bisection (the inverse iteration's scratch is still free)
+    if ((ce = bisect_f64(st, d, eabs, n, r, reinterpret_cast<float*>(Ls), lam, batch)) != cudaSuccess) return ce;
+  } else {
+    ProfScope ps(st, K_BISECT);
+    bisect_kernel<R><<<(total * 32 + 255) / 256, 256, 0, st>>>(d, eabs, n, r, ldde, lam, r, total);
+  }
+  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  const long long sS = (long long)n * r;
+  {
+    ProfScope ps(st, K_INVITER);
+    inviter_kernel<R><<<(total + 127) / 128, 128, 0, st>>>(d, eabs, n, r, ldde, lam, r, Z, sS, Ls, U0, U1, U2, u8b,
+                                                           sS, total, 32);
+  }
+  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  ce = backtransform_wy<R>(st, Vh, (long long)n * n, n, Z, sS, phi, ldde, r, U, sU, Tw, wyws, batch);
+  if (ce != cudaSuccess) return ce;
+  // orthonormalise the eigenvector block (QR; Q written over U)
+  return qr<R>(st, U, sU, n, r, U, sU, nullptr, 0, qrws, batch);
+}
+
+// Eigenvalues per warp of the float64 inverse iteration (measured at n = 640,
+// 2 x 512 eigenvalues: 32 per warp 2.87 ms, 8 per warp 2.52 ms, 2 per warp 2.78 ms).
+constexpr int INVITER64_PER_WARP = 8;
+
+// ---------------------------------------------------------------- mixed precision
 __global__ void cx_f2d_kernel(const cx<float>* X, long long sX, int rows, int cols, int ldx, cx<double>* Y,
                               long long sY) {
   const long long count = (long long)rows * cols;
@@ -799,9 +826,7 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
   double* U2 = reinterpret_cast<double*>(take(q, 8 * nr * B));
   float* Zf = reinterpret_cast<float*>(take(q, 4 * nr * B));
   float2* Kp = reinterpret_cast<float2*>(take(q, 8 * 32 * B));
-  float* df = reinterpret_cast<float*>(take(q, 4 * (size_t)n * B));
-  float* ef = reinterpret_cast<float*>(take(q, 4 * (size_t)n * B));
-  float* lamf = reinterpret_cast<float*>(take(q, 4 * (size_t)r * B));
+  float* df = reinterpret_cast<float*>(take(q, 4 * (2 * (size_t)n + r) * B));
   uint8_t* piv = reinterpret_cast<uint8_t*>(u8_ws);
   cudaError_t ce;
   if (n <= EIGH_F64_MAX) {
@@ -829,22 +854,7 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
   const int total = batch * r;
-  {
-    // float32 multisection of the rounded tridiagonal brackets every eigenvalue
-    // to about eps_32 ||T||; float64 bisection narrows the brackets
-    ProfScope ps(st, K_BISECT);
-    re_d2f_pair_kernel<<<64, 256, 0, st>>>(dd, eabs, df, ef, (long long)n * batch);
-    bisect_kernel<float><<<(total * 32 + 255) / 256, 256, 0, st>>>(df, ef, n, r, n, lamf, r, total);
-  }
-  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  {
-    ProfScope ps(st, K_BISECT64);
-    const dim3 grid((r + BIS64_THREADS / 4 - 1) / (BIS64_THREADS / 4), batch);
-    const size_t bsm = 2 * sizeof(double) * (size_t)n;
-    if ((ce = ensure_kernel_smem((const void*)bisect64_kernel, bsm, false)) != cudaSuccess) return ce;
-    bisect64_kernel<<<grid, BIS64_THREADS, bsm, st>>>(dd, eabs, n, r, n, lamf, lam, r);
-  }
-  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  if ((ce = bisect_f64(st, dd, eabs, n, r, df, lam, batch)) != cudaSuccess) return ce;
   {
     ProfScope ps(st, K_INVITER);
     const int pw = INVITER64_PER_WARP;

@@ -6,6 +6,8 @@
 // through distributed shared memory.  Each panel also yields the compact-WY
 // factor T (P_0 ... P_{b-1} = I - V T V^H).  Trailing updates and the explicit Q then apply each panel's
 // block reflector (wy_apply).  All reductions are in a fixed order (deterministic).
+#include <type_traits>
+
 #include "kernels.cuh"
 
 namespace cg = cooperative_groups;
@@ -689,6 +691,8 @@ static cudaError_t panel_factor(cudaStream_t st, cx<R>* A, long long sA, int m, 
   ProfScope ps(st, K_QR_FACTOR, 1, work * batch);
   // register-resident panel when every CTA's rows fit 16 warps x 16 registers
   int csr = mp >= 512 ? 8 : (mp >= 128 ? 4 : (mp >= 32 ? 2 : 1));
+  // float64 runs at two lanes per SM and bounds the panel: more CTAs per matrix
+  if (std::is_same<R, double>::value && mp >= 64) csr = 8;
   if ((mp + csr - 1) / csr > 16 * QR_WARPS) csr = 16;
   const int nl = (mp + csr - 1) / csr;
   if (nl <= 1 * QR_WARPS)

@@ -7,6 +7,8 @@
 // writes its partial product, and a second kernel sums the partials in chunk
 // order (deterministic) and multiplies by op(T).  The rank-bw update of C is
 // then a GEMM with inner dimension bw.
+#include <type_traits>
+
 #include "kernels.cuh"
 
 namespace nne {
@@ -21,22 +23,23 @@ long long wy_workspace(int N) { return (long long)(WY_SPLIT_MAX + 1) * WY_B * N;
 // Partial s of W = V^H C over rows [s * kc, min((s + 1) * kc, K)), written to
 // P[z][s] (WY_B x N, rows >= bw zero).  VROWS: V is passed as V^H, row c at
 // Vb + c * ldv; otherwise V is K x bw with row i at Vb + i * ldv.
-template <typename R, bool VROWS>
+// TN output columns per CTA (the sums do not depend on it).
+template <typename R, bool VROWS, int TN>
 __global__ void __launch_bounds__(256) wy_partial_kernel(const cx<R>* __restrict__ Vb, long long sV, int ldv, int bw,
                                                          int K, int N, int kc, const cx<R>* __restrict__ Cb,
                                                          long long sC, int ldc, cx<R>* __restrict__ Pb, int S) {
   __shared__ cx<R> Vs[WY_KS][WY_B + 1];   // conj(V[i][c])
-  __shared__ cx<R> Cs[WY_KS][WY_TN];
-  const int z = blockIdx.z, s = blockIdx.y, j0 = blockIdx.x * WY_TN;
+  __shared__ cx<R> Cs[WY_KS][TN];
+  const int z = blockIdx.z, s = blockIdx.y, j0 = blockIdx.x * TN;
   const cx<R>* V = Vb + z * sV;
   const cx<R>* C = Cb + z * sC;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int i_begin = s * kc, i_end = min(K, i_begin + kc);
-  cx<R> acc[2][4];
+  cx<R> acc[2][TN / 16];
 #pragma unroll
   for (int p = 0; p < 2; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[p][q] = mk<R>(0, 0);
+    for (int q = 0; q < TN / 16; ++q) acc[p][q] = mk<R>(0, 0);
   for (int i0 = i_begin; i0 < i_end; i0 += WY_KS) {
     for (int e = tid; e < WY_KS * WY_B; e += 256) {
       int k, c;
@@ -46,8 +49,8 @@ __global__ void __launch_bounds__(256) wy_partial_kernel(const cx<R>* __restrict
       if (gi < i_end && c < bw) v = VROWS ? V[(long long)c * ldv + gi] : conj(V[(long long)gi * ldv + c]);
       Vs[k][c] = v;
     }
-    for (int e = tid; e < WY_KS * WY_TN; e += 256) {
-      const int k = e / WY_TN, j = e % WY_TN;
+    for (int e = tid; e < WY_KS * TN; e += 256) {
+      const int k = e / TN, j = e % TN;
       const int gi = i0 + k, gj = j0 + j;
       Cs[k][j] = (gi < i_end && gj < N) ? C[(long long)gi * ldc + gj] : mk<R>(0, 0);
     }
@@ -56,7 +59,7 @@ __global__ void __launch_bounds__(256) wy_partial_kernel(const cx<R>* __restrict
     for (int k = 0; k < WY_KS; ++k) {
       const cx<R> a0 = Vs[k][ty], a1 = Vs[k][ty + 16];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < TN / 16; ++q) {
         const cx<R> b = Cs[k][tx + 16 * q];
         fma_(acc[0][q], a0, b);
         fma_(acc[1][q], a1, b);
@@ -68,7 +71,7 @@ __global__ void __launch_bounds__(256) wy_partial_kernel(const cx<R>* __restrict
 #pragma unroll
   for (int p = 0; p < 2; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < TN / 16; ++q) {
       const int gj = j0 + tx + 16 * q;
       if (gj < N) P[(long long)(ty + 16 * p) * N + gj] = acc[p][q];
     }
@@ -128,11 +131,13 @@ cudaError_t wy_apply(cudaStream_t st, bool v_rows, const cx<R>* V, long long sV,
   cudaError_t e;
   {
     ProfScope ps(st, K_WY, 2, 8.0 * bw * (double)N * K * batch);
-    dim3 g1(tiles, S, batch);
+    // float64 runs at two lanes per SM: narrower tiles put the product on more of them
+    constexpr int TN = std::is_same<R, double>::value ? 16 : WY_TN;
+    dim3 g1((N + TN - 1) / TN, S, batch);
     if (v_rows)
-      wy_partial_kernel<R, true><<<g1, 256, 0, st>>>(V, sV, ldv, bw, K, N, kc, C, sC, ldc, P, S);
+      wy_partial_kernel<R, true, TN><<<g1, 256, 0, st>>>(V, sV, ldv, bw, K, N, kc, C, sC, ldc, P, S);
     else
-      wy_partial_kernel<R, false><<<g1, 256, 0, st>>>(V, sV, ldv, bw, K, N, kc, C, sC, ldc, P, S);
+      wy_partial_kernel<R, false, TN><<<g1, 256, 0, st>>>(V, sV, ldv, bw, K, N, kc, C, sC, ldc, P, S);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     dim3 g2((N + WY_B - 1) / WY_B, batch);
     wy_reduce_kernel<R><<<g2, 256, 0, st>>>(P, S, N, bw, T, sT, ldt, t_adj ? 1 : 0, W2, sW2);
