@@ -304,17 +304,12 @@ __device__ __forceinline__ unsigned long long splitmix(unsigned long long x) {
 // Inverse iteration for eigenvalue lam[t] of the real tridiagonal (d, e):
 // 3 solves with the partially pivoted LU of (T - lam I); tiny pivots are
 // replaced by eps*||T||.  Output column t of Z (n x r, row-major).  The
-// factorisation keeps the pivots' reciprocals, so the solves multiply (a
-// divide costs several FMAs, dear in float64).  per_warp eigenvalues share a
-// warp (the rest of its lanes idle), which spreads the sequential float64
-// recurrences over more of the SMs' sub-partitions.
+// factorisation keeps the pivots' reciprocals, so the solves multiply.  One
+// thread per eigenvector (float32; float64 has its own, k_tri64.cu).
 template <typename R>
 __global__ void inviter_kernel(const R* db, const R* eb, int n, int r, int ldde, const R* lamb, int ldl, R* Zb,
-                               long long sZ, R* Lb, R* U0b, R* U1b, R* U2b, uint8_t* pivb, long long sS, int total,
-                               int per_warp) {
-  const int wg = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5), ln = threadIdx.x & 31;
-  if (ln >= per_warp) return;
-  const int gid = wg * per_warp + ln;
+                               long long sZ, R* Lb, R* U0b, R* U1b, R* U2b, uint8_t* pivb, long long sS, int total) {
+  const int gid = (int)(blockIdx.x * (long long)blockDim.x + threadIdx.x);
   if (gid >= total) return;
   const int z = gid / r, t = gid % r;
   const R* d = db + (long long)z * ldde;
@@ -502,125 +497,6 @@ static cudaError_t tridiag_global(cudaStream_t st, cx<R>* H, long long sH, int n
   return launch_cluster(tridiag_kernel<R, lower>, cs, batch, smem, st, H, sH, n, d, e, ldde, P, Kp, Vh, sVh);
 }
 
-// Top r eigenvalues (descending) of the real tridiagonal (d, e) in float64.
-// Four lanes per eigenvalue, eight eigenvalues per warp: each round the four
-// lanes count at four interior points of the bracket (it shrinks five-fold)
-// until it is 4 eps_64 ||T|| wide.  The bracket starts at lamf[t] -/+
-// 8 eps_32 ||T|| around the float32 eigenvalue of the rounded tridiagonal
-// when Sturm counts confirm that it holds the wanted eigenvalue, else at the
-// Gershgorin interval.  The counts use the three-term recurrence of the
-// leading principal minors p_k of T - x I (eigenvalues below x = sign changes
-// of 1, p_0, ..., p_{n-1}; Sturm): three float64 operations per step and no
-// divide, where the quotient form q_k = p_k / p_{k-1} costs a float64 divide,
-// several FMAs at GB300's 1/64 float64 rate.  T is scaled by a power of two
-// (exactly) to norm <= 1, so |p_k| grows at most 3x per step and a pair
-// (p_{k-1}, p_k) is rescaled by a power of two when its larger exponent
-// leaves [-600, 600]; a minor that is zero (or underflows) is replaced by
-// -2^-1000 p_{k-1}, the quotient form's -pivmin convention.
-constexpr int BIS64_THREADS = 64;   // 16 eigenvalues per block: blocks spread over the SMs
-
-__device__ __forceinline__ int sturm_minors(const double* ds, const double* b, int n, double x) {
-  double p0 = 1.0, p1 = ds[0] - x;
-  if (((__double2hiint(p1) & 0x7fffffff) | __double2loint(p1)) == 0) p1 = -0x1p-1000;
-  int c = __double2hiint(p1) < 0;
-  for (int k = 1; k < n; ++k) {
-    double p = fma(-b[k - 1], p0, (ds[k] - x) * p1);
-    if (((__double2hiint(p) & 0x7fffffff) | __double2loint(p)) == 0) p = -0x1p-1000 * p1;
-    c += (__double2hiint(p) ^ __double2hiint(p1)) < 0;
-    p0 = p1;
-    p1 = p;
-    const int em = max((__double2hiint(p1) >> 20) & 0x7ff, (__double2hiint(p0) >> 20) & 0x7ff);
-    if (em > 1023 + 600 || em < 1023 - 600) {
-      const double sc = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em)
-      p0 *= sc;
-      p1 *= sc;
-    }
-  }
-  return c;
-}
-
-__global__ void __launch_bounds__(BIS64_THREADS) bisect64_kernel(const double* db, const double* eb, int n, int r,
-                                                                 int ldde, const float* lamfb, double* lamb, int ldl) {
-  extern __shared__ double bis_smem[];
-  double* ds = bis_smem;        // n: d scaled
-  double* bs = bis_smem + n;    // n: e^2 scaled
-  __shared__ double red[2][BIS64_THREADS / 32];
-  __shared__ int sexp;
-  const int z = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const double* d = db + (long long)z * ldde;
-  const double* e = eb + (long long)z * ldde;
-  // Gershgorin interval and the power-of-two scale
-  double glo = 1e300, ghi = -1e300;
-  for (int k = tid; k < n; k += BIS64_THREADS) {
-    const double rad = (k > 0 ? e[k - 1] : 0.0) + (k + 1 < n ? e[k] : 0.0);
-    glo = fmin(glo, d[k] - rad);
-    ghi = fmax(ghi, d[k] + rad);
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
-    ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
-  }
-  if (lane == 0) {
-    red[0][wid] = glo;
-    red[1][wid] = ghi;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < BIS64_THREADS / 32; ++w) {
-      red[0][0] = fmin(red[0][0], red[0][w]);
-      red[1][0] = fmax(red[1][0], red[1][w]);
-    }
-    const double tn = fmax(fabs(red[0][0]), fabs(red[1][0]));
-    sexp = tn > 0 ? ((__double2hiint(tn) >> 20) & 0x7ff) - 1023 + 1 : 0;   // tn < 2^sexp
-  }
-  __syncthreads();
-  const double sc = __hiloint2double((1023 - sexp) << 20, 0);   // 2^-sexp
-  for (int k = tid; k < n; k += BIS64_THREADS) {
-    ds[k] = d[k] * sc;
-    const double es = k + 1 < n ? e[k] * sc : 0.0;
-    bs[k] = es * es;
-  }
-  glo = red[0][0] * sc;
-  ghi = red[1][0] * sc;
-  __syncthreads();
-  const double tnorm = fmax(fabs(glo), fabs(ghi));
-  const double tol = 4 * DBL_EPSILON * tnorm + 0x1p-1000;
-  glo -= 4 * DBL_EPSILON * tnorm;
-  ghi += 4 * DBL_EPSILON * tnorm;
-  const int g = lane >> 2, sub = lane & 3;
-  const int t = blockIdx.x * (BIS64_THREADS / 4) + wid * 8 + g;
-  const bool live = t < r;
-  const int idx = n - 1 - (live ? t : 0);
-  double lo = glo, hi = ghi;
-  {
-    // the float32 bracket, checked by two lanes of the group
-    const double lf = live ? (double)lamfb[(long long)z * ldl + t] * sc : 0.0;
-    const double w = 8.0 * (double)FLT_EPSILON * tnorm;
-    const double x = sub == 0 ? lf - w : lf + w;
-    const int cnt = sub < 2 ? sturm_minors(ds, bs, n, x) : 0;
-    const int c0 = __shfl_sync(0xffffffffu, cnt, lane & ~3), c1 = __shfl_sync(0xffffffffu, cnt, (lane & ~3) + 1);
-    if (c0 <= idx && c1 > idx) {
-      lo = lf - w;
-      hi = lf + w;
-    }
-  }
-  for (int it = 0; it < 40; ++it) {
-    const bool open = live && (hi - lo) > tol;
-    if (!__any_sync(0xffffffffu, open)) break;
-    const double x = lo + (hi - lo) * ((double)(sub + 1) / 5.0);
-    const int cnt = open ? sturm_minors(ds, bs, n, x) : 0;
-    const unsigned m = __ballot_sync(0xffffffffu, cnt <= idx);
-    const int K = __popc((m >> (lane & ~3)) & 0xfu);   // points at or below the eigenvalue (a prefix)
-    if (open) {
-      const double nlo = K > 0 ? lo + (hi - lo) * ((double)K / 5.0) : lo;
-      const double nhi = K < 4 ? lo + (hi - lo) * ((double)(K + 1) / 5.0) : hi;
-      lo = nlo;
-      hi = nhi;
-    }
-  }
-  if (live && sub == 0) lamb[(long long)z * ldl + t] = 0.5 * (lo + hi) / sc;
-}
-
 __global__ void re_d2f_pair_kernel(const double* a, const double* b, float* fa, float* fb, long long count) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
     fa[i] = (float)a[i];
@@ -644,12 +520,7 @@ static cudaError_t bisect_f64(cudaStream_t st, const double* d, const double* e,
     bisect_kernel<float><<<(total * 32 + 255) / 256, 256, 0, st>>>(df, ef, n, r, n, lamf, r, total);
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  ProfScope ps(st, K_BISECT64);
-  const dim3 grid((r + BIS64_THREADS / 4 - 1) / (BIS64_THREADS / 4), batch);
-  const size_t bsm = 2 * sizeof(double) * (size_t)n;
-  if ((ce = ensure_kernel_smem((const void*)bisect64_kernel, bsm, false)) != cudaSuccess) return ce;
-  bisect64_kernel<<<grid, BIS64_THREADS, bsm, st>>>(d, e, n, r, n, lamf, lam, r);
-  return cudaGetLastError();
+  return bisect64(st, d, e, n, r, lamf, lam, batch);
 }
 
 EighWork eigh_workspace(int n, int r) {
@@ -718,10 +589,12 @@ cudaError_t eigh_top(cudaStream_t st, cx<R>* H, long long sH, int n, int r, cx<R
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
   const long long sS = (long long)n * r;
-  {
+  if constexpr (std::is_same<R, double>::value) {
+    if ((ce = inviter64<double>(st, d, eabs, n, r, lam, Z, Z, Ls, U0, U1, U2, u8b, batch)) != cudaSuccess) return ce;
+  } else {
     ProfScope ps(st, K_INVITER);
     inviter_kernel<R><<<(total + 127) / 128, 128, 0, st>>>(d, eabs, n, r, ldde, lam, r, Z, sS, Ls, U0, U1, U2, u8b,
-                                                           sS, total, 32);
+                                                           sS, total);
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
   ce = backtransform_wy<R>(st, Vh, (long long)n * n, n, Z, sS, phi, ldde, r, U, sU, Tw, wyws, batch);
@@ -729,10 +602,6 @@ cudaError_t eigh_top(cudaStream_t st, cx<R>* H, long long sH, int n, int r, cx<R
   // orthonormalise the eigenvector block (QR; Q written over U)
   return qr<R>(st, U, sU, n, r, U, sU, nullptr, 0, qrws, batch);
 }
-
-// Eigenvalues per warp of the float64 inverse iteration (measured at n = 640,
-// 2 x 512 eigenvalues: 32 per warp 2.87 ms, 8 per warp 2.52 ms, 2 per warp 2.78 ms).
-constexpr int INVITER64_PER_WARP = 8;
 
 // ---------------------------------------------------------------- mixed precision
 __global__ void cx_f2d_kernel(const cx<float>* X, long long sX, int rows, int cols, int ldx, cx<double>* Y,
@@ -748,11 +617,6 @@ __global__ void cx_f2d_kernel(const cx<float>* X, long long sX, int rows, int co
 __global__ void cx_d2f_kernel(const cx<double>* X, cx<float>* Y, long long count) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
     Y[i] = mk<float>((float)X[i].re, (float)X[i].im);
-}
-
-__global__ void re_d2f_kernel(const double* X, float* Y, long long count) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
-    Y[i] = (float)X[i];
 }
 
 static inline size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -853,20 +717,11 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
     tridiag_phases_kernel<double><<<batch, 256, 0, st>>>(ed, n, n, eabs, phid);
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  const int total = batch * r;
   if ((ce = bisect_f64(st, dd, eabs, n, r, df, lam, batch)) != cudaSuccess) return ce;
-  {
-    ProfScope ps(st, K_INVITER);
-    const int pw = INVITER64_PER_WARP;
-    const int warps = (total + pw - 1) / pw;
-    inviter_kernel<double><<<(warps + 3) / 4, 128, 0, st>>>(dd, eabs, n, r, n, lam, r, Z, (long long)nr, Ls, U0, U1, U2,
-                                                            piv, (long long)nr, total, pw);
-  }
-  if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  if ((ce = inviter64<float>(st, dd, eabs, n, r, lam, Zf, Z, Ls, U0, U1, U2, piv, batch)) != cudaSuccess) return ce;
   {
     ProfScope ps(st, K_ELEMWISE);
     cx_d2f_kernel<<<64, 256, 0, st>>>(phid, phif, (long long)(n * B));
-    re_d2f_kernel<<<1024, 256, 0, st>>>(Z, Zf, (long long)(nr * B));
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
   ce = backtransform_wy<float>(st, Vhf, (long long)nn, n, Zf, (long long)nr, phif, n, r, U, sU, Tw, wyws, batch);

@@ -106,6 +106,14 @@ template <typename R>
 cudaError_t gram_entropy(cudaStream_t st, cx<R>* H, long long sH, int n, void* cx_ws, void* re_ws, int batch,
                          double* S, long long sS);
 
+// ---- k_tri64.cu (float64 eigenpairs of real tridiagonals; d, e: batch x n)
+// Top r eigenvalues (descending) from float32 estimates lamf (batch x r each).
+cudaError_t bisect64(cudaStream_t st, const double* d, const double* e, int n, int r, const float* lamf, double* lam,
+                     int batch);
+// Their unit eigenvectors, columns of Z (n x r).  Y (may be Z), L, U0, U1, U2, piv: n x r scratch per matrix.
+template <typename OUT>
+cudaError_t inviter64(cudaStream_t st, const double* d, const double* e, int n, int r, const double* lam, OUT* Z,
+                      double* Y, double* L, double* U0, double* U1, double* U2, uint8_t* piv, int batch);
 // ---- k_tridiag_df.cu (double-float reduction of complex64 eigenproblems)
 cudaError_t tridiag_df(cudaStream_t st, const cx<float>* H, long long sH, int n, float4* work, float4* P, float2* Kp,
                        double* d, cx<double>* e, cx<float>* Vh, int batch);
