@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <cooperative_groups.h>
 #include <stdint.h>
+
+#include <memory>
 #include <math.h>
 
 #include "../../include/nne.h"
@@ -118,4 +120,42 @@ nne_status set_cuda_error(cudaError_t e, const char* what, const char* file, int
 // sizes from other host threads stay valid.
 cudaError_t ensure_kernel_smem(const void* func, size_t bytes, bool nonportable_cluster);
 nne_status set_error(nne_status s, const char* fmt, ...);
+
+// Stream-ordered device memory from the library's pool on the calling context's
+// device.
+//
+// The device's default pool gives unused memory back at every synchronisation
+// (its release threshold is 0), so each call that allocated scratch paid for
+// mapping it again: 1.0 of the 1.67 ms of a 2048 x 2048 x 512 batch-8 GEMM call.
+// The library's pool, one per device and shared by its contexts (it exists while
+// any does), keeps up to MEM_POOL_KEEP between calls and gives all of it back
+// with the last context, or when an allocation fails (every pool is then trimmed
+// and the allocation tried once more).  The pool in force is the one of the
+// innermost PoolScope of the calling thread (every entry point that allocates
+// opens one); without a scope dev_alloc uses the device's default pool.  Frees
+// need no scope.
+constexpr size_t MEM_POOL_KEEP = (size_t)1 << 30;
+cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
+template <typename T>
+cudaError_t dev_alloc(T** p, size_t bytes, cudaStream_t st) {
+  return dev_alloc(reinterpret_cast<void**>(p), bytes, st);
+}
+class MemPool {
+ public:
+  static std::shared_ptr<MemPool> of_device(int device);
+  explicit MemPool(int device);
+  ~MemPool();
+  MemPool(const MemPool&) = delete;
+  MemPool& operator=(const MemPool&) = delete;
+  cudaMemPool_t handle() const { return pool_; }
+ private:
+  cudaMemPool_t pool_ = nullptr;
+};
+class PoolScope {
+ public:
+  explicit PoolScope(const MemPool* p);
+  ~PoolScope();
+ private:
+  cudaMemPool_t prev_;
+};
 }  // namespace nne

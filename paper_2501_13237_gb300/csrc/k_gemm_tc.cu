@@ -474,7 +474,7 @@ static cudaError_t launch_tc(cudaStream_t st, int M, int N, int K, float2 alpha,
     return cudaGetLastError();
   }
   float2* P = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&P, sizeof(float2) * (size_t)M * N * S * batch, st);
+  cudaError_t e = dev_alloc((void**)&P, sizeof(float2) * (size_t)M * N * S * batch, st);
   if (e != cudaSuccess) return e;
   dim3 grid((N + tc::BN - 1) / tc::BN, (M + tc::BM - 1) / tc::BM, batch * S);
   cgemm_tc_kernel<OPA, OPB><<<grid, 256, tc::SMEM_BYTES, st>>>(M, N, K, make_float2(1.f, 0.f), A, sA, lda, B, sB,

@@ -477,7 +477,7 @@ cudaError_t split_a(cudaStream_t st, int opA, int M, int K, const float2* a, lon
 
 cudaError_t tma_hold_a(cudaStream_t st, int opA, int M, int K, const cx<float>* A, long long sA, int lda, int batch) {
   float* p = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&p, sizeof(float) * (size_t)2 * M * plane_pitch(K) * batch, st);
+  cudaError_t e = dev_alloc((void**)&p, sizeof(float) * (size_t)2 * M * plane_pitch(K) * batch, st);
   if (e != cudaSuccess) return e;
   e = split_a(st, opA, M, K, reinterpret_cast<const float2*>(A), sA, lda, batch, p);
   if (e != cudaSuccess) {
@@ -520,7 +520,7 @@ cudaError_t cgemm_tma(cudaStream_t st, int opA, int opB, int M, int N, int K, cx
       held = h.planes;
   const size_t a_floats = held ? 0 : (size_t)2 * M * ldp * batch, b_floats = (size_t)2 * N2 * ldp * batch;
   float* planes = nullptr;
-  if ((e = cudaMallocAsync((void**)&planes, sizeof(float) * (a_floats + b_floats) + 1024, st)) != cudaSuccess) return e;
+  if ((e = dev_alloc((void**)&planes, sizeof(float) * (a_floats + b_floats) + 1024, st)) != cudaSuccess) return e;
   float* PA = held ? held : planes;
   float* PB = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(planes + a_floats) + 255) & ~uintptr_t(255));
   // (pad columns of the pitch lie outside the tensor maps' extent: the loads fill zeros there)
@@ -559,7 +559,7 @@ cudaError_t cgemm_tma(cudaStream_t st, int opA, int opB, int M, int N, int K, cx
       e = launch(1, Kr, al, be, reinterpret_cast<float2*>(C), sC, ldc);
     } else {
       float2* P = nullptr;
-      e = cudaMallocAsync((void**)&P, sizeof(float2) * (size_t)M * N * S * batch, st);
+      e = dev_alloc((void**)&P, sizeof(float2) * (size_t)M * N * S * batch, st);
       if (e == cudaSuccess) {
         e = launch(S, kc, make_float2(1.f, 0.f), make_float2(0.f, 0.f), P, (long long)M * N, N);
         if (e == cudaSuccess) e = cgemm_split_reduce(st, M, N, S, P, al, be, reinterpret_cast<float2*>(C), sC, ldc, batch);

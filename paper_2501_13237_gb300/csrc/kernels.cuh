@@ -196,5 +196,6 @@ size_t state_bytes(int n, int chi, int n_inst, int dtype, int sketch_rows, int s
 
 // Device ordinal and stream of a context (defined with the context in nne_api.cu).
 void ctx_device_stream(const nne_ctx* ctx, int* device, cudaStream_t* stream);
+MemPool* ctx_pool(const nne_ctx* ctx);
 
 }  // namespace nne

@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -47,6 +48,7 @@ struct nne_ctx {
   size_t budget = 0;
   size_t used = 0;
   ScratchF64 snoise;   // superoperator-build scratch, grown on demand
+  std::shared_ptr<MemPool> pool;
   ~nne_ctx() {
     if (snoise.p) {
       cudaFreeAsync(snoise.p, stream);
@@ -60,6 +62,7 @@ void ctx_device_stream(const nne_ctx* ctx, int* device, cudaStream_t* stream) {
   *device = ctx->device;
   *stream = ctx->stream;
 }
+MemPool* ctx_pool(const nne_ctx* ctx) { return ctx->pool.get(); }
 }  // namespace nne
 
 namespace {
@@ -74,8 +77,8 @@ struct DevAlloc {
     if (ctx->budget && ctx->used + bytes > ctx->budget)
       return set_error(NNE_ERR_OOM, "HBM budget exceeded: %zu + %zu > %zu bytes", ctx->used, bytes, ctx->budget);
     // stream-ordered: no device-wide synchronisation, so states on other streams keep running
-    cudaError_t e = cudaMallocAsync(p, bytes, ctx->stream);
-    if (e != cudaSuccess) return set_cuda_error(e, "cudaMallocAsync", __FILE__, __LINE__);
+    cudaError_t e = dev_alloc(p, bytes, ctx->stream);
+    if (e != cudaSuccess) return set_cuda_error(e, "dev_alloc", __FILE__, __LINE__);
     ctx->used += bytes;
     blocks.push_back({*p, bytes});
     return NNE_OK;
@@ -97,7 +100,7 @@ ScratchF64& scratch_snoise(nne_ctx* ctx, int n_inst) {
     if (ctx->snoise.p) cudaFreeAsync(ctx->snoise.p, ctx->stream);
     ctx->snoise.p = nullptr;
     ctx->snoise.n = 0;
-    if (cudaMallocAsync(&ctx->snoise.p, need * sizeof(double), ctx->stream) == cudaSuccess) ctx->snoise.n = need;
+    if (dev_alloc(&ctx->snoise.p, need * sizeof(double), ctx->stream) == cudaSuccess) ctx->snoise.n = need;
     else ctx->snoise.p = nullptr;
   }
   return ctx->snoise;
@@ -168,7 +171,7 @@ size_t state_bytes(int n, int chi, int n_inst, int dtype, int sketch_rows, int s
   total += round256((size_t)ew.u8_elems * n_inst);
   total += round256((size_t)qr_workspace((int)N4, (int)N4).cx_elems * n_inst * esz);
   total += round256(n);
-  total += round256(sizeof(int) * (n + 1)) + round256(sizeof(void*) * n) + round256(sizeof(long long) * n);
+  total += round256(sizeof(void*) * n) + round256(sizeof(long long) * n);
   total += round256(sizeof(double) * 2 * 2 * (size_t)(n + 1) * D * n_inst);
   total += round256(sizeof(double) * 2 * (size_t)(n + 1) * n_inst);
   if (sketch_cols > 0) {
@@ -215,7 +218,6 @@ struct nne_state {
   cudaEvent_t ev_fork = nullptr;
   std::vector<cudaEvent_t> ev_join;
   // sweep
-  int* d_dims = nullptr;
   void** d_site = nullptr;
   long long* d_stride = nullptr;
   double* d_env = nullptr;
@@ -626,6 +628,28 @@ nne_status entropy_sweep(nne_state* s, double* S) {
   return NNE_OK;
 }
 
+// [log F of every instance | state status | tensor-core status] into one block.
+__global__ void gather_results_kernel(const double* logfid, int n_inst, const int* err, const int* tc_err, double* out) {
+  for (int i = threadIdx.x; i < n_inst; i += blockDim.x) out[i] = logfid[i];
+  int* words = reinterpret_cast<int*>(out + n_inst);
+  if (threadIdx.x == 0) words[0] = *err;
+  if (threadIdx.x == 1) words[1] = tc_err ? *tc_err : 0;
+}
+
+// The status words read back from the device: the state's (h) and the
+// tensor-core GEMM's (t, at te; reported once and cleared).
+nne_status report_err(nne_state* s, int h, int t, int* te) {
+  if (t != 0 && te) {
+    // reported once: the word is cleared so that the next call starts clean
+    cudaError_t e = cudaMemsetAsync(te, 0, sizeof(int), s->ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->ctx->stream);
+    if (e != cudaSuccess) return set_cuda_error(e, "cudaMemsetAsync", __FILE__, __LINE__);
+  }
+  if (h != 0) return set_error(h, "device-side failure status %d (non-finite or zero norm in a gate step)", h);
+  if (t != 0) return set_error(t, "tensor-core GEMM reported status %d (a bounded wait expired)", t);
+  return NNE_OK;
+}
+
 nne_status read_err(nne_state* s) {
   int h = 0, t = 0;
   cudaError_t e = cudaMemcpyAsync(&h, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->ctx->stream);
@@ -635,17 +659,8 @@ nne_status read_err(nne_state* s) {
   if (e != cudaSuccess) return set_cuda_error(e, "cudaMemcpyAsync", __FILE__, __LINE__);
   e = cudaStreamSynchronize(s->ctx->stream);
   if (e != cudaSuccess) return set_cuda_error(e, "cudaStreamSynchronize", __FILE__, __LINE__);
-  if (t != 0 && te) {
-    // reported once: the word is cleared so that the next call starts clean
-    e = cudaMemsetAsync(te, 0, sizeof(int), s->ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->ctx->stream);
-    if (e != cudaSuccess) return set_cuda_error(e, "cudaMemsetAsync", __FILE__, __LINE__);
-  }
-  if (h != 0) return set_error(h, "device-side failure status %d (non-finite or zero norm in a gate step)", h);
-  if (t != 0) return set_error(t, "tensor-core GEMM reported status %d (a bounded wait expired)", t);
-  return NNE_OK;
+  return report_err(s, h, t, te);
 }
-
 bool is_device_ptr(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -655,11 +670,13 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// An entry point's device and memory pool.
 struct DeviceGuard {
   int prev = -1;
-  explicit DeviceGuard(int dev) {
+  PoolScope pool;
+  explicit DeviceGuard(const nne_ctx* ctx) : pool(ctx->pool.get()) {
     cudaGetDevice(&prev);
-    if (prev != dev) cudaSetDevice(dev);
+    if (prev != ctx->device) cudaSetDevice(ctx->device);
   }
   ~DeviceGuard() {
     int cur = -1;
@@ -685,6 +702,7 @@ nne_status nne_ctx_create(int device, void* cuda_stream, size_t hbm_budget_bytes
   c->device = device;
   c->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   c->budget = hbm_budget_bytes;
+  c->pool = MemPool::of_device(device);
   *out = c;
   return NNE_OK;
 }
@@ -697,7 +715,7 @@ nne_status nne_build_superops(nne_ctx* ctx, int n_gates, const double* U, int n_
                               void* G_out) {
   if (!ctx || n_gates < 0 || n_inst < 1 || !rates || (n_gates > 0 && (!U || !G_out)))
     return set_error(NNE_ERR_ARG, "nne_build_superops: bad arguments");
-  DeviceGuard g(ctx->device);
+  DeviceGuard g(ctx);
   const bool u_dev = is_device_ptr(U), r_dev = is_device_ptr(rates);
   if (!r_dev)
     for (int i = 0; i < n_inst; ++i)
@@ -716,9 +734,9 @@ nne_status nne_build_superops(nne_ctx* ctx, int n_gates, const double* U, int n_
   double *dU = nullptr, *dR = nullptr, *dS = nullptr;
   const size_t bu = sizeof(double) * 32 * (size_t)std::max(n_gates, 1), br = sizeof(double) * 4 * n_inst,
                bs = sizeof(double) * 512 * n_inst;
-  NNE_CUDA_TRY(cudaMallocAsync(&dU, bu, ctx->stream));
-  NNE_CUDA_TRY(cudaMallocAsync(&dR, br, ctx->stream));
-  NNE_CUDA_TRY(cudaMallocAsync(&dS, bs, ctx->stream));
+  NNE_CUDA_TRY(dev_alloc(&dU, bu, ctx->stream));
+  NNE_CUDA_TRY(dev_alloc(&dR, br, ctx->stream));
+  NNE_CUDA_TRY(dev_alloc(&dS, bs, ctx->stream));
   nne_status rc = NNE_OK;
   cudaError_t e = cudaSuccess;
   if (n_gates > 0) e = cudaMemcpyAsync(dU, U, sizeof(double) * 32 * n_gates, cudaMemcpyDefault, ctx->stream);
@@ -737,7 +755,7 @@ nne_status nne_build_pauli_superops(nne_ctx* ctx, int n_gates, const double* U, 
   if (!ctx || n_gates < 0 || n_inst < 1 || !lambdas || (n_gates > 0 && (!U || !pauli_rates || !G_out)))
     return set_error(NNE_ERR_ARG, "nne_build_pauli_superops: bad arguments");
   if (n_gates == 0) return NNE_OK;
-  DeviceGuard g(ctx->device);
+  DeviceGuard g(ctx);
   const bool u_dev = is_device_ptr(U), p_dev = is_device_ptr(pauli_rates), l_dev = is_device_ptr(lambdas);
   if (!p_dev && !l_dev)
     for (int i = 0; i < n_inst; ++i)
@@ -759,9 +777,9 @@ nne_status nne_build_pauli_superops(nne_ctx* ctx, int n_gates, const double* U, 
   double *dU = nullptr, *dP = nullptr, *dL = nullptr;
   const size_t bu = sizeof(double) * 32 * (size_t)n_gates, bp = sizeof(double) * 32 * (size_t)n_gates,
                bl = sizeof(double) * n_inst;
-  NNE_CUDA_TRY(cudaMallocAsync(&dU, bu, ctx->stream));
-  NNE_CUDA_TRY(cudaMallocAsync(&dP, bp, ctx->stream));
-  NNE_CUDA_TRY(cudaMallocAsync(&dL, bl, ctx->stream));
+  NNE_CUDA_TRY(dev_alloc(&dU, bu, ctx->stream));
+  NNE_CUDA_TRY(dev_alloc(&dP, bp, ctx->stream));
+  NNE_CUDA_TRY(dev_alloc(&dL, bl, ctx->stream));
   nne_status rc = NNE_OK;
   cudaError_t e = cudaMemcpyAsync(dU, U, bu, cudaMemcpyDefault, ctx->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dP, pauli_rates, bp, cudaMemcpyDefault, ctx->stream);
@@ -782,7 +800,7 @@ nne_status nne_create_state(nne_ctx* ctx, int n_qubits, int chi, int n_inst, nne
     return set_error(NNE_ERR_ARG, "nne_create_state: bad arguments");
   if (chi > 4096) return set_error(NNE_ERR_ARG, "chi %d above the supported maximum 4096", chi);
   *out = nullptr;
-  DeviceGuard g(ctx->device);
+  DeviceGuard g(ctx);
   nne_state* s = new nne_state();
   s->ctx = ctx;
   s->mem.ctx = ctx;
@@ -816,26 +834,6 @@ nne_status nne_create_state(nne_ctx* ctx, int n_qubits, int chi, int n_inst, nne
   if (rc != NNE_OK) return fail(rc);
   s->site.resize(n);
   for (int k = 0; k < n; ++k) s->site[k] = reinterpret_cast<char*>(arena) + off[k];
-  // initial product state |b><b| : s = 3 b
-  {
-    std::vector<char> host(total, 0);
-    for (int k = 0; k < n; ++k) {
-      const int b = init_bits ? (init_bits[k] ? 1 : 0) : 0;
-      for (int i = 0; i < n_inst; ++i) {
-        char* p = host.data() + off[k] + (size_t)i * s->sstride[k] * s->esz + (size_t)(3 * b) * s->esz;
-        if (dtype == NNE_C64) {
-          const float one = 1.0f;
-          memcpy(p, &one, sizeof(float));
-        } else {
-          const double one = 1.0;
-          memcpy(p, &one, sizeof(double));
-        }
-      }
-    }
-    cudaError_t e = cudaMemcpyAsync(arena, host.data(), total, cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return fail(set_cuda_error(e, "cudaMemcpyAsync", __FILE__, __LINE__));
-  }
   // scalars
   void* p = nullptr;
   if ((rc = s->mem.alloc(&p, sizeof(double) * (3 * n_inst + 3 * (size_t)n_inst * PARTS) + 64)) != NNE_OK)
@@ -877,8 +875,6 @@ nne_status nne_create_state(nne_ctx* ctx, int n_qubits, int chi, int n_inst, nne
   if (cudaMemcpyAsync(s->d_bits, s->bits.data(), n, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
     return fail(set_error(NNE_ERR_CUDA, "cudaMemcpyAsync bits"));
   // sweep buffers
-  if ((rc = s->mem.alloc(&p, sizeof(int) * (n + 1))) != NNE_OK) return fail(rc);
-  s->d_dims = reinterpret_cast<int*>(p);
   if ((rc = s->mem.alloc(&p, sizeof(void*) * n)) != NNE_OK) return fail(rc);
   s->d_site = reinterpret_cast<void**>(p);
   if ((rc = s->mem.alloc(&p, sizeof(long long) * n)) != NNE_OK) return fail(rc);
@@ -888,12 +884,17 @@ nne_status nne_create_state(nne_ctx* ctx, int n_qubits, int chi, int n_inst, nne
   if ((rc = s->mem.alloc(&p, sizeof(double) * 2 * (size_t)(n + 1) * n_inst)) != NNE_OK) return fail(rc);
   s->d_envscale = reinterpret_cast<double*>(p);
   {
+    // initial product state |b><b|
     std::vector<void*> hs(s->site.begin(), s->site.end());
     cudaError_t e = cudaMemcpyAsync(s->d_site, hs.data(), sizeof(void*) * n, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(s->d_stride, s->sstride.data(), sizeof(long long) * n, cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(arena, 0, total, ctx->stream);
+    if (e == cudaSuccess)
+      e = dtype == NNE_C64 ? product_state<float>(ctx->stream, n, s->d_site, s->d_stride, n_inst, s->d_bits)
+                           : product_state<double>(ctx->stream, n, s->d_site, s->d_stride, n_inst, s->d_bits);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return fail(set_cuda_error(e, "cudaMemcpyAsync", __FILE__, __LINE__));
+    if (e != cudaSuccess) return fail(set_cuda_error(e, "initial state", __FILE__, __LINE__));
   }
   // concurrent sub-batches of the gate steps (streams and fork/join events); only where the
   // kernels are large (bonds of 256 and more): small states are launch-bound, and splitting
@@ -920,7 +921,7 @@ nne_status nne_create_state(nne_ctx* ctx, int n_qubits, int chi, int n_inst, nne
 
 void nne_destroy_state(nne_state* st) {
   if (!st) return;
-  DeviceGuard g(st->ctx->device);
+  DeviceGuard g(st->ctx);
   cudaStreamSynchronize(st->ctx->stream);
   for (cudaStream_t q : st->sub_st) cudaStreamSynchronize(q);
   destroy_streams(st);
@@ -933,7 +934,7 @@ nne_status nne_set_sketch(nne_state* st, const void* omega, int rows, int cols, 
     return set_error(NNE_ERR_ARG, "nne_set_sketch: need rows >= 4*chi_max (%d), 1 <= cols <= 4*chi_max, 0 <= q <= 16",
                      4 * st->dmax);
   if (st->d_omega) return set_error(NNE_ERR_ARG, "nne_set_sketch: sketch already set");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   void* p = nullptr;
   nne_status rc;
   const size_t es = st->esz;
@@ -962,7 +963,7 @@ nne_status nne_apply_layer(nne_state* st, int n_gates, const int* left_qubit, co
   for (int g = 0; g < n_gates; ++g)
     if (left_qubit[g] < 0 || left_qubit[g] > st->n - 2)
       return set_error(NNE_ERR_ARG, "gate %d: left qubit %d out of range", g, left_qubit[g]);
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   const double* Gd = reinterpret_cast<const double*>(G);
   const long long sG = (long long)n_gates * 256;   // complex elements between instances
   // the instances split into nsub views, each on its own stream, forked from and joined back
@@ -991,7 +992,7 @@ nne_status nne_apply_layer(nne_state* st, int n_gates, const int* left_qubit, co
 
 nne_status nne_truncate(nne_state* st, int chi_new, double* log_fid_out) {
   if (!st || chi_new < 1 || chi_new > st->chi) return set_error(NNE_ERR_ARG, "nne_truncate: bad arguments");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   std::vector<double> before(st->n_inst), after(st->n_inst);
   NNE_CUDA_TRY(cudaMemcpyAsync(before.data(), st->d_logfid, sizeof(double) * st->n_inst, cudaMemcpyDeviceToHost,
                                st->ctx->stream));
@@ -1008,10 +1009,10 @@ nne_status nne_truncate(nne_state* st, int chi_new, double* log_fid_out) {
 nne_status nne_entropy(nne_state* st, double* S_out) {
   if (!st || !S_out) return set_error(NNE_ERR_ARG, "nne_entropy: bad arguments");
   if (st->n < 2) return NNE_OK;
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   const size_t bytes = sizeof(double) * (size_t)st->n_inst * (st->n - 1);
   double* dS = nullptr;
-  NNE_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&dS), bytes, st->ctx->stream));
+  NNE_CUDA_TRY(dev_alloc(reinterpret_cast<void**>(&dS), bytes, st->ctx->stream));
   nne_status rc = st->dtype == NNE_C64 ? entropy_sweep<float>(st, dS) : entropy_sweep<double>(st, dS);
   cudaError_t ce = cudaSuccess;
   if (rc == NNE_OK) ce = cudaMemcpyAsync(S_out, dS, bytes, cudaMemcpyDeviceToHost, st->ctx->stream);
@@ -1025,7 +1026,7 @@ nne_status nne_expect(nne_state* st, int n_obs, const uint8_t* paulis, double* r
                       double* log_fid_out) {
   if (!st || n_obs < 0 || (n_obs > 0 && (!paulis || !re_out || !im_out)))
     return set_error(NNE_ERR_ARG, "nne_expect: bad arguments");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   const int n = st->n;
   std::vector<int> first(std::max(n_obs, 1), -1), last(std::max(n_obs, 1), -1);
   for (int o = 0; o < n_obs; ++o)
@@ -1043,50 +1044,53 @@ nne_status nne_expect(nne_state* st, int n_obs, const uint8_t* paulis, double* r
     if (first[o] >= 0 && last[o] - first[o] > 1) general.push_back(o);
   const int n_general = (int)general.size();
   cudaStream_t s = st->ctx->stream;
-  void *dp = nullptr, *df = nullptr, *dl = nullptr, *dout = nullptr, *dgen = nullptr, *dv = nullptr;
-  const size_t bp = (size_t)std::max(n_obs, 1) * n, bf = sizeof(int) * std::max(n_obs, 1),
-               bo = sizeof(double) * 2 * (size_t)std::max(n_obs, 1) * st->n_inst,
-               bv = sizeof(double) * 2 * 2 * 4 * (size_t)n * st->dmax * st->n_inst;
-  NNE_CUDA_TRY(cudaMallocAsync(&dp, bp, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&df, bf, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dl, bf, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dgen, bf, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dout, bo, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dv, bv, s));
-  std::vector<double> hout(2 * (size_t)std::max(n_obs, 1) * st->n_inst);
-  cudaError_t e = cudaMemcpyAsync(st->d_dims, st->dims.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && n_obs > 0) e = cudaMemcpyAsync(dp, paulis, (size_t)n_obs * n, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(df, first.data(), bf, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dl, last.data(), bf, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && n_general > 0)
-    e = cudaMemcpyAsync(dgen, general.data(), sizeof(int) * n_general, cudaMemcpyHostToDevice, s);
+  // one block: inputs [paulis | first | last | general | dims], results [values | log F | status words], the sweep's vectors
+  auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
+  const size_t no1 = std::max(n_obs, 1), bi = sizeof(int) * no1;
+  const size_t o_first = al(no1 * n), o_last = o_first + al(bi), o_gen = o_last + al(bi), o_dims = o_gen + al(bi),
+               in_bytes = o_dims + al(sizeof(int) * (n + 1));
+  const size_t b_val = sizeof(double) * 2 * (size_t)n_obs * st->n_inst, b_lf = sizeof(double) * st->n_inst,
+               out_bytes = b_val + b_lf + 2 * sizeof(int);
+  const size_t o_out = in_bytes, o_vec = o_out + al(out_bytes);
+  std::vector<char> hin(in_bytes), hout(out_bytes);
+  if (n_obs > 0) memcpy(hin.data(), paulis, (size_t)n_obs * n);
+  memcpy(hin.data() + o_first, first.data(), bi);
+  memcpy(hin.data() + o_last, last.data(), bi);
+  if (n_general > 0) memcpy(hin.data() + o_gen, general.data(), sizeof(int) * n_general);
+  memcpy(hin.data() + o_dims, st->dims.data(), sizeof(int) * (n + 1));
+  char* blk = nullptr;
+  NNE_CUDA_TRY(dev_alloc((void**)&blk, o_vec + sizeof(double) * 2 * 2 * 4 * (size_t)n * st->dmax * st->n_inst, s));
+  const uint8_t* dp = reinterpret_cast<const uint8_t*>(blk);
+  const int *df = reinterpret_cast<const int*>(blk + o_first), *dl = reinterpret_cast<const int*>(blk + o_last),
+            *dgen = reinterpret_cast<const int*>(blk + o_gen), *ddims = reinterpret_cast<const int*>(blk + o_dims);
+  double *dout = reinterpret_cast<double*>(blk + o_out), *dv = reinterpret_cast<double*>(blk + o_vec);
+  cudaError_t e = cudaMemcpyAsync(blk, hin.data(), in_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = st->dtype == NNE_C64
-            ? expect_sweep<float>(s, n, st->d_dims, (const void* const*)st->d_site, st->d_stride, st->n_inst, st->dmax,
-                                  n_obs, (const uint8_t*)dp, (const int*)df, (const int*)dl, (const int*)dgen,
-                                  n_general, st->d_env, st->d_envscale, (double*)dv, (double*)dout)
-            : expect_sweep<double>(s, n, st->d_dims, (const void* const*)st->d_site, st->d_stride, st->n_inst,
-                                   st->dmax, n_obs, (const uint8_t*)dp, (const int*)df, (const int*)dl,
-                                   (const int*)dgen, n_general, st->d_env, st->d_envscale, (double*)dv, (double*)dout);
-  if (e == cudaSuccess && n_obs > 0)
-    e = cudaMemcpyAsync(hout.data(), dout, sizeof(double) * 2 * (size_t)n_obs * st->n_inst, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && log_fid_out)
-    e = cudaMemcpyAsync(log_fid_out, st->d_logfid, sizeof(double) * st->n_inst, cudaMemcpyDeviceToHost, s);
-  nne_status rc = NNE_OK;
-  if (e != cudaSuccess) rc = set_cuda_error(e, "nne_expect", __FILE__, __LINE__);
-  if (rc == NNE_OK) rc = read_err(st);
-  cudaFreeAsync(dp, s);
-  cudaFreeAsync(df, s);
-  cudaFreeAsync(dl, s);
-  cudaFreeAsync(dgen, s);
-  cudaFreeAsync(dout, s);
-  cudaFreeAsync(dv, s);
+            ? expect_sweep<float>(s, n, ddims, (const void* const*)st->d_site, st->d_stride, st->n_inst, st->dmax,
+                                  n_obs, dp, df, dl, dgen, n_general, st->d_env, st->d_envscale, dv, dout)
+            : expect_sweep<double>(s, n, ddims, (const void* const*)st->d_site, st->d_stride, st->n_inst, st->dmax,
+                                   n_obs, dp, df, dl, dgen, n_general, st->d_env, st->d_envscale, dv, dout);
+  int* te = tc_error_ptr();
+  if (e == cudaSuccess) {
+    ProfScope ps(s, K_ELEMWISE);
+    gather_results_kernel<<<1, 128, 0, s>>>(st->d_logfid, st->n_inst, st->d_err, te, dout + 2 * (size_t)n_obs * st->n_inst);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hout.data(), dout, out_bytes, cudaMemcpyDeviceToHost, s);
+  cudaFreeAsync(blk, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return set_cuda_error(e, "nne_expect", __FILE__, __LINE__);
+  int words[2];
+  memcpy(words, hout.data() + b_val + b_lf, sizeof(words));
+  if (log_fid_out) memcpy(log_fid_out, hout.data() + b_val, b_lf);
+  const nne_status rc = report_err(st, words[0], words[1], te);
   if (rc != NNE_OK) return rc;
-  for (int i = 0; i < st->n_inst; ++i)
-    for (int o = 0; o < n_obs; ++o) {
-      re_out[(size_t)i * n_obs + o] = hout[2 * ((size_t)i * n_obs + o)];
-      im_out[(size_t)i * n_obs + o] = hout[2 * ((size_t)i * n_obs + o) + 1];
-    }
+  const double* v = reinterpret_cast<const double*>(hout.data());
+  for (size_t i = 0; i < (size_t)n_obs * st->n_inst; ++i) {
+    re_out[i] = v[2 * i];
+    im_out[i] = v[2 * i + 1];
+  }
   return NNE_OK;
 }
 
@@ -1097,35 +1101,32 @@ nne_status nne_extrapolate(nne_ctx* ctx, int n_lambda, const double* lambdas, co
       method < 0 || method > 2 || (method == NNE_FIT_POLY && (degree < 1 || degree > 15)))
     return set_error(NNE_ERR_ARG, "nne_extrapolate: bad arguments");
   if (n_obs == 0) return NNE_OK;
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx);
   cudaStream_t s = ctx->stream;
-  double *dl = nullptr, *dv = nullptr, *df = nullptr, *dy = nullptr, *dout = nullptr;
-  int* dst = nullptr;
-  NNE_CUDA_TRY(cudaMallocAsync(&dl, sizeof(double) * n_lambda, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dv, sizeof(double) * n_lambda * (size_t)n_obs, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&df, sizeof(double) * n_lambda, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dy, sizeof(double) * (size_t)n_obs, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dout, sizeof(double) * (size_t)n_obs, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dst, sizeof(int) * (size_t)n_obs, s));
-  cudaError_t e = cudaMemcpyAsync(dl, lambdas, sizeof(double) * n_lambda, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(dv, values, sizeof(double) * n_lambda * (size_t)n_obs, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && log_fid) e = cudaMemcpyAsync(df, log_fid, sizeof(double) * n_lambda, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && y_zero) e = cudaMemcpyAsync(dy, y_zero, sizeof(double) * n_obs, cudaMemcpyHostToDevice, s);
+  // one block: inputs [lambdas | values | log F | y_zero], results [estimates | statuses]
+  const size_t nl = n_lambda, no = n_obs;
+  std::vector<double> hin(nl + nl * no + nl + no, 0.0);
+  memcpy(hin.data(), lambdas, sizeof(double) * nl);
+  memcpy(hin.data() + nl, values, sizeof(double) * nl * no);
+  if (log_fid) memcpy(hin.data() + nl + nl * no, log_fid, sizeof(double) * nl);
+  if (y_zero) memcpy(hin.data() + 2 * nl + nl * no, y_zero, sizeof(double) * no);
+  const size_t out_bytes = (sizeof(double) + sizeof(int)) * no;
+  std::vector<char> hout(out_bytes);
+  double* blk = nullptr;
+  NNE_CUDA_TRY(dev_alloc((void**)&blk, sizeof(double) * hin.size() + out_bytes, s));
+  double *dl = blk, *dv = dl + nl, *df = dv + nl * no, *dy = df + nl, *dout = dy + no;
+  int* dst = reinterpret_cast<int*>(dout + no);
+  cudaError_t e = cudaMemcpyAsync(blk, hin.data(), sizeof(double) * hin.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = extrapolate_fit(s, n_lambda, dl, dv, log_fid ? df : nullptr, n_obs, method, degree, lambda_star,
                         y_zero ? dy : nullptr, dout, dst);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out, dout, sizeof(double) * n_obs, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(per_obs_status, dst, sizeof(int) * n_obs, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hout.data(), dout, out_bytes, cudaMemcpyDeviceToHost, s);
+  cudaFreeAsync(blk, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  nne_status rc = e == cudaSuccess ? NNE_OK : set_cuda_error(e, "nne_extrapolate", __FILE__, __LINE__);
-  cudaFreeAsync(dl, s);
-  cudaFreeAsync(dv, s);
-  cudaFreeAsync(df, s);
-  cudaFreeAsync(dy, s);
-  cudaFreeAsync(dout, s);
-  cudaFreeAsync(dst, s);
-  return rc;
+  if (e != cudaSuccess) return set_cuda_error(e, "nne_extrapolate", __FILE__, __LINE__);
+  memcpy(out, hout.data(), sizeof(double) * no);
+  memcpy(per_obs_status, hout.data() + sizeof(double) * no, sizeof(int32_t) * no);
+  return NNE_OK;
 }
 
 nne_status nne_extrapolate_ladder(nne_ctx* ctx, int k, int n_lambda, const double* lambdas, const double* values,
@@ -1136,20 +1137,20 @@ nne_status nne_extrapolate_ladder(nne_ctx* ctx, int k, int n_lambda, const doubl
       !out || !per_obs_status || method < 0 || method > 2 || (method == NNE_FIT_POLY && (degree < 1 || degree > 15)))
     return set_error(NNE_ERR_ARG, "nne_extrapolate_ladder: bad arguments");
   if (n_obs == 0) return NNE_OK;
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx);
   cudaStream_t s = ctx->stream;
   const size_t cells = (size_t)n_lambda * n_obs;
   double *dl = nullptr, *dv = nullptr, *df = nullptr, *dy = nullptr, *dob = nullptr, *dout = nullptr;
   uint8_t* dc = nullptr;
   int* dst = nullptr;
-  NNE_CUDA_TRY(cudaMallocAsync(&dl, sizeof(double) * n_lambda, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dv, sizeof(double) * k * cells, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&df, sizeof(double) * k * (size_t)n_lambda, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dy, sizeof(double) * (size_t)n_obs, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dob, sizeof(double) * cells, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dc, cells, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dout, sizeof(double) * (size_t)n_obs, s));
-  NNE_CUDA_TRY(cudaMallocAsync(&dst, sizeof(int) * (size_t)n_obs, s));
+  NNE_CUDA_TRY(dev_alloc(&dl, sizeof(double) * n_lambda, s));
+  NNE_CUDA_TRY(dev_alloc(&dv, sizeof(double) * k * cells, s));
+  NNE_CUDA_TRY(dev_alloc(&df, sizeof(double) * k * (size_t)n_lambda, s));
+  NNE_CUDA_TRY(dev_alloc(&dy, sizeof(double) * (size_t)n_obs, s));
+  NNE_CUDA_TRY(dev_alloc(&dob, sizeof(double) * cells, s));
+  NNE_CUDA_TRY(dev_alloc(&dc, cells, s));
+  NNE_CUDA_TRY(dev_alloc(&dout, sizeof(double) * (size_t)n_obs, s));
+  NNE_CUDA_TRY(dev_alloc(&dst, sizeof(int) * (size_t)n_obs, s));
   cudaError_t e = cudaMemcpyAsync(dl, lambdas, sizeof(double) * n_lambda, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dv, values, sizeof(double) * k * cells, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(df, log_fid, sizeof(double) * k * (size_t)n_lambda, cudaMemcpyHostToDevice, s);
@@ -1176,7 +1177,7 @@ nne_status nne_extrapolate_ladder(nne_ctx* ctx, int k, int n_lambda, const doubl
 
 nne_status nne_reset_state(nne_state* st, const uint8_t* init_bits) {
   if (!st) return set_error(NNE_ERR_ARG, "null state");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   cudaStream_t s = st->ctx->stream;
   if (init_bits) {
     for (int k = 0; k < st->n; ++k) st->bits[k] = init_bits[k] ? 1 : 0;
@@ -1212,7 +1213,7 @@ nne_status nne_cgemm_c64(nne_ctx* ctx, int op_a, int op_b, int M, int N, int K, 
   if (!ctx || !alpha || !beta || !A || !B || !C || M < 0 || N < 0 || K < 0 || batch < 0 || op_a < 0 || op_a > 1 ||
       op_b < 0 || op_b > 1)
     return set_error(NNE_ERR_ARG, "nne_cgemm_c64: bad arguments");
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx);
   cudaError_t e = cgemm<float>(ctx->stream, op_a, op_b, M, N, K, mk<float>(alpha[0], alpha[1]),
                                reinterpret_cast<const cx<float>*>(A), stride_a, lda,
                                reinterpret_cast<const cx<float>*>(B), stride_b, ldb, mk<float>(beta[0], beta[1]),
@@ -1233,13 +1234,13 @@ nne_status nne_cgemm_c64(nne_ctx* ctx, int op_a, int op_b, int M, int N, int K, 
 
 nne_status nne_sync(nne_state* st) {
   if (!st) return set_error(NNE_ERR_ARG, "null state");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   return read_err(st);
 }
 
 nne_status nne_state_info(nne_state* st, int* dims_out, int* centre_out, double* log_norm_out, double* log_fid_out) {
   if (!st) return set_error(NNE_ERR_ARG, "null state");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   if (log_norm_out)
     NNE_CUDA_TRY(cudaMemcpyAsync(log_norm_out, st->d_lognorm, sizeof(double) * st->n_inst, cudaMemcpyDeviceToHost,
                                  st->ctx->stream));
@@ -1257,7 +1258,7 @@ nne_status nne_state_info(nne_state* st, int* dims_out, int* centre_out, double*
 nne_status nne_state_read_site(nne_state* st, int inst, int k, void* host_out, size_t cap_bytes) {
   if (!st || inst < 0 || inst >= st->n_inst || k < 0 || k >= st->n || !host_out)
     return set_error(NNE_ERR_ARG, "nne_state_read_site: bad arguments");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   const size_t bytes = (size_t)st->dims[k] * 4 * st->dims[k + 1] * st->esz;
   if (cap_bytes < bytes) return set_error(NNE_ERR_ARG, "buffer too small: %zu < %zu", cap_bytes, bytes);
   NNE_CUDA_TRY(cudaMemcpyAsync(host_out, st->site[k] + (size_t)inst * st->sstride[k] * st->esz, bytes,
@@ -1269,7 +1270,7 @@ nne_status nne_state_write_site(nne_state* st, int inst, int k, int dl, int dr, 
   if (!st || inst < 0 || inst >= st->n_inst || k < 0 || k >= st->n || !host_in || dl < 1 || dr < 1 ||
       dl > st->cap[k] || dr > st->cap[k + 1])
     return set_error(NNE_ERR_ARG, "nne_state_write_site: bad arguments (dims above capacity?)");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   const size_t bytes = (size_t)dl * 4 * dr * st->esz;
   NNE_CUDA_TRY(cudaMemcpyAsync(st->site[k] + (size_t)inst * st->sstride[k] * st->esz, host_in, bytes,
                                cudaMemcpyHostToDevice, st->ctx->stream));
@@ -1286,7 +1287,7 @@ nne_status nne_state_set_centre(nne_state* st, int centre) {
 
 nne_status nne_state_set_log(nne_state* st, const double* log_norm, const double* log_fid) {
   if (!st) return set_error(NNE_ERR_ARG, "nne_state_set_log: null state");
-  DeviceGuard dg(st->ctx->device);
+  DeviceGuard dg(st->ctx);
   const size_t b = sizeof(double) * st->n_inst;
   if (log_norm) NNE_CUDA_TRY(cudaMemcpyAsync(st->d_lognorm, log_norm, b, cudaMemcpyHostToDevice, st->ctx->stream));
   if (log_fid) NNE_CUDA_TRY(cudaMemcpyAsync(st->d_logfid, log_fid, b, cudaMemcpyHostToDevice, st->ctx->stream));

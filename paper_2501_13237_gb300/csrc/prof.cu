@@ -3,7 +3,10 @@
 // timing is enabled the scope records an event pair on the launching stream
 // (events come from a reusable pool), and nne_prof_collect sums the elapsed
 // times per class after synchronising.
+#include <cuda.h>
+
 #include <atomic>
+#include <map>
 #include <mutex>
 #include <unordered_map>
 #include <vector>
@@ -87,6 +90,58 @@ cudaError_t ensure_kernel_smem(const void* func, size_t bytes, bool nonportable_
     a.second = true;
   }
   return cudaSuccess;
+}
+
+// ---------------------------------------------------------------- device memory
+static thread_local cudaMemPool_t t_pool = nullptr;
+static std::mutex g_pools_mu;
+static std::map<int, std::weak_ptr<MemPool>> g_pools;   // per device, while any context holds it
+
+std::shared_ptr<MemPool> MemPool::of_device(int device) {
+  std::lock_guard<std::mutex> lk(g_pools_mu);
+  std::weak_ptr<MemPool>& w = g_pools[device];
+  std::shared_ptr<MemPool> p = w.lock();
+  if (!p) w = p = std::make_shared<MemPool>(device);
+  return p;
+}
+
+MemPool::MemPool(int device) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  if (cudaMemPoolCreate(&pool_, &props) != cudaSuccess) {
+    cudaGetLastError();
+    pool_ = nullptr;   // dev_alloc then takes the default pool
+    return;
+  }
+  cuuint64_t keep = MEM_POOL_KEEP;
+  cudaMemPoolSetAttribute(pool_, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
+MemPool::~MemPool() {
+  if (pool_) cudaMemPoolDestroy(pool_);   // outstanding allocations stay valid until they are freed
+}
+
+PoolScope::PoolScope(const MemPool* p) : prev_(t_pool) { t_pool = p ? p->handle() : nullptr; }
+PoolScope::~PoolScope() { t_pool = prev_; }
+
+cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
+  auto once = [&] {
+    return t_pool ? cudaMallocFromPoolAsync(p, bytes, t_pool, st) : cudaMallocAsync(p, bytes, st);
+  };
+  cudaError_t e = once();
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  std::vector<std::shared_ptr<MemPool>> live;
+  {
+    std::lock_guard<std::mutex> lk(g_pools_mu);
+    for (auto& q : g_pools)
+      if (std::shared_ptr<MemPool> m = q.second.lock()) live.push_back(m);
+  }
+  for (auto& m : live)
+    if (m->handle()) cudaMemPoolTrimTo(m->handle(), 0);
+  return once();
 }
 
 }  // namespace nne

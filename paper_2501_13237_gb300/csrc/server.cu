@@ -108,6 +108,7 @@ void log_job(FILE* f, const JobCopy& j, const ResultRec& r) {
 }
 
 nne_status run_job(nne_ctx* ctx, cudaStream_t st, const JobCopy& j, ResultRec& r) {
+  const nne::PoolScope pool(nne::ctx_pool(ctx));
   nne_state* s = nullptr;
   nne_status rc = nne_create_state(ctx, j.n, j.chi, j.n_lambda, (nne_dtype)j.dtype, (nne_trunc)j.trunc,
                                    j.has_bits ? j.bits.data() : nullptr, &s);
@@ -131,10 +132,10 @@ nne_status run_job(nne_ctx* ctx, cudaStream_t st, const JobCopy& j, ResultRec& r
   // rate channels: dRates = n_lambda x 4; Pauli channels: 32 per gate (c0, c1), then the n_lambda levels
   const bool pauli = !j.pauli.empty();
   const size_t n_rates = pauli ? (size_t)32 * j.gates + j.n_lambda : (size_t)4 * j.n_lambda;
-  cudaError_t e = cudaMallocAsync((void**)&dU, sizeof(double) * 32 * (size_t)std::max<long long>(j.gates, 1), st);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&dRates, sizeof(double) * n_rates, st);
+  cudaError_t e = nne::dev_alloc((void**)&dU, sizeof(double) * 32 * (size_t)std::max<long long>(j.gates, 1), st);
+  if (e == cudaSuccess) e = nne::dev_alloc((void**)&dRates, sizeof(double) * n_rates, st);
   if (e == cudaSuccess)
-    e = cudaMallocAsync((void**)&dG, sizeof(double) * 512 * (size_t)j.n_lambda * std::max(j.max_layer_gates, 1), st);
+    e = nne::dev_alloc((void**)&dG, sizeof(double) * 512 * (size_t)j.n_lambda * std::max(j.max_layer_gates, 1), st);
   if (e == cudaSuccess && j.gates > 0)
     e = cudaMemcpyAsync(dU, j.U.data(), sizeof(double) * 32 * j.gates, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !pauli)
