@@ -589,6 +589,293 @@ __global__ void __launch_bounds__(QR_THREADS) qr_panel_reg_kernel(cx<R>* Ab, lon
   }
 }
 
+// Register-resident panel factorisation with one pass over the panel and one
+// cluster exchange per column.
+//
+// Layout as above: warp w of a CTA holds its local rows w, w + 16, ... (RPW of
+// them), lane c holds column c; rows are dealt to the CTAs cyclically.  What
+// bounds a column is the chain pass - block sum - exchange - pivot, so
+//   * the update with reflector j and the products with the raw next column x
+//     (S_c = sum conj(a_c) x over rows > j) share one pass; with h_c = (S_c -
+//     alpha conj(row[c])) / un, row = row j+1 of the panel, both v^H a_c (c to the
+//     right) and the v_c^H v of T (c to the left) follow after the exchange, and
+//     S of the column itself is its exact squared norm: nothing is downdated
+//     and no column needs a second round;
+//   * after the exchange one warp of each CTA sums the shares and forms the
+//     pivot (all 16 doing so cost more issue slots than the broadcast, and in
+//     float64 queue for the SM's two lanes); a 17th warp without rows extends T.
+// A 32-column panel of 8 matrices, complex64 (us, the kernel above in brackets):
+// 2048 rows 90 (138), 512 rows 58 (91), 256 rows 55 (64); complex128, 256 rows of
+// 4 matrices, 267 (332).
+__device__ __forceinline__ void fused_pivot(double xn2, cx<double> x0, cx<double>* alpha, double* inv, double* tau) {
+  hh_pivot<double>(xn2, x0, alpha, inv, tau);
+}
+// 1 / sqrt(x), x > 0: the hardware estimate (2 ulp) and one Newton step.
+__device__ __forceinline__ float rsqrt_newton(float x) {
+  const float y = rsqrtf(x);
+  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
+}
+// hh_pivot without divides and square roots on the column's chain (440 -> about
+// 150 cycles); |x0| below 2^-50 is scaled away from denormal squares.
+__device__ __forceinline__ void fused_pivot(float xn2, cx<float> x0, cx<float>* alpha, float* inv, float* tau) {
+  const float s = fmaxf(fabsf(x0.re), fabsf(x0.im));
+  const float up = s < 0x1p-50f ? 0x1p70f : 1.f, dn = s < 0x1p-50f ? 0x1p-70f : 1.f;
+  const float a = x0.re * up, b = x0.im * up, q2 = fmaf(a, a, b * b);
+  const bool nz = q2 > 0.f;
+  const float qi = nz ? rsqrt_newton(q2) : 0.f;
+  const float pr = nz ? a * qi : 1.f, pi = b * qi, ax0 = q2 * qi * dn;
+  const bool live = xn2 > 0.f;
+  const float xn = live ? xn2 * rsqrt_newton(xn2) : 0.f;
+  *alpha = mk<float>(-xn * pr, -xn * pi);
+  const float un2 = 2.f * fmaf(xn, ax0, xn2);
+  *inv = live ? rsqrt_newton(un2) : 0.f;
+  *tau = live ? 2.f : 0.f;
+}
+template <typename R>
+struct __align__(4 * sizeof(R)) VX {
+  cx<R> v, x;
+};
+template <typename R>
+struct FusedMsg {
+  cx<R> s[QB];     // this CTA's S_c
+  cx<R> row[QB];   // row j of the panel (from its owner only)
+};
+template <typename R, int RPW>
+struct FusedShared {
+  FusedMsg<R> msg[2][QR_CS_MAX];
+  cx<R> row[QB];                 // row j of the panel (its owner)
+  cx<R> g[QB];                   // the T warp's copy of h
+  cx<R> sum[QB];                 // complex128: the block sums
+  cx<R> raw[QR_WARPS][RPW][2];   // a warp's rows: entries of the last and of this column,
+  VX<R> vx[QR_WARPS][RPW];       // and what becomes of them
+  cx<R> red[QR_WARPS][QB + 1];
+  cx<R> alphas[QB];
+  cx<R> h[QB];                   // of the column: h_c, 1 / un
+  R inv;
+  cx<R> Ts[QB][QB + 1];
+};
+
+constexpr int FUSED_THREADS = QR_THREADS + 32;   // and the T warp
+
+template <typename R, int RPW>
+__global__ void __launch_bounds__(FUSED_THREADS) qr_panel_fused_kernel(cx<R>* Ab, long long sA, int lda, int m, int pb,
+                                                                     int bw, cx<R>* Vb, long long sV, int ldv,
+                                                                     cx<R>* Tb, long long sT, int zr) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CS = (int)cluster.num_blocks(), lcs = __ffs(CS) - 1;   // a power of two (integer divides cost more than the pass)
+  const int rank = (int)cluster.block_rank();
+  const int z = blockIdx.y;
+  cx<R>* A = Ab + z * sA;
+  cx<R>* V = Vb + z * sV;
+  cx<R>* T = Tb + z * sT;
+  constexpr bool F64 = std::is_same<R, double>::value;
+  __shared__ FusedShared<R, RPW> sh;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int mp = m - pb;
+  const int nloc = mp > rank ? (mp - rank + CS - 1) >> lcs : 0;
+  const bool t_warp = wid == QR_WARPS;   // holds no rows
+  const int kmax = !t_warp && nloc > wid ? (nloc - wid + QR_WARPS - 1) / QR_WARPS : 0;   // this warp's live registers
+  cx<R> a[RPW];
+#pragma unroll
+  for (int k = 0; k < RPW; ++k) {
+    const int li = wid + QR_WARPS * k;
+    a[k] = mk<R>(0, 0);
+    if (!t_warp && li < nloc && lane < bw) a[k] = A[(long long)(pb + rank + li * CS) * lda + pb + lane];
+  }
+  for (int e = tid; e < QB * QB; e += FUSED_THREADS) sh.Ts[e / QB][e % QB] = mk<R>(0, 0);
+  // every CTA of the cluster is running before anyone writes into its shared memory
+  cluster.sync();
+  cx<R> alpha = mk<R>(0, 0), wf = mk<R>(0, 0);   // of the last column; wf: this lane's 2 v^H a_c
+  R inv = 0;
+  for (int j = 0; j < bw; ++j) {
+    const int buf = j & 1;
+    // register of row j - 1 (the last pivot row) and of row j, -1 if not in this warp
+    const int lstep = lcs + 4, mask = (QR_WARPS << lcs) - 1, d1 = j - 1 - rank - (wid << lcs), d0 = d1 + 1;
+    const int k1 = (j > 0 && d1 >= 0 && (d1 & mask) == 0) ? d1 >> lstep : -1;
+    const int k0 = (d0 >= 0 && (d0 & mask) == 0 && j < mp) ? d0 >> lstep : -1;
+    // first register with a row >= j - 1
+    const int jr = j > 0 ? j - 1 : 0;
+    const int l1 = jr > rank ? (jr - rank + CS - 1) >> lcs : 0;
+    const int kmin = l1 > wid ? (l1 - wid + QR_WARPS - 1) / QR_WARPS : 0;
+    cx<R> acc0 = mk<R>(0, 0), acc1 = mk<R>(0, 0);
+    if (t_warp) {
+    } else if (j == 0) {
+#pragma unroll
+      for (int k = 0; k < RPW; ++k)
+        if (k < kmax) {
+          const cx<R> x = shfl_idx(a[k], 0);
+          if (k & 1) fmac_(acc1, a[k], x); else fmac_(acc0, a[k], x);
+        }
+    } else {
+      // the last column's and this column's raw entries to shared memory; lane k
+      // turns row k's into v and the updated x (0 where the row takes no part);
+      // every lane then reads (v, x) of a row with one broadcast load
+      const cx<R> wj = shfl_idx(wf, j);
+      if (lane == j - 1 || lane == j) {
+#pragma unroll
+        for (int k = 0; k < RPW; ++k) sh.raw[wid][k][lane - (j - 1)] = a[k];
+      }
+      if (!F64) __syncwarp();
+      if (!F64 && lane < RPW) {
+        cx<R> u = sh.raw[wid][lane][0], x = sh.raw[wid][lane][1];
+        const bool live = lane >= kmin && lane < kmax;
+        if (lane == k1) u = u - alpha;
+        const cx<R> v = live ? inv * u : mk<R>(0, 0);
+        x = hh_upd(x, v, wj);
+        if (!live || lane == k1) x = mk<R>(0, 0);
+        sh.vx[wid][lane] = VX<R>{v, x};
+      }
+      if (!F64) __syncwarp();
+    }
+    if (F64 && j > 0) {
+      // float64 instructions cost the SM 19 cycles each however few lanes they use:
+      // lane = row for the CTA's rows, 32 at a time, by as few warps as that takes
+      __syncthreads();
+      const cx<R> wj = shfl_idx(wf, j);
+      for (int q = wid; 32 * q < QR_WARPS * RPW; q += QR_WARPS) {
+        const int w = lane & (QR_WARPS - 1), k = 2 * q + (lane >> 4);
+        const int pi = rank + ((w + QR_WARPS * k) << lcs);
+        if (k < RPW) {
+          cx<R> u = sh.raw[w][k][0], x = sh.raw[w][k][1];
+          const bool live = pi >= j - 1 && pi < mp;
+          if (pi == j - 1) u = u - alpha;
+          const cx<R> v = live ? inv * u : mk<R>(0, 0);
+          x = hh_upd(x, v, wj);
+          if (!live || pi == j - 1) x = mk<R>(0, 0);
+          sh.vx[w][k] = VX<R>{v, x};
+        }
+      }
+      __syncthreads();
+    }
+    if (!t_warp && j > 0) {
+#pragma unroll
+      for (int k = 0; k < RPW; ++k) {
+        const VX<R> q = sh.vx[wid][k];
+        if (lane != j - 1) a[k] = hh_upd(a[k], q.v, wf);   // wf = 0 left of the column
+        else if (k >= kmin) a[k] = q.v;
+        if (k & 1) fmac_(acc1, a[k], q.x); else fmac_(acc0, a[k], q.x);
+      }
+    }
+    if (!t_warp) sh.red[wid][lane] = acc0 + acc1;
+    if (!t_warp && k0 >= 0) {
+      cx<R> r = mk<R>(0, 0);
+#pragma unroll
+      for (int k = 0; k < RPW; ++k)
+        if (k == k0) r = a[k];
+      sh.row[lane] = r;
+    }
+    __syncthreads();
+    // warp d forms the block sums (lane = column) and stores them to CTA d in one piece:
+    // stores that scatter over the CTAs cost their number of pieces (a shared-memory
+    // pipe 92 % busy, and about 680 cycles more per column).  In float64 two warps
+    // form the real and the imaginary sums once.
+    if (F64) {
+      if (wid < 2) {
+        R t = 0;
+#pragma unroll
+        for (int w = 0; w < QR_WARPS; ++w) t += wid ? sh.red[w][lane].im : sh.red[w][lane].re;
+        (wid ? sh.sum[lane].im : sh.sum[lane].re) = t;
+      }
+      __syncthreads();
+    }
+    if (wid < CS) {
+      cx<R> t0 = mk<R>(0, 0), t1 = t0, t2 = t0, t3 = t0;
+      if (F64) {
+        t0 = sh.sum[lane];
+      } else {
+#pragma unroll
+        for (int w = 0; w < QR_WARPS; w += 4) {
+          t0 = t0 + sh.red[w][lane];
+          t1 = t1 + sh.red[w + 1][lane];
+          t2 = t2 + sh.red[w + 2][lane];
+          t3 = t3 + sh.red[w + 3][lane];
+        }
+        t0 = (t0 + t1) + (t2 + t3);
+      }
+      FusedMsg<R>* dst = cluster.map_shared_rank(&sh.msg[buf][rank], wid);
+      dst->s[lane] = t0;
+      if (rank == (j & (CS - 1))) dst->row[lane] = sh.row[lane];
+    }
+    cluster.sync();
+    if (wid == 0) {   // one warp: lane c forms h_c of the column, and all its pivot
+      cx<R> s0 = mk<R>(0, 0), s1 = s0;
+#pragma unroll
+      for (int src = 0; src < QR_CS_MAX; src += 2) {   // independent loads
+        if (src < CS) s0 = s0 + sh.msg[buf][src].s[lane];
+        if (src + 1 < CS) s1 = s1 + sh.msg[buf][src + 1].s[lane];
+      }
+      const cx<R> S = s0 + s1;
+      const R xn2 = __shfl_sync(0xffffffffu, S.re, j);
+      const cx<R> rc = j < mp ? sh.msg[buf][j & (CS - 1)].row[lane] : mk<R>(0, 0);
+      R tau;
+      fused_pivot(xn2, shfl_idx(rc, j), &alpha, &inv, &tau);
+      sh.h[lane] = inv * (S - alpha * conj(rc));
+      if (lane == 0) {
+        sh.alphas[j] = alpha;
+        sh.inv = inv;
+      }
+    }
+    __syncthreads();
+    const cx<R> h = sh.h[lane];
+    alpha = sh.alphas[j];
+    inv = sh.inv;
+    wf = (lane > j && lane < bw) ? mk<R>(R(2) * h.re, -R(2) * h.im) : mk<R>(0, 0);
+    // T[0:j, j] = -tau T[0:j, 0:j] (V^H v_j), T[j][j] = tau: up to 31 dependent steps, by a
+    // warp that has no rows, while the others are at the next column
+    if (rank == 0 && t_warp) {
+      const R tau = inv > R(0) ? R(2) : R(0);
+      sh.g[lane] = h;
+      __syncwarp();
+      cx<R> ta0 = mk<R>(0, 0), ta1 = ta0;
+      if (lane < j) {
+        int l = lane;
+        for (; l + 1 < j; l += 2) {
+          fma_(ta0, sh.Ts[lane][l], sh.g[l]);
+          fma_(ta1, sh.Ts[lane][l + 1], sh.g[l + 1]);
+        }
+        if (l < j) fma_(ta0, sh.Ts[lane][l], sh.g[l]);
+        const cx<R> ta = ta0 + ta1;
+        sh.Ts[lane][j] = mk<R>(-tau * ta.re, -tau * ta.im);
+      }
+      if (lane == j) sh.Ts[j][j] = mk<R>(tau, 0);
+      __syncwarp();
+    }
+  }
+  // the last column's reflector
+  {
+    const int j = bw - 1, d1 = j - rank - (wid << lcs);
+    const int k1 = (d1 >= 0 && (d1 & ((QR_WARPS << lcs) - 1)) == 0) ? d1 >> (lcs + 4) : -1;
+    const int l1 = j > rank ? (j - rank + CS - 1) >> lcs : 0;
+    const int kmin = l1 > wid ? (l1 - wid + QR_WARPS - 1) / QR_WARPS : 0;
+#pragma unroll
+    for (int k = 0; k < RPW; ++k)
+      if (k >= kmin && k < kmax && lane == j) {
+        cx<R> u = a[k];
+        if (k == k1) u = u - alpha;
+        a[k] = inv * u;
+      }
+  }
+  __syncthreads();
+  // write back V and the R part of A
+#pragma unroll
+  for (int k = 0; k < RPW; ++k) {
+    const int li = wid + QR_WARPS * k;
+    if (!t_warp && li < nloc && lane < bw) {
+      const int pi = rank + li * CS;
+      const long long gi = pb + pi;
+      V[gi * ldv + pb + lane] = pi >= lane ? a[k] : mk<R>(0, 0);
+      A[gi * lda + pb + lane] = pi < lane ? a[k] : (pi == lane ? sh.alphas[lane] : mk<R>(0, 0));
+    }
+  }
+  if (rank == 0) {
+    for (int e = tid; e < QB * QB; e += FUSED_THREADS) T[e] = sh.Ts[e / QB][e % QB];
+    // rows of the outer block above this panel: zero in its reflector columns
+    for (int e = tid; e < zr * QB; e += FUSED_THREADS)
+      if (e % QB < bw) V[(long long)(pb - zr + e / QB) * ldv + pb + e % QB] = mk<R>(0, 0);
+  }
+}
+
+constexpr int QR_KEEP_MAX = 160;
 constexpr int QNB = 128;   // outer block: 4 panels applied to the trailing matrix together
 
 // Compact-WY factor of an outer block of np_in <= 4 panels from the panels'
@@ -648,12 +935,13 @@ __global__ void qr_extract_r2_kernel(const cx<R>* Ab, long long sA, int lda, int
 }
 
 template <typename K, typename... Args>
-static cudaError_t launch_cluster_qr(K kernel, int cs, int batch, size_t smem, cudaStream_t st, Args... args) {
+static cudaError_t launch_cluster_qr(K kernel, int cs, int batch, int threads, size_t smem, cudaStream_t st,
+                                     Args... args) {
   cudaError_t e = ensure_kernel_smem((const void*)kernel, smem, cs > 8);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cs, batch, 1);
-  cfg.blockDim = dim3(QR_THREADS, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -695,17 +983,24 @@ static cudaError_t panel_factor(cudaStream_t st, cx<R>* A, long long sA, int m, 
   if (std::is_same<R, double>::value && mp >= 64) csr = 8;
   if ((mp + csr - 1) / csr > 16 * QR_WARPS) csr = 16;
   const int nl = (mp + csr - 1) / csr;
-  if (nl <= 1 * QR_WARPS)
-    return launch_cluster_qr(qr_panel_reg_kernel<R, 1>, csr, batch, 0, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT, zr);
-  if (nl <= 2 * QR_WARPS)
-    return launch_cluster_qr(qr_panel_reg_kernel<R, 2>, csr, batch, 0, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT, zr);
-  if (nl <= 4 * QR_WARPS)
-    return launch_cluster_qr(qr_panel_reg_kernel<R, 4>, csr, batch, 0, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT, zr);
-  if (nl <= 8 * QR_WARPS)
-    return launch_cluster_qr(qr_panel_reg_kernel<R, 8>, csr, batch, 0, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT, zr);
-  if (nl <= 16 * QR_WARPS)
-    return launch_cluster_qr(qr_panel_reg_kernel<R, 16>, csr, batch, 0, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT,
-                             zr);
+  // The fused kernel is the faster at every size; complex64 matrices of up to
+  // QR_KEEP_MAX rows keep the other one so that small jobs' results stay as they
+  // were (see EIGH_F64_MAX).
+  const bool fused = std::is_same<R, double>::value || m > QR_KEEP_MAX;
+  auto go = [&](auto kernel) {
+    return launch_cluster_qr(kernel, csr, batch, fused ? FUSED_THREADS : QR_THREADS, 0, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT, zr);
+  };
+#define NNE_PANEL(RPW)                                                                       \
+  if (nl <= RPW * QR_WARPS) {                                                                \
+    if (fused) return go(qr_panel_fused_kernel<R, RPW>);                                     \
+    if constexpr (std::is_same<R, float>::value) return go(qr_panel_reg_kernel<R, RPW>);     \
+  }
+  NNE_PANEL(1)
+  NNE_PANEL(2)
+  NNE_PANEL(4)
+  NNE_PANEL(8)
+  NNE_PANEL(16)
+#undef NNE_PANEL
   int cs = mp >= 512 ? 8 : (mp >= 128 ? 4 : (mp >= 32 ? 2 : 1));
   int maxloc = (mp + cs - 1) / cs;
   size_t smem = sizeof(cx<R>) * (size_t)maxloc * PS;
@@ -714,7 +1009,8 @@ static cudaError_t panel_factor(cudaStream_t st, cx<R>* A, long long sA, int m, 
     maxloc = (mp + cs - 1) / cs;
     smem = sizeof(cx<R>) * (size_t)maxloc * PS;
   }
-  return launch_cluster_qr(qr_panel_kernel<R>, cs, batch, smem, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT, maxloc, zr);
+  return launch_cluster_qr(qr_panel_kernel<R>, cs, batch, QR_THREADS, smem, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT,
+                           maxloc, zr);
 }
 
 // Blocked Householder QR.  Outer blocks of 128 columns: their four 32-column

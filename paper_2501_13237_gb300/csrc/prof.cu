@@ -117,6 +117,10 @@ MemPool::MemPool(int device) {
   }
   cuuint64_t keep = MEM_POOL_KEEP;
   cudaMemPoolSetAttribute(pool_, cudaMemPoolAttrReleaseThreshold, &keep);
+  // no reuse that makes one stream wait for another: with it a state's sub-batch
+  // streams ran one after the other (they all allocate GEMM planes)
+  int off = 0;
+  cudaMemPoolSetAttribute(pool_, cudaMemPoolReuseAllowInternalDependencies, &off);
 }
 
 MemPool::~MemPool() {
