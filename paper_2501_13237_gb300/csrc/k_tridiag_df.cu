@@ -3,10 +3,10 @@
 // quality on the float32 pipes.
 //
 // tridiag_df_kernel   the matrix in L2, lower triangle only: the first jend
-//                     columns of matrices that do not fit in shared memory;
-// tridiag_dfs_kernel  the (trailing) matrix in the shared memory of one
-//                     cluster: the whole reduction of the sizes that fit and
-//                     the rest of larger ones.
+//                     columns of matrices of more than 1024 rows;
+// tridiag_dfs_kernel  one exchange per column, the rows in the shared memory of
+//                     one cluster (sizes that fit, and the rest of larger
+//                     ones) or in L2 (up to 1024 rows).
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -18,12 +18,26 @@ namespace cg = cooperative_groups;
 
 namespace nne {
 
+// Double-float copy of a Hermitian complex64 matrix, both triangles from the lower one.
 __global__ void cx_f2df_kernel(const cx<float>* X, long long sX, int n, float4* Y, long long sY) {
   const long long count = (long long)n * n;
   const int z = blockIdx.y;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
-    const cx<float> v = X[z * sX + i];
-    Y[z * sY + i] = make_float4(v.re, 0.f, v.im, 0.f);
+    const int r = (int)(i / n), c = (int)(i % n);
+    const cx<float> v = X[z * sX + (c <= r ? i : (long long)c * n + r)];
+    Y[z * sY + i] = make_float4(v.re, 0.f, c < r ? v.im : (c > r ? -v.im : 0.f), 0.f);
+  }
+}
+
+// Upper triangle of the trailing block from row and column `off` on <- conjugate of the lower.
+__global__ void df_mirror_kernel(float4* Y, long long sY, int n0, int off) {
+  const int n = n0 - off, z = blockIdx.y;
+  const long long count = (long long)n * n;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
+    const int r = (int)(i / n), c = (int)(i % n);
+    if (c <= r) continue;
+    const float4 a = Y[z * sY + (long long)(off + c) * n0 + off + r];
+    Y[z * sY + (long long)(off + r) * n0 + off + c] = make_float4(a.x, a.y, -a.z, -a.w);
   }
 }
 
@@ -197,35 +211,53 @@ __global__ void __launch_bounds__(512) tridiag_df_kernel(float4* Hb, long long s
   }
 }
 
-// ---------------------------------------------------------------- shared-memory resident
+// ---------------------------------------------------------------- one exchange per column
 // One cluster per matrix; the rows, both triangles, are dealt cyclically to
-// its CTAs and stay in shared memory.  Thread t of every CTA owns entry t of
-// the current column, so n <= NT.
+// its CTAs.  Thread t of every CTA owns entries t, t + NT, ... (EPT of them) of
+// the current column.
 //
-// What bounds it: per column a chain of one exchange and two block sums, and
-// 3 complex multiply-adds per entry of the trailing matrix on the float32
-// pipes.  Hence
+// What bounds it: per column a chain of one exchange and two sums, and 3
+// complex multiply-adds per entry of the trailing matrix on the float32 pipes.
+// Hence
 //   * one cluster barrier per column: the CTAs push their part of p = A v to
 //     all others before it; after it every CTA forms K = v^H p, w, the next
-//     column (the stored row j+1 of its owner, read through distributed shared
-//     memory, minus its part of the rank-2 update) and the next reflector
-//     itself, with the same operations in the same order, so no second
-//     exchange is needed;
+//     column (the stored row j+1 of its owner, minus its part of the rank-2
+//     update) and the next reflector itself, with the same operations in the
+//     same order, so no second exchange is needed;
 //   * one pass over the matrix per column: the rank-2 update of column j and
 //     the product with v_{j+1} read and write each entry once;
+//   * the pivot is formed by one warp (all warps doing so cost more issue slots
+//     than the broadcast; for K, and for gathering p to push it in one piece, the
+//     extra block barrier cost more than it saved);
 //   * no float64: GB300 has two float64 lanes per SM.
 // The matrix is scaled by a power of two to a largest diagonal entry in
 // [1, 2); columns below norm 2^-50 then count as null (their squares would
 // leave float32's range, and an inaccurate norm makes a reflector that is not
 // unitary), a backward error below eps_64 ||H||.
 //
-// Source: complex64 (SRC_DF false) or the double-float trailing block of
-// tridiag_df_kernel (true), both n0 x n0 with the lower triangle valid; the
-// block starts at row and column `off` and has n = n0 - off rows.
-template <int NT, bool SRC_DF>
-__global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict__ Hsrc, long long sH, int n0, int off,
+// ROWS_C64   rows in shared memory, from the complex64 matrix (lower triangle read);
+// ROWS_DF    rows in shared memory, from the double-float trailing block at
+//            `off` that ROWS_GLOBAL left (lower triangle read), scaled by *pre already;
+// ROWS_GLOBAL  rows in place in a double-float matrix (both triangles), columns
+//            off .. jend - 1 only, the trailing block then up to date; *pre is set.
+// The block starts at row and column `off` and has n = n0 - off rows.
+enum DfRows { ROWS_C64, ROWS_DF, ROWS_GLOBAL };
+
+struct DfsLayout {   // shared memory, in float4 from the base
+  int n, cs, maxloc, nw;
+  bool global;
+  __host__ __device__ size_t rows() const { return 0; }
+  __host__ __device__ size_t v() const { return global ? 0 : (size_t)maxloc * n; }   // [2][n] reflectors of this and the last column
+  __host__ __device__ size_t w() const { return v() + 2 * (size_t)n; }               // n: w of the last column
+  __host__ __device__ size_t p() const { return w() + n; }                           // [2][n] p of all rows, pushed by their owners
+  __host__ __device__ size_t k() const { return p() + 2 * (size_t)n; }               // [2][cs][nw] float2: shares of K
+  __host__ __device__ size_t bytes() const { return 16 * k() + 2 * sizeof(float2) * (size_t)cs * nw; }
+};
+
+template <int NT, int EPT, int ROWS>
+__global__ void __launch_bounds__(NT) tridiag_dfs_kernel(void* Hsrc, long long sH, int n0, int off, int jend,
                                                          double* db, cx<double>* eb, int ldde, cx<float>* Vhb,
-                                                         long long sVh, int maxloc) {
+                                                         long long sVh, float* pre, int maxloc) {
   cg::cluster_group cluster = cg::this_cluster();
   const int CS = (int)cluster.num_blocks();
   const int rank = (int)cluster.block_rank();
@@ -233,26 +265,33 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict_
   double* d = db + (long long)z * ldde + off;
   cx<double>* e = eb + (long long)z * ldde + off;
   cx<float>* Vh = Vhb + z * sVh + (long long)off * n0 + off;
-  extern __shared__ __align__(16) unsigned char dfs_smem[];
-  float4* Hl = reinterpret_cast<float4*>(dfs_smem);     // [maxloc][n] own rows
-  float4* vb = Hl + (long long)maxloc * n;              // [2][n] reflectors of this and the last column
-  float4* wb = vb + 2 * n;                              // n: w of the last column
-  float4* pb = wb + n;                                  // [2][n] p of all rows, pushed by their owners
-  float2* kbuf = reinterpret_cast<float2*>(pb + 2 * n); // [2][CS][NW] shares of K, pushed by their warps
+  extern __shared__ __align__(16) float4 dfs_smem[];
   constexpr int NW = NT / 32;
+  const DfsLayout lay{n, CS, maxloc, NW, ROWS == ROWS_GLOBAL};
+  float4* vb = dfs_smem + lay.v();
+  float4* wb = dfs_smem + lay.w();
+  float4* pb = dfs_smem + lay.p();
+  float2* kbuf = reinterpret_cast<float2*>(dfs_smem + lay.k());
   __shared__ float2 redN[NW];
   __shared__ float redM[NW];
-  __shared__ float4 x0_s;
+  __shared__ float4 x0_s, alpha_s;
+  __shared__ float2 inv_s, K_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nloc = n > rank ? (n - rank + CS - 1) / CS : 0;
   auto source = [&](int i, int c) {   // entry (i, c), c <= i
-    if (SRC_DF)
-      return reinterpret_cast<const float4*>(Hsrc)[z * sH + (long long)(off + i) * n0 + off + c];
-    const cx<float> a = reinterpret_cast<const cx<float>*>(Hsrc)[z * sH + (long long)(off + i) * n0 + off + c];
+    const long long at = z * sH + (long long)(off + i) * n0 + off + c;
+    if (ROWS != ROWS_C64) return reinterpret_cast<const float4*>(Hsrc)[at];
+    const cx<float> a = reinterpret_cast<const cx<float>*>(Hsrc)[at];
     return make_float4(a.re, 0.f, a.im, 0.f);
   };
+  auto row_of = [&](int li) -> float4* {   // own row li
+    if (ROWS == ROWS_GLOBAL)
+      return reinterpret_cast<float4*>(Hsrc) + z * sH + (long long)(off + rank + li * CS) * n0 + off;
+    return dfs_smem + (long long)li * n;
+  };
   // power-of-two scale from the largest diagonal entry
-  float mx = tid < n ? fabsf(source(tid, tid).x) : 0.f;
+  float mx = 0.f;
+  for (int t = tid; t < n; t += NT) mx = fmaxf(mx, fabsf(source(t, t).x));
   for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (lane == 0) redM[warp] = mx;
   __syncthreads();
@@ -260,37 +299,47 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict_
   int ex = 0;
   if (mx > 0.f && mx < INFINITY) ex = min(max(ilogbf(mx), -120), 120);
   const float sc = ldexpf(1.f, -ex);
-  const double back = ldexp(1.0, ex);
-  for (long long q = tid; q < (long long)nloc * n; q += NT) {
-    const int li = (int)(q / n), c = (int)(q % n), i = rank + li * CS;
-    float4 a;
-    if (c <= i) {
-      a = source(i, c);
-    } else {
-      a = source(c, i);
-      a.z = -a.z;
-      a.w = -a.w;
+  const double back = ROWS == ROWS_DF ? ldexp((double)pre[z], ex) : ldexp(1.0, ex);
+  float4 x[EPT];   // the current column below its diagonal
+#pragma unroll
+  for (int q = 0; q < EPT; ++q) {
+    const int t = tid + q * NT;
+    x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t < n - 1) {
+      const float4 a = source(t + 1, 0);
+      x[q] = make_float4(a.x * sc, a.y * sc, a.z * sc, a.w * sc);
     }
-    if (c == i) a.z = a.w = 0.f;
-    Hl[q] = make_float4(a.x * sc, a.y * sc, a.z * sc, a.w * sc);
   }
-  // sum over the block, in the same order in every CTA (s: NW shared partials)
-  auto block_df = [&](float hi, float lo, float2* s) {
+  const float4 a00 = source(0, 0);
+  if (ROWS == ROWS_GLOBAL) {
+    cluster.sync();   // the unscaled entries have been read
+    if (rank == 0 && tid == 0) pre[z] = ldexpf(1.f, ex);
+    for (long long q = tid; q < (long long)nloc * n; q += NT) {
+      float4* a = row_of((int)(q / n)) + q % n;
+      *a = make_float4(a->x * sc, a->y * sc, a->z * sc, a->w * sc);
+    }
+  } else {
+    for (long long q = tid; q < (long long)nloc * n; q += NT) {
+      const int li = (int)(q / n), c = (int)(q % n), i = rank + li * CS;
+      float4 a;
+      if (c <= i) {
+        a = source(i, c);
+      } else {
+        a = source(c, i);
+        a.z = -a.z;
+        a.w = -a.w;
+      }
+      if (c == i) a.z = a.w = 0.f;
+      dfs_smem[q] = make_float4(a.x * sc, a.y * sc, a.z * sc, a.w * sc);
+    }
+  }
+  // warp sum of a double-float, the same bits on every lane
+  auto warp_df = [&](float hi, float lo) {
     for (int o = 16; o > 0; o >>= 1) {
       const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
       df_add(hi, lo, bh, bl);
     }
-    if (lane == 0) s[warp] = make_float2(hi, lo);
-    __syncthreads();
-    float2 t = s[lane % NW];
-    for (int o = NW / 2; o > 0; o >>= 1) {
-      const float bh = __shfl_xor_sync(0xffffffffu, t.x, o), bl = __shfl_xor_sync(0xffffffffu, t.y, o);
-      df_add(t.x, t.y, bh, bl);
-    }
-    t.x = __shfl_sync(0xffffffffu, t.x, 0);
-    t.y = __shfl_sync(0xffffffffu, t.y, 0);
-    df_norm(t.x, t.y);
-    return t;
+    return make_float2(__shfl_sync(0xffffffffu, hi, 0), __shfl_sync(0xffffffffu, lo, 0));
   };
   // b -= v conj(wk) + w conj(vk)
   auto rank2 = [](float4& b, float4 vt, float4 wt, float4 vk, float4 wk) {
@@ -305,76 +354,91 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict_
     df_norm(b.x, b.y);
     df_norm(b.z, b.w);
   };
-  // reflector r (column r below the diagonal: entry t of it is x, held by thread t < m) -> vout, Vh row r, e[r]
-  auto reflector = [&](int r, int m, float4 x, float4* vout) {
+  // reflector r (column r below the diagonal: m entries x) -> vout, Vh row r, e[r]
+  auto reflector = [&](int r, int m, float4* vout) {
     float nh = 0.f, nl = 0.f;
-    if (tid < m) {
-      df_mac(nh, nl, x.x, x.y, x.x, x.y);
-      df_mac(nh, nl, x.z, x.w, x.z, x.w);
-    }
-    if (tid == 0) x0_s = x;
-    const float2 xn2 = block_df(nh, nl, redN);
-    const float4 x0 = x0_s;
-    float2 ar = make_float2(0.f, 0.f), ai = ar, inv = ar;   // alpha, 1 / ||x - alpha e_0||
-    if (xn2.x >= 0x1p-100f) {
-      // alpha = -e^{i arg x_0} ||x||, the phase from x_0 scaled away from float32's denormal squares
-      const bool small = fmaxf(fabsf(x0.x), fabsf(x0.z)) < 0x1p-30f;
-      const float up = small ? 0x1p60f : 1.f, dn = small ? 0x1p-60f : 1.f;
-      const float2 a = make_float2(x0.x * up, x0.y * up), b = make_float2(x0.z * up, x0.w * up);
-      const float2 q2 = df_add2(df_mul2(a, a), df_mul2(b, b));
-      const float2 xn = df_mul2(xn2, df_rsqrt(xn2));
-      float2 pr = make_float2(1.f, 0.f), pi = make_float2(0.f, 0.f), ax0 = pi;
-      if (q2.x > 0x1p-100f) {
-        const float2 qi = df_rsqrt(q2);
-        pr = df_mul2(a, qi);
-        pi = df_mul2(b, qi);
-        ax0 = df_mul2(q2, qi);
-        ax0 = make_float2(ax0.x * dn, ax0.y * dn);
+#pragma unroll
+    for (int q = 0; q < EPT; ++q)
+      if (tid + q * NT < m) {
+        df_mac(nh, nl, x[q].x, x[q].y, x[q].x, x[q].y);
+        df_mac(nh, nl, x[q].z, x[q].w, x[q].z, x[q].w);
       }
-      ar = df_mul(-pr.x, -pr.y, xn.x, xn.y);
-      ai = df_mul(-pi.x, -pi.y, xn.x, xn.y);
-      const float2 u2 = df_add2(xn2, df_mul2(xn, ax0));
-      inv = df_rsqrt(make_float2(2.f * u2.x, 2.f * u2.y));
-    }
-    if (tid < m) {
-      if (tid == 0) {
-        df_add(x.x, x.y, -ar.x, -ar.y);
-        df_add(x.z, x.w, -ai.x, -ai.y);
+    if (tid == 0) x0_s = x[0];
+    const float2 part = warp_df(nh, nl);
+    if (lane == 0) redN[warp] = part;
+    __syncthreads();
+    float2 inv;
+    if (warp == 0) {
+      float2 ar = make_float2(0.f, 0.f), ai = ar;   // alpha; inv = 1 / ||x - alpha e_0||
+      inv = ar;
+      const float2 mine = lane < NW ? redN[lane] : make_float2(0.f, 0.f);
+      float2 xn2 = warp_df(mine.x, mine.y);
+      df_norm(xn2.x, xn2.y);
+      const float4 x0 = x0_s;
+      if (xn2.x >= 0x1p-100f) {
+        // alpha = -e^{i arg x_0} ||x||, the phase from x_0 scaled away from float32's denormal squares
+        const bool small = fmaxf(fabsf(x0.x), fabsf(x0.z)) < 0x1p-30f;
+        const float up = small ? 0x1p60f : 1.f, dn = small ? 0x1p-60f : 1.f;
+        const float2 a = make_float2(x0.x * up, x0.y * up), b = make_float2(x0.z * up, x0.w * up);
+        const float2 q2 = df_add2(df_mul2(a, a), df_mul2(b, b));
+        const float2 xn = df_mul2(xn2, df_rsqrt(xn2));
+        float2 pr = make_float2(1.f, 0.f), pi = make_float2(0.f, 0.f), ax0 = pi;
+        if (q2.x > 0x1p-100f) {
+          const float2 qi = df_rsqrt(q2);
+          pr = df_mul2(a, qi);
+          pi = df_mul2(b, qi);
+          ax0 = df_mul2(q2, qi);
+          ax0 = make_float2(ax0.x * dn, ax0.y * dn);
+        }
+        ar = df_mul(-pr.x, -pr.y, xn.x, xn.y);
+        ai = df_mul(-pi.x, -pi.y, xn.x, xn.y);
+        const float2 u2 = df_add2(xn2, df_mul2(xn, ax0));
+        inv = df_rsqrt(make_float2(2.f * u2.x, 2.f * u2.y));
       }
-      const float2 vr = df_mul(x.x, x.y, inv.x, inv.y), vi = df_mul(x.z, x.w, inv.x, inv.y);
-      vout[tid] = make_float4(vr.x, vr.y, vi.x, vi.y);
-      if (rank == r % CS) Vh[(long long)r * n0 + r + 1 + tid] = mk<float>(vr.x, -vi.x);
+      if (lane == 0) {
+        alpha_s = make_float4(ar.x, ar.y, ai.x, ai.y);
+        inv_s = inv;
+        if (rank == 0) e[r] = mk<double>(df_to_d(ar.x, ar.y) * back, df_to_d(ai.x, ai.y) * back);
+      }
     }
-    if (rank == 0 && tid == 0) e[r] = mk<double>(df_to_d(ar.x, ar.y) * back, df_to_d(ai.x, ai.y) * back);
+    __syncthreads();
+    inv = inv_s;
+#pragma unroll
+    for (int q = 0; q < EPT; ++q) {
+      const int t = tid + q * NT;
+      if (t < m) {
+        float4 u = x[q];
+        if (t == 0) {
+          const float4 al = alpha_s;
+          df_add(u.x, u.y, -al.x, -al.y);
+          df_add(u.z, u.w, -al.z, -al.w);
+        }
+        const float2 vr = df_mul(u.x, u.y, inv.x, inv.y), vi = df_mul(u.z, u.w, inv.x, inv.y);
+        vout[t] = make_float4(vr.x, vr.y, vi.x, vi.y);
+        if (rank == 0) Vh[(long long)r * n0 + r + 1 + t] = mk<float>(vr.x, -vi.x);
+      }
+    }
   };
-  {
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid < n - 1) {
-      const float4 a = source(tid + 1, 0);
-      x = make_float4(a.x * sc, a.y * sc, a.z * sc, a.w * sc);
-    }
-    reflector(0, n - 1, x, vb);
-    if (rank == 0 && tid == 0) {
-      const float4 a = source(0, 0);
-      d[0] = df_to_d(a.x, a.y);
-    }
-  }
+  reflector(0, n - 1, vb);
+  if (rank == 0 && tid == 0) d[0] = df_to_d(a00.x, a00.y) * (ROWS == ROWS_DF ? (double)pre[z] : 1.0);
+  int oc = 1 % CS, ol = 1 / CS;   // row j + 1: its CTA and place there
   cluster.sync();   // every CTA of the cluster runs before anyone writes into its shared memory
-  for (int j = 0; j + 2 < n; ++j) {
-    const int m = n - j - 1;
-    const float4* v = vb + (j & 1) * n;              // v_j: entry t is row j + 1 + t
-    const float4* vo = vb + ((j & 1) ^ 1) * n + 1;   // v_{j-1} at row j + 1
-    const float4* wo = wb + 1;                       // w_{j-1} at row j + 1
-    float4* p = pb + (j & 1) * n;
+  const int jlast = ROWS == ROWS_GLOBAL ? jend - off : n - 2;   // columns 0 .. jlast - 1
+  for (int j = 0; j < jlast; ++j) {
+    const int m = n - j - 1, buf = j & 1;
+    const float4* v = vb + buf * n;              // v_j: entry t is row j + 1 + t
+    const float4* vo = vb + (buf ^ 1) * n + 1;   // v_{j-1} at row j + 1
+    const float4* wo = wb + 1;                   // w_{j-1} at row j + 1
+    float4* p = pb + buf * n;
     // own rows i > j, two per warp at a time: A <- A - v_{j-1} w^H - w v_{j-1}^H
     // on columns > j, p_i = row . v_j, and this warp's share of K = v_j^H p
-    const int l0 = j + 1 > rank ? (j + 1 - rank + CS - 1) / CS : 0;
+    const int l0 = ol + (oc > rank ? 1 : 0);   // first own row > j
     float kh = 0.f, kl = 0.f;
     for (int li = l0 + warp; li < nloc; li += 2 * NW) {
       const bool two = li + NW < nloc;
       const int t = rank + li * CS - j - 1, t2 = t + NW * CS;
-      float4* row = Hl + (long long)li * n + (j + 1);
-      float4* row2 = row + (long long)NW * n;
+      float4* row = row_of(li) + (j + 1);
+      float4* row2 = row_of(two ? li + NW : li) + (j + 1);
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), acc2 = acc;
       if (j == 0) {
         for (int k = lane; k < m; k += 32) {
@@ -384,15 +448,23 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict_
         }
       } else if (two) {
         const float4 vt = vo[t], wt = wo[t], vt2 = vo[t2], wt2 = wo[t2];
+        float4 b = row[min(lane, m - 1)], b2 = row2[min(lane, m - 1)];
         for (int k = lane; k < m; k += 32) {
+          const int kn = min(k + 32, m - 1);
+          float4 nb, nb2;
+          if (ROWS == ROWS_GLOBAL) {   // the next entries' loads ahead of this one's arithmetic
+            nb = row[kn];
+            nb2 = row2[kn];
+          }
           const float4 wk = wo[k], vk = vo[k], vn = v[k];
-          float4 b = row[k], b2 = row2[k];
           rank2(b, vt, wt, vk, wk);
           rank2(b2, vt2, wt2, vk, wk);
           row[k] = b;
           row2[k] = b2;
           df_cmac<false>(acc, b, vn);
           df_cmac<false>(acc2, b2, vn);
+          b = ROWS == ROWS_GLOBAL ? nb : row[kn];
+          b2 = ROWS == ROWS_GLOBAL ? nb2 : row2[kn];
         }
       } else {
         const float4 vt = vo[t], wt = wo[t];
@@ -419,48 +491,51 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict_
         df_add(acc.x, acc.y, bh, bl);
         df_add(acc.z, acc.w, ch, cl);
       }
+      if ((lane & 15) == 0 && (!up || two)) {
+        const float4 vt = v[up ? t2 : t];
+        df_mac(kh, kl, vt.x, vt.y, acc.x, acc.y);
+        df_mac(kh, kl, vt.z, vt.w, acc.z, acc.w);
+      }
       // every CTA gets the same bits (the lanes' lo parts may differ by rounding)
       const int src = lane & 16;
       acc.x = __shfl_sync(0xffffffffu, acc.x, src);
       acc.y = __shfl_sync(0xffffffffu, acc.y, src);
       acc.z = __shfl_sync(0xffffffffu, acc.z, src);
       acc.w = __shfl_sync(0xffffffffu, acc.w, src);
-      const int tr = up ? t2 : t;
-      if (!up || two) {
-        const float4 vt = v[tr];
-        df_mac(kh, kl, vt.x, vt.y, acc.x, acc.y);
-        df_mac(kh, kl, vt.z, vt.w, acc.z, acc.w);
-        if ((lane & 15) < CS) *cluster.map_shared_rank(p + tr, lane & 15) = acc;
-      }
+      if ((!up || two) && (lane & 15) < CS) *cluster.map_shared_rank(p + (up ? t2 : t), lane & 15) = acc;
     }
     {
-      float2* kb = kbuf + (j & 1) * CS * NW;
       const float bh = __shfl_xor_sync(0xffffffffu, kh, 16), bl = __shfl_xor_sync(0xffffffffu, kl, 16);
       df_add(kh, kl, bh, bl);
       kh = __shfl_sync(0xffffffffu, kh, 0);
       kl = __shfl_sync(0xffffffffu, kl, 0);
-      if (lane < CS) *cluster.map_shared_rank(kb + rank * NW + warp, lane) = make_float2(kh, kl);
+      if (lane < CS) cluster.map_shared_rank(kbuf + ((size_t)buf * CS + rank) * NW, lane)[warp] = make_float2(kh, kl);
     }
     cluster.sync();
-    // row j + 1 (its owner's last word on it), K = v^H p
-    const int own = (j + 1) % CS;
-    const float4* rj1 = cluster.map_shared_rank(Hl + (long long)((j + 1) / CS) * n + (j + 1), own);
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid + 1 < m) {
-      a = rj1[tid + 1];
-      a.z = -a.z;   // entry (j + 2 + tid, j + 1) by symmetry
-      a.w = -a.w;
+    // row j + 1 (its owner's last word on it), and K = v^H p by every warp
+    float4 a[EPT];
+    {
+      const float4* rj1 =
+          ROWS == ROWS_GLOBAL
+              ? reinterpret_cast<const float4*>(Hsrc) + z * sH + (long long)(off + j + 1) * n0 + off + (j + 1)
+              : cluster.map_shared_rank(dfs_smem + (long long)ol * n + (j + 1), oc);
+#pragma unroll
+      for (int q = 0; q < EPT; ++q) {
+        const int t = tid + q * NT;
+        a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t + 1 < m) {
+          a[q] = ROWS == ROWS_GLOBAL ? __ldcg(rj1 + t + 1) : rj1[t + 1];
+          a[q].z = -a[q].z;   // entry (j + 2 + t, j + 1) by symmetry
+          a[q].w = -a[q].w;
+        }
+      }
     }
     float2 K = make_float2(0.f, 0.f);
     {
-      const float2* kb = kbuf + (j & 1) * CS * NW;
+      const float2* kb = kbuf + (size_t)buf * CS * NW;
       for (int q = lane; q < CS * NW; q += 32) df_add(K.x, K.y, kb[q].x, kb[q].y);
-      for (int o = 16; o > 0; o >>= 1) {
-        const float bh = __shfl_xor_sync(0xffffffffu, K.x, o), bl = __shfl_xor_sync(0xffffffffu, K.y, o);
-        df_add(K.x, K.y, bh, bl);
-      }
-      K.x = __shfl_sync(0xffffffffu, K.x, 0);
-      K.y = __shfl_sync(0xffffffffu, K.y, 0);
+      K = warp_df(K.x, K.y);
+      if (ROWS == ROWS_GLOBAL && tid == 0) K_s = K;   // for the last column's update
     }
     const float k2h = -2.f * K.x, k2l = -2.f * K.y;
     auto wof = [&](float4 vt, float4 pt) {   // w = 2 p - 2 K v
@@ -472,26 +547,35 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict_
       return w;
     };
     const float4 v0 = v[0], w0 = wof(v0, p[0]);
-    if (tid + 1 < m) {
-      const float4 vt = v[tid + 1], wt = wof(vt, p[tid + 1]);
-      wb[tid + 1] = wt;
-      rank2(a, vt, wt, v0, w0);
+#pragma unroll
+    for (int q = 0; q < EPT; ++q) {
+      const int t = tid + q * NT;
+      if (t + 1 < m) {
+        const float4 vt = v[t + 1], wt = wof(vt, p[t + 1]);
+        wb[t + 1] = wt;
+        rank2(a[q], vt, wt, v0, w0);
+      }
+      x[q] = a[q];
     }
-    if (rank == own && tid == 0) {
+    if (rank == oc && tid == 0) {
       // d[j + 1] = A[j+1][j+1] - 2 Re(v_0 conj(w_0))
-      const float4 g = Hl[(long long)((j + 1) / CS) * n + (j + 1)];
+      const float4 g = row_of(ol)[j + 1];
       float gh = g.x, gl = g.y;
       df_mac(gh, gl, -2.f * v0.x, -2.f * v0.y, w0.x, w0.y);
       df_mac(gh, gl, -2.f * v0.z, -2.f * v0.w, w0.z, w0.w);
       d[j + 1] = df_to_d(gh, gl) * back;
     }
-    if (j + 3 < n) {
-      reflector(j + 1, m - 1, a, vb + ((j & 1) ^ 1) * n);
-    } else if (tid == 0) {
+    if (++oc == CS) {   // to row j + 2
+      oc = 0;
+      ++ol;
+    }
+    if (ROWS == ROWS_GLOBAL ? j + 1 < jlast : j + 3 < n) {
+      reflector(j + 1, m - 1, vb + (buf ^ 1) * n);
+    } else if (ROWS != ROWS_GLOBAL && tid == 0) {
       // the last 2 x 2 block: subdiagonal, and the corner by its owner
-      if (rank == 0) e[n - 2] = mk<double>(df_to_d(a.x, a.y) * back, df_to_d(a.z, a.w) * back);
+      if (rank == 0) e[n - 2] = mk<double>(df_to_d(x[0].x, x[0].y) * back, df_to_d(x[0].z, x[0].w) * back);
       if (rank == (n - 1) % CS) {
-        const float4 g = Hl[(long long)((n - 1) / CS) * n + (n - 1)], v1 = v[1], w1 = wof(v1, p[1]);
+        const float4 g = dfs_smem[(long long)((n - 1) / CS) * n + (n - 1)], v1 = v[1], w1 = wb[1];
         float gh = g.x, gl = g.y;
         df_mac(gh, gl, -2.f * v1.x, -2.f * v1.y, w1.x, w1.y);
         df_mac(gh, gl, -2.f * v1.z, -2.f * v1.w, w1.z, w1.w);
@@ -499,6 +583,34 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(const void* __restrict_
       }
     }
     __syncthreads();
+  }
+  if (ROWS == ROWS_GLOBAL) {
+    // the last column's rank-2 update of the trailing block (rows and columns jlast and on; v_{jlast-1}
+    // and w at row jlast are entries 0, which wb does not hold: w_0 is not needed beyond row jlast)
+    const int j = jlast - 1, m = n - j - 1;
+    const float4* v = vb + (j & 1) * n;
+    const float k2h = -2.f * K_s.x, k2l = -2.f * K_s.y;
+    if (tid == 0) {
+      const float4 pt = pb[(j & 1) * n], vt = v[0];
+      float4 w = make_float4(2.f * pt.x, 2.f * pt.y, 2.f * pt.z, 2.f * pt.w);
+      df_mac(w.x, w.y, k2h, k2l, vt.x, vt.y);
+      df_mac(w.z, w.w, k2h, k2l, vt.z, vt.w);
+      df_norm(w.x, w.y);
+      df_norm(w.z, w.w);
+      wb[0] = w;
+    }
+    __syncthreads();
+    for (int li = warp; li < nloc; li += NW) {
+      const int t = rank + li * CS - j - 1;
+      if (t < 0) continue;
+      float4* row = row_of(li) + (j + 1);
+      const float4 vt = v[t], wt = wb[t];
+      for (int k = lane; k < m; k += 32) {
+        float4 b = row[k];
+        rank2(b, vt, wt, v[k], wb[k]);
+        row[k] = b;
+      }
+    }
   }
   cluster.sync();   // rows of this CTA may still be read by others
 }
@@ -531,52 +643,43 @@ cudaError_t launch_df(void (*kernel)(KArgs...), int cs, int batch, int threads, 
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-size_t dfs_bytes(int n, int cs) {
-  return 16 * ((size_t)((n + cs - 1) / cs) * n + 5 * (size_t)n) + 2 * sizeof(float2) * cs * (512 / 32);
-}
 constexpr size_t DFS_SMEM = 226 * 1024;   // dynamic shared memory per CTA (227 KB less the static part)
 
-template <int NT, bool SRC_DF>
-cudaError_t dfs_nt(cudaStream_t st, const void* H, long long sH, int n0, int off, double* d, cx<double>* e, int ldde,
-                   cx<float>* Vh, long long sVh, int batch, int cs) {
-  const int n = n0 - off, maxloc = (n + cs - 1) / cs;
-  return launch_df(tridiag_dfs_kernel<NT, SRC_DF>, cs, batch, NT, dfs_bytes(n, cs), st, H, sH, n0, off, d, e, ldde, Vh,
-                   sVh, maxloc);
+// CTAs per matrix: more of them shorten a column's pass over the matrix until
+// the exchange dominates.  Twelve is the most that lets eight clusters run at once
+// on the GPU's GPCs, and 384 rows of 12 CTAs fill their shared memory.  Measured
+// (us per launch, batch of 8; in brackets the float64 kernel, above 384 rows
+// L2 kernel down to 384 rows, batch of 8): DFS_FIGURES
+constexpr int DFS_CS = 12, DFS_MAX = 384, DFS_GLOBAL_MAX = 1024;
+
+template <int NT, int EPT, int ROWS>
+cudaError_t dfs_launch(cudaStream_t st, void* H, long long sH, int n0, int off, int jend, double* d, cx<double>* e,
+                       int ldde, cx<float>* Vh, long long sVh, float* pre, int batch) {
+  const int n = n0 - off, maxloc = (n + DFS_CS - 1) / DFS_CS;
+  const size_t smem = DfsLayout{n, DFS_CS, maxloc, NT / 32, ROWS == ROWS_GLOBAL}.bytes();
+  if (n < 3 || n > NT * EPT || smem > DFS_SMEM) return cudaErrorInvalidValue;
+  return launch_df(tridiag_dfs_kernel<NT, EPT, ROWS>, DFS_CS, batch, NT, smem, st, H, sH, n0, off, jend, d, e, ldde, Vh,
+                   sVh, pre, maxloc);
 }
 
 }  // namespace
 
-// CTAs per matrix: more of them shorten a column's pass over the matrix until
-// the exchange (about 2.5 us per column) dominates.  Measured on batches of 5 (us
-// per launch on 4 / 8 / 12 CTAs; the float64 kernel in brackets): n = 180: 959 /
-// 740 / 670 (1866), 256: - / 1373 / 1239 (4175), 384: - / - / 2764.  Twelve is the
-// most that lets eight clusters run at once on the GPU's GPCs (sixteen: 2572 for
-// five matrices of 384, two waves for eight), and 384 rows of 12 CTAs fill their
-// shared memory.
-constexpr int DFS_CS = 12, DFS_MAX = 384;
-
-static cudaError_t tridiag_dfs(cudaStream_t st, bool src_df, const void* H, long long sH, int n0, int off, double* d,
-                               cx<double>* e, int ldde, cx<float>* Vh, long long sVh, int batch) {
-  const int n = n0 - off;
-  if (n < 3 || n > DFS_MAX || dfs_bytes(n, DFS_CS) > DFS_SMEM) return cudaErrorInvalidValue;
-  if (src_df) return dfs_nt<512, true>(st, H, sH, n0, off, d, e, ldde, Vh, sVh, batch, DFS_CS);
-  if (n <= 256) return dfs_nt<256, false>(st, H, sH, n0, off, d, e, ldde, Vh, sVh, batch, DFS_CS);
-  return dfs_nt<512, false>(st, H, sH, n0, off, d, e, ldde, Vh, sVh, batch, DFS_CS);
-}
-
 // d, e (T[k+1][k] = e[k]) and the float32 reflectors (row j of Vh, conjugated,
 // columns j + 1 on; the rest of Vh untouched) of the Hermitian H[z] (n x n,
 // lower triangle read).  Up to DFS_MAX rows the whole reduction runs in shared
-// memory; above, the L2-resident kernel takes the columns until the trailing
-// block fits.  work: batch x n x n float4 (n > DFS_MAX only), P: batch x n
-// float4, Kp: batch x 32 float2.
+// memory; above, on rows in L2 until the trailing block fits (beyond
+// DFS_GLOBAL_MAX rows with the two-barrier kernel first, whose vectors are not
+// tied to a thread each).  work: batch x n x n float4 (n > DFS_MAX only), P:
+// batch x n float4, Kp: batch x 32 float2.
 cudaError_t tridiag_df(cudaStream_t st, const cx<float>* H, long long sH, int n, float4* work, float4* P, float2* Kp,
                        double* d, cx<double>* e, cx<float>* Vh, int batch) {
   const long long nn = (long long)n * n;
   cudaError_t ce;
   if (n <= DFS_MAX) {
     ProfScope ps(st, K_TRIDIAG, 1, 16.0 / 3.0 * (double)n * n * n * batch);
-    return tridiag_dfs(st, false, H, sH, n, 0, d, e, n, Vh, nn, batch);
+    void* h = const_cast<cx<float>*>(H);
+    if (n <= 256) return dfs_launch<256, 1, ROWS_C64>(st, h, sH, n, 0, 0, d, e, n, Vh, nn, nullptr, batch);
+    return dfs_launch<512, 1, ROWS_C64>(st, h, sH, n, 0, 0, d, e, n, Vh, nn, nullptr, batch);
   }
   {
     ProfScope ps(st, K_ELEMWISE);
@@ -584,14 +687,23 @@ cudaError_t tridiag_df(cudaStream_t st, const cx<float>* H, long long sH, int n,
     cx_f2df_kernel<<<grid, 256, 0, st>>>(H, sH, n, work, nn);
     if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
   }
-  ProfScope ps(st, K_TRIDIAG, 2, 16.0 / 3.0 * (double)n * n * n * batch);
-  const int cs = tridiag64_cluster_size((const void*)tridiag_df_kernel<TRIDIAG_DF_UNROLL>);
-  const size_t smem = std::max<size_t>(32 * (size_t)n, TRIDIAG64_SMEM);
-  const int jend = n - DFS_MAX;
-  if ((ce = launch_df(tridiag_df_kernel<TRIDIAG_DF_UNROLL>, cs, batch, TRIDIAG_DF_THREADS, smem, st, work, nn, n, d, e,
-                      n, P, Kp, Vh, nn, jend)) != cudaSuccess)
+  ProfScope ps(st, K_TRIDIAG, n > DFS_GLOBAL_MAX ? 4 : 2, 16.0 / 3.0 * (double)n * n * n * batch);
+  int off = 0;
+  if (n > DFS_GLOBAL_MAX) {
+    const int cs = tridiag64_cluster_size((const void*)tridiag_df_kernel<TRIDIAG_DF_UNROLL>);
+    const size_t smem = std::max<size_t>(32 * (size_t)n, TRIDIAG64_SMEM);
+    off = n - DFS_GLOBAL_MAX;
+    if ((ce = launch_df(tridiag_df_kernel<TRIDIAG_DF_UNROLL>, cs, batch, TRIDIAG_DF_THREADS, smem, st, work, nn, n, d,
+                        e, n, P, Kp, Vh, nn, off)) != cudaSuccess)
+      return ce;
+    df_mirror_kernel<<<dim3(1024, batch), 256, 0, st>>>(work, nn, n, off);
+    if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
+  }
+  float* pre = reinterpret_cast<float*>(Kp);
+  if ((ce = dfs_launch<512, 2, ROWS_GLOBAL>(st, work, nn, n, off, n - DFS_MAX, d, e, n, Vh, nn, pre, batch)) !=
+      cudaSuccess)
     return ce;
-  return tridiag_dfs(st, true, work, nn, n, jend, d, e, n, Vh, nn, batch);
+  return dfs_launch<512, 1, ROWS_DF>(st, work, nn, n, n - DFS_MAX, 0, d, e, n, Vh, nn, pre, batch);
 }
 
 }  // namespace nne

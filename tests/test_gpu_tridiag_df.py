@@ -1,6 +1,6 @@
 """Double-float reduction of the truncation's eigenproblem at the edges of its
 launch shapes: 4 chi x 4 chi Gram matrices below the double-float sizes, of 256
-and 512 threads, at the shared-memory limit (384) and above it (the first columns in L2).
+and 512 threads, at the shared-memory limit (384) and above it (the first columns on rows in L2).
 One complex64 gate step of a product gate with weak noise per size -- the middle
 bond equals the kept rank, so the cut is gapped -- against the exact SVD update."""
 import math
@@ -22,7 +22,7 @@ def haar_u2(rng):
 
 
 @pytest.mark.parametrize("direction", [+1, -1])
-@pytest.mark.parametrize("chi", [40, 41, 53, 64, 65, 96, 97, 110])
+@pytest.mark.parametrize("chi", [40, 41, 53, 64, 65, 96, 97, 110, 256])
 def test_gate_step_sizes(chi, direction):
     require_gpu()
     from paper_2501_13237_gb300 import nne
