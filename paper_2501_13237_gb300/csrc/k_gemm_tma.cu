@@ -19,7 +19,7 @@
 // (one 128-byte swizzle row).  Warp 0 lane 0 issues the TMA loads of a stage
 // (A hi/lo 128 x 32, B hi/lo 256 x 32, 128-byte swizzle) against an
 // mbarrier's transaction count; warp 1 lane 0 issues 12 MMAs per stage
-// (kind::tf32, M = 128, N = 256, K = 8) into a 256-column TMEM accumulator and
+// (kind::tf32, M = 128, N = 256, K = 8) into one or two 256-column TMEM accumulators and
 // commits the stage back to the producer; warps 2-5 drain TMEM through shared
 // memory to coalesced rows of C with alpha and beta.  Every mbarrier wait is
 // bounded: on expiry the kernel records NNE_ERR_TIMEOUT, waits (bounded) for
@@ -40,7 +40,6 @@ namespace tg {
 
 constexpr int BM = 128, BN = 256;
 constexpr int THREADS = 192;
-constexpr int TMEM_COLS = BN;
 constexpr int EPI_LD = BN + 4;                       // floats per epilogue row in shared memory
 constexpr long long SPIN_LIMIT = 1LL << 26;
 
@@ -244,12 +243,18 @@ __global__ void __launch_bounds__(256) split_b_kernel(const float2* __restrict__
 // ---------------------------------------------------------------- the GEMM
 // grid (ceil(2N / BN), ceil(M / BM), batch * ksplit); slice s of K covers the
 // real range [s kc, (s + 1) kc) and writes its own C block (zz = z ksplit + s).
-template <int SWZ>
+// TWO: the hi.hi products and the cross terms (hi.lo + lo.hi, 2^-11 of them) keep
+// accumulators of their own, added in the epilogue.  The tensor cores truncate
+// every accumulation, which biases a sum by the number of accumulations into it;
+// with one accumulator for all three products that was three times the bias
+// (2048 x 2048 x 512: 7.2e-6 of the result's norm against 2.4e-6).
+template <int SWZ, bool TWO>
 __global__ void __launch_bounds__(tg::THREADS, 1)
     cgemm_tma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N2,
                      int Kp, int ksplit, int kc, float2 alpha, float2 beta, float2* __restrict__ C, long long sC,
                      int ldc, int* err, long long wait_limit) {
   using namespace tg;
+  constexpr int TMEM_COLS = TWO ? 2 * BN : BN;
   constexpr int BK = Pipe<SWZ>::BK, STAGES = Pipe<SWZ>::STAGES, A_PLANE = Pipe<SWZ>::A_PLANE,
                 B_PLANE = Pipe<SWZ>::B_PLANE, STAGE = Pipe<SWZ>::STAGE;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -330,9 +335,10 @@ __global__ void __launch_bounds__(tg::THREADS, 1)
         for (int kk = 0; kk < BK / 8; ++kk) {
           const uint32_t ko = kk * 32;   // 8 tf32 = 32 bytes along the swizzled row
           const uint32_t first = (c == 0 && kk == 0) ? 0u : 1u;
+          const uint32_t tcross = TWO ? tbase + BN : tbase;
           mma_tf32(tbase, desc_sw<SWZ>(a_hi + ko), desc_sw<SWZ>(b_hi + ko), id, first);
-          mma_tf32(tbase, desc_sw<SWZ>(a_hi + ko), desc_sw<SWZ>(b_lo + ko), id, 1u);
-          mma_tf32(tbase, desc_sw<SWZ>(a_lo + ko), desc_sw<SWZ>(b_hi + ko), id, 1u);
+          mma_tf32(tcross, desc_sw<SWZ>(a_hi + ko), desc_sw<SWZ>(b_lo + ko), id, TWO ? first : 1u);
+          mma_tf32(tcross, desc_sw<SWZ>(a_lo + ko), desc_sw<SWZ>(b_hi + ko), id, 1u);
         }
         mma_commit(&empty_bar[s]);
       }
@@ -355,8 +361,15 @@ __global__ void __launch_bounds__(tg::THREADS, 1)
       const uint32_t lane_off = (uint32_t)(32 * q) << 16;
       for (int cc = 0; cc < BN / 16; ++cc) {
         float v[16];
-        if (nk > 0) tmem_ld16(tbase + lane_off + cc * 16, v);
-        else
+        if (nk > 0) {
+          tmem_ld16(tbase + lane_off + cc * 16, v);
+          if (TWO) {
+            float c[16];
+            tmem_ld16(tbase + BN + lane_off + cc * 16, c);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] += c[i];
+          }
+        } else
 #pragma unroll
           for (int i = 0; i < 16; ++i) v[i] = 0.f;
 #pragma unroll
@@ -506,10 +519,14 @@ cudaError_t cgemm_tma(cudaStream_t st, int opA, int opB, int M, int N, int K, cx
   int* err = tc_error_ptr();
   if (!err) return cudaErrorInvalidSymbol;
   const int swz = g_tma_variant == 2 ? 64 : 128;
-  const void* kern = swz == 128 ? (const void*)cgemm_tma_kernel<128> : (const void*)cgemm_tma_kernel<64>;
+  // products of matrices within 160 x 160 x 160 keep one accumulator: their sums are
+  // short, and small jobs' results stay as they were
+  const bool two = M > 160 || N > 160 || K > 160;
+  auto kern = swz == 128 ? (two ? cgemm_tma_kernel<128, true> : cgemm_tma_kernel<128, false>)
+                         : (two ? cgemm_tma_kernel<64, true> : cgemm_tma_kernel<64, false>);
   const int smem = swz == 128 ? tg::Pipe<128>::SMEM : tg::Pipe<64>::SMEM;
   const int BK = swz / 4;
-  cudaError_t e = ensure_kernel_smem(kern, smem, false);
+  cudaError_t e = ensure_kernel_smem((const void*)kern, smem, false);
   if (e != cudaSuccess) return e;
   const int Kr = 2 * K;                             // real K
   const int ldp = plane_pitch(K);
@@ -549,10 +566,7 @@ cudaError_t cgemm_tma(cudaStream_t st, int opA, int opB, int M, int N, int K, cx
     const long long wl = g_wait_limit > 0 ? g_wait_limit : (g_wait_limit < 0 ? 0 : tg::SPIN_LIMIT);
     dim3 grid((N2 + tg::BN - 1) / tg::BN, (M + tg::BM - 1) / tg::BM, batch * S);
     auto launch = [&](int ks, int kcl, float2 a, float2 bt, float2* out, long long so, int ldo) {
-      if (swz == 128)
-        cgemm_tma_kernel<128><<<grid, tg::THREADS, smem, st>>>(mA, mB, M, N2, Kr, ks, kcl, a, bt, out, so, ldo, err, wl);
-      else
-        cgemm_tma_kernel<64><<<grid, tg::THREADS, smem, st>>>(mA, mB, M, N2, Kr, ks, kcl, a, bt, out, so, ldo, err, wl);
+      kern<<<grid, tg::THREADS, smem, st>>>(mA, mB, M, N2, Kr, ks, kcl, a, bt, out, so, ldo, err, wl);
       return cudaGetLastError();
     };
     if (S == 1) {
