@@ -20,12 +20,19 @@
 // through the interior sites.
 // Accumulation: float64 for complex128 states; for complex64 states the
 // products are formed in float32, summed in float32 over at most 16 terms and
-// then added into float64 accumulators.  Each environment is rescaled to
-// max-abs 1 and its log-scale carried separately, so long chains neither
-// overflow nor underflow.
+// then added into double-float accumulators (48 bits).  A float64 instruction of a
+// warp takes 64 cycles here, and the float64 folds, warp sums, reciprocals and
+// logarithms of an earlier build were most of the sweep's time; the per-site
+// vectors and the environments travel as double-floats too.  Each environment is
+// rescaled by a power of two to max-abs in [1, 2) (exact, an integer addition) and
+// its exponent carried separately, so long chains neither overflow nor underflow.
+// 40 sites of bonds 512, 4 instances, complex64: 1.55 -> 0.78 ms (2.08 GB: 2.7 TB/s).
 #include <map>
 #include <mutex>
 
+#include <type_traits>
+
+#include "df.cuh"
 #include "kernels.cuh"
 
 namespace cg = cooperative_groups;
@@ -63,6 +70,54 @@ constexpr int RING_STAGES = 4;   // batches in flight per thread (cp.async ring 
 template <typename R> struct Vec;
 template <> struct Vec<float> { static constexpr int V = 2; };
 template <> struct Vec<double> { static constexpr int V = 1; };
+
+// Accumulators, environments and per-site vectors: double-float for complex64
+// states, float64 for complex128 ones; 16 bytes either way.
+template <typename R> struct Env;
+template <> struct Env<float> { using T = float4; };    // {re_hi, re_lo, im_hi, im_lo}
+template <> struct Env<double> { using T = cx<double>; };
+
+__device__ __forceinline__ void env_zero(float4& a) { a = make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ void env_zero(cx<double>& a) { a = mk<double>(0, 0); }
+__device__ __forceinline__ void env_fold(float4& a, cx<float> s) {
+  df_add(a.x, a.y, s.re, 0.f);
+  df_add(a.z, a.w, s.im, 0.f);
+}
+__device__ __forceinline__ void env_fold(cx<double>& a, cx<double> s) { a = a + s; }
+__device__ __forceinline__ float4 env_add(float4 a, float4 b) {
+  df_add(a.x, a.y, b.x, b.y);
+  df_add(a.z, a.w, b.z, b.w);
+  df_norm(a.x, a.y);
+  df_norm(a.z, a.w);
+  return a;
+}
+__device__ __forceinline__ cx<double> env_add(cx<double> a, cx<double> b) { return a + b; }
+__device__ __forceinline__ float4 env_shfl_xor(float4 a, int o) {
+  return make_float4(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o),
+                     __shfl_xor_sync(0xffffffffu, a.z, o), __shfl_xor_sync(0xffffffffu, a.w, o));
+}
+__device__ __forceinline__ cx<double> env_shfl_xor(cx<double> a, int o) { return shfl_xor(a, o); }
+__device__ __forceinline__ cx<double> env_d(float4 a) { return mk<double>(df_to_d(a.x, a.y), df_to_d(a.z, a.w)); }
+__device__ __forceinline__ cx<double> env_d(cx<double> a) { return a; }
+// Leading bits of the larger component: orders magnitudes, and holds the exponent.
+__device__ __forceinline__ int env_key(float4 a) { return max(__float_as_int(a.x) & 0x7fffffff, __float_as_int(a.z) & 0x7fffffff); }
+__device__ __forceinline__ int env_key(cx<double> a) { return max(__double2hiint(a.re) & 0x7fffffff, __double2hiint(a.im) & 0x7fffffff); }
+template <typename R>
+__device__ __forceinline__ int key_exp(int key) {   // binary exponent, 0 for a zero environment
+  const int f = std::is_same<R, float>::value ? key >> 23 : key >> 20;
+  return f == 0 ? 0 : f - (std::is_same<R, float>::value ? 127 : 1023);
+}
+// a 2^-e
+__device__ __forceinline__ float4 env_scale(float4 a, int e) {
+  const float h0 = __int_as_float((127 - e / 2) << 23), h1 = __int_as_float((127 - (e - e / 2)) << 23);
+  return make_float4(a.x * h0 * h1, a.y * h0 * h1, a.z * h0 * h1, a.w * h0 * h1);
+}
+__device__ __forceinline__ cx<double> env_scale(cx<double> a, int e) {
+  const double h0 = __hiloint2double((1023 - e / 2) << 20, 0), h1 = __hiloint2double((1023 - (e - e / 2)) << 20, 0);
+  return mk<double>(a.re * h0 * h1, a.im * h0 * h1);
+}
+__device__ __forceinline__ cx<float> env_coef(float4 a) { return mk<float>(a.x, a.z); }
+__device__ __forceinline__ cx<double> env_coef(cx<double> a) { return a; }
 
 // Streaming loads (site tensors are read once per pass).
 template <typename R, int V>
@@ -108,17 +163,13 @@ __device__ __forceinline__ void ring_read(const unsigned char* ring_ptr, int st,
   for (int v = 0; v < V; ++v) o[v] = reinterpret_cast<const cx<R>*>(p)[v];
 }
 
-__device__ __forceinline__ cx<double> up(cx<float> a) { return mk<double>(a.re, a.im); }
-__device__ __forceinline__ cx<double> up(cx<double> a) { return a; }
-
-// Shared-memory layout of env_cluster_kernel, in cx<double> units from the base.
+// Shared-memory layout of env_cluster_kernel, in 16-byte units from the base.
 struct Layout {
   int D, SL;
-  __host__ __device__ int cur() const { return 0; }                 // D: current environment (float64)
-  __host__ __device__ int slice() const { return D; }               // 2 x SL: this CTA's slice of the next one
-  __host__ __device__ int fin() const { return D + 2 * SL; }        // 4 x SL: left-pass results of this CTA
-  __host__ __device__ int part() const { return D + 6 * SL; }       // 2 x THREADS: row-group partial sums
-  __host__ __device__ int scal() const { return D + 6 * SL + 2 * THREADS; }   // 8 doubles (maxes, reduction)
+  __host__ __device__ int slice() const { return 0; }           // 2 x SL: this CTA's slice of the next environment
+  __host__ __device__ int fin() const { return 2 * SL; }        // 4 x SL: left-pass results of this CTA
+  __host__ __device__ int part() const { return 6 * SL; }       // 2 x THREADS: row-group partial sums
+  __host__ __device__ int scal() const { return 6 * SL + 2 * THREADS; }   // 32 ints: every CTA's key, double-buffered
   __host__ __device__ int coef() const { return scal() + 8; }       // D x cx<R>: environment in the state's precision
   // per-thread rings of asynchronous copies (RING_STAGES x NB 16-byte slots per thread), 16-byte aligned
   __host__ __device__ size_t ring_off(size_t esz) const { return (16 * (size_t)coef() + esz * (size_t)D + 15) & ~size_t(15); }
@@ -127,13 +178,13 @@ struct Layout {
 
 __host__ __device__ inline int slice_cap(int D, int cs) { return (D + cs - 1) / cs + 2; }
 
-__device__ __forceinline__ double block_max_sw(double v, double* red) {
-  for (int m = 16; m > 0; m >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, m));
+__device__ __forceinline__ int block_max_key(int v, int* red) {
+  for (int m = 16; m > 0; m >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, m));
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  double t = 0;
-  for (int i = 0; i < THREADS / 32; ++i) t = fmax(t, red[i]);
+  int t = 0;
+  for (int i = 0; i < THREADS / 32; ++i) t = max(t, red[i]);
   return t;
 }
 
@@ -143,7 +194,8 @@ __device__ __forceinline__ double block_max_sw(double v, double* red) {
 // in flight.
 template <typename R, int V>
 __device__ void left_site(const cx<R>* __restrict__ M, int dl, int dr, int b0, int w, const cx<R>* coef,
-                          cx<double>* fin, int SL, cx<double>* part, unsigned char* ring_ptr) {
+                          typename Env<R>::T* fin, int SL, typename Env<R>::T* part, unsigned char* ring_ptr) {
+  using T = typename Env<R>::T;
   constexpr int BYTES = (int)sizeof(cx<R>) * V;
   const uint32_t ring = (uint32_t)__cvta_generic_to_shared(ring_ptr);
   const int t = threadIdx.x;
@@ -153,9 +205,9 @@ __device__ void left_site(const cx<R>* __restrict__ M, int dl, int dr, int b0, i
   for (int u0 = 0; u0 < U; u0 += THREADS) {
     const int u = u0 + (G > 1 ? t % U : t), g = G > 1 ? t / U : 0;
     const bool act = u < U && g < G;
-    cx<double> acc[V];
+    T acc[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) acc[v] = mk<double>(0, 0);
+    for (int v = 0; v < V; ++v) env_zero(acc[v]);
     if (act) {
       const int s = u / wu, j = (u % wu) * V;
       const cx<R>* col = M + (long long)s * dr + b0 + j;
@@ -191,7 +243,7 @@ __device__ void left_site(const cx<R>* __restrict__ M, int dl, int dr, int b0, i
           for (int v = 0; v < V; ++v) fma_(s32[v], c, m[v]);
         }
 #pragma unroll
-        for (int v = 0; v < V; ++v) acc[v] = acc[v] + up(s32[v]);
+        for (int v = 0; v < V; ++v) env_fold(acc[v], s32[v]);
       }
       cp_wait_all();
     }
@@ -211,8 +263,8 @@ __device__ void left_site(const cx<R>* __restrict__ M, int dl, int dr, int b0, i
         const int s = t / wu, j = (t % wu) * V;
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-          cx<double> tot = mk<double>(0, 0);
-          for (int gg = 0; gg < G; ++gg) tot = tot + part[(gg * U + t) * V + v];
+          T tot = part[t * V + v];
+          for (int gg = 1; gg < G; ++gg) tot = env_add(tot, part[(gg * U + t) * V + v]);
           fin[s * SL + j + v] = tot;
         }
       }
@@ -221,12 +273,13 @@ __device__ void left_site(const cx<R>* __restrict__ M, int dl, int dr, int b0, i
 }
 
 // Right pass at one site: rho[tt][a] = sum_b M[a][tt][b] coef[b] for this CTA's rows, one warp per row.
-// Writes rho to global memory and R[a] = rho[0][a] + rho[3][a] into the slice; returns the row max-abs.
+// Writes rho to global memory and R[a] = rho[0][a] + rho[3][a] into the slice; returns the rows' largest key.
 // A warp's work is a flat list of jobs (row, segment tt, batch of 32 NB units),
 // streamed through each lane's ring of asynchronous copies.
 template <typename R, int V>
-__device__ double right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, const cx<R>* coef, cx<double>* rho,
-                             int D, cx<double>* slice, unsigned char* ring_ptr) {
+__device__ int right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, const cx<R>* coef,
+                          typename Env<R>::T* rho, int D, typename Env<R>::T* slice, unsigned char* ring_ptr) {
+  using T = typename Env<R>::T;
   constexpr int BYTES = (int)sizeof(cx<R>) * V;
   const uint32_t ring = (uint32_t)__cvta_generic_to_shared(ring_ptr);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = THREADS / 32;
@@ -254,12 +307,14 @@ __device__ double right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1
   };
 #pragma unroll
   for (int b = 0; b < RING_STAGES - 1; ++b) issue(b);
-  double mx = 0;
-  cx<double> acc = mk<double>(0, 0), seg0 = mk<double>(0, 0);
+  int key = 0;
+  T acc0, acc1, acc2, acc3;   // the four segments of the row
+  env_zero(acc0);
+  acc1 = acc2 = acc3 = acc0;
+  int ri = 0, tt = 0, bb = 0;
   for (int jb = 0; jb < jobs; ++jb) {
     issue(jb + RING_STAGES - 1);
     cp_wait_ring();
-    const int ri = jb / (4 * nbs), rem = jb % (4 * nbs), tt = rem / nbs, bb = rem % nbs;
     cx<R> s32 = mk<R>(0, 0);
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
@@ -270,128 +325,145 @@ __device__ double right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1
 #pragma unroll
         for (int v = 0; v < V; ++v) fma_(s32, m[v], coef[uu * V + v]);
     }
-    acc = acc + up(s32);
-    if (bb == nbs - 1) {   // segment tt of row a complete
-      const cx<double> tot = warp_sum(acc);
-      acc = mk<double>(0, 0);
+    if (tt == 0) env_fold(acc0, s32);
+    else if (tt == 1) env_fold(acc1, s32);
+    else if (tt == 2) env_fold(acc2, s32);
+    else env_fold(acc3, s32);
+    if (++bb == nbs) {
+      bb = 0;
+      ++tt;
+    }
+    if (tt == 4) {
+      // row complete: the four sums over the warp in five steps; lanes 8 q .. 8 q + 7 end with segment q's
+      const bool up = lane & 16, up8 = lane & 8;
+      T x = up ? acc2 : acc0, y = up ? acc3 : acc1;
+      x = env_add(x, env_shfl_xor(up ? acc0 : acc2, 16));
+      y = env_add(y, env_shfl_xor(up ? acc1 : acc3, 16));
+      T w = env_add(up8 ? y : x, env_shfl_xor(up8 ? x : y, 8));
+      for (int o = 4; o > 0; o >>= 1) w = env_add(w, env_shfl_xor(w, o));
       const int a = a0 + warp + ri * nw;
-      if (lane == 0) rho[(long long)tt * D + a] = tot;
-      if (tt == 0) seg0 = tot;
-      if (tt == 3 && lane == 0) {
-        const cx<double> Ra = seg0 + tot;
+      if ((lane & 7) == 0) rho[(long long)(lane >> 3) * D + a] = w;
+      const T Ra = env_add(w, env_shfl_xor(w, 24));   // lane 0: segments 0 and 3
+      if (lane == 0) {
         slice[a - a0] = Ra;
-        mx = fmax(mx, fmax(fabs(Ra.re), fabs(Ra.im)));
+        key = max(key, env_key(Ra));
       }
+      env_zero(acc0);
+      acc1 = acc2 = acc3 = acc0;
+      tt = 0;
+      ++ri;
     }
   }
   cp_wait_all();
-  return mx;
+  return key;
 }
+
+// sum_s v_P[s] x_s: two of the four vectors, with a sign or a factor +-i.
+__device__ __forceinline__ float4 env_neg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
+__device__ __forceinline__ cx<double> env_neg(cx<double> a) { return mk<double>(-a.re, -a.im); }
+__device__ __forceinline__ float4 env_times_i(float4 a) { return make_float4(-a.z, -a.w, a.x, a.y); }
+__device__ __forceinline__ cx<double> env_times_i(cx<double> a) { return mk<double>(-a.im, a.re); }
+template <typename T>
+__device__ __forceinline__ T pauli_sum(int p, T x0, T x1, T x2, T x3) {
+  if (p == 0) return env_add(x0, x3);
+  if (p == 1) return env_add(x1, x2);
+  if (p == 2) return env_times_i(env_add(x1, env_neg(x2)));
+  return env_add(x0, env_neg(x3));
+}
+__device__ __forceinline__ void env_mac(float4& acc, float4 a, float4 b) { df_cmac<false>(acc, a, b); }
+__device__ __forceinline__ void env_mac(cx<double>& acc, cx<double> a, cx<double> b) { fma_(acc, a, b); }
+__device__ __forceinline__ float4 env_from_d(cx<double> a, float4) { return df_from_cd(a); }
+__device__ __forceinline__ cx<double> env_from_d(cx<double> a, cx<double>) { return a; }
 
 }  // namespace sweep
 
 // Both environment sweeps and the per-site partial contractions in one launch.
 // grid (cs, 2, n_inst), cluster (cs, 1, 1): cluster (pass, z); pass 0 left, 1 right.
-// env: [z][pass][k = 0..n][D] complex double, envscale: [z][pass][k], vecs: [z][pass][k = 0..n-1][4][D].
+// env: [z][pass][k = 0..n][D] complex double, envscale: [z][pass][k], vecs: [z][pass][k = 0..n-1][4][D] Env<R>::T.
 template <typename R>
 __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, const int* __restrict__ dims,
                                                                     const void* const* __restrict__ site,
                                                                     const long long* __restrict__ stride, int D,
                                                                     double* env, double* envscale, double* vecs) {
   using namespace sweep;
+  using T = typename Env<R>::T;
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int pass = blockIdx.y, z = blockIdx.z, t = threadIdx.x;
   constexpr int VV = Vec<R>::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Layout L{D, slice_cap(D, cs)};
-  cx<double>* base = reinterpret_cast<cx<double>*>(smem_raw);
-  cx<double>* cur = base + L.cur();
-  cx<double>* slice = base + L.slice();
-  cx<double>* fin = base + L.fin();
-  cx<double>* part = base + L.part();
-  double* scal = reinterpret_cast<double*>(base + L.scal());   // [0..1] maxes (double-buffered), [8..15] reduction
+  T* base = reinterpret_cast<T*>(smem_raw);
+  T* slice = base + L.slice();
+  T* fin = base + L.fin();
+  T* part = base + L.part();
+  int* keys = reinterpret_cast<int*>(base + L.scal());   // [2][16]
+  __shared__ int red[THREADS / 32];
   cx<R>* coef = reinterpret_cast<cx<R>*>(base + L.coef());
   unsigned char* ring_ptr = smem_raw + L.ring_off(sizeof(cx<R>));
   cx<double>* E = reinterpret_cast<cx<double>*>(env) + ((long long)z * 2 + pass) * (n + 1) * D;
   double* ls = envscale + ((long long)z * 2 + pass) * (n + 1);
-  cx<double>* VK = reinterpret_cast<cx<double>*>(vecs) + ((long long)z * 2 + pass) * n * 4 * D;
+  T* VK = reinterpret_cast<T*>(vecs) + ((long long)z * 2 + pass) * n * 4 * D;
   const int first = pass == 0 ? 0 : n;
   if (t == 0) {
-    cur[0] = mk<double>(1, 0);
     coef[0] = mk<R>(1, 0);
     if (rank == 0) {
       E[(long long)first * D] = mk<double>(1, 0);
       ls[first] = 0;
     }
   }
-  __syncthreads();
-  double lsc = 0;
+  cluster.sync();   // every CTA of the cluster runs before anyone writes into its shared memory
+  long long esum = 0;   // binary exponent of the environment
   int pb = 0;
   for (int step = 0; step < n; ++step) {
     const int k = pass == 0 ? step : n - 1 - step;
     const int dl = dims[k], dr = dims[k + 1];
     const cx<R>* M = reinterpret_cast<const cx<R>*>(site[k]) + z * stride[k];
     const bool vec = VV > 1 && dr % VV == 0 && (reinterpret_cast<uintptr_t>(M) & 15) == 0;
-    cx<double>* sl = slice + pb * L.SL;
-    double mx = 0;
-    int own0, own1;   // entries of the next environment this CTA owns
+    T* sl = slice + pb * L.SL;
+    int key = 0;
+    int width;   // entries of the next environment per CTA
     if (pass == 0) {
       const int v = vec ? VV : 1;
-      const int bs = ((dr + cs - 1) / cs + v - 1) / v * v;
-      const int b0 = min(dr, rank * bs), b1 = min(dr, b0 + bs);
-      own0 = b0;
-      own1 = b1;
+      width = ((dr + cs - 1) / cs + v - 1) / v * v;
+      const int b0 = min(dr, rank * width), b1 = min(dr, b0 + width);
       if (vec) left_site<R, VV>(M, dl, dr, b0, b1 - b0, coef, fin, L.SL, part, ring_ptr);
       else left_site<R, 1>(M, dl, dr, b0, b1 - b0, coef, fin, L.SL, part, ring_ptr);
       __syncthreads();
-      cx<double>* ell = VK + (long long)k * 4 * D;
+      T* ell = VK + (long long)k * 4 * D;
       for (int q = t; q < 4 * (b1 - b0); q += THREADS) {
         const int s = q / (b1 - b0), j = q % (b1 - b0);
         ell[(long long)s * D + b0 + j] = fin[s * L.SL + j];
       }
       for (int j = t; j < b1 - b0; j += THREADS) {
-        const cx<double> Lb = fin[j] + fin[3 * L.SL + j];
+        const T Lb = env_add(fin[j], fin[3 * L.SL + j]);
         sl[j] = Lb;
-        mx = fmax(mx, fmax(fabs(Lb.re), fabs(Lb.im)));
+        key = max(key, env_key(Lb));
       }
     } else {
-      const int rs = (dl + cs - 1) / cs;
-      const int a0 = min(dl, rank * rs), a1 = min(dl, a0 + rs);
-      own0 = a0;
-      own1 = a1;
-      cx<double>* rho = VK + (long long)k * 4 * D;
-      mx = vec ? right_site<R, VV>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr)
-               : right_site<R, 1>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr);
-    }
-    mx = block_max_sw(mx, scal + 8);
-    if (t == 0) scal[pb] = mx;
-    (void)own0;
-    (void)own1;
-    cluster.sync();   // every slice and max of this site is published
-    // the next environment, normalised to max-abs 1, gathered from the cluster's slices
-    double m = 0;
-    for (int r = 0; r < cs; ++r) m = fmax(m, *cluster.map_shared_rank(scal + pb, r));
-    const double inv = m > 0 ? 1.0 / m : 1.0;
-    const int nd = pass == 0 ? dr : dl;               // length of the next environment
-    int width;
-    if (pass == 0) {
-      const int v = vec ? VV : 1;
-      width = ((dr + cs - 1) / cs + v - 1) / v * v;
-    } else {
       width = (dl + cs - 1) / cs;
+      const int a0 = min(dl, rank * width), a1 = min(dl, a0 + width);
+      T* rho = VK + (long long)k * 4 * D;
+      key = vec ? right_site<R, VV>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr)
+                : right_site<R, 1>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr);
     }
+    key = block_max_key(key, red);
+    if (t < cs) cluster.map_shared_rank(keys, t)[16 * pb + rank] = key;
+    cluster.sync();   // every slice and key of this site is published
+    // the next environment, scaled to max-abs in [1, 2), gathered from the cluster's slices
+    int m = 0;
+    for (int r = 0; r < cs; ++r) m = max(m, keys[16 * pb + r]);
+    const int e = key_exp<R>(m);
+    const int nd = pass == 0 ? dr : dl;               // length of the next environment
     const int knext = pass == 0 ? k + 1 : k;
     for (int i = t; i < nd; i += THREADS) {
       const int r = i / width;
-      const cx<double> val = cluster.map_shared_rank(slice + pb * L.SL, r)[i - r * width];
-      const cx<double> nv = inv * val;
-      cur[i] = nv;
-      coef[i] = mk<R>((R)nv.re, (R)nv.im);
-      if (rank == 0) E[(long long)knext * D + i] = nv;
+      const T nv = env_scale(cluster.map_shared_rank(slice + pb * L.SL, r)[i - r * width], e);
+      coef[i] = env_coef(nv);
+      if (r == rank) E[(long long)knext * D + i] = env_d(nv);
     }
-    lsc += m > 0 ? log(m) : 0.0;
-    if (rank == 0 && t == 0) ls[knext] = lsc;
+    esum += e;
+    if (rank == 0 && t == 0) ls[knext] = (double)esum * 0.6931471805599453094;   // ln 2
     pb ^= 1;
     __syncthreads();
   }
@@ -481,11 +553,14 @@ __global__ void __launch_bounds__(256) obs_kernel(int n, const int* dims, const 
 // (string, instance), dot products of the stored per-site vectors:
 //   one site k:      sum_b (sum_s v_P[s] ell_k[s][b]) R_{k+1}[b]
 //   sites k, k + 1:  sum_c (sum_s v_P[s] ell_k[s][c]) (sum_t v_Q[t] rho_{k+1}[t][c])
+template <typename R>
 __global__ void __launch_bounds__(256) obs_local_kernel(int n, const int* __restrict__ dims, int D,
                                                         const double* env, const double* envscale,
                                                         const double* vecs, const uint8_t* __restrict__ paulis,
                                                         const int* __restrict__ first, const int* __restrict__ last,
                                                         int n_obs, double* out) {
+  using namespace sweep;
+  using T = typename Env<R>::T;
   const int lane = threadIdx.x & 31;
   const int o = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), z = blockIdx.y;
   if (o >= n_obs) return;
@@ -500,47 +575,32 @@ __global__ void __launch_bounds__(256) obs_local_kernel(int n, const int* __rest
   const cx<double>* ER = reinterpret_cast<const cx<double>*>(env) + ((long long)z * 2 + 1) * (n + 1) * D;
   const double* lsL = envscale + ((long long)z * 2 + 0) * (n + 1);
   const double* lsR = envscale + ((long long)z * 2 + 1) * (n + 1);
-  const cx<double>* ell = reinterpret_cast<const cx<double>*>(vecs) + (((long long)z * 2 + 0) * n + f) * 4 * D;
+  const T* ell = reinterpret_cast<const T*>(vecs) + (((long long)z * 2 + 0) * n + f) * 4 * D;
   const int P = paulis[(long long)o * n + f];
-  const cx<double> p0 = pvec(P, 0), p1 = pvec(P, 1), p2 = pvec(P, 2), p3 = pvec(P, 3);
   const int d = dims[f + 1];
-  cx<double> acc = mk<double>(0, 0);
+  T acc;
+  env_zero(acc);
   double lscale;
   if (l == f) {
     const cx<double>* Rn = ER + (long long)(f + 1) * D;
-    for (int b = lane; b < d; b += 32) {
-      cx<double> u = mk<double>(0, 0);
-      fma_(u, p0, ell[b]);
-      fma_(u, p1, ell[D + b]);
-      fma_(u, p2, ell[2 * D + b]);
-      fma_(u, p3, ell[3 * D + b]);
-      fma_(acc, u, Rn[b]);
-    }
+    for (int b = lane; b < d; b += 32)
+      env_mac(acc, pauli_sum(P, ell[b], ell[D + b], ell[2 * D + b], ell[3 * D + b]), env_from_d(Rn[b], acc));
     lscale = lsL[f] + lsR[f + 1];
   } else {
-    const cx<double>* rho = reinterpret_cast<const cx<double>*>(vecs) + (((long long)z * 2 + 1) * n + l) * 4 * D;
+    const T* rho = reinterpret_cast<const T*>(vecs) + (((long long)z * 2 + 1) * n + l) * 4 * D;
     const int Q = paulis[(long long)o * n + l];
-    const cx<double> q0 = pvec(Q, 0), q1 = pvec(Q, 1), q2 = pvec(Q, 2), q3 = pvec(Q, 3);
-    for (int c = lane; c < d; c += 32) {
-      cx<double> u = mk<double>(0, 0), w = mk<double>(0, 0);
-      fma_(u, p0, ell[c]);
-      fma_(u, p1, ell[D + c]);
-      fma_(u, p2, ell[2 * D + c]);
-      fma_(u, p3, ell[3 * D + c]);
-      fma_(w, q0, rho[c]);
-      fma_(w, q1, rho[D + c]);
-      fma_(w, q2, rho[2 * D + c]);
-      fma_(w, q3, rho[3 * D + c]);
-      fma_(acc, u, w);
-    }
+    for (int c = lane; c < d; c += 32)
+      env_mac(acc, pauli_sum(P, ell[c], ell[D + c], ell[2 * D + c], ell[3 * D + c]),
+              pauli_sum(Q, rho[c], rho[D + c], rho[2 * D + c], rho[3 * D + c]));
     lscale = lsL[f] + lsR[l + 1];
   }
-  acc = warp_sum(acc);
+  for (int m = 16; m > 0; m >>= 1) acc = env_add(acc, env_shfl_xor(acc, m));
   if (lane == 0) {
     const cx<double> tr = EL[(long long)n * D];
     const double scale = exp(lscale - lsL[n]);
     const double den = tr.re * tr.re + tr.im * tr.im;
-    const double qr = (acc.re * tr.re + acc.im * tr.im) / den, qi = (acc.im * tr.re - acc.re * tr.im) / den;
+    const cx<double> av = env_d(acc);
+    const double qr = (av.re * tr.re + av.im * tr.im) / den, qi = (av.im * tr.re - av.re * tr.im) / den;
     res[0] = qr * scale;
     res[1] = qi * scale;
   }
@@ -638,7 +698,7 @@ cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* 
   if (n_obs <= 0) return cudaSuccess;
   {
     ProfScope ps(st, K_SWEEP_OBS);
-    obs_local_kernel<<<dim3((n_obs + 7) / 8, n_inst), 256, 0, st>>>(n, d_dims, max_dim, d_env, d_envscale, d_vecs,
+    obs_local_kernel<R><<<dim3((n_obs + 7) / 8, n_inst), 256, 0, st>>>(n, d_dims, max_dim, d_env, d_envscale, d_vecs,
                                                                    d_paulis, d_first, d_last, n_obs, d_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
