@@ -1,14 +1,6 @@
 // Hermitian eigensolver pieces for matrices that fit in one cluster's shared
 // memory (n <= 640 complex64 / 448 complex128 with 16 CTAs), plus the
 // blocked (compact-WY) back-transformation shared by both reduction paths.
-//
-// Reduction: rows are spread cyclically over the CTAs of a cluster and stay
-// in shared memory for the whole reduction; column j is read from its owner
-// through distributed shared memory, every CTA forms the Householder vector
-// redundantly (identical arithmetic, so identical results; the FP64 parts on
-// one thread per CTA), the products
-// p = A v are pushed to every CTA, and one more barrier closes the rank-2
-// update.  Reflector j is stored conjugated as row j of Vh (n x n).
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -190,6 +182,290 @@ __global__ void __launch_bounds__(256) tridiag_smem_kernel(const cx<R>* Hb, long
   }
 }
 
+// Householder tridiagonalisation of the Hermitian H[z] (n x n) by one
+// cluster, the rows dealt to the CTAs cyclically and in shared memory.
+//
+// One exchange per column, as the double-float kernel (k_tridiag_df.cu): the
+// rank-2 update of column j shares a pass with the product p = A v_{j+1}; the
+// CTAs push their part of p to all others before the column's only cluster
+// barrier, and after it every CTA forms K = v^H p, w = 2p - 2Kv, the next column
+// (row j+1 of its owner, less its part of the update) and its reflector itself.
+//
+// In float64 the time is the number of float64 instructions on a column's chain
+// times 64 cycles (an SM issues one per 19 cycles, a warp one per 64, whatever
+// the lanes): two rows share a warp's reduction, single values (K, norm, pivot)
+// are formed by one warp, the pivot's parts on lanes of one instruction stream
+// and from reciprocal square roots by series instead of divides.  us per launch
+// (the earlier two-barrier kernel in brackets), float64: n = 64:
+// 387 (515), 256: 3129 (4163); float32, n = 128: 234 (328).
+// Sums run in a fixed order.
+__device__ __forceinline__ float rsqrt_series(float x) {   // hardware estimate (2 ulp), one Newton step
+  const float y = rsqrtf(x);
+  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
+}
+// From a 20-bit estimate y with r = 1 - x y^2: y (1 + r/2 + 3 r^2/8 + 5 r^3 / 16), error r^4 = 2^-76 before rounding.
+__device__ __forceinline__ double rsqrt_series(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double r = fma(-x * y, y, 1.0);
+  return fma(y * r, fma(r, fma(r, 0.3125, 0.375), 0.5), y);
+}
+// Pivots smaller than SMALL are scaled by UP before they are squared (their squares
+// would be denormal and |x0| inaccurate, and the reflector not unitary).
+template <typename R> struct PivotScale;
+template <> struct PivotScale<float> {
+  static __device__ __forceinline__ float small() { return 0x1p-50f; }
+  static __device__ __forceinline__ float up() { return 0x1p70f; }
+  static __device__ __forceinline__ float dn() { return 0x1p-70f; }
+  static __device__ __forceinline__ float floor2() { return 0.f; }         // squared norms at or below count as null
+};
+template <> struct PivotScale<double> {
+  static __device__ __forceinline__ double small() { return 0x1p-400; }
+  static __device__ __forceinline__ double up() { return 0x1p500; }
+  static __device__ __forceinline__ double dn() { return 0x1p-500; }
+  static __device__ __forceinline__ double floor2() { return 0x1p-1000; }  // the estimate flushes denormals
+};
+
+constexpr int TRI_THREADS = 256, TRI_NW = TRI_THREADS / 32;
+
+template <typename R, int EPT>
+__global__ void __launch_bounds__(TRI_THREADS) tridiag_fused_kernel(const cx<R>* Hb, long long sH, int n, R* db,
+                                                                     cx<R>* eb, int ldde, cx<R>* Vhb, long long sVh,
+                                                                     int maxloc) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CS = (int)cluster.num_blocks();
+  const int rank = (int)cluster.block_rank();
+  const int z = blockIdx.y;
+  const cx<R>* H = Hb + z * sH;
+  R* d = db + (long long)z * ldde;
+  cx<R>* e = eb + (long long)z * ldde;
+  cx<R>* Vh = Vhb + z * sVh;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<R>* Hl = reinterpret_cast<cx<R>*>(smem_raw);     // [maxloc][n] own rows
+  cx<R>* vb = Hl + (long long)maxloc * n;             // [2][n] reflectors of this and the last column
+  cx<R>* pb = vb + 2 * n;                             // [2][n] p of all rows, then w in its place
+  R* kbuf = reinterpret_cast<R*>(pb + 2 * n);         // [2][CS][NW] shares of K, pushed by their warps
+  __shared__ R redN[TRI_NW];
+  __shared__ cx<R> x0_s, alpha_s;
+  __shared__ R inv_s, K_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nloc = n > rank ? (n - rank + CS - 1) / CS : 0;
+  auto in = [&](int i, int c) { return H[(long long)i * n + c]; };
+  for (long long q = tid; q < (long long)nloc * n; q += TRI_THREADS) {
+    const int li = (int)(q / n), c = (int)(q % n), i = rank + li * CS;
+    Hl[q] = in(i, c);
+  }
+  auto warp_real = [&](R v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  cx<R> x[EPT];   // the current column below its diagonal, entries tid, tid + 256, ...
+#pragma unroll
+  for (int q = 0; q < EPT; ++q) x[q] = tid + q * TRI_THREADS < n - 1 ? conj(in(0, tid + q * TRI_THREADS + 1)) : mk<R>(0, 0);
+  // reflector r from the column x (m entries) -> vout, Vh row r, e[r]
+  auto reflector = [&](int r, int m, cx<R>* vout) {
+    if (32 * warp < m) {
+      R s = 0;
+#pragma unroll
+      for (int q = 0; q < EPT; ++q)
+        if (tid + q * TRI_THREADS < m) s += norm2(x[q]);
+      s = warp_real(s);
+      if (lane == 0) redN[warp] = s;
+    } else if (lane == 0) {
+      redN[warp] = R(0);
+    }
+    if (tid == 0) x0_s = x[0];
+    __syncthreads();
+    if (warp == 0) {
+      R xn2 = lane < TRI_NW ? redN[lane] : R(0);
+      for (int o = TRI_NW / 2; o > 0; o >>= 1) xn2 += __shfl_xor_sync(0xffffffffu, xn2, o);
+      xn2 = __shfl_sync(0xffffffffu, xn2, 0);
+      using PS = PivotScale<R>;
+      cx<R> x0 = x0_s;
+      const bool tiny = fmax(fabs(x0.re), fabs(x0.im)) < PS::small();
+      if (tiny) x0 = PS::up() * x0;
+      const R q2 = norm2(x0);
+      // lane 0: 1 / |x0|, lane 1: 1 / ||x||, in one evaluation
+      const R arg = lane == 0 ? q2 : xn2;
+      const R is = arg > PS::floor2() ? rsqrt_series(arg) : R(0);
+      const R root = arg * is;   // |x0|, ||x||
+      const R qi = __shfl_sync(0xffffffffu, is, 0), ax0s = __shfl_sync(0xffffffffu, root, 0),
+              xn = __shfl_sync(0xffffffffu, root, 1);
+      // alpha = -e^{i arg x0} ||x||: real part on lane 0, imaginary on lane 1
+      const R ph = ((lane == 0 ? x0.re : x0.im) * qi);
+      const R al = -(qi > R(0) ? ph : (lane == 0 ? R(1) : R(0))) * xn;
+      const R ax0 = tiny ? ax0s * PS::dn() : ax0s;
+      const R un2 = R(2) * fma(xn, ax0, xn2);
+      const R inv = xn > R(0) ? rsqrt_series(un2) : R(0);
+      const R al_im = __shfl_sync(0xffffffffu, al, 1);
+      if (lane == 0) {
+        alpha_s = mk<R>(al, al_im);
+        inv_s = inv;
+        if (rank == 0) e[r] = mk<R>(al, al_im);
+      }
+    }
+    __syncthreads();
+    const R inv = inv_s;
+#pragma unroll
+    for (int q = 0; q < EPT; ++q) {
+      const int t = tid + q * TRI_THREADS;
+      if (t < m) {
+        cx<R> u = x[q];
+        if (t == 0) u = u - alpha_s;
+        const cx<R> v = inv * u;
+        vout[t] = v;
+        if (rank == r % CS) {
+          Vh[(long long)r * n + r + 1 + t] = conj(v);   // conjugated, for the back-transformation
+        }
+      }
+    }
+    // left of the reflector: zeros
+    if (rank == r % CS)
+      for (int t = tid; t <= r; t += TRI_THREADS) Vh[(long long)r * n + t] = mk<R>(0, 0);
+  };
+  // a -= v conj(wk) + w conj(vk)
+  auto rank2 = [](cx<R>& a, cx<R> vt, cx<R> wt, cx<R> vk, cx<R> wk) {
+    a.re -= vt.re * wk.re + vt.im * wk.im + wt.re * vk.re + wt.im * vk.im;
+    a.im -= vt.im * wk.re - vt.re * wk.im + wt.im * vk.re - wt.re * vk.im;
+  };
+  if (n > 2) reflector(0, n - 1, vb);
+  if (rank == 0 && tid == 0) d[0] = in(0, 0).re;
+  int oc = 1 % CS, ol = 1 / CS;   // row j + 1: its CTA and place there
+  cluster.sync();   // every CTA of the cluster runs before anyone writes into its shared memory
+  for (int j = 0; j + 2 < n; ++j) {
+    const int m = n - j - 1, buf = j & 1;
+    const cx<R>* v = vb + buf * n;               // v_j: entry t is row j + 1 + t
+    const cx<R>* vo = vb + (buf ^ 1) * n + 1;    // v_{j-1}, w_{j-1} at row j + 1
+    const cx<R>* wo = pb + (buf ^ 1) * n + 1;
+    cx<R>* p = pb + buf * n;
+    // own rows i > j, two per warp at a time: update with column j - 1, product with v_j
+    const int l0 = ol + (oc > rank ? 1 : 0);
+    R ks = 0;
+    for (int li = l0 + warp; li < nloc; li += 2 * TRI_NW) {
+      const bool two = li + TRI_NW < nloc;
+      const int t = rank + li * CS - j - 1, t2 = t + TRI_NW * CS;
+      cx<R>* row = Hl + (long long)li * n + (j + 1);
+      cx<R>* row2 = Hl + (long long)(two ? li + TRI_NW : li) * n + (j + 1);
+      cx<R> a0 = mk<R>(0, 0), a1 = a0, b0 = a0, b1 = a0;
+      if (j == 0) {
+        for (int k = lane; k < m; k += 32) {
+          fma_(a0, row[k], v[k]);
+          if (two) fma_(b0, row2[k], v[k]);
+        }
+      } else {
+        const cx<R> vt = vo[t], wt = wo[t], vt2 = two ? vo[t2] : vt, wt2 = two ? wo[t2] : wt;
+        int k = lane;
+        for (; k + 32 < m; k += 64) {
+          cx<R> r0 = row[k], r1 = row[k + 32];
+          const cx<R> wk0 = wo[k], vk0 = vo[k], wk1 = wo[k + 32], vk1 = vo[k + 32];
+          const cx<R> v0 = v[k], v1 = v[k + 32];
+          rank2(r0, vt, wt, vk0, wk0);
+          rank2(r1, vt, wt, vk1, wk1);
+          row[k] = r0;
+          row[k + 32] = r1;
+          fma_(a0, r0, v0);
+          fma_(a1, r1, v1);
+          if (two) {
+            r0 = row2[k];
+            r1 = row2[k + 32];
+            rank2(r0, vt2, wt2, vk0, wk0);
+            rank2(r1, vt2, wt2, vk1, wk1);
+            row2[k] = r0;
+            row2[k + 32] = r1;
+            fma_(b0, r0, v0);
+            fma_(b1, r1, v1);
+          }
+        }
+        for (; k < m; k += 32) {
+          cx<R> r0 = row[k];
+          rank2(r0, vt, wt, vo[k], wo[k]);
+          row[k] = r0;
+          fma_(a0, r0, v[k]);
+          if (two) {
+            r0 = row2[k];
+            rank2(r0, vt2, wt2, vo[k], wo[k]);
+            row2[k] = r0;
+            fma_(b0, r0, v[k]);
+          }
+        }
+        a0 = a0 + a1;
+        b0 = b0 + b1;
+      }
+      // both rows' sums in five steps: lanes 0-15 end with the first row's, 16-31 with the second's
+      const bool up = lane & 16;
+      cx<R> s = (up ? b0 : a0) + shfl_xor(up ? a0 : b0, 16);
+      for (int o = 8; o > 0; o >>= 1) s = s + shfl_xor(s, o);
+      if (!up || two) {
+        const int tr = up ? t2 : t;
+        const cx<R> vt = v[tr];
+        ks += vt.re * s.re + vt.im * s.im;   // the same on 16 lanes
+        if ((lane & 15) < CS) *cluster.map_shared_rank(p + tr, lane & 15) = s;
+      }
+    }
+    {
+      const R kw = ks + __shfl_xor_sync(0xffffffffu, ks, 16);
+      if (lane < CS) cluster.map_shared_rank(kbuf + (buf * CS + rank) * TRI_NW, lane)[warp] = kw;
+    }
+    cluster.sync();
+    // row j + 1 (its owner's last word on it)
+    cx<R> a[EPT];
+    const cx<R>* rj1 = cluster.map_shared_rank(Hl + (long long)ol * n + (j + 1), oc);
+#pragma unroll
+    for (int q = 0; q < EPT; ++q) {
+      const int t = tid + q * TRI_THREADS;
+      a[q] = t + 1 < m ? conj(rj1[t + 1]) : mk<R>(0, 0);   // entry (j + 2 + t, j + 1) by symmetry
+    }
+    if (warp == 0) {
+      R K = 0;
+      for (int q = lane; q < CS * TRI_NW; q += 32) K += kbuf[buf * CS * TRI_NW + q];
+      K = warp_real(K);
+      if (lane == 0) K_s = R(2) * K;
+    }
+    __syncthreads();
+    const R twoK = K_s;
+    auto wof = [&](cx<R> vt, cx<R> pt) { return mk<R>(pt.re + pt.re - twoK * vt.re, pt.im + pt.im - twoK * vt.im); };
+    if (32 * warp + 1 < m) {
+      const cx<R> v0 = v[0], w0 = wof(v0, p[0]);
+#pragma unroll
+      for (int q = 0; q < EPT; ++q) {
+        const int t = tid + q * TRI_THREADS;
+        if (t + 1 < m) {
+          const cx<R> vt = v[t + 1], wt = wof(vt, p[t + 1]);
+          p[t + 1] = wt;   // (entry 0 stays p: no row needs w_0 again)
+          rank2(a[q], vt, wt, v0, w0);
+        }
+        x[q] = a[q];
+      }
+      if (rank == oc && tid == 0) {
+        // d[j + 1] = A[j+1][j+1] - 2 Re(v_0 conj(w_0))
+        d[j + 1] = Hl[(long long)ol * n + (j + 1)].re - R(2) * (v0.re * w0.re + v0.im * w0.im);
+      }
+    }
+    if (++oc == CS) {   // to row j + 2
+      oc = 0;
+      ++ol;
+    }
+    if (j + 3 < n) {
+      reflector(j + 1, m - 1, vb + (buf ^ 1) * n);
+    } else if (tid == 0) {
+      // the last 2 x 2 block: subdiagonal, and the corner by its owner
+      if (rank == (n - 1) % CS) {
+        const cx<R> v0 = v[0], w0 = wof(v0, p[0]), v1 = v[1], w1 = p[1];
+        cx<R> sub = Hl[(long long)((n - 1) / CS) * n + (n - 2)];
+        rank2(sub, v1, w1, v0, w0);
+        e[n - 2] = sub;
+        d[n - 1] = Hl[(long long)((n - 1) / CS) * n + (n - 1)].re - R(2) * (v1.re * w1.re + v1.im * w1.im);
+      }
+    }
+    __syncthreads();
+  }
+  if (n == 2 && rank == 0 && tid == 0) {
+    d[1] = in(1, 1).re;
+    e[0] = in(1, 0);
+  }
+  cluster.sync();   // rows of this CTA may still be read by others
+}
+
 // U[k][c] = phi_k Z[k][c] (complex from the real tridiagonal eigenvectors).
 template <typename R>
 __global__ void phase_scale_kernel(const R* Zb, long long sZ, const cx<R>* phib, int ldde, int n, int r, cx<R>* Ub,
@@ -266,12 +542,12 @@ static cudaError_t launch_cl(K kernel, int cs, int batch, size_t smem, cudaStrea
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-constexpr size_t SMEM_LIMIT = 224 * 1024;   // dynamic shared memory per CTA (227 KB less the static part)
+constexpr size_t SMEM_LIMIT = 226 * 1024;   // dynamic shared memory per CTA (227 KB less the static part)
 
 template <typename R>
 static size_t tridiag_smem_bytes(int n, int cs) {
   const size_t maxloc = (n + cs - 1) / cs;
-  return sizeof(cx<R>) * (maxloc * n + 4 * (size_t)n);
+  return sizeof(cx<R>) * (maxloc * n + 4 * (size_t)n) + sizeof(R) * 2 * 16 * TRI_NW;
 }
 
 // Smallest power-of-two cluster whose shared memory holds the matrix (0: none does).
@@ -285,31 +561,30 @@ int smem_cluster_size(int n) {
 }
 
 // Cluster size for `batch` matrices: among the sizes from smem_cluster_size(n)
-// up to 16 that hold the matrix, the largest whose clusters all fit on the GPU
+// up to `most` that hold the matrix, the largest whose clusters all fit on the GPU
 // at once (cudaOccupancyMaxActiveClusters); a cluster of 16 does not fit on
 // every GPC, so for a batch of 8 a size of 13 or 14 can finish in one wave
-// where 16 needs two.  Cached per (n, batch) and device.
+// where 16 needs two.  Cached per kernel, (n, batch) and device.
 template <typename R>
-static int tridiag_cluster_size(int n, int batch, cudaStream_t st) {
+static int tridiag_cluster_size(const void* kernel, int n, int batch, int most) {
   static std::mutex mu;
-  static std::map<std::tuple<int, int, int>, int> cache;
+  static std::map<std::tuple<const void*, int, int, int>, int> cache;
   int dev = 0;
   cudaGetDevice(&dev);
   std::lock_guard<std::mutex> lk(mu);
-  auto key = std::make_tuple(n, batch, dev);
+  auto key = std::make_tuple(kernel, n, batch, dev);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
   const int cs0 = smem_cluster_size<R>(n);
   int best = cs0, best_waves = 1 << 30;
-  for (int cs = std::max(cs0, 2); cs <= 16 && cs0 > 0; ++cs) {
+  for (int cs = std::max(cs0, 2); cs <= std::max(cs0, std::min(16, most)) && cs0 > 0; ++cs) {
     const size_t smem = tridiag_smem_bytes<R>(n, cs);
     if (smem > SMEM_LIMIT) continue;
-    if (ensure_kernel_smem((const void*)tridiag_smem_kernel<R>, smem, cs > 8) != cudaSuccess) continue;
+    if (ensure_kernel_smem(kernel, smem, cs > 8) != cudaSuccess) continue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs, batch, 1);
     cfg.blockDim = dim3(256, 1, 1);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
@@ -318,7 +593,7 @@ static int tridiag_cluster_size(int n, int batch, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int active = 0;
-    if (cudaOccupancyMaxActiveClusters(&active, (const void*)tridiag_smem_kernel<R>, &cfg) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) != cudaSuccess ||
         active < 1) {
       cudaGetLastError();
       continue;
@@ -336,12 +611,23 @@ static int tridiag_cluster_size(int n, int batch, cudaStream_t st) {
 template <typename R>
 cudaError_t tridiag_smem(cudaStream_t st, const cx<R>* H, long long sH, int n, R* d, cx<R>* e, int ldde, cx<R>* Vh,
                          long long sVh, int batch) {
-  if (smem_cluster_size<R>(n) == 0) return cudaErrorInvalidValue;
-  const int cs = tridiag_cluster_size<R>(n, batch, st);
-  const int maxloc = (n + cs - 1) / cs;
+  if (smem_cluster_size<R>(n) == 0 || n > 3 * TRI_THREADS) return cudaErrorInvalidValue;
+  auto kernel = n <= TRI_THREADS ? tridiag_fused_kernel<R, 1> : tridiag_fused_kernel<R, 3>;
+  const int cs = tridiag_cluster_size<R>((const void*)kernel, n, batch, (n + 7) / 8);
   const size_t smem = tridiag_smem_bytes<R>(n, cs);
   ProfScope ps(st, K_TRIDIAG, 1, 16.0 / 3.0 * (double)n * n * n * batch);   // Hermitian tridiagonalisation flops
-  return launch_cl(tridiag_smem_kernel<R>, cs, batch, smem, st, H, sH, n, d, e, ldde, Vh, sVh, maxloc);
+  return launch_cl(kernel, cs, batch, smem, st, H, sH, n, d, e, ldde, Vh, sVh, (n + cs - 1) / cs);
+}
+
+// The two-barrier kernel, for the float64 reduction of complex64 states' small
+// eigenproblems (n <= EIGH_F64_MAX), whose last bits small jobs' results follow.
+cudaError_t tridiag_smem_keep(cudaStream_t st, const cx<double>* H, long long sH, int n, double* d, cx<double>* e,
+                              int ldde, cx<double>* Vh, long long sVh, int batch) {
+  if (smem_cluster_size<double>(n) == 0) return cudaErrorInvalidValue;
+  const int cs = tridiag_cluster_size<double>((const void*)tridiag_smem_kernel<double>, n, batch, 16);
+  const size_t smem = tridiag_smem_bytes<double>(n, cs);
+  ProfScope ps(st, K_TRIDIAG, 1, 16.0 / 3.0 * (double)n * n * n * batch);
+  return launch_cl(tridiag_smem_kernel<double>, cs, batch, smem, st, H, sH, n, d, e, ldde, Vh, sVh, (n + cs - 1) / cs);
 }
 
 template <typename R>

@@ -566,11 +566,11 @@ cudaError_t eigh_top(cudaStream_t st, cx<R>* H, long long sH, int n, int r, cx<R
   double* Kp = reinterpret_cast<double*>(U2 + (long long)batch * n * r + 1);
   Kp = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(Kp) + 15) & ~uintptr_t(15));
   (void)w;
-  cudaError_t ce = cudaMemsetAsync(Vh, 0, sizeof(cx<R>) * (size_t)batch * n * n, st);
-  if (ce != cudaSuccess) return ce;
+  cudaError_t ce;
   if (smem_cluster_size<R>(n) > 0) {
     ce = tridiag_smem<R>(st, H, sH, n, d, e, ldde, Vh, (long long)n * n, batch);
   } else {
+    if ((ce = cudaMemsetAsync(Vh, 0, sizeof(cx<R>) * (size_t)batch * n * n, st)) != cudaSuccess) return ce;
     ce = tridiag_global<R>(st, H, sH, n, d, e, ldde, P, Kp, Vh, (long long)n * n, batch);
   }
   if (ce != cudaSuccess) return ce;
@@ -702,7 +702,7 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
     }
     if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
     if ((ce = cudaMemsetAsync(Vhd, 0, 16 * nn * B, st)) != cudaSuccess) return ce;
-    if ((ce = tridiag_smem<double>(st, Hd, (long long)nn, n, dd, ed, n, Vhd, (long long)nn, batch)) != cudaSuccess)
+    if ((ce = tridiag_smem_keep(st, Hd, (long long)nn, n, dd, ed, n, Vhd, (long long)nn, batch)) != cudaSuccess)
       return ce;
     ProfScope ps(st, K_ELEMWISE);
     cx_d2f_kernel<<<1024, 256, 0, st>>>(Vhd, Vhf, (long long)(nn * B));
@@ -743,11 +743,11 @@ cudaError_t gram_entropy(cudaStream_t st, cx<R>* H, long long sH, int n, void* c
   R* lam = eabs + (long long)batch * n;             // batch x n
   double* Kp = reinterpret_cast<double*>(lam + (long long)batch * n + 1);
   Kp = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(Kp) + 15) & ~uintptr_t(15));
-  cudaError_t ce = cudaMemsetAsync(Vh, 0, sizeof(cx<R>) * (size_t)batch * n * n, st);
-  if (ce != cudaSuccess) return ce;
+  cudaError_t ce;
   if (smem_cluster_size<R>(n) > 0) {
     ce = tridiag_smem<R>(st, H, sH, n, d, e, n, Vh, (long long)n * n, batch);
   } else {
+    if ((ce = cudaMemsetAsync(Vh, 0, sizeof(cx<R>) * (size_t)batch * n * n, st)) != cudaSuccess) return ce;
     ce = tridiag_global<R>(st, H, sH, n, d, e, n, P, Kp, Vh, (long long)n * n, batch);
   }
   if (ce != cudaSuccess) return ce;

@@ -124,9 +124,13 @@ constexpr size_t TRIDIAG64_SMEM = 120 * 1024;
 
 template <typename R>
 int smem_cluster_size(int n);
+// Reduction of matrices that fit in one cluster's shared memory; reflectors as rows of Vh,
+// conjugated, zeros left of them.  _keep: the earlier kernel (Vh's zeros are the caller's).
 template <typename R>
 cudaError_t tridiag_smem(cudaStream_t st, const cx<R>* H, long long sH, int n, R* d, cx<R>* e, int ldde, cx<R>* Vh,
                          long long sVh, int batch);
+cudaError_t tridiag_smem_keep(cudaStream_t st, const cx<double>* H, long long sH, int n, double* d, cx<double>* e,
+                              int ldde, cx<double>* Vh, long long sVh, int batch);
 template <typename R>
 cudaError_t backtransform_wy(cudaStream_t st, const cx<R>* Vh, long long sVh, int n, const R* Z, long long sZ,
                              const cx<R>* phi, int ldde, int r, cx<R>* U, long long sU, cx<R>* Tw, cx<R>* wy_ws,
