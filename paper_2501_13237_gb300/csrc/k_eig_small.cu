@@ -11,161 +11,179 @@ namespace cg = cooperative_groups;
 
 namespace nne {
 
-// Reflector of row r (the owner's own row, stored at Hl_row): x = conj of the
-// row's entries right of the diagonal (the column below it, by symmetry),
-// v = (x - alpha e_0) / ||x - alpha e_0||, alpha = -e^{i arg x_0} ||x||.
-// Writes v to vpub, conj(v) to row r of Vh, d[r] and e[r] = alpha.  Called by
-// every thread of the owning CTA; the norm is summed in R.
-template <typename R>
-__device__ __forceinline__ void tridiag_publish(const cx<R>* Hl_row, int n, int r, cx<R>* vpub, cx<R>* Vh, R* d,
-                                                cx<R>* e, R* red, cx<R>* alpha_s, R* inv_s) {
-  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
+constexpr int KEEP_THREADS = 256;
+struct PublishShared {
+  double red[KEEP_THREADS / 32];
+  double ax0, ph[2], xn, inv;
+};
+// Named barriers of a part of the block's warps.
+__device__ __forceinline__ void barrier_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void barrier_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// The reflector of row r (x0 = conj of its first entry) by the 256 threads of the
+// owning CTA: v goes to vd of every CTA of the cluster, conj(v) to row r of Vh, and
+// d[r], e[r] = alpha.  The last warp forms |x0| and its phase, a divide per lane, while the
+// others sum the norm: as one thread's chain the three square roots and five
+// divides (some 650 cycles each) were 40 % of a column.
+__device__ __forceinline__ void tridiag_publish(cg::cluster_group& cluster, const cx<double>* Hl_row, int n, int r,
+                                                cx<double>* vd, cx<double>* Vh, double* d, cx<double>* e,
+                                                PublishShared& sh) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, last = KEEP_THREADS / 32 - 1;
   const int m = n - r - 1;
-  R sp = 0;
-  for (int t = tid; t < m; t += nth) sp += norm2(Hl_row[r + 1 + t]);
-  sp = warp_sum_r(sp);
-  if (lane == 0) red[warp] = sp;
-  __syncthreads();
-  if (tid == 0) {
-    R xn2 = 0;
-    for (int w2 = 0; w2 < nw; ++w2) xn2 += red[w2];
-    const cx<R> x0 = conj(Hl_row[r + 1]);
-    R pr, pi, ax0;
-    unit_phase_of(x0, &pr, &pi, &ax0);
-    const R xn = sqrt(xn2);
-    cx<R> alpha = mk<R>(0, 0);
-    R un = 0;
-    if (xn > R(0)) {
-      alpha = mk<R>(-xn * pr, -xn * pi);
-      un = sqrt(R(2) * xn2 + R(2) * xn * ax0);
+  if (warp == last) {
+    const cx<double> x0 = conj(Hl_row[r + 1]);
+    const double s = fmax(fabs(x0.re), fabs(x0.im)), mine = lane & 1 ? x0.im : x0.re;
+    const bool nz = s > 0.0;
+    const double q = mine / (nz ? s : 1.0);
+    const double a = __shfl_sync(0xffffffffu, q, 0), b = __shfl_sync(0xffffffffu, q, 1);
+    const double rr = sqrt(a * a + b * b);
+    if (lane == 0) sh.ax0 = nz ? s * rr : 0.0;
+    __syncwarp();
+    barrier_arrive(2, 64);
+    const double ph = q / (nz ? rr : 1.0);
+    if (lane < 2) sh.ph[lane] = nz ? ph : (lane ? 0.0 : 1.0);
+  } else {
+    double sp = 0;
+    if (tid < m) sp += norm2(Hl_row[r + 1 + tid]);
+    sp = warp_sum_r(sp);
+    if (lane == 0) sh.red[warp] = sp;
+    __syncwarp();
+    barrier_sync(1, KEEP_THREADS - 32);
+    if (warp == 0) {
+      double xn2 = 0;
+      for (int w2 = 0; 32 * w2 < m; ++w2) xn2 += sh.red[w2];
+      const double xn = sqrt(xn2);
+      barrier_sync(2, 64);
+      double un = 0;
+      if (xn > 0.0) un = sqrt(2.0 * xn2 + 2.0 * xn * sh.ax0);
+      if (lane == 0) {
+        sh.xn = xn;
+        sh.inv = un > 0.0 ? 1.0 / un : 0.0;
+      }
     }
-    *alpha_s = alpha;
-    *inv_s = un > R(0) ? R(1) / un : R(0);
+  }
+  __syncthreads();
+  const double xn = sh.xn, inv = sh.inv;
+  const cx<double> alpha = xn > 0.0 ? mk<double>(-xn * sh.ph[0], -xn * sh.ph[1]) : mk<double>(0, 0);
+  if (tid == KEEP_THREADS - 1) {
     d[r] = Hl_row[r].re;
     e[r] = alpha;
   }
-  __syncthreads();
-  const cx<R> alpha = *alpha_s;
-  const R inv = *inv_s;
-  cx<R>* vr = Vh + (long long)r * n + (r + 1);
-  for (int t = tid; t < m; t += nth) {
-    cx<R> u = conj(Hl_row[r + 1 + t]);
-    if (t == 0) u = u - alpha;
-    const cx<R> v = inv * u;
-    vpub[t] = v;
-    vr[t] = conj(v);
+  if (tid < m) {
+    cx<double> u = conj(Hl_row[r + 1 + tid]);
+    if (tid == 0) u = u - alpha;
+    const cx<double> v = inv * u;
+    for (int c = 0; c < (int)cluster.num_blocks(); ++c) cluster.map_shared_rank(vd, c)[tid] = v;
+    Vh[(long long)r * n + (r + 1) + tid] = conj(v);
   }
 }
 
-// Householder tridiagonalisation of the Hermitian H[z] (n x n) by one
+// Householder tridiagonalisation of the Hermitian H[z] (n x n, n <= 224) by one
 // cluster.  Rows are dealt to the CTAs cyclically and stay in shared memory.
-// Column j: every CTA pulls v_j from the owner of row j, forms p = A v on
-// its rows and publishes p and its share of K = v^H p; after a cluster
-// barrier it pulls all of p and K, applies A <- A - v w^H - w v^H with
-// w = 2p - 2Kv to its rows, and the owner of row j+1 forms and publishes
-// v_{j+1}; a second barrier closes the column.  Sums run in a fixed order.
-template <typename R>
-__global__ void __launch_bounds__(256) tridiag_smem_kernel(const cx<R>* Hb, long long sH, int n, R* db, cx<R>* eb,
-                                                            int ldde, cx<R>* Vhb, long long sVh, int maxloc) {
+// Column j: every CTA forms p = A v on its rows and stores p and its warps' shares of
+// K = v^H p into every CTA; after a cluster barrier each applies
+// A <- A - v w^H - w v^H with w = 2p - 2Kv to its rows, and the owner of row j+1 forms
+// v_{j+1} and stores it into every CTA; a second barrier closes the column.  Sums run in
+// a fixed order: the results, to the last bit, are those that small jobs follow.
+// Bound by its chain of float64 instructions (64 cycles each).  Stores into the other CTAs
+// in place of loads from them, no add of a zero share and the reflector's chain over
+// two warps: 1 to 5 matrices of 64 rows 532 -> 378 us, of 160 rows 1904 -> 1490; 40 of
+// 64 rows 732 -> 585.
+__global__ void __launch_bounds__(KEEP_THREADS) tridiag_smem_kernel(const cx<double>* Hb, long long sH, int n, double* db,
+                                                                    cx<double>* eb, int ldde, cx<double>* Vhb,
+                                                                    long long sVh, int maxloc) {
   cg::cluster_group cluster = cg::this_cluster();
   const int CS = (int)cluster.num_blocks();
   const int rank = (int)cluster.block_rank();
   const int z = blockIdx.y;
-  const cx<R>* H = Hb + z * sH;
-  R* d = db + (long long)z * ldde;
-  cx<R>* e = eb + (long long)z * ldde;
-  cx<R>* Vh = Vhb + z * sVh;
+  const cx<double>* H = Hb + z * sH;
+  double* d = db + (long long)z * ldde;
+  cx<double>* e = eb + (long long)z * ldde;
+  cx<double>* Vh = Vhb + z * sVh;
   extern __shared__ unsigned char smem_raw[];
-  cx<R>* Hl = reinterpret_cast<cx<R>*>(smem_raw);     // [maxloc][n] own rows
-  cx<R>* vpub = Hl + (long long)maxloc * n;           // n: v published by the owner of the pivot row
-  cx<R>* vloc = vpub + n;                             // n: this CTA's copy of v
-  cx<R>* ppub = vloc + n;                             // n: p of own rows, at their offsets
-  cx<R>* w = ppub + n;                                // n: w = 2p - 2Kv
-  __shared__ R kpub;                                  // this CTA's share of K
-  __shared__ R red[32];
-  __shared__ cx<R> alpha_s;
-  __shared__ R inv_s, twoK_s;
-  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
+  cx<double>* Hl = reinterpret_cast<cx<double>*>(smem_raw);     // [maxloc][n] own rows
+  cx<double>* vbuf = Hl + (long long)maxloc * n;                // 2 x n: v of even and of odd columns
+  cx<double>* p = vbuf + 2 * n;                                 // n
+  cx<double>* w = p + n;                                        // n: w = 2p - 2Kv
+  constexpr int NW = KEEP_THREADS / 32;
+  __shared__ double kpart[16][NW];                              // all warps' shares of K
+  __shared__ PublishShared sh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nloc = n > rank ? (n - rank + CS - 1) / CS : 0;
-  for (long long e2 = tid; e2 < (long long)nloc * n; e2 += nth) {
+  for (long long e2 = tid; e2 < (long long)nloc * n; e2 += KEEP_THREADS) {
     const int li = (int)(e2 / n), c = (int)(e2 % n);
     Hl[e2] = H[(long long)(rank + li * CS) * n + c];
   }
-  __syncthreads();
-  if (n > 2 && rank == 0) tridiag_publish(Hl, n, 0, vpub, Vh, d, e, red, &alpha_s, &inv_s);
+  // every CTA of the cluster is running before anyone writes into its shared memory
+  cluster.sync();
+  if (n > 2 && rank == 0) tridiag_publish(cluster, Hl, n, 0, vbuf, Vh, d, e, sh);
   cluster.sync();
   for (int j = 0; j + 2 < n; ++j) {
-    const int m = n - j - 1, owner = j % CS;
-    // pull v_j
-    {
-      const cx<R>* src = cluster.map_shared_rank(vpub, owner);
-      for (int t = tid; t < m; t += nth) vloc[t] = src[t];
-    }
-    __syncthreads();
+    const int m = n - j - 1;
+    const cx<double>* v = vbuf + (j & 1) * n;
     // p = A v on own rows i > j; K share = sum Re(conj(v_t) p_t)
     const int lstart = (j + 1 - rank + CS - 1) / CS;
-    R kp = 0;
-    for (int li = lstart + warp; li < nloc; li += nw) {
+    double kp = 0;
+    for (int li = lstart + warp; li < nloc; li += NW) {
       const int i = rank + li * CS, t = i - j - 1;
-      const cx<R>* row = Hl + (long long)li * n + (j + 1);
-      cx<R> a0 = mk<R>(0, 0), a1 = a0, a2 = a0, a3 = a0;
+      const cx<double>* row = Hl + (long long)li * n + (j + 1);
+      cx<double> a0 = mk<double>(0, 0), a1 = a0, a2 = a0, a3 = a0;
       int k = lane;
       for (; k + 96 < m; k += 128) {
-        fma_(a0, row[k], vloc[k]);
-        fma_(a1, row[k + 32], vloc[k + 32]);
-        fma_(a2, row[k + 64], vloc[k + 64]);
-        fma_(a3, row[k + 96], vloc[k + 96]);
+        fma_(a0, row[k], v[k]);
+        fma_(a1, row[k + 32], v[k + 32]);
+        fma_(a2, row[k + 64], v[k + 64]);
+        fma_(a3, row[k + 96], v[k + 96]);
       }
-      for (; k < m; k += 32) fma_(a0, row[k], vloc[k]);
-      cx<R> acc = (a0 + a1) + (a2 + a3);
-      acc = warp_sum(acc);
-      if (lane == 0) {
-        ppub[t] = acc;
-        kp += vloc[t].re * acc.re + vloc[t].im * acc.im;
-      }
+      for (; k < m; k += 32) fma_(a0, row[k], v[k]);
+      if (m > 96) a0 = (a0 + a1) + (a2 + a3);
+      // lanes 0-15 sum the real parts, 16-31 the imaginary
+      const bool im = lane >= 16;
+      double s = (im ? a0.im : a0.re) + __shfl_xor_sync(0xffffffffu, im ? a0.re : a0.im, 16);
+      for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const cx<double> acc = mk<double>(__shfl_sync(0xffffffffu, s, 0), __shfl_sync(0xffffffffu, s, 16));
+      if (lane < CS) cluster.map_shared_rank(p, lane)[t] = acc;
+      kp += v[t].re * acc.re + v[t].im * acc.im;
     }
-    if (lane == 0) red[warp] = kp;
-    __syncthreads();
-    if (tid == 0) {
-      R t = 0;
-      for (int w2 = 0; w2 < nw; ++w2) t += red[w2];
-      kpub = t;
-    }
+    if (lane < CS) *cluster.map_shared_rank(&kpart[rank][warp], lane) = kp;
+    const int nact = min(NW, (m + CS - 1) / CS);   // warps with rows, at most, in any CTA
     cluster.sync();
-    // pull p and K; w = 2p - 2Kv
-    if (warp == 0) {
-      R kk = lane < CS ? *cluster.map_shared_rank(&kpub, lane) : R(0);
+    if (32 * warp < m) {
+      double kk = 0;
+      if (lane < CS)
+        for (int w2 = 0; w2 < nact; ++w2) kk += kpart[lane][w2];
       for (int o = 1; o < 32; o <<= 1) {
-        const R other = __shfl_down_sync(0xffffffffu, kk, o);
-        kk += (lane + o < 32) ? other : R(0);
+        const double other = __shfl_down_sync(0xffffffffu, kk, o);
+        kk += (lane + o < 32) ? other : 0.0;
       }
-      if (lane == 0) twoK_s = R(2) * kk;
-    }
-    for (int t = tid; t < m; t += nth) w[t] = *cluster.map_shared_rank(ppub + t, (j + 1 + t) % CS);
-    __syncthreads();
-    {
-      const R twoK = twoK_s;
-      for (int t = tid; t < m; t += nth)
-        w[t] = mk<R>(2 * w[t].re - twoK * vloc[t].re, 2 * w[t].im - twoK * vloc[t].im);
+      const double twoK = 2.0 * __shfl_sync(0xffffffffu, kk, 0);
+      if (tid < m) {
+        const cx<double> pt = p[tid], vt = v[tid];
+        w[tid] = mk<double>(2 * pt.re - twoK * vt.re, 2 * pt.im - twoK * vt.im);
+      }
     }
     __syncthreads();
-    for (int li = lstart + warp; li < nloc; li += nw) {
+    for (int li = lstart + warp; li < nloc; li += NW) {
       const int i = rank + li * CS, t = i - j - 1;
-      cx<R>* row = Hl + (long long)li * n + (j + 1);
-      const cx<R> vt = vloc[t], wt = w[t];
+      cx<double>* row = Hl + (long long)li * n + (j + 1);
+      const cx<double> vt = v[t], wt = w[t];
 #pragma unroll 4
       for (int k = lane; k < m; k += 32) {
-        cx<R> a = row[k];
-        const cx<R> wk = w[k], vk = vloc[k];
+        cx<double> a = row[k];
+        const cx<double> wk = w[k], vk = v[k];
         a.re -= vt.re * wk.re + vt.im * wk.im + wt.re * vk.re + wt.im * vk.im;
         a.im -= vt.im * wk.re - vt.re * wk.im + wt.im * vk.re - wt.re * vk.im;
         row[k] = a;
       }
     }
-    // the owner of row j+1 forms and publishes the next reflector
+    // the owner of row j+1 forms the next reflector
     if (j + 3 < n && rank == (j + 1) % CS) {
       __syncthreads();
-      tridiag_publish(Hl + (long long)((j + 1) / CS) * n, n, j + 1, vpub, Vh, d, e, red, &alpha_s, &inv_s);
+      tridiag_publish(cluster, Hl + (long long)((j + 1) / CS) * n, n, j + 1, vbuf + ((j + 1) & 1) * n, Vh, d, e, sh);
     }
     cluster.sync();
   }
@@ -623,11 +641,11 @@ cudaError_t tridiag_smem(cudaStream_t st, const cx<R>* H, long long sH, int n, R
 // eigenproblems (n <= EIGH_F64_MAX), whose last bits small jobs' results follow.
 cudaError_t tridiag_smem_keep(cudaStream_t st, const cx<double>* H, long long sH, int n, double* d, cx<double>* e,
                               int ldde, cx<double>* Vh, long long sVh, int batch) {
-  if (smem_cluster_size<double>(n) == 0) return cudaErrorInvalidValue;
-  const int cs = tridiag_cluster_size<double>((const void*)tridiag_smem_kernel<double>, n, batch, 16);
+  if (smem_cluster_size<double>(n) == 0 || n > KEEP_THREADS - 32) return cudaErrorInvalidValue;
+  const int cs = tridiag_cluster_size<double>((const void*)tridiag_smem_kernel, n, batch, 16);
   const size_t smem = tridiag_smem_bytes<double>(n, cs);
   ProfScope ps(st, K_TRIDIAG, 1, 16.0 / 3.0 * (double)n * n * n * batch);
-  return launch_cl(tridiag_smem_kernel<double>, cs, batch, smem, st, H, sH, n, d, e, ldde, Vh, sVh, (n + cs - 1) / cs);
+  return launch_cl(tridiag_smem_kernel, cs, batch, smem, st, H, sH, n, d, e, ldde, Vh, sVh, (n + cs - 1) / cs);
 }
 
 template <typename R>
