@@ -502,43 +502,74 @@ __global__ void phase_scale_kernel(const R* Zb, long long sZ, const cx<R>* phib,
 // Compact-WY factors of blocks of 32 consecutive tridiagonal reflectors:
 // block b (reflectors 32b .. 32b+bw-1) gives T_b with
 // P_{32b} ... P_{32b+bw-1} = I - V_b T_b V_b^H, V_b^H = Vh rows 32b...
+// The Gram matrix by 2 x 2 entries per thread (upper triangle only) over WT_C staged
+// columns, then T with one row per lane: column l, once known, goes into the sums of
+// all columns right of it.  Both sum in ascending order.  One CTA per block of
+// reflectors, bound by the Gram's chains (64 rows 56 -> 14 us; the complex64 eigenproblems of
+// chi 64, 256 rows, 160 -> 25 us: each entry used to walk two rows in global memory).
+constexpr int WT_C = 32;
 template <typename R>
 __global__ void __launch_bounds__(256) wy_t_kernel(const cx<R>* Vhb, long long sVh, int n, int nref, cx<R>* Tb,
                                                     long long sT) {
-  __shared__ cx<R> G[32][32];
-  __shared__ cx<R> Ts[32][32];
+  __shared__ cx<R> G[32][33];
+  __shared__ cx<R> Vs[32][WT_C + 1];
   const int b = blockIdx.x, z = blockIdx.y;
   const cx<R>* Vh = Vhb + z * sVh;
   cx<R>* T = Tb + z * sT + (long long)b * 1024;
   const int j0 = 32 * b, bw = min(32, nref - j0);
-  const int tid = threadIdx.x;
-  for (int e = tid; e < 1024; e += blockDim.x) {
-    const int a = e / 32, c = e % 32;
-    cx<R> acc = mk<R>(0, 0);
-    if (a < bw && c < bw) {
-      const cx<R>* ra = Vh + (long long)(j0 + a) * n;
-      const cx<R>* rc = Vh + (long long)(j0 + c) * n;
-      for (int i = j0 + 1; i < n; ++i) fmac_(acc, rc[i], ra[i]);   // G[a][c] = v_a^H v_c = sum conj(v_a) v_c
-      // rows hold conj(v): ra[i] = conj(v_a[i]) -> acc = sum conj(rc) ra = sum v_c conj(v_a)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // thread q of the first 136 forms entries (a, c), (a, c + 16), (a + 16, c), (a + 16, c + 16), a <= c < 16
+  int a = 0, c = 0;
+  if (tid < 136) {
+    int q = tid;
+    while (q >= 16 - a) q -= 16 - a++;
+    c = a + q;
+  }
+  cx<R> g00 = mk<R>(0, 0), g01 = g00, g11 = g00, g10 = g00;
+  for (int c0 = j0 + 1; c0 < n; c0 += WT_C) {
+    for (int r = warp; r < 32; r += 8)
+      Vs[r][lane] = r < bw && c0 + lane < n ? Vh[(long long)(j0 + r) * n + c0 + lane] : mk<R>(0, 0);
+    __syncthreads();
+    if (tid < 136) {
+      const int m = min(WT_C, n - c0);
+#pragma unroll 4
+      for (int i = 0; i < m; ++i) {
+        // rows hold conj(v): G[a][c] = v_a^H v_c = sum conj(Vh_c) Vh_a
+        const cx<R> a0 = Vs[a][i], a1 = Vs[a + 16][i], b0 = Vs[c][i], b1 = Vs[c + 16][i];
+        fmac_(g00, b0, a0);
+        fmac_(g01, b1, a0);
+        fmac_(g10, a1, b0);   // (c, a + 16), the mirror of (a + 16, c), which lies below the diagonal
+        fmac_(g11, b1, a1);
+      }
     }
-    G[a][c] = acc;
-    Ts[a][c] = mk<R>(0, 0);
+    __syncthreads();
+  }
+  if (tid < 136) {
+    G[a][c] = g00;
+    G[a][c + 16] = g01;
+    G[c][a + 16] = g10;
+    G[a + 16][c + 16] = g11;
   }
   __syncthreads();
-  if (tid < 32) {
-    for (int i = 0; i < bw; ++i) {
-      const R tau = G[i][i].re > R(0.5) ? R(2) : R(0);
-      cx<R> acc = mk<R>(0, 0);
-      if (tid < i)
-        for (int l = tid; l < i; ++l) fma_(acc, Ts[tid][l], G[l][i]);
-      __syncwarp();
-      if (tid < i) Ts[tid][i] = mk<R>(-tau * acc.re, -tau * acc.im);
-      if (tid == i) Ts[i][i] = mk<R>(tau, 0);
-      __syncwarp();
+  if (warp == 0) {
+    cx<R> acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = mk<R>(0, 0);
+#pragma unroll
+    for (int l = 0; l < 32; ++l) {
+      cx<R> t = mk<R>(0, 0);
+      if (l < bw) {
+        const R tau = G[l][l].re > R(0.5) ? R(2) : R(0);
+        if (lane < l) t = mk<R>(-tau * acc[l].re, -tau * acc[l].im);
+        if (lane == l) t = mk<R>(tau, 0);
+      }
+      T[lane * 32 + l] = t;
+      if (lane <= l && l < bw) {
+#pragma unroll
+        for (int i = l + 1; i < 32; ++i) fma_(acc[i], t, G[l][i]);
+      }
     }
   }
-  __syncthreads();
-  for (int e = tid; e < 1024; e += blockDim.x) T[e] = Ts[e / 32][e % 32];
 }
 
 template <typename K, typename... Args>
