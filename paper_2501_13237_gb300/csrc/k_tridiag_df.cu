@@ -645,21 +645,57 @@ cudaError_t launch_df(void (*kernel)(KArgs...), int cs, int batch, int threads, 
 
 constexpr size_t DFS_SMEM = 226 * 1024;   // dynamic shared memory per CTA (227 KB less the static part)
 
-// CTAs per matrix: more of them shorten a column's pass over the matrix until
-// the exchange dominates.  Twelve is the most that lets eight clusters run at once
-// on the GPU's GPCs, and 384 rows of 12 CTAs fill their shared memory.  Measured
-// (us per launch, batch of 8; in brackets the float64 kernel, above 384 rows
-// L2 kernel down to 384 rows, batch of 8): DFS_FIGURES
-constexpr int DFS_CS = 12, DFS_MAX = 384, DFS_GLOBAL_MAX = 1024;
+// CTAs per matrix: more of them shorten a column's pass over the matrix.  Sixteen is
+// the most a cluster holds, but only seven such clusters run at once on the GPU's GPCs
+// (one CTA per SM), of twelve eight: sixteen where that takes no more waves.  384 rows
+// of 12 CTAs fill their shared memory.  Measured, us, 12 and 16 CTAs: 161 rows 561 and
+// 554, 256 rows 1226 and 1120, 384 rows 2634 and 2425, 512 rows 5303 and 4245, 640 rows
+// 9096 and 7547 (five to seven matrices).  The kernels before: 256 rows, five matrices, 4.17 ms
+// (float64); 512 rows, eight, 9.9 and 640 rows 17.0 (lower triangle in L2, two barriers a column).
+constexpr int DFS_CS = 12, DFS_CS_FEW = 16, DFS_MAX = 384, DFS_GLOBAL_MAX = 1024;
+
+// Clusters of `cs` CTAs that run at once, a CTA to an SM; cached per kernel, size and device.
+int dfs_active(const void* kernel, int cs, int threads) {
+  static std::mutex mu;
+  static std::map<std::tuple<const void*, int, int>, int> cache;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lk(mu);
+  auto key = std::make_tuple(kernel, cs, dev);
+  auto it = cache.find(key);
+  if (it != cache.end()) return it->second;
+  int active = 0;
+  if (ensure_kernel_smem(kernel, DFS_SMEM, cs > 8) == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cs, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = DFS_SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      active = 0;
+    }
+  }
+  cache[key] = active;
+  return active;
+}
 
 template <int NT, int EPT, int ROWS>
 cudaError_t dfs_launch(cudaStream_t st, void* H, long long sH, int n0, int off, int jend, double* d, cx<double>* e,
                        int ldde, cx<float>* Vh, long long sVh, float* pre, int batch) {
-  const int n = n0 - off, maxloc = (n + DFS_CS - 1) / DFS_CS;
-  const size_t smem = DfsLayout{n, DFS_CS, maxloc, NT / 32, ROWS == ROWS_GLOBAL}.bytes();
+  auto kernel = tridiag_dfs_kernel<NT, EPT, ROWS>;
+  const int few = dfs_active((const void*)kernel, DFS_CS_FEW, NT), many = dfs_active((const void*)kernel, DFS_CS, NT);
+  const int cs = few > 0 && (many < 1 || (batch + few - 1) / few <= (batch + many - 1) / many) ? DFS_CS_FEW : DFS_CS;
+  const int n = n0 - off, maxloc = (n + cs - 1) / cs;
+  const size_t smem = DfsLayout{n, cs, maxloc, NT / 32, ROWS == ROWS_GLOBAL}.bytes();
   if (n < 3 || n > NT * EPT || smem > DFS_SMEM) return cudaErrorInvalidValue;
-  return launch_df(tridiag_dfs_kernel<NT, EPT, ROWS>, DFS_CS, batch, NT, smem, st, H, sH, n0, off, jend, d, e, ldde, Vh,
-                   sVh, pre, maxloc);
+  return launch_df(kernel, cs, batch, NT, smem, st, H, sH, n0, off, jend, d, e, ldde, Vh, sVh, pre, maxloc);
 }
 
 }  // namespace
