@@ -277,7 +277,7 @@ nne_status nne_cgemm_c64(nne_ctx* ctx, int op_a, int op_b, int M, int N, int K, 
  * 160 rows) or in double-float arithmetic on the float32 pipes (larger ones;
  * about 2^-46 relative, in one cluster's shared memory up to 384 rows), bisection and inverse
  * iteration in float64, the back-transformation in float32; 0 runs them in
- * float32 (about 1.5x the gate-step rate at chi = 512, with a float32
+ * float32 (about 1.14x the gate-step rate at chi = 512, with a float32
  * reduction's error of eps_32 times the largest eigenvalue, which turns the
  * eigenvectors next to a flat cut).  complex128 states always use float64.
  * NNE_OPT_GEMM_TMA (default 2): large complex64 GEMMs (M >= 128, N >= 64,
