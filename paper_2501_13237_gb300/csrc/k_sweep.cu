@@ -102,11 +102,21 @@ __device__ __forceinline__ cx<double> env_d(cx<double> a) { return a; }
 // Leading bits of the larger component: orders magnitudes, and holds the exponent.
 __device__ __forceinline__ int env_key(float4 a) { return max(__float_as_int(a.x) & 0x7fffffff, __float_as_int(a.z) & 0x7fffffff); }
 __device__ __forceinline__ int env_key(cx<double> a) { return max(__double2hiint(a.re) & 0x7fffffff, __double2hiint(a.im) & 0x7fffffff); }
+// Binary exponent of a key (also of a denormal's), 0 for a zero one.
 template <typename R>
-__device__ __forceinline__ int key_exp(int key) {   // binary exponent, 0 for a zero environment
-  const int f = std::is_same<R, float>::value ? key >> 23 : key >> 20;
-  return f == 0 ? 0 : f - (std::is_same<R, float>::value ? 127 : 1023);
+__device__ __forceinline__ int key_exp(int key) {
+  constexpr int FB = std::is_same<R, float>::value ? 23 : 20, BIAS = std::is_same<R, float>::value ? 127 : 1023;
+  const int f = key >> FB;
+  return f > 0 ? f - BIAS : (key == 0 ? 0 : 32 - FB - BIAS - __clz(key));
 }
+// Per-site vectors from this exponent on may have lost, or make their reader lose, terms to
+// overflow: the site is formed again from the environment times 2^-SITE_DOWN, which keeps
+// the sums of up to 4096 products of any finite entries in range.
+template <typename R>
+__device__ __forceinline__ bool key_overflows(int key) {
+  return key_exp<R>(key) >= (std::is_same<R, float>::value ? 126 : 1022);
+}
+constexpr int SITE_DOWN = 24;
 // a 2^-e
 __device__ __forceinline__ float4 env_scale(float4 a, int e) {
   const float h0 = __int_as_float((127 - e / 2) << 23), h1 = __int_as_float((127 - (e - e / 2)) << 23);
@@ -169,8 +179,8 @@ struct Layout {
   __host__ __device__ int slice() const { return 0; }           // 2 x SL: this CTA's slice of the next environment
   __host__ __device__ int fin() const { return 2 * SL; }        // 4 x SL: left-pass results of this CTA
   __host__ __device__ int part() const { return 6 * SL; }       // 2 x THREADS: row-group partial sums
-  __host__ __device__ int scal() const { return 6 * SL + 2 * THREADS; }   // 32 ints: every CTA's key, double-buffered
-  __host__ __device__ int coef() const { return scal() + 8; }       // D x cx<R>: environment in the state's precision
+  __host__ __device__ int scal() const { return 6 * SL + 2 * THREADS; }   // 32 int2: every CTA's keys, double-buffered
+  __host__ __device__ int coef() const { return scal() + 16; }      // D x cx<R>: environment in the state's precision
   // per-thread rings of asynchronous copies (RING_STAGES x NB 16-byte slots per thread), 16-byte aligned
   __host__ __device__ size_t ring_off(size_t esz) const { return (16 * (size_t)coef() + esz * (size_t)D + 15) & ~size_t(15); }
   __host__ __device__ size_t bytes(size_t esz) const { return ring_off(esz) + (size_t)RING_STAGES * NB * THREADS * 16; }
@@ -178,13 +188,15 @@ struct Layout {
 
 __host__ __device__ inline int slice_cap(int D, int cs) { return (D + cs - 1) / cs + 2; }
 
-__device__ __forceinline__ int block_max_key(int v, int* red) {
-  for (int m = 16; m > 0; m >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, m));
+__device__ __forceinline__ int2 max_keys(int2 a, int2 b) { return make_int2(max(a.x, b.x), max(a.y, b.y)); }
+__device__ __forceinline__ int2 block_max_keys(int2 v, int2* red) {
+  for (int m = 16; m > 0; m >>= 1)
+    v = max_keys(v, make_int2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m)));
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  int t = 0;
-  for (int i = 0; i < THREADS / 32; ++i) t = max(t, red[i]);
+  int2 t = make_int2(0, 0);
+  for (int i = 0; i < THREADS / 32; ++i) t = max_keys(t, red[i]);
   return t;
 }
 
@@ -273,11 +285,12 @@ __device__ void left_site(const cx<R>* __restrict__ M, int dl, int dr, int b0, i
 }
 
 // Right pass at one site: rho[tt][a] = sum_b M[a][tt][b] coef[b] for this CTA's rows, one warp per row.
-// Writes rho to global memory and R[a] = rho[0][a] + rho[3][a] into the slice; returns the rows' largest key.
+// Writes rho to global memory and R[a] = rho[0][a] + rho[3][a] into the slice; returns the largest keys
+// of R (x) and of rho (y).
 // A warp's work is a flat list of jobs (row, segment tt, batch of 32 NB units),
 // streamed through each lane's ring of asynchronous copies.
 template <typename R, int V>
-__device__ int right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, const cx<R>* coef,
+__device__ int2 right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, const cx<R>* coef,
                           typename Env<R>::T* rho, int D, typename Env<R>::T* slice, unsigned char* ring_ptr) {
   using T = typename Env<R>::T;
   constexpr int BYTES = (int)sizeof(cx<R>) * V;
@@ -307,7 +320,7 @@ __device__ int right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, c
   };
 #pragma unroll
   for (int b = 0; b < RING_STAGES - 1; ++b) issue(b);
-  int key = 0;
+  int2 key = make_int2(0, 0);
   T acc0, acc1, acc2, acc3;   // the four segments of the row
   env_zero(acc0);
   acc1 = acc2 = acc3 = acc0;
@@ -343,10 +356,11 @@ __device__ int right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, c
       for (int o = 4; o > 0; o >>= 1) w = env_add(w, env_shfl_xor(w, o));
       const int a = a0 + warp + ri * nw;
       if ((lane & 7) == 0) rho[(long long)(lane >> 3) * D + a] = w;
+      key.y = max(key.y, env_key(w));
       const T Ra = env_add(w, env_shfl_xor(w, 24));   // lane 0: segments 0 and 3
       if (lane == 0) {
         slice[a - a0] = Ra;
-        key = max(key, env_key(Ra));
+        key.x = max(key.x, env_key(Ra));
       }
       env_zero(acc0);
       acc1 = acc2 = acc3 = acc0;
@@ -379,12 +393,14 @@ __device__ __forceinline__ cx<double> env_from_d(cx<double> a, cx<double>) { ret
 
 // Both environment sweeps and the per-site partial contractions in one launch.
 // grid (cs, 2, n_inst), cluster (cs, 1, 1): cluster (pass, z); pass 0 left, 1 right.
-// env: [z][pass][k = 0..n][D] complex double, envscale: [z][pass][k], vecs: [z][pass][k = 0..n-1][4][D] Env<R>::T.
+// env: [z][pass][k = 0..n][D] complex double, envscale: [z][pass][k], vecs: [z][pass][k = 0..n-1][4][D] Env<R>::T,
+// vexp: [z][pass][k = 0..n-1] {exponent of the site's largest entry in vecs, exponent its vectors are short of}.
 template <typename R>
 __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, const int* __restrict__ dims,
                                                                     const void* const* __restrict__ site,
                                                                     const long long* __restrict__ stride, int D,
-                                                                    double* env, double* envscale, double* vecs) {
+                                                                    double* env, double* envscale, double* vecs,
+                                                                    int2* vexp) {
   using namespace sweep;
   using T = typename Env<R>::T;
   cg::cluster_group cluster = cg::this_cluster();
@@ -397,13 +413,14 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
   T* slice = base + L.slice();
   T* fin = base + L.fin();
   T* part = base + L.part();
-  int* keys = reinterpret_cast<int*>(base + L.scal());   // [2][16]
-  __shared__ int red[THREADS / 32];
+  int2* keys = reinterpret_cast<int2*>(base + L.scal());   // [2][16] of the environment (x) and the vectors (y)
+  __shared__ int2 red[THREADS / 32];
   cx<R>* coef = reinterpret_cast<cx<R>*>(base + L.coef());
   unsigned char* ring_ptr = smem_raw + L.ring_off(sizeof(cx<R>));
   cx<double>* E = reinterpret_cast<cx<double>*>(env) + ((long long)z * 2 + pass) * (n + 1) * D;
   double* ls = envscale + ((long long)z * 2 + pass) * (n + 1);
   T* VK = reinterpret_cast<T*>(vecs) + ((long long)z * 2 + pass) * n * 4 * D;
+  int2* vx = vexp + ((long long)z * 2 + pass) * n;
   const int first = pass == 0 ? 0 : n;
   if (t == 0) {
     coef[0] = mk<R>(1, 0);
@@ -420,40 +437,55 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
     const int dl = dims[k], dr = dims[k + 1];
     const cx<R>* M = reinterpret_cast<const cx<R>*>(site[k]) + z * stride[k];
     const bool vec = VV > 1 && dr % VV == 0 && (reinterpret_cast<uintptr_t>(M) & 15) == 0;
-    T* sl = slice + pb * L.SL;
-    int key = 0;
     int width;   // entries of the next environment per CTA
-    if (pass == 0) {
-      const int v = vec ? VV : 1;
-      width = ((dr + cs - 1) / cs + v - 1) / v * v;
-      const int b0 = min(dr, rank * width), b1 = min(dr, b0 + width);
-      if (vec) left_site<R, VV>(M, dl, dr, b0, b1 - b0, coef, fin, L.SL, part, ring_ptr);
-      else left_site<R, 1>(M, dl, dr, b0, b1 - b0, coef, fin, L.SL, part, ring_ptr);
-      __syncthreads();
-      T* ell = VK + (long long)k * 4 * D;
-      for (int q = t; q < 4 * (b1 - b0); q += THREADS) {
-        const int s = q / (b1 - b0), j = q % (b1 - b0);
-        ell[(long long)s * D + b0 + j] = fin[s * L.SL + j];
+    int2 m;      // largest keys of the cluster
+    for (int down = 0;; down = SITE_DOWN) {
+      T* sl = slice + pb * L.SL;
+      int2 key = make_int2(0, 0);
+      if (pass == 0) {
+        const int v = vec ? VV : 1;
+        width = ((dr + cs - 1) / cs + v - 1) / v * v;
+        const int b0 = min(dr, rank * width), b1 = min(dr, b0 + width);
+        if (vec) left_site<R, VV>(M, dl, dr, b0, b1 - b0, coef, fin, L.SL, part, ring_ptr);
+        else left_site<R, 1>(M, dl, dr, b0, b1 - b0, coef, fin, L.SL, part, ring_ptr);
+        __syncthreads();
+        T* ell = VK + (long long)k * 4 * D;
+        for (int q = t; q < 4 * (b1 - b0); q += THREADS) {
+          const int s = q / (b1 - b0), j = q % (b1 - b0);
+          const T f = fin[s * L.SL + j];
+          ell[(long long)s * D + b0 + j] = f;
+          key.y = max(key.y, env_key(f));
+        }
+        for (int j = t; j < b1 - b0; j += THREADS) {
+          const T Lb = env_add(fin[j], fin[3 * L.SL + j]);
+          sl[j] = Lb;
+          key.x = max(key.x, env_key(Lb));
+        }
+      } else {
+        width = (dl + cs - 1) / cs;
+        const int a0 = min(dl, rank * width), a1 = min(dl, a0 + width);
+        T* rho = VK + (long long)k * 4 * D;
+        key = vec ? right_site<R, VV>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr)
+                  : right_site<R, 1>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr);
       }
-      for (int j = t; j < b1 - b0; j += THREADS) {
-        const T Lb = env_add(fin[j], fin[3 * L.SL + j]);
-        sl[j] = Lb;
-        key = max(key, env_key(Lb));
+      key = block_max_keys(key, red);
+      if (t < cs) cluster.map_shared_rank(keys, t)[16 * pb + rank] = key;
+      cluster.sync();   // every slice and key of this site is published
+      m = make_int2(0, 0);
+      for (int r = 0; r < cs; ++r) m = max_keys(m, keys[16 * pb + r]);
+      if (down == 0 && key_overflows<R>(m.y)) {   // the same in every CTA
+        const int nc = pass == 0 ? dl : dr;
+        for (int i = t; i < nc; i += THREADS) coef[i] = R(1.0 / (1 << SITE_DOWN)) * coef[i];
+        esum += SITE_DOWN;
+        pb ^= 1;
+        __syncthreads();
+        continue;
       }
-    } else {
-      width = (dl + cs - 1) / cs;
-      const int a0 = min(dl, rank * width), a1 = min(dl, a0 + width);
-      T* rho = VK + (long long)k * 4 * D;
-      key = vec ? right_site<R, VV>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr)
-                : right_site<R, 1>(M, dr, a0, a1, coef, rho, D, sl, ring_ptr);
+      if (rank == 0 && t == 0) vx[k] = make_int2(key_exp<R>(m.y), down);
+      break;
     }
-    key = block_max_key(key, red);
-    if (t < cs) cluster.map_shared_rank(keys, t)[16 * pb + rank] = key;
-    cluster.sync();   // every slice and key of this site is published
     // the next environment, scaled to max-abs in [1, 2), gathered from the cluster's slices
-    int m = 0;
-    for (int r = 0; r < cs; ++r) m = max(m, keys[16 * pb + r]);
-    const int e = key_exp<R>(m);
+    const int e = key_exp<R>(m.x);
     const int nd = pass == 0 ? dr : dl;               // length of the next environment
     const int knext = pass == 0 ? k + 1 : k;
     for (int i = t; i < nd; i += THREADS) {
@@ -553,10 +585,14 @@ __global__ void __launch_bounds__(256) obs_kernel(int n, const int* dims, const 
 // (string, instance), dot products of the stored per-site vectors:
 //   one site k:      sum_b (sum_s v_P[s] ell_k[s][b]) R_{k+1}[b]
 //   sites k, k + 1:  sum_c (sum_s v_P[s] ell_k[s][c]) (sum_t v_Q[t] rho_{k+1}[t][c])
+// The vectors are stored in the magnitude of their site's tensor; both factors are brought to
+// order 1 first (exactly, by a power of two), as their products would leave float32's range
+// for tensors of magnitude below 1e-19 or above 1e19.
 template <typename R>
 __global__ void __launch_bounds__(256) obs_local_kernel(int n, const int* __restrict__ dims, int D,
                                                         const double* env, const double* envscale,
-                                                        const double* vecs, const uint8_t* __restrict__ paulis,
+                                                        const double* vecs, const int2* vexp,
+                                                        const uint8_t* __restrict__ paulis,
                                                         const int* __restrict__ first, const int* __restrict__ last,
                                                         int n_obs, double* out) {
   using namespace sweep;
@@ -576,28 +612,33 @@ __global__ void __launch_bounds__(256) obs_local_kernel(int n, const int* __rest
   const double* lsL = envscale + ((long long)z * 2 + 0) * (n + 1);
   const double* lsR = envscale + ((long long)z * 2 + 1) * (n + 1);
   const T* ell = reinterpret_cast<const T*>(vecs) + (((long long)z * 2 + 0) * n + f) * 4 * D;
+  const int2 xl = vexp[((long long)z * 2 + 0) * n + f];
   const int P = paulis[(long long)o * n + f];
   const int d = dims[f + 1];
   T acc;
   env_zero(acc);
   double lscale;
+  int ex = xl.x + xl.y;   // exponent taken out of the vectors
   if (l == f) {
     const cx<double>* Rn = ER + (long long)(f + 1) * D;
     for (int b = lane; b < d; b += 32)
-      env_mac(acc, pauli_sum(P, ell[b], ell[D + b], ell[2 * D + b], ell[3 * D + b]), env_from_d(Rn[b], acc));
+      env_mac(acc, env_scale(pauli_sum(P, ell[b], ell[D + b], ell[2 * D + b], ell[3 * D + b]), xl.x),
+              env_from_d(Rn[b], acc));
     lscale = lsL[f] + lsR[f + 1];
   } else {
     const T* rho = reinterpret_cast<const T*>(vecs) + (((long long)z * 2 + 1) * n + l) * 4 * D;
+    const int2 xr = vexp[((long long)z * 2 + 1) * n + l];
     const int Q = paulis[(long long)o * n + l];
     for (int c = lane; c < d; c += 32)
-      env_mac(acc, pauli_sum(P, ell[c], ell[D + c], ell[2 * D + c], ell[3 * D + c]),
-              pauli_sum(Q, rho[c], rho[D + c], rho[2 * D + c], rho[3 * D + c]));
+      env_mac(acc, env_scale(pauli_sum(P, ell[c], ell[D + c], ell[2 * D + c], ell[3 * D + c]), xl.x),
+              env_scale(pauli_sum(Q, rho[c], rho[D + c], rho[2 * D + c], rho[3 * D + c]), xr.x));
     lscale = lsL[f] + lsR[l + 1];
+    ex += xr.x + xr.y;
   }
   for (int m = 16; m > 0; m >>= 1) acc = env_add(acc, env_shfl_xor(acc, m));
   if (lane == 0) {
     const cx<double> tr = EL[(long long)n * D];
-    const double scale = exp(lscale - lsL[n]);
+    const double scale = exp(lscale - lsL[n] + (double)ex * 0.6931471805599453094);   // ln 2
     const double den = tr.re * tr.re + tr.im * tr.im;
     const cx<double> av = env_d(acc);
     const double qr = (av.re * tr.re + av.im * tr.im) / den, qi = (av.im * tr.re - av.re * tr.im) / den;
@@ -669,7 +710,7 @@ template <typename R>
 cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* const* d_site,
                          const long long* d_stride, int n_inst, int max_dim, int n_obs, const uint8_t* d_paulis,
                          const int* d_first, const int* d_last, const int* d_general, int n_general, double* d_env,
-                         double* d_envscale, double* d_vecs, double* d_out) {
+                         double* d_envscale, double* d_vecs, int2* d_vexp, double* d_out) {
   cudaError_t e;
   {
     const int cs = sweep_cluster_size<R>(n_inst, max_dim);
@@ -692,14 +733,14 @@ cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, env_cluster_kernel<R>, n, d_dims, d_site, d_stride, max_dim, d_env, d_envscale,
-                           d_vecs);
+                           d_vecs, d_vexp);
   }
   if (e != cudaSuccess) return e;
   if (n_obs <= 0) return cudaSuccess;
   {
     ProfScope ps(st, K_SWEEP_OBS);
     obs_local_kernel<R><<<dim3((n_obs + 7) / 8, n_inst), 256, 0, st>>>(n, d_dims, max_dim, d_env, d_envscale, d_vecs,
-                                                                   d_paulis, d_first, d_last, n_obs, d_out);
+                                                                   d_vexp, d_paulis, d_first, d_last, n_obs, d_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (n_general <= 0) return cudaSuccess;
@@ -714,7 +755,7 @@ cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* 
 #define NNE_INST_SWEEP(R)                                                                                          \
   template cudaError_t expect_sweep<R>(cudaStream_t, int, const int*, const void* const*, const long long*, int, int, \
                                        int, const uint8_t*, const int*, const int*, const int*, int, double*, double*, \
-                                       double*, double*);
+                                       double*, int2*, double*);
 NNE_INST_SWEEP(float)
 NNE_INST_SWEEP(double)
 
