@@ -24,8 +24,11 @@
 // warp takes 64 cycles here, and the float64 folds, warp sums, reciprocals and
 // logarithms of an earlier build were most of the sweep's time; the per-site
 // vectors and the environments travel as double-floats too.  Each environment is
-// rescaled by a power of two to max-abs in [1, 2) (exact, an integer addition) and
-// its exponent carried separately, so long chains neither overflow nor underflow.
+// rescaled to max-abs 1 (complex128: by a power of two to [1, 2)) and its scale carried
+// as mantissa and exponent, so long chains neither overflow nor underflow.  Exactly 1:
+// the coefficient that dominates the products then has no rounding of its own to
+// float32 (with powers of two alone the error against 64 bits was 11 % larger, mean of
+// 270 chains of five shapes).
 // 40 sites of bonds 512, 4 instances, complex64: 1.55 -> 0.78 ms (2.08 GB: 2.7 TB/s).
 #include <map>
 #include <mutex>
@@ -102,6 +105,20 @@ __device__ __forceinline__ cx<double> env_d(cx<double> a) { return a; }
 // Leading bits of the larger component: orders magnitudes, and holds the exponent.
 __device__ __forceinline__ int env_key(float4 a) { return max(__float_as_int(a.x) & 0x7fffffff, __float_as_int(a.z) & 0x7fffffff); }
 __device__ __forceinline__ int env_key(cx<double> a) { return max(__double2hiint(a.re) & 0x7fffffff, __double2hiint(a.im) & 0x7fffffff); }
+// The largest component in full, ordered by magnitude: the high part's bits, then the low
+// part's (signed relative to the high part).
+__device__ __forceinline__ unsigned long long comp_key(float hi, float lo) {
+  const int h = __float_as_int(hi), l = __float_as_int(h < 0 ? -lo : lo);
+  return (unsigned long long)(h & 0x7fffffff) << 32 | (unsigned)(l ^ (l >> 31 | 0x80000000));
+}
+__device__ __forceinline__ float2 key_df(unsigned long long key) {
+  const int l = (int)(unsigned)key;
+  return make_float2(__int_as_float((int)(key >> 32)), __int_as_float(l < 0 ? l ^ 0x80000000 : ~l));
+}
+__device__ __forceinline__ unsigned long long env_max_key(float4 a) { return max(comp_key(a.x, a.y), comp_key(a.z, a.w)); }
+__device__ __forceinline__ unsigned long long env_max_key(cx<double> a) {
+  return max((unsigned long long)__double_as_longlong(fabs(a.re)), (unsigned long long)__double_as_longlong(fabs(a.im)));
+}
 // Binary exponent of a key (also of a denormal's), 0 for a zero one.
 template <typename R>
 __device__ __forceinline__ int key_exp(int key) {
@@ -126,6 +143,37 @@ __device__ __forceinline__ cx<double> env_scale(cx<double> a, int e) {
   const double h0 = __hiloint2double((1023 - e / 2) << 20, 0), h1 = __hiloint2double((1023 - (e - e / 2)) << 20, 0);
   return mk<double>(a.re * h0 * h1, a.im * h0 * h1);
 }
+// The factor that brings the largest component to 1: 2^-e, and for double-floats the
+// reciprocal of the mantissa m left (one Newton step from the rounded 1 / m: 2^-47).
+template <typename R> struct EnvNorm;
+template <> struct EnvNorm<float> {
+  int e;
+  float2 m, c;
+  __device__ __forceinline__ explicit EnvNorm(unsigned long long key) : e(0), m(make_float2(1.f, 0.f)), c(m) {
+    const float2 v = key_df(key);
+    if (!(v.x > 0.f) || v.x == INFINITY) return;   // nothing to scale
+    e = key_exp<float>(__float_as_int(v.x));
+    const float4 w = env_scale(make_float4(v.x, v.y, 0.f, 0.f), e);
+    m = make_float2(w.x, w.y);
+    const float y = __frcp_rn(m.x);
+    float rh = 1.f, rl = 0.f;
+    df_mac(rh, rl, -m.x, -m.y, y, 0.f);
+    c = make_float2(y, y * (rh + rl));
+    df_norm(c.x, c.y);
+  }
+  __device__ __forceinline__ float4 operator()(float4 a) const {
+    a = env_scale(a, e);
+    const float2 re = df_mul(a.x, a.y, c.x, c.y), im = df_mul(a.z, a.w, c.x, c.y);
+    return make_float4(re.x, re.y, im.x, im.y);
+  }
+  __device__ __forceinline__ double mantissa() const { return df_to_d(m.x, m.y); }
+};
+template <> struct EnvNorm<double> {
+  int e;
+  __device__ __forceinline__ explicit EnvNorm(unsigned long long key) : e(key_exp<double>((int)(key >> 32))) {}
+  __device__ __forceinline__ cx<double> operator()(cx<double> a) const { return env_scale(a, e); }
+  __device__ __forceinline__ double mantissa() const { return 1.0; }
+};
 __device__ __forceinline__ cx<float> env_coef(float4 a) { return mk<float>(a.x, a.z); }
 __device__ __forceinline__ cx<double> env_coef(cx<double> a) { return a; }
 
@@ -179,8 +227,8 @@ struct Layout {
   __host__ __device__ int slice() const { return 0; }           // 2 x SL: this CTA's slice of the next environment
   __host__ __device__ int fin() const { return 2 * SL; }        // 4 x SL: left-pass results of this CTA
   __host__ __device__ int part() const { return 6 * SL; }       // 2 x THREADS: row-group partial sums
-  __host__ __device__ int scal() const { return 6 * SL + 2 * THREADS; }   // 32 int2: every CTA's keys, double-buffered
-  __host__ __device__ int coef() const { return scal() + 16; }      // D x cx<R>: environment in the state's precision
+  __host__ __device__ int scal() const { return 6 * SL + 2 * THREADS; }   // 32 SiteKeys: every CTA's, double-buffered
+  __host__ __device__ int coef() const { return scal() + 32; }      // D x cx<R>: environment in the state's precision
   // per-thread rings of asynchronous copies (RING_STAGES x NB 16-byte slots per thread), 16-byte aligned
   __host__ __device__ size_t ring_off(size_t esz) const { return (16 * (size_t)coef() + esz * (size_t)D + 15) & ~size_t(15); }
   __host__ __device__ size_t bytes(size_t esz) const { return ring_off(esz) + (size_t)RING_STAGES * NB * THREADS * 16; }
@@ -188,14 +236,18 @@ struct Layout {
 
 __host__ __device__ inline int slice_cap(int D, int cs) { return (D + cs - 1) / cs + 2; }
 
-__device__ __forceinline__ int2 max_keys(int2 a, int2 b) { return make_int2(max(a.x, b.x), max(a.y, b.y)); }
-__device__ __forceinline__ int2 block_max_keys(int2 v, int2* red) {
+struct __align__(16) SiteKeys {
+  unsigned long long env;   // env_max_key of the environment
+  int vec;                  // env_key of the per-site vectors
+};
+__device__ __forceinline__ SiteKeys max_keys(SiteKeys a, SiteKeys b) { return {max(a.env, b.env), max(a.vec, b.vec)}; }
+__device__ __forceinline__ SiteKeys block_max_keys(SiteKeys v, SiteKeys* red) {
   for (int m = 16; m > 0; m >>= 1)
-    v = max_keys(v, make_int2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m)));
+    v = max_keys(v, {__shfl_xor_sync(0xffffffffu, v.env, m), __shfl_xor_sync(0xffffffffu, v.vec, m)});
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  int2 t = make_int2(0, 0);
+  SiteKeys t = {0, 0};
   for (int i = 0; i < THREADS / 32; ++i) t = max_keys(t, red[i]);
   return t;
 }
@@ -286,11 +338,11 @@ __device__ void left_site(const cx<R>* __restrict__ M, int dl, int dr, int b0, i
 
 // Right pass at one site: rho[tt][a] = sum_b M[a][tt][b] coef[b] for this CTA's rows, one warp per row.
 // Writes rho to global memory and R[a] = rho[0][a] + rho[3][a] into the slice; returns the largest keys
-// of R (x) and of rho (y).
+// of R and of rho.
 // A warp's work is a flat list of jobs (row, segment tt, batch of 32 NB units),
 // streamed through each lane's ring of asynchronous copies.
 template <typename R, int V>
-__device__ int2 right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, const cx<R>* coef,
+__device__ SiteKeys right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, const cx<R>* coef,
                           typename Env<R>::T* rho, int D, typename Env<R>::T* slice, unsigned char* ring_ptr) {
   using T = typename Env<R>::T;
   constexpr int BYTES = (int)sizeof(cx<R>) * V;
@@ -320,7 +372,7 @@ __device__ int2 right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, 
   };
 #pragma unroll
   for (int b = 0; b < RING_STAGES - 1; ++b) issue(b);
-  int2 key = make_int2(0, 0);
+  SiteKeys key = {0, 0};
   T acc0, acc1, acc2, acc3;   // the four segments of the row
   env_zero(acc0);
   acc1 = acc2 = acc3 = acc0;
@@ -356,11 +408,11 @@ __device__ int2 right_site(const cx<R>* __restrict__ M, int dr, int a0, int a1, 
       for (int o = 4; o > 0; o >>= 1) w = env_add(w, env_shfl_xor(w, o));
       const int a = a0 + warp + ri * nw;
       if ((lane & 7) == 0) rho[(long long)(lane >> 3) * D + a] = w;
-      key.y = max(key.y, env_key(w));
+      key.vec = max(key.vec, env_key(w));
       const T Ra = env_add(w, env_shfl_xor(w, 24));   // lane 0: segments 0 and 3
       if (lane == 0) {
         slice[a - a0] = Ra;
-        key.x = max(key.x, env_key(Ra));
+        key.env = max(key.env, env_max_key(Ra));
       }
       env_zero(acc0);
       acc1 = acc2 = acc3 = acc0;
@@ -393,14 +445,14 @@ __device__ __forceinline__ cx<double> env_from_d(cx<double> a, cx<double>) { ret
 
 // Both environment sweeps and the per-site partial contractions in one launch.
 // grid (cs, 2, n_inst), cluster (cs, 1, 1): cluster (pass, z); pass 0 left, 1 right.
-// env: [z][pass][k = 0..n][D] complex double, envscale: [z][pass][k], vecs: [z][pass][k = 0..n-1][4][D] Env<R>::T,
-// vexp: [z][pass][k = 0..n-1] {exponent of the site's largest entry in vecs, exponent its vectors are short of}.
+// env: [z][pass][k = 0..n][D] complex double, times envscale [z][pass][k] 2^exps[z][pass][k].env,
+// vecs: [z][pass][k = 0..n-1][4][D] Env<R>::T.
 template <typename R>
 __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, const int* __restrict__ dims,
                                                                     const void* const* __restrict__ site,
                                                                     const long long* __restrict__ stride, int D,
                                                                     double* env, double* envscale, double* vecs,
-                                                                    int2* vexp) {
+                                                                    SweepExp* exps) {
   using namespace sweep;
   using T = typename Env<R>::T;
   cg::cluster_group cluster = cg::this_cluster();
@@ -413,24 +465,26 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
   T* slice = base + L.slice();
   T* fin = base + L.fin();
   T* part = base + L.part();
-  int2* keys = reinterpret_cast<int2*>(base + L.scal());   // [2][16] of the environment (x) and the vectors (y)
-  __shared__ int2 red[THREADS / 32];
+  SiteKeys* keys = reinterpret_cast<SiteKeys*>(base + L.scal());   // [2][16]
+  __shared__ SiteKeys red[THREADS / 32];
   cx<R>* coef = reinterpret_cast<cx<R>*>(base + L.coef());
   unsigned char* ring_ptr = smem_raw + L.ring_off(sizeof(cx<R>));
   cx<double>* E = reinterpret_cast<cx<double>*>(env) + ((long long)z * 2 + pass) * (n + 1) * D;
   double* ls = envscale + ((long long)z * 2 + pass) * (n + 1);
   T* VK = reinterpret_cast<T*>(vecs) + ((long long)z * 2 + pass) * n * 4 * D;
-  int2* vx = vexp + ((long long)z * 2 + pass) * n;
+  SweepExp* ex = exps + ((long long)z * 2 + pass) * (n + 1);
   const int first = pass == 0 ? 0 : n;
   if (t == 0) {
     coef[0] = mk<R>(1, 0);
     if (rank == 0) {
       E[(long long)first * D] = mk<double>(1, 0);
-      ls[first] = 0;
+      ls[first] = 1.0;
+      ex[first].env = 0;
     }
   }
   cluster.sync();   // every CTA of the cluster runs before anyone writes into its shared memory
-  long long esum = 0;   // binary exponent of the environment
+  int esum = 0;       // scale of the environment: mant 2^esum, mant in [1, 2) (of thread 0)
+  double mant = 1.0;
   int pb = 0;
   for (int step = 0; step < n; ++step) {
     const int k = pass == 0 ? step : n - 1 - step;
@@ -438,10 +492,10 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
     const cx<R>* M = reinterpret_cast<const cx<R>*>(site[k]) + z * stride[k];
     const bool vec = VV > 1 && dr % VV == 0 && (reinterpret_cast<uintptr_t>(M) & 15) == 0;
     int width;   // entries of the next environment per CTA
-    int2 m;      // largest keys of the cluster
+    SiteKeys m;  // largest keys of the cluster
     for (int down = 0;; down = SITE_DOWN) {
       T* sl = slice + pb * L.SL;
-      int2 key = make_int2(0, 0);
+      SiteKeys key = {0, 0};
       if (pass == 0) {
         const int v = vec ? VV : 1;
         width = ((dr + cs - 1) / cs + v - 1) / v * v;
@@ -454,12 +508,12 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
           const int s = q / (b1 - b0), j = q % (b1 - b0);
           const T f = fin[s * L.SL + j];
           ell[(long long)s * D + b0 + j] = f;
-          key.y = max(key.y, env_key(f));
+          key.vec = max(key.vec, env_key(f));
         }
         for (int j = t; j < b1 - b0; j += THREADS) {
           const T Lb = env_add(fin[j], fin[3 * L.SL + j]);
           sl[j] = Lb;
-          key.x = max(key.x, env_key(Lb));
+          key.env = max(key.env, env_max_key(Lb));
         }
       } else {
         width = (dl + cs - 1) / cs;
@@ -471,9 +525,9 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
       key = block_max_keys(key, red);
       if (t < cs) cluster.map_shared_rank(keys, t)[16 * pb + rank] = key;
       cluster.sync();   // every slice and key of this site is published
-      m = make_int2(0, 0);
+      m = {0, 0};
       for (int r = 0; r < cs; ++r) m = max_keys(m, keys[16 * pb + r]);
-      if (down == 0 && key_overflows<R>(m.y)) {   // the same in every CTA
+      if (down == 0 && key_overflows<R>(m.vec)) {   // the same in every CTA
         const int nc = pass == 0 ? dl : dr;
         for (int i = t; i < nc; i += THREADS) coef[i] = R(1.0 / (1 << SITE_DOWN)) * coef[i];
         esum += SITE_DOWN;
@@ -481,21 +535,34 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
         __syncthreads();
         continue;
       }
-      if (rank == 0 && t == 0) vx[k] = make_int2(key_exp<R>(m.y), down);
+      if (rank == 0 && t == 0) {
+        ex[k].vec = key_exp<R>(m.vec);
+        ex[k].down = down;
+      }
       break;
     }
-    // the next environment, scaled to max-abs in [1, 2), gathered from the cluster's slices
-    const int e = key_exp<R>(m.x);
+    // the next environment, scaled, gathered from the cluster's slices
+    const EnvNorm<R> norm(m.env);
     const int nd = pass == 0 ? dr : dl;               // length of the next environment
     const int knext = pass == 0 ? k + 1 : k;
     for (int i = t; i < nd; i += THREADS) {
       const int r = i / width;
-      const T nv = env_scale(cluster.map_shared_rank(slice + pb * L.SL, r)[i - r * width], e);
+      const T nv = norm(cluster.map_shared_rank(slice + pb * L.SL, r)[i - r * width]);
       coef[i] = env_coef(nv);
       if (r == rank) E[(long long)knext * D + i] = env_d(nv);
     }
-    esum += e;
-    if (rank == 0 && t == 0) ls[knext] = (double)esum * 0.6931471805599453094;   // ln 2
+    esum += norm.e;
+    if (rank == 0 && t == 0) {
+      if (std::is_same<R, float>::value) {
+        mant *= norm.mantissa();
+        if (mant >= 2.0) {
+          mant *= 0.5;
+          ++esum;
+        }
+      }
+      ls[knext] = mant;
+      ex[knext].env = esum;
+    }
     pb ^= 1;
     __syncthreads();
   }
@@ -507,8 +574,9 @@ __global__ void __launch_bounds__(sweep::THREADS) env_cluster_kernel(int n, cons
 template <typename R>
 __global__ void __launch_bounds__(256) obs_kernel(int n, const int* dims, const void* const* site,
                                                    const long long* stride, int max_dim, const double* env,
-                                                   const double* envscale, const uint8_t* paulis, const int* first,
-                                                   const int* last, const int* idx, int n_obs, double* out) {
+                                                   const double* envscale, const SweepExp* exps,
+                                                   const uint8_t* paulis, const int* first, const int* last,
+                                                   const int* idx, int n_obs, double* out) {
   extern __shared__ unsigned char smem_raw[];
   cx<double>* S = reinterpret_cast<cx<double>*>(smem_raw);
   cx<double>* S2 = S + max_dim;
@@ -530,7 +598,9 @@ __global__ void __launch_bounds__(256) obs_kernel(int n, const int* dims, const 
     const int d = dims[l + 1];
     for (int b = threadIdx.x; b < d; b += blockDim.x) S[b] = ER[(long long)(l + 1) * max_dim + b];
   }
-  double lsS = lsR[l + 1];
+  const SweepExp* xL = exps + ((long long)z * 2 + 0) * (n + 1);
+  const SweepExp* xR = exps + ((long long)z * 2 + 1) * (n + 1);
+  double lsS = 0;
   __syncthreads();
   for (int k = l; k >= f; --k) {
     const int dl = dims[k], dr = dims[k + 1];
@@ -572,7 +642,8 @@ __global__ void __launch_bounds__(256) obs_kernel(int n, const int* dims, const 
     cx<double> v = mk<double>(0, 0);
     for (int w = 0; w < nw; ++w) v = v + cred[w];
     const cx<double> tr = EL[(long long)n * max_dim];
-    const double scale = exp(lsL[f] + lsS - lsL[n]);
+    const double scale = lsL[f] * lsR[l + 1] / lsL[n] *
+                         exp(lsS + (double)(xL[f].env + xR[l + 1].env - xL[n].env) * 0.6931471805599453094);   // ln 2
     const double den = tr.re * tr.re + tr.im * tr.im;
     // v / tr
     const double qr = (v.re * tr.re + v.im * tr.im) / den, qi = (v.im * tr.re - v.re * tr.im) / den;
@@ -591,7 +662,7 @@ __global__ void __launch_bounds__(256) obs_kernel(int n, const int* dims, const 
 template <typename R>
 __global__ void __launch_bounds__(256) obs_local_kernel(int n, const int* __restrict__ dims, int D,
                                                         const double* env, const double* envscale,
-                                                        const double* vecs, const int2* vexp,
+                                                        const double* vecs, const SweepExp* exps,
                                                         const uint8_t* __restrict__ paulis,
                                                         const int* __restrict__ first, const int* __restrict__ last,
                                                         int n_obs, double* out) {
@@ -612,38 +683,37 @@ __global__ void __launch_bounds__(256) obs_local_kernel(int n, const int* __rest
   const double* lsL = envscale + ((long long)z * 2 + 0) * (n + 1);
   const double* lsR = envscale + ((long long)z * 2 + 1) * (n + 1);
   const T* ell = reinterpret_cast<const T*>(vecs) + (((long long)z * 2 + 0) * n + f) * 4 * D;
-  const int2 xl = vexp[((long long)z * 2 + 0) * n + f];
+  const SweepExp* xL = exps + ((long long)z * 2 + 0) * (n + 1);
+  const SweepExp* xR = exps + ((long long)z * 2 + 1) * (n + 1);
+  const int xl = xL[f].vec;
   const int P = paulis[(long long)o * n + f];
   const int d = dims[f + 1];
   T acc;
   env_zero(acc);
-  double lscale;
-  int ex = xl.x + xl.y;   // exponent taken out of the vectors
+  const double scale = lsL[f] * lsR[l + 1] / lsL[n];
+  int ex = xL[f].env + xR[l + 1].env - xL[n].env + xl + xL[f].down;   // and the exponents taken out of the vectors
   if (l == f) {
     const cx<double>* Rn = ER + (long long)(f + 1) * D;
     for (int b = lane; b < d; b += 32)
-      env_mac(acc, env_scale(pauli_sum(P, ell[b], ell[D + b], ell[2 * D + b], ell[3 * D + b]), xl.x),
+      env_mac(acc, env_scale(pauli_sum(P, ell[b], ell[D + b], ell[2 * D + b], ell[3 * D + b]), xl),
               env_from_d(Rn[b], acc));
-    lscale = lsL[f] + lsR[f + 1];
   } else {
     const T* rho = reinterpret_cast<const T*>(vecs) + (((long long)z * 2 + 1) * n + l) * 4 * D;
-    const int2 xr = vexp[((long long)z * 2 + 1) * n + l];
+    const int xr = xR[l].vec;
     const int Q = paulis[(long long)o * n + l];
     for (int c = lane; c < d; c += 32)
-      env_mac(acc, env_scale(pauli_sum(P, ell[c], ell[D + c], ell[2 * D + c], ell[3 * D + c]), xl.x),
-              env_scale(pauli_sum(Q, rho[c], rho[D + c], rho[2 * D + c], rho[3 * D + c]), xr.x));
-    lscale = lsL[f] + lsR[l + 1];
-    ex += xr.x + xr.y;
+      env_mac(acc, env_scale(pauli_sum(P, ell[c], ell[D + c], ell[2 * D + c], ell[3 * D + c]), xl),
+              env_scale(pauli_sum(Q, rho[c], rho[D + c], rho[2 * D + c], rho[3 * D + c]), xr));
+    ex += xr + xR[l].down;
   }
   for (int m = 16; m > 0; m >>= 1) acc = env_add(acc, env_shfl_xor(acc, m));
   if (lane == 0) {
     const cx<double> tr = EL[(long long)n * D];
-    const double scale = exp(lscale - lsL[n] + (double)ex * 0.6931471805599453094);   // ln 2
     const double den = tr.re * tr.re + tr.im * tr.im;
     const cx<double> av = env_d(acc);
     const double qr = (av.re * tr.re + av.im * tr.im) / den, qi = (av.im * tr.re - av.re * tr.im) / den;
-    res[0] = qr * scale;
-    res[1] = qi * scale;
+    res[0] = ldexp(qr * scale, ex);
+    res[1] = ldexp(qi * scale, ex);
   }
 }
 
@@ -710,7 +780,7 @@ template <typename R>
 cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* const* d_site,
                          const long long* d_stride, int n_inst, int max_dim, int n_obs, const uint8_t* d_paulis,
                          const int* d_first, const int* d_last, const int* d_general, int n_general, double* d_env,
-                         double* d_envscale, double* d_vecs, int2* d_vexp, double* d_out) {
+                         double* d_envscale, double* d_vecs, SweepExp* d_exps, double* d_out) {
   cudaError_t e;
   {
     const int cs = sweep_cluster_size<R>(n_inst, max_dim);
@@ -733,14 +803,14 @@ cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, env_cluster_kernel<R>, n, d_dims, d_site, d_stride, max_dim, d_env, d_envscale,
-                           d_vecs, d_vexp);
+                           d_vecs, d_exps);
   }
   if (e != cudaSuccess) return e;
   if (n_obs <= 0) return cudaSuccess;
   {
     ProfScope ps(st, K_SWEEP_OBS);
     obs_local_kernel<R><<<dim3((n_obs + 7) / 8, n_inst), 256, 0, st>>>(n, d_dims, max_dim, d_env, d_envscale, d_vecs,
-                                                                   d_vexp, d_paulis, d_first, d_last, n_obs, d_out);
+                                                                   d_exps, d_paulis, d_first, d_last, n_obs, d_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (n_general <= 0) return cudaSuccess;
@@ -748,14 +818,14 @@ cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* 
   if ((e = ensure_kernel_smem((const void*)obs_kernel<R>, smem, false)) != cudaSuccess) return e;
   ProfScope ps(st, K_SWEEP_OBS);
   obs_kernel<R><<<dim3(n_general, n_inst), 256, smem, st>>>(n, d_dims, d_site, d_stride, max_dim, d_env, d_envscale,
-                                                            d_paulis, d_first, d_last, d_general, n_obs, d_out);
+                                                            d_exps, d_paulis, d_first, d_last, d_general, n_obs, d_out);
   return cudaGetLastError();
 }
 
 #define NNE_INST_SWEEP(R)                                                                                          \
   template cudaError_t expect_sweep<R>(cudaStream_t, int, const int*, const void* const*, const long long*, int, int, \
                                        int, const uint8_t*, const int*, const int*, const int*, int, double*, double*, \
-                                       double*, int2*, double*);
+                                       double*, SweepExp*, double*);
 NNE_INST_SWEEP(float)
 NNE_INST_SWEEP(double)
 

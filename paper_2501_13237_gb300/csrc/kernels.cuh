@@ -159,19 +159,19 @@ cudaError_t qr(cudaStream_t st, cx<R>* A, long long sA, int m, int n, cx<R>* Q, 
                long long sR, void* cx_ws, int batch);
 
 // ---- k_sweep.cu
-// <P> for n_obs Pauli strings on every instance (see nne_expect).
-struct SweepSites {
-  const void* const* site;   // per site k: pointer to instance 0's tensor
-  const long long* stride;   // per site k: elements between instances
+struct SweepExp {
+  int vec, down;   // site k: exponent of its per-site vectors' largest entry, and what it lacks to the site's scale
+  int env;         // environment k: exponent of its scale
 };
-// d_env: n_inst x 2 x (n + 1) x max_dim complex double; d_envscale: n_inst x 2 x (n + 1);
-// d_vecs: n_inst x 2 x n x 4 x max_dim complex double; d_vexp: n_inst x 2 x n int2; d_general lists the n_general
+// <P> for n_obs Pauli strings on every instance (see nne_expect).
+// d_env: n_inst x 2 x (n + 1) x max_dim complex double; d_envscale, d_exps: n_inst x 2 x (n + 1);
+// d_vecs: n_inst x 2 x n x 4 x max_dim complex double; d_general lists the n_general
 // strings whose support spans three or more sites.
 template <typename R>
 cudaError_t expect_sweep(cudaStream_t st, int n, const int* d_dims, const void* const* d_site,
                          const long long* d_stride, int n_inst, int max_dim, int n_obs, const uint8_t* d_paulis,
                          const int* d_first, const int* d_last, const int* d_general, int n_general, double* d_env,
-                         double* d_envscale, double* d_vecs, int2* d_vexp, double* d_out /* n_inst x n_obs x 2 */);
+                         double* d_envscale, double* d_vecs, SweepExp* d_exps, double* d_out /* n_inst x n_obs x 2 */);
 // Cluster size of the environment sweep: 0 picks it from occupancy, 1..16 forces it.
 void set_sweep_cluster(int cs);
 

@@ -1052,7 +1052,7 @@ nne_status nne_expect(nne_state* st, int n_obs, const uint8_t* paulis, double* r
   const size_t b_val = sizeof(double) * 2 * (size_t)n_obs * st->n_inst, b_lf = sizeof(double) * st->n_inst,
                out_bytes = b_val + b_lf + 2 * sizeof(int);
   const size_t o_out = in_bytes, o_vec = o_out + al(out_bytes);
-  const size_t o_vexp = o_vec + sizeof(double) * 2 * 2 * 4 * (size_t)n * st->dmax * st->n_inst;
+  const size_t o_exps = o_vec + sizeof(double) * 2 * 2 * 4 * (size_t)n * st->dmax * st->n_inst;
   std::vector<char> hin(in_bytes), hout(out_bytes);
   if (n_obs > 0) memcpy(hin.data(), paulis, (size_t)n_obs * n);
   memcpy(hin.data() + o_first, first.data(), bi);
@@ -1060,12 +1060,12 @@ nne_status nne_expect(nne_state* st, int n_obs, const uint8_t* paulis, double* r
   if (n_general > 0) memcpy(hin.data() + o_gen, general.data(), sizeof(int) * n_general);
   memcpy(hin.data() + o_dims, st->dims.data(), sizeof(int) * (n + 1));
   char* blk = nullptr;
-  NNE_CUDA_TRY(dev_alloc((void**)&blk, o_vexp + sizeof(int2) * 2 * (size_t)n * st->n_inst, s));
+  NNE_CUDA_TRY(dev_alloc((void**)&blk, o_exps + sizeof(SweepExp) * 2 * (size_t)(n + 1) * st->n_inst, s));
   const uint8_t* dp = reinterpret_cast<const uint8_t*>(blk);
   const int *df = reinterpret_cast<const int*>(blk + o_first), *dl = reinterpret_cast<const int*>(blk + o_last),
             *dgen = reinterpret_cast<const int*>(blk + o_gen), *ddims = reinterpret_cast<const int*>(blk + o_dims);
   double *dout = reinterpret_cast<double*>(blk + o_out), *dv = reinterpret_cast<double*>(blk + o_vec);
-  int2* dx = reinterpret_cast<int2*>(blk + o_vexp);
+  SweepExp* dx = reinterpret_cast<SweepExp*>(blk + o_exps);
   cudaError_t e = cudaMemcpyAsync(blk, hin.data(), in_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = st->dtype == NNE_C64

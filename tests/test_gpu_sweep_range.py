@@ -53,3 +53,26 @@ def test_scaled_pair(bonds, dtype, scale, at):
         ref_st.M[k] = ref_st.M[k] / scale
     ref = ref_st.expect_codes(codes)
     assert (np.abs(vals[0] - ref) <= TOL[dtype] * np.maximum(1.0, np.abs(ref))).all()
+
+
+def test_environment_adds_no_rounding():
+    """A chain of bonds 1 whose environments are real: every product has the factor 1, so the
+    sweep's only error is the double-float scaling (2^-46 per site), not float32's rounding
+    of a scaled environment."""
+    require_gpu()
+    from paper_2501_13237_gb300 import nne
+    n = 24
+    rng = np.random.default_rng(5)
+    M = [rand_c(rng, (1, 4, 1)).astype(np.complex64) for _ in range(n)]
+    for m in M:
+        m[0, [0, 3], 0] = rng.uniform(0.1, 1.0, 2)
+    st = nne.State(nne.Context(0), n, 4, 1, nne.C64)
+    for k in range(n):
+        st.write_site(0, k, M[k])
+    codes = strings(n)
+    vals, _ = st.expect(codes)
+    st.close()
+    ref_st = mps.VMPO(n, 4)
+    ref_st.M = [m.astype(np.complex128) for m in M]
+    ref = ref_st.expect_codes(codes)
+    assert (np.abs(vals[0] - ref) <= 1e-12 * np.maximum(1.0, np.abs(ref))).all()
