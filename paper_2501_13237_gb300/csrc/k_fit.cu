@@ -1,6 +1,6 @@
 // a8 -- noise-strength extrapolation to lambda* in float64 (Sec. 2.2.3 (B);
 // App. B.2): one thread per observable for POLY and EXP_LOGLIN (fit_kernel),
-// one cluster per observable that needs EXP3 (exp3_kernel).
+// clusters that take the observables that need EXP3 (exp3_kernel).
 //   POLY(m):     least squares in t = (lambda - lambda*)/max|lambda - lambda*| by
 //                Householder QR; estimate = constant coefficient.
 //   EXP_LOGLIN:  criterion 2 (|y| >= 1e-10), criterion 3 (sign of the
@@ -252,8 +252,8 @@ __global__ void fit_kernel(int nl, const double* lam, const double* vals, const 
   store_fit(nl, lam, vals, n_obs, o, ls, mask, fb, est, st, out, status);
 }
 
-// EXP3 of the observables fit_kernel marked: one cluster of EXP3_CS CTAs each
-// (the other clusters leave at once).
+// EXP3 of the observables fit_kernel marked.  Clusters of EXP3_CS CTAs each take `per`
+// neighbouring observables at a time, EXP3_CLUSTERS of them at most.
 //
 // Bound by float64 arithmetic, which runs at 1/64 of the float32 rate: a
 // profile at one b costs about 40 operations per level (the exponential most
@@ -264,92 +264,29 @@ __global__ void fit_kernel(int nl, const double* lam, const double* vals, const 
 // lowest index among equal ones, as a scan in order finds it); the golden
 // section that follows is a serial chain of about 60 profiles, each formed by
 // one warp with a level per lane and the sums in level order (whole call of
-// that table: 22.8 ms -> 0.33 ms).
+// that table: 22.8 ms -> 0.3 ms).  The warp's lanes repeat each other's sums, a
+// third of the work on top of the grid's: where every cluster has more than
+// EXP3_WARP observables that need it (a large table), a thread takes one instead,
+// with the same operations in the same order.  EXP3 of 50000 observables at 5
+// levels: 68.1 ms by one thread each, 91.2 with a warp each throughout, 69.6 now;
+// a call over 10^6 observables of which none needs it: 13.3 ms with a cluster for
+// each, 8.6 now.
 constexpr int EXP3_CS = 8, EXP3_THREADS = 128, EXP3_GRID = 4001;
+constexpr int EXP3_CLUSTERS = 4 * 152, EXP3_MOST = 128, EXP3_WARP = 8;
 
-__global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS)
-    exp3_kernel(int nl, const double* lam, const double* vals, int n_obs, double ls, const uint8_t* mask,
-                const double* fb, double* out, int* status, int o0) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int o = o0 + (int)(blockIdx.x / EXP3_CS);
-  if (status[o] != FIT_NEEDS_EXP3) return;   // the same for every CTA of the cluster
-  __shared__ double y[FIT_MAXL], lc[FIT_MAXL];
-  __shared__ double wbest[EXP3_THREADS / 32];
-  __shared__ int widx[EXP3_THREADS / 32];
-  __shared__ double cbest[EXP3_CS];
-  __shared__ int cidx[EXP3_CS];
-  __shared__ int m_s, ok_s;
-  __shared__ double B_s;
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid == 0) {
-    m_s = gather_levels(nl, lam, vals, nullptr, n_obs, o, mask, y, lc, nullptr);
-    double B = 0;
-    ok_s = exp3_range(m_s, lc, &B) ? 1 : 0;
-    B_s = B;
-  }
-  cluster.sync();   // also: every CTA has read status[o], and runs, before rank 0 is written to
-  const int m = m_s;
-  if (!ok_s) {
-    if (rank == 0 && tid == 0) {
-      double est;
-      int st;
-      nofit(m, lc, y, ls, &est, &st);
-      store_fit(nl, lam, vals, n_obs, o, ls, mask, fb, est, st, out, status);
-    }
-    return;
-  }
-  const double B = B_s, step = (2 * B) / (EXP3_GRID - 1);
-  auto gridb = [&](int i) { return (i == EXP3_GRID - 1) ? B : i * step - B; };
-  double best = 1e300, a, c;
-  int bi = 0;
-  for (int i = rank * EXP3_THREADS + tid; i < EXP3_GRID; i += EXP3_CS * EXP3_THREADS) {
-    const double b = gridb(i);
-    const double l = (b == 0.0) ? 1e300 : exp3_profile(b, m, lc, y, &a, &c);
-    if (l < best) { best = l; bi = i; }
-  }
-  for (int d = 16; d > 0; d >>= 1) {
-    const double l2 = __shfl_xor_sync(0xffffffffu, best, d);
-    const int i2 = __shfl_xor_sync(0xffffffffu, bi, d);
-    if (l2 < best || (l2 == best && i2 < bi)) { best = l2; bi = i2; }
-  }
-  if (lane == 0) {
-    wbest[tid >> 5] = best;
-    widx[tid >> 5] = bi;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < EXP3_THREADS / 32; ++w)
-      if (wbest[w] < best || (wbest[w] == best && widx[w] < bi)) { best = wbest[w]; bi = widx[w]; }
-    *cluster.map_shared_rank(&cbest[rank], 0) = best;
-    *cluster.map_shared_rank(&cidx[rank], 0) = bi;
-  }
-  cluster.sync();
-  if (rank != 0 || tid >= 32) return;
-  best = cbest[0];
-  bi = cidx[0];
-  for (int r = 1; r < EXP3_CS; ++r)
-    if (cbest[r] < best || (cbest[r] == best && cidx[r] < bi)) { best = cbest[r]; bi = cidx[r]; }
-  // one profile by the warp: lane j forms the exponentials of levels j and j + 32
-  auto profile = [&](double b) {
-    double e0 = lane < m ? exp(-b * lc[lane]) : 0.0, e1 = lane + 32 < m ? exp(-b * lc[lane + 32]) : 0.0;
-    auto e = [&](int j) { return __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31); };
-    double em = 0, ym = 0;
-    for (int j = 0; j < m; ++j) { em += e(j); ym += y[j]; }
-    em /= m;
-    ym /= m;
-    double see = 0, sey = 0;
-    for (int j = 0; j < m; ++j) { const double ej = e(j); see += (ej - em) * (ej - em); sey += (ej - em) * (y[j] - ym); }
-    a = see > 0 ? sey / see : 0.0;
-    c = ym - a * em;
-    double loss = 0;
-    for (int j = 0; j < m; ++j) { const double r = a * e(j) + c - y[j]; loss += r * r; }
-    return loss;
-  };
-  double lo = gridb(max(bi - 1, 0)), hi = gridb(min(bi + 1, EXP3_GRID - 1));
+__device__ __forceinline__ double exp3_step(double B) { return (2 * B) / (EXP3_GRID - 1); }
+__device__ __forceinline__ double exp3_gridb(int i, double B, double step) {
+  return (i == EXP3_GRID - 1) ? B : i * step - B;
+}
+
+// Golden section around grid point bi: the estimate at ls.  profile(b, &a, &c) is the loss.
+template <typename F>
+__device__ __forceinline__ double exp3_golden(int bi, double B, double step, double ls, F profile) {
+  double a, c;
+  double lo = exp3_gridb(max(bi - 1, 0), B, step), hi = exp3_gridb(min(bi + 1, EXP3_GRID - 1), B, step);
   const double g = (sqrt(5.0) - 1.0) / 2.0;
   double x1 = hi - g * (hi - lo), x2 = lo + g * (hi - lo);
-  auto f = [&](double b) { return b == 0.0 ? 1e300 : profile(b); };
+  auto f = [&](double b) { return b == 0.0 ? 1e300 : profile(b, &a, &c); };
   double f1 = f(x1), f2 = f(x2);
   const double tol = 1e-12 * B;
   for (int it = 0; it < 200 && hi - lo > tol; ++it) {
@@ -365,10 +302,145 @@ __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS)
   }
   double b = 0.5 * (lo + hi);
   if (b == 0.0) b = lo;
-  profile(b);
-  if (lane == 0) {
-    out[o] = a * exp(-b * ls) + c;
-    status[o] = NNE_OK;
+  profile(b, &a, &c);
+  return a * exp(-b * ls) + c;
+}
+
+// The golden section and the result of observable o by one thread.
+__device__ __noinline__ void exp3_finish_thread(int bi, int nl, const double* lam, const double* vals, int n_obs, int o,
+                                                double ls, const uint8_t* mask, const double* fb, double* out,
+                                                int* status) {
+  double y[FIT_MAXL], lc[FIT_MAXL], B = 0, est = 0;
+  const int m = gather_levels(nl, lam, vals, nullptr, n_obs, o, mask, y, lc, nullptr);
+  int st = NNE_OK;
+  if (exp3_range(m, lc, &B))
+    est = exp3_golden(bi, B, exp3_step(B), ls,
+                      [&](double b, double* a, double* c) { return exp3_profile(b, m, lc, y, a, c); });
+  else
+    nofit(m, lc, y, ls, &est, &st);
+  store_fit(nl, lam, vals, n_obs, o, ls, mask, fb, est, st, out, status);
+}
+
+struct Exp3Best {
+  double loss;
+  int at;
+  __device__ __forceinline__ void take(double l, int i) {
+    if (l < loss || (l == loss && i < at)) { loss = l; at = i; }
+  }
+};
+
+__global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 8)
+    exp3_kernel(int nl, const double* lam, const double* vals, int n_obs, double ls, const uint8_t* mask,
+                const double* fb, double* out, int* status, int per) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int cl = (int)(blockIdx.x / EXP3_CS), ncl = (int)(gridDim.x / EXP3_CS);
+  constexpr int NW = EXP3_THREADS / 32;
+  __shared__ double ys[NW + 1][FIT_MAXL], lams[NW + 1][FIT_MAXL];   // of each warp's golden section, of the grid's observable
+  __shared__ int list[EXP3_MOST], count[NW];
+  __shared__ double wbest[NW];
+  __shared__ int widx[NW];
+  __shared__ Exp3Best best_s[EXP3_MOST / EXP3_CS][EXP3_CS];   // by observable of this CTA and CTA of the cluster
+  __shared__ int m_s, ok_s;
+  __shared__ double B_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double *y = ys[NW], *lc = lams[NW];
+  for (long long o0 = (long long)cl * per; o0 < n_obs; o0 += (long long)ncl * per) {
+    // the marked observables, the same list in every CTA
+    const bool mine = tid < per && o0 + tid < n_obs && status[o0 + tid] == FIT_NEEDS_EXP3;
+    if (!__syncthreads_or(mine)) continue;
+    const unsigned votes = __ballot_sync(0xffffffffu, mine);
+    if (lane == 0) count[warp] = __popc(votes);
+    __syncthreads();
+    int n_fit = 0, before = 0;
+    for (int w = 0; w < NW; ++w) {
+      if (w < warp) before += count[w];
+      n_fit += count[w];
+    }
+    if (mine) list[before + __popc(votes & ((1u << lane) - 1))] = (int)(o0 + tid);
+    // also: every CTA runs, has read its statuses and is done with best_s
+    cluster.sync();
+    double step = 0;   // of the last observable
+    for (int q = 0; q < n_fit; ++q) {
+      if (tid == 0) {
+        m_s = gather_levels(nl, lam, vals, nullptr, n_obs, list[q], mask, y, lc, nullptr);
+        double B = 0;
+        ok_s = exp3_range(m_s, lc, &B) ? 1 : 0;
+        B_s = B;
+      }
+      __syncthreads();
+      const int m = m_s;
+      const double B = B_s;
+      if (ok_s) {
+        Exp3Best best{1e300, 0};
+        step = exp3_step(B);
+        for (int i = rank * EXP3_THREADS + tid; i < EXP3_GRID; i += EXP3_CS * EXP3_THREADS) {
+          const double b = exp3_gridb(i, B, step);
+          double a, c;
+          const double l = (b == 0.0) ? 1e300 : exp3_profile(b, m, lc, y, &a, &c);
+          if (l < best.loss) { best.loss = l; best.at = i; }
+        }
+        for (int d = 16; d > 0; d >>= 1)
+          best.take(__shfl_xor_sync(0xffffffffu, best.loss, d), __shfl_xor_sync(0xffffffffu, best.at, d));
+        if (lane == 0) {
+          wbest[warp] = best.loss;
+          widx[warp] = best.at;
+        }
+        __syncthreads();
+        if (tid == 0) {
+          for (int w = 1; w < NW; ++w) best.take(wbest[w], widx[w]);
+          *cluster.map_shared_rank(&best_s[q / EXP3_CS][rank], q % EXP3_CS) = best;
+        }
+      }
+      __syncthreads();   // y, lc, m_s are free
+    }
+    cluster.sync();
+    // observable q by CTA q % EXP3_CS
+    auto best_of = [&](int q) {
+      Exp3Best best = best_s[q / EXP3_CS][0];
+      for (int r = 1; r < EXP3_CS; ++r) best.take(best_s[q / EXP3_CS][r].loss, best_s[q / EXP3_CS][r].at);
+      return best.at;
+    };
+    if (n_fit > EXP3_WARP) {   // a thread each
+      const int q = tid * EXP3_CS + rank;
+      if (q < n_fit) exp3_finish_thread(best_of(q), nl, lam, vals, n_obs, list[q], ls, mask, fb, out, status);
+    } else if (warp * EXP3_CS + rank < n_fit) {   // a warp each
+      const int q = warp * EXP3_CS + rank, o = list[q];
+      const bool last = q == n_fit - 1;   // whose levels are still at hand
+      double *yt = ys[last ? NW : warp], *lt = lams[last ? NW : warp];
+      int m = m_s, st = NNE_OK;
+      bool ok = ok_s;
+      double B = B_s, est = 0;
+      if (!last) {
+        if (lane == 0) m = gather_levels(nl, lam, vals, nullptr, n_obs, o, mask, yt, lt, nullptr);
+        m = __shfl_sync(0xffffffffu, m, 0);
+        ok = exp3_range(m, lt, &B);
+        step = exp3_step(B);
+      }
+      if (ok) {
+        // lane j forms the exponentials of levels j and j + 32
+        est = exp3_golden(best_of(q), B, step, ls, [&](double b, double* a, double* c) {
+          const double e0 = lane < m ? exp(-b * lt[lane]) : 0.0, e1 = lane + 32 < m ? exp(-b * lt[lane + 32]) : 0.0;
+          auto e = [&](int j) { return __shfl_sync(0xffffffffu, j < 32 ? e0 : e1, j & 31); };
+          double em = 0, ym = 0;
+          for (int j = 0; j < m; ++j) { em += e(j); ym += yt[j]; }
+          em /= m;
+          ym /= m;
+          double see = 0, sey = 0;
+          for (int j = 0; j < m; ++j) { const double ej = e(j); see += (ej - em) * (ej - em); sey += (ej - em) * (yt[j] - ym); }
+          *a = see > 0 ? sey / see : 0.0;
+          *c = ym - *a * em;
+          double loss = 0;
+          for (int j = 0; j < m; ++j) { const double r = *a * e(j) + *c - yt[j]; loss += r * r; }
+          return loss;
+        });
+      } else {
+        nofit(m, lt, yt, ls, &est, &st);
+      }
+      if (lane == 0) store_fit(nl, lam, vals, n_obs, o, ls, mask, fb, est, st, out, status);
+      __syncwarp();
+    }
+    __syncthreads();   // list is free
   }
 }
 
@@ -380,13 +452,12 @@ static cudaError_t launch_fit(cudaStream_t st, int nl, const double* lam, const 
                                               status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || method == NNE_FIT_POLY) return e;
-  constexpr int PER_LAUNCH = 1 << 24;   // observables per launch: the grid stays below 2^31 CTAs
-  for (int o0 = 0; o0 < n_obs && e == cudaSuccess; o0 += std::min(PER_LAUNCH, n_obs - o0)) {
-    exp3_kernel<<<std::min(PER_LAUNCH, n_obs - o0) * EXP3_CS, EXP3_THREADS, 0, st>>>(nl, lam, vals, n_obs, ls, mask, fb,
-                                                                                  out, status, o0);
-    e = cudaGetLastError();
-  }
-  return e;
+  // equal shares in as few passes as EXP3_MOST allows
+  const long long passes = (n_obs - 1) / ((long long)EXP3_CLUSTERS * EXP3_MOST) + 1;
+  const int per = (int)((n_obs - 1) / (passes * EXP3_CLUSTERS) + 1);
+  const int clusters = std::min(EXP3_CLUSTERS, (n_obs - 1) / per + 1);
+  exp3_kernel<<<clusters * EXP3_CS, EXP3_THREADS, 0, st>>>(nl, lam, vals, n_obs, ls, mask, fb, out, status, per);
+  return cudaGetLastError();
 }
 
 // (A) over k rungs: vals (k x nl x n_obs), logf (k x nl) -> obar (nl x n_obs), conv (nl x n_obs).
