@@ -265,12 +265,12 @@ __global__ void fit_kernel(int nl, const double* lam, const double* vals, const 
 // section that follows is a serial chain of about 60 profiles, each formed by
 // one warp with a level per lane and the sums in level order (whole call of
 // that table: 22.8 ms -> 0.3 ms).  The warp's lanes repeat each other's sums, a
-// third of the work on top of the grid's: where every cluster has more than
-// EXP3_WARP observables that need it (a large table), a thread takes one instead,
-// with the same operations in the same order.  EXP3 of 50000 observables at 5
-// levels: 68.1 ms by one thread each, 91.2 with a warp each throughout, 69.6 now;
-// a call over 10^6 observables of which none needs it: 13.3 ms with a cluster for
-// each, 8.6 now.
+// third of the work on top of the grid's: where a cluster has more than EXP3_WARP
+// observables that need it (a large table), its CTAs take a grid each and a thread
+// a golden section, with the same operations in the same order.  Whole calls, ms, one
+// thread per observable throughout, a cluster each throughout, now: EXP3 of 50000
+// observables at 5 levels 68.2, 91.2, 68.6; of 200000 250, 364, 261; a fit of 100000
+// observables of which 1 % fall back 57.3, 2.6, 2.4; none of 10^6 3.3, 9.0, 3.3.
 constexpr int EXP3_CS = 8, EXP3_THREADS = 128, EXP3_GRID = 4001;
 constexpr int EXP3_CLUSTERS = 4 * 152, EXP3_MOST = 128, EXP3_WARP = 8;
 
@@ -360,8 +360,9 @@ __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 
     if (mine) list[before + __popc(votes & ((1u << lane) - 1))] = (int)(o0 + tid);
     // also: every CTA runs, has read its statuses and is done with best_s
     cluster.sync();
-    double step = 0;   // of the last observable
-    for (int q = 0; q < n_fit; ++q) {
+    const bool many = n_fit > EXP3_WARP;   // then a CTA for a grid
+    double step = 0;                       // of the last observable
+    for (int q = many ? rank : 0; q < n_fit; q += many ? EXP3_CS : 1) {
       if (tid == 0) {
         m_s = gather_levels(nl, lam, vals, nullptr, n_obs, list[q], mask, y, lc, nullptr);
         double B = 0;
@@ -374,7 +375,7 @@ __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 
       if (ok_s) {
         Exp3Best best{1e300, 0};
         step = exp3_step(B);
-        for (int i = rank * EXP3_THREADS + tid; i < EXP3_GRID; i += EXP3_CS * EXP3_THREADS) {
+        for (int i = (many ? 0 : rank * EXP3_THREADS) + tid; i < EXP3_GRID; i += (many ? 1 : EXP3_CS) * EXP3_THREADS) {
           const double b = exp3_gridb(i, B, step);
           double a, c;
           const double l = (b == 0.0) ? 1e300 : exp3_profile(b, m, lc, y, &a, &c);
@@ -389,7 +390,8 @@ __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 
         __syncthreads();
         if (tid == 0) {
           for (int w = 1; w < NW; ++w) best.take(wbest[w], widx[w]);
-          *cluster.map_shared_rank(&best_s[q / EXP3_CS][rank], q % EXP3_CS) = best;
+          if (many) best_s[q / EXP3_CS][0] = best;
+          else *cluster.map_shared_rank(&best_s[q / EXP3_CS][rank], q % EXP3_CS) = best;
         }
       }
       __syncthreads();   // y, lc, m_s are free
@@ -398,10 +400,10 @@ __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 
     // observable q by CTA q % EXP3_CS
     auto best_of = [&](int q) {
       Exp3Best best = best_s[q / EXP3_CS][0];
-      for (int r = 1; r < EXP3_CS; ++r) best.take(best_s[q / EXP3_CS][r].loss, best_s[q / EXP3_CS][r].at);
+      for (int r = 1; r < (many ? 1 : EXP3_CS); ++r) best.take(best_s[q / EXP3_CS][r].loss, best_s[q / EXP3_CS][r].at);
       return best.at;
     };
-    if (n_fit > EXP3_WARP) {   // a thread each
+    if (many) {   // a thread each
       const int q = tid * EXP3_CS + rank;
       if (q < n_fit) exp3_finish_thread(best_of(q), nl, lam, vals, n_obs, list[q], ls, mask, fb, out, status);
     } else if (warp * EXP3_CS + rank < n_fit) {   // a warp each
