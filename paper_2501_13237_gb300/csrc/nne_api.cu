@@ -1105,29 +1105,47 @@ nne_status nne_extrapolate(nne_ctx* ctx, int n_lambda, const double* lambdas, co
   if (n_obs == 0) return NNE_OK;
   DeviceGuard dg(ctx);
   cudaStream_t s = ctx->stream;
-  // one block: inputs [lambdas | values | log F | y_zero], results [estimates | statuses]
-  const size_t nl = n_lambda, no = n_obs;
-  std::vector<double> hin(nl + nl * no + nl + no, 0.0);
-  memcpy(hin.data(), lambdas, sizeof(double) * nl);
-  memcpy(hin.data() + nl, values, sizeof(double) * nl * no);
-  if (log_fid) memcpy(hin.data() + nl + nl * no, log_fid, sizeof(double) * nl);
-  if (y_zero) memcpy(hin.data() + 2 * nl + nl * no, y_zero, sizeof(double) * no);
+  // one block: inputs [lambdas | log F | y_zero | values], results [estimates | statuses].  A small table goes over
+  // in one copy each way; a large one straight from and to the caller's arrays (its copy on the host cost more
+  // than the fit: 10^6 observables at 5 levels, POLY, 6.5 -> 1.1 ms)
+  constexpr size_t STAGE_MAX = 64 * 1024;
+  const size_t nl = n_lambda, no = n_obs, n_in = 2 * nl + no + nl * no;
   const size_t out_bytes = (sizeof(double) + sizeof(int)) * no;
-  std::vector<char> hout(out_bytes);
+  const bool staged = sizeof(double) * n_in <= STAGE_MAX;
   double* blk = nullptr;
-  NNE_CUDA_TRY(dev_alloc((void**)&blk, sizeof(double) * hin.size() + out_bytes, s));
-  double *dl = blk, *dv = dl + nl, *df = dv + nl * no, *dy = df + nl, *dout = dy + no;
+  NNE_CUDA_TRY(dev_alloc((void**)&blk, sizeof(double) * n_in + out_bytes, s));
+  double *dl = blk, *df = dl + nl, *dy = df + nl, *dv = dy + no, *dout = dv + nl * no;
   int* dst = reinterpret_cast<int*>(dout + no);
-  cudaError_t e = cudaMemcpyAsync(blk, hin.data(), sizeof(double) * hin.size(), cudaMemcpyHostToDevice, s);
+  std::vector<double> hin;
+  std::vector<char> hout;
+  cudaError_t e = cudaSuccess;
+  if (staged) {
+    hin.assign(n_in, 0.0);
+    hout.resize(out_bytes);
+  }
+  auto put = [&](double* dst_at, const double* src, size_t count) {
+    if (!src || e != cudaSuccess) return;
+    if (staged) memcpy(hin.data() + (dst_at - blk), src, sizeof(double) * count);
+    else e = cudaMemcpyAsync(dst_at, src, sizeof(double) * count, cudaMemcpyHostToDevice, s);
+  };
+  put(dl, lambdas, nl);
+  put(df, log_fid, nl);
+  put(dy, y_zero, no);
+  put(dv, values, nl * no);
+  if (staged) e = cudaMemcpyAsync(blk, hin.data(), sizeof(double) * n_in, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = extrapolate_fit(s, n_lambda, dl, dv, log_fid ? df : nullptr, n_obs, method, degree, lambda_star,
                         y_zero ? dy : nullptr, dout, dst);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(hout.data(), dout, out_bytes, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && staged) e = cudaMemcpyAsync(hout.data(), dout, out_bytes, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && !staged) e = cudaMemcpyAsync(out, dout, sizeof(double) * no, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && !staged) e = cudaMemcpyAsync(per_obs_status, dst, sizeof(int) * no, cudaMemcpyDeviceToHost, s);
   cudaFreeAsync(blk, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return set_cuda_error(e, "nne_extrapolate", __FILE__, __LINE__);
-  memcpy(out, hout.data(), sizeof(double) * no);
-  memcpy(per_obs_status, hout.data() + sizeof(double) * no, sizeof(int32_t) * no);
+  if (staged) {
+    memcpy(out, hout.data(), sizeof(double) * no);
+    memcpy(per_obs_status, hout.data() + sizeof(double) * no, sizeof(int32_t) * no);
+  }
   return NNE_OK;
 }
 

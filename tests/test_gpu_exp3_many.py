@@ -51,3 +51,22 @@ def test_too_few_levels_in_a_large_table():
     lams, y, lf = table(2, 9000, 3)
     est, st = nne.Context(0).extrapolate(lams, y, lf, method=ofit.M_EXP3, lambda_star=1.0)
     assert (st == -6).all() and (est == y[0]).all()
+
+
+@pytest.mark.parametrize("n_obs", [1363, 1364, 5000])
+@pytest.mark.parametrize("given", [False, True])
+def test_tables_around_the_staged_size(n_obs, given):
+    """4 levels of 1363 observables (with their y_zero) are the last to go over in one 64 KB
+    copy: the same estimates above and below, with and without the optional inputs."""
+    require_gpu()
+    from paper_2501_13237_gb300 import nne
+    ctx = nne.Context(0)
+    lams, y, lf = table(4, n_obs, 7)
+    opt = dict(log_fid=lf, y_zero=y[0]) if given else {}
+    for method, tol in [(ofit.M_POLY, 1e-10), (ofit.M_EXP_LOGLIN, 1e-10)]:
+        est, st = ctx.extrapolate(lams, y, method=method, degree=2, lambda_star=1.0, **opt)
+        few = np.r_[0:20, n_obs - 20:n_obs]
+        sub = dict(log_fid=lf, y_zero=y[0, few]) if given else {}
+        ref, rst = ofit.extrapolate(method, lams, y[:, few], 1.0, degree=2, **sub)
+        assert (st[few] == rst).all() and (st == 0).all()
+        assert (np.abs(est[few] - ref) <= tol).all()
