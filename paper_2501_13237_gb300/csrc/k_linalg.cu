@@ -528,7 +528,7 @@ EighWork eigh_workspace(int n, int r) {
   const long long qn = std::max(n, r);
   // cx: e, phi, P (n each), Vh (n x n), WY factors (ceil(n/32) x 32 x 32), WY application workspace
   //     (for r columns), QR workspace of an n x r matrix
-  w.cx_elems = 3LL * n + (long long)n * n + ((n + 31) / 32) * 1024LL + wy_workspace(r) + qr_workspace(n, r).cx_elems +
+  w.cx_elems = 3LL * n + (long long)n * n + ((n + 31) / 32) * 1024LL + wy_workspace(n, r) + qr_workspace(n, r).cx_elems +
                32;
   // re: d, eabs (n each), lam (r), Z (n r), L/U0/U1/U2 (4 n r), Kpart (32 doubles = 64 floats)
   w.re_elems = 2LL * n + r + 5LL * n * r + 64 + qn;
@@ -553,8 +553,8 @@ cudaError_t eigh_top(cudaStream_t st, cx<R>* H, long long sH, int n, int r, cx<R
   cx<R>* Vh = P + (long long)batch * n;             // batch x n x n
   cx<R>* Tw = Vh + (long long)batch * n * n;        // batch x nb x 1024
   const int nbw = (n + 31) / 32;
-  cx<R>* wyws = Tw + (long long)batch * nbw * 1024;          // batch x wy_workspace(r)
-  cx<R>* qrws = wyws + (long long)batch * wy_workspace(r);   // QR workspace for batch n x r matrices
+  cx<R>* wyws = Tw + (long long)batch * nbw * 1024;          // batch x wy_workspace(n, r)
+  cx<R>* qrws = wyws + (long long)batch * wy_workspace(n, r);   // QR workspace for batch n x r matrices
   R* d = reb;                                       // batch x n
   R* eabs = d + (long long)batch * n;               // batch x n
   R* lam = eabs + (long long)batch * n;             // batch x r
@@ -638,7 +638,7 @@ MixedEighWork eigh_mixed_workspace(int n, int r) {
   const int nbw = (n + 31) / 32;
   const size_t nf = (size_t)std::min(n, EIGH_F64_MAX);   // a state's smaller problems take the float64 path
   w.cx_bytes = al256(std::max(16 * nn, 32 * nf * nf)) + al256(16 * (size_t)n) * 3 + al256(8 * nn) + al256(8 * (size_t)n) +
-               al256(8 * (size_t)nbw * 1024) + al256(8 * (size_t)wy_workspace(r)) +
+               al256(8 * (size_t)nbw * 1024) + al256(8 * (size_t)wy_workspace(n, r)) +
                al256(8 * (size_t)qr_workspace(n, r).cx_elems) + 1024;
   w.re_bytes = al256(8 * (size_t)n) * 2 + al256(8 * (size_t)r) + al256(8 * nr) * 5 + al256(4 * nr) + 512 +
                al256(4 * (size_t)n) * 2 + al256(4 * (size_t)r) + 1024;
@@ -677,7 +677,7 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
   cx<float>* Vhf = reinterpret_cast<cx<float>*>(take(c, 8 * nn * B));
   cx<float>* phif = reinterpret_cast<cx<float>*>(take(c, 8 * (size_t)n * B));
   cx<float>* Tw = reinterpret_cast<cx<float>*>(take(c, 8 * (size_t)nbw * 1024 * B));
-  cx<float>* wyws = reinterpret_cast<cx<float>*>(take(c, 8 * (size_t)wy_workspace(r) * B));
+  cx<float>* wyws = reinterpret_cast<cx<float>*>(take(c, 8 * (size_t)wy_workspace(n, r) * B));
   cx<float>* qrws = reinterpret_cast<cx<float>*>(take(c, 8 * (size_t)qr_workspace(n, r).cx_elems * B));
   unsigned char* q = reinterpret_cast<unsigned char*>(re_ws);
   double* dd = reinterpret_cast<double*>(take(q, 8 * (size_t)n * B));

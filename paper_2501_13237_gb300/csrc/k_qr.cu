@@ -990,9 +990,9 @@ QrWork qr_workspace(int m, int n) {
   const int k = std::min(m, n);
   const int np = (k + QB - 1) / QB;
   const int nblk = (k + QNB - 1) / QNB;
-  // V (m x n) + panel T (np x 32 x 32) + WY application workspace (n columns)
+  // V (m x n) + panel T (np x 32 x 32) + WY application workspace (a block's own columns)
   // + block T (nblk x 128 x 128) + Gram (128 x 128) + W1, W2 (128 x n each)
-  w.cx_elems = (long long)m * n + (long long)np * QB * QB + wy_workspace(n) + (long long)nblk * QNB * QNB +
+  w.cx_elems = (long long)m * n + (long long)np * QB * QB + wy_workspace(m, std::min(n, QNB - QB)) + (long long)nblk * QNB * QNB +
                (long long)QNB * QNB + 2LL * QNB * n + 64;
   return w;
 }
@@ -1060,7 +1060,7 @@ cudaError_t qr(cudaStream_t st, cx<R>* A, long long sA, int m, int n, cx<R>* Q, 
   cx<R>* T = V + sV * batch;
   const long long sT = (long long)np * QB * QB;
   cx<R>* wyws = T + sT * batch;
-  cx<R>* Tb = wyws + wy_workspace(n) * batch;
+  cx<R>* Tb = wyws + wy_workspace(m, std::min(n, QNB - QB)) * batch;   // a block's own columns
   const long long sTb = (long long)nblk * QNB * QNB;
   cx<R>* G = Tb + sTb * batch;
   const long long sG = (long long)QNB * QNB;

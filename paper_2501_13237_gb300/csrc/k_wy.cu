@@ -19,7 +19,10 @@ constexpr int WY_RN = 8;          // output columns per CTA of the reduction
 constexpr int WY_TN = 64;         // output columns per CTA of the partial product
 constexpr int WY_KS = 16;         // rows of V and C per shared-memory stage
 
-long long wy_workspace(int N) { return (long long)(WY_SPLIT_MAX + 1) * WY_B * N; }
+// Chunks of at least 64 rows (each 16 of them one barrier-to-barrier stage: the chunk is a
+// chain of loads).
+static int wy_chunks(int K) { return std::min(WY_SPLIT_MAX, (K + 63) / 64); }
+long long wy_workspace(int K, int N) { return (long long)(wy_chunks(K) + 1) * WY_B * N; }
 
 // Partial s of W = V^H C over rows [s * kc, min((s + 1) * kc, K)), written to
 // P[z][s] (WY_B x N, rows >= bw zero).  VROWS: V is passed as V^H, row c at
@@ -127,16 +130,15 @@ cudaError_t wy_apply(cudaStream_t st, bool v_rows, const cx<R>* V, long long sV,
   if (bw <= 0 || K <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   if (bw > WY_B) return cudaErrorInvalidValue;
   const int tiles = (N + WY_TN - 1) / WY_TN;
-  // about four waves of partial-product CTAs, chunks of at least 64 rows (each 16 of them one
-  // barrier-to-barrier stage: the chunk is a chain of loads)
+  // about four waves of partial-product CTAs
   int S = (4 * 152 + tiles * batch - 1) / (tiles * batch);
-  S = std::max(1, std::min(S, std::min(WY_SPLIT_MAX, (K + 63) / 64)));
+  S = std::max(1, std::min(S, wy_chunks(K)));
   int kc = (K + S - 1) / S;
   kc = (kc + WY_KS - 1) / WY_KS * WY_KS;
   S = (K + kc - 1) / kc;
-  // workspace (batch x wy_workspace(N) elements): partials [z][s] (WY_B x N each), then W2[z] (WY_B x N)
+  // workspace (batch x wy_workspace(K, N) elements): partials [z][s] (WY_B x N each), then W2[z] (WY_B x N)
   cx<R>* P = ws;
-  cx<R>* W2 = ws + (long long)batch * WY_SPLIT_MAX * WY_B * N;
+  cx<R>* W2 = ws + (long long)batch * S * WY_B * N;
   const long long sW2 = (long long)WY_B * N;
   cudaError_t e;
   {
