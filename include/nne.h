@@ -80,7 +80,10 @@ typedef struct nne_state nne_state;
  *   device           CUDA ordinal made current by every call on this context.
  *   cuda_stream      cudaStream_t (NULL = the legacy default stream).
  *   hbm_budget_bytes cap on the memory states created on this context may
- *                    allocate (0 = no cap); exceeding it gives NNE_ERR_OOM. */
+ *                    allocate (0 = no cap); exceeding it gives NNE_ERR_OOM.
+ * While any context of a device exists the library keeps up to 1 GB of freed device
+ * memory for its next allocations there (one pool per device, not counted in the
+ * budget); the last context gives it back. */
 nne_status nne_ctx_create(int device, void* cuda_stream, size_t hbm_budget_bytes, nne_ctx** out);
 void nne_ctx_destroy(nne_ctx* ctx);
 /* Bytes currently allocated by states of this context. */

@@ -129,8 +129,10 @@ nne_status set_error(nne_status s, const char* fmt, ...);
 // mapping it again: 1.0 of the 1.67 ms of a 2048 x 2048 x 512 batch-8 GEMM call.
 // The library's pool, one per device and shared by its contexts (it exists while
 // any does), keeps up to MEM_POOL_KEEP between calls and gives all of it back
-// with the last context, or when an allocation fails (every pool is then trimmed
-// and the allocation tried once more).  The pool in force is the one of the
+// with the last context, or when an allocation fails: every pool is then trimmed, and
+// the allocation may take memory whose free is still pending on another stream (its
+// stream then waits for that free, as in the default pool); if that fails too, it is
+// tried a last time with no work pending on the device.  The pool in force is the one of the
 // innermost PoolScope of the calling thread (every entry point that allocates
 // opens one); without a scope dev_alloc uses the device's default pool.  Frees
 // need no scope.
@@ -143,7 +145,7 @@ cudaError_t dev_alloc(T** p, size_t bytes, cudaStream_t st) {
 class MemPool {
  public:
   static std::shared_ptr<MemPool> of_device(int device);
-  explicit MemPool(int device);
+  explicit MemPool(int device, size_t max_bytes = 0);   // max_bytes 0: what the device holds
   ~MemPool();
   MemPool(const MemPool&) = delete;
   MemPool& operator=(const MemPool&) = delete;

@@ -105,11 +105,12 @@ std::shared_ptr<MemPool> MemPool::of_device(int device) {
   return p;
 }
 
-MemPool::MemPool(int device) {
+MemPool::MemPool(int device, size_t max_bytes) {
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = device;
+  props.maxSize = max_bytes;
   if (cudaMemPoolCreate(&pool_, &props) != cudaSuccess) {
     cudaGetLastError();
     pool_ = nullptr;   // dev_alloc then takes the default pool
@@ -118,7 +119,8 @@ MemPool::MemPool(int device) {
   cuuint64_t keep = MEM_POOL_KEEP;
   cudaMemPoolSetAttribute(pool_, cudaMemPoolAttrReleaseThreshold, &keep);
   // no reuse that makes one stream wait for another: with it a state's sub-batch
-  // streams ran one after the other (they all allocate GEMM planes)
+  // streams ran one after the other (they all allocate GEMM planes); dev_alloc allows it
+  // when memory runs out
   int off = 0;
   cudaMemPoolSetAttribute(pool_, cudaMemPoolReuseAllowInternalDependencies, &off);
 }
@@ -134,17 +136,32 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
   auto once = [&] {
     return t_pool ? cudaMallocFromPoolAsync(p, bytes, t_pool, st) : cudaMallocAsync(p, bytes, st);
   };
+  auto trim = [] {
+    std::vector<std::shared_ptr<MemPool>> live;
+    {
+      std::lock_guard<std::mutex> lk(g_pools_mu);
+      for (auto& q : g_pools)
+        if (std::shared_ptr<MemPool> m = q.second.lock()) live.push_back(m);
+    }
+    for (auto& m : live)
+      if (m->handle()) cudaMemPoolTrimTo(m->handle(), 0);
+  };
   cudaError_t e = once();
   if (e != cudaErrorMemoryAllocation) return e;
   cudaGetLastError();
-  std::vector<std::shared_ptr<MemPool>> live;
-  {
-    std::lock_guard<std::mutex> lk(g_pools_mu);
-    for (auto& q : g_pools)
-      if (std::shared_ptr<MemPool> m = q.second.lock()) live.push_back(m);
+  static std::mutex short_mu;   // one short allocation at a time
+  std::lock_guard<std::mutex> lk(short_mu);
+  trim();
+  if (t_pool) {
+    int on = 1, off = 0;
+    cudaMemPoolSetAttribute(t_pool, cudaMemPoolReuseAllowInternalDependencies, &on);
+    e = once();
+    cudaMemPoolSetAttribute(t_pool, cudaMemPoolReuseAllowInternalDependencies, &off);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
   }
-  for (auto& m : live)
-    if (m->handle()) cudaMemPoolTrimTo(m->handle(), 0);
+  if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
+  trim();
   return once();
 }
 

@@ -1,5 +1,5 @@
 """Device memory of a job (nne_job_bytes: the state's and its workspaces' allocation plan)
-against the smallest plan the library has had.  A server or context with a memory budget
+against an earlier plan of the library.  A server or context with a memory budget
 admits what fits in it, so a workspace that grows refuses jobs that used to run."""
 import numpy as np
 import pytest
