@@ -269,7 +269,8 @@ nne_status nne_cgemm_c64(nne_ctx* ctx, int op_a, int op_b, int M, int N, int K, 
  * back to the context stream), so that the latency-bound kernels of one
  * overlap the GEMMs of another.  States whose largest bond is below 256 use
  * one stream (their kernels are small and splitting multiplies launches).
- * Results do not depend on it beyond the rounding of GEMM split choices.
+ * Results do not depend on it beyond the rounding of sums whose split follows the batch: the GEMMs',
+ * the compact-WY products', and the reductions' of eigenproblems of up to 160 rows and of float64.
  * NNE_OPT_SERIAL_LAYERS (default 0): when 1, nne_apply_layer runs all of a
  * state's instances as one batch on the context stream, whatever the state's
  * sub-batch count -- for per-launch timing of the kernels alone.
@@ -278,7 +279,7 @@ nne_status nne_cgemm_c64(nne_ctx* ctx, int op_a, int op_b, int M, int N, int K, 
  * Rayleigh-Ritz matrix of the subspace iteration, the centre compression)
  * with float64 quality: the Householder reduction in float64 (matrices of up to
  * 160 rows) or in double-float arithmetic on the float32 pipes (larger ones;
- * about 2^-46 relative, in one cluster's shared memory up to 384 rows), bisection and inverse
+ * about 2^-46 relative, in one cluster's shared memory up to 380 rows), bisection and inverse
  * iteration in float64, the back-transformation in float32; 0 runs them in
  * float32 (about 1.14x the gate-step rate at chi = 512, with a float32
  * reduction's error of eps_32 times the largest eigenvalue, which turns the

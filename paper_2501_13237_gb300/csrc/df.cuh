@@ -33,6 +33,15 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float bh, float bl)
   hi = s;
   lo = __fadd_rn(lo, __fadd_rn(e, bl));
 }
+// The same with the lo parts first: the bits do not depend on which addend is which (the
+// rounding error of the hi parts is exact), so lanes that exchange partial sums agree.
+__device__ __forceinline__ void df_add_sym(float& hi, float& lo, float bh, float bl) {
+  const float s = __fadd_rn(hi, bh);
+  const float bb = __fsub_rn(s, hi);
+  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(bh, bb));
+  hi = s;
+  lo = __fadd_rn(__fadd_rn(lo, bl), e);
+}
 __device__ __forceinline__ void df_norm(float& hi, float& lo) {
   const float s = __fadd_rn(hi, lo);
   lo = __fsub_rn(lo, __fsub_rn(s, hi));

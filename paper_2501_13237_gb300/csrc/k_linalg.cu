@@ -12,7 +12,9 @@
 //     orthonormalise the eigenvector block and for the centre moves.
 // Precision follows the state: float for complex64 states, double for
 // complex128.  The reductions are written in a fixed order, so results are
-// bitwise reproducible run to run and independent of what else is batched.
+// bitwise reproducible run to run.  The double-float and the L2-resident reductions do not
+// depend on what else is batched either; those in one cluster's shared memory (tridiag_smem,
+// _keep) sum K over as many CTAs as the batch lets run at once.
 #include <map>
 #include <mutex>
 

@@ -244,14 +244,13 @@ __global__ void __launch_bounds__(512) tridiag_df_kernel(float4* Hb, long long s
 enum DfRows { ROWS_C64, ROWS_DF, ROWS_GLOBAL };
 
 struct DfsLayout {   // shared memory, in float4 from the base
-  int n, cs, maxloc, nw;
+  int n, maxloc;
   bool global;
-  __host__ __device__ size_t rows() const { return 0; }
   __host__ __device__ size_t v() const { return global ? 0 : (size_t)maxloc * n; }   // [2][n] reflectors of this and the last column
   __host__ __device__ size_t w() const { return v() + 2 * (size_t)n; }               // n: w of the last column
   __host__ __device__ size_t p() const { return w() + n; }                           // [2][n] p of all rows, pushed by their owners
-  __host__ __device__ size_t k() const { return p() + 2 * (size_t)n; }               // [2][cs][nw] float2: shares of K
-  __host__ __device__ size_t bytes() const { return 16 * k() + 2 * sizeof(float2) * (size_t)cs * nw; }
+  __host__ __device__ size_t k() const { return p() + 2 * (size_t)n; }               // [2][n] float2: the rows' terms of K, pushed with p
+  __host__ __device__ size_t bytes() const { return 16 * k() + 2 * sizeof(float2) * (size_t)n; }
 };
 
 template <int NT, int EPT, int ROWS>
@@ -267,12 +266,12 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(void* Hsrc, long long s
   cx<float>* Vh = Vhb + z * sVh + (long long)off * n0 + off;
   extern __shared__ __align__(16) float4 dfs_smem[];
   constexpr int NW = NT / 32;
-  const DfsLayout lay{n, CS, maxloc, NW, ROWS == ROWS_GLOBAL};
+  const DfsLayout lay{n, maxloc, ROWS == ROWS_GLOBAL};
   float4* vb = dfs_smem + lay.v();
   float4* wb = dfs_smem + lay.w();
   float4* pb = dfs_smem + lay.p();
   float2* kbuf = reinterpret_cast<float2*>(dfs_smem + lay.k());
-  __shared__ float2 redN[NW];
+  __shared__ float2 redN[NW], redK[NW];
   __shared__ float redM[NW];
   __shared__ float4 x0_s, alpha_s;
   __shared__ float2 inv_s, K_s;
@@ -337,9 +336,9 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(void* Hsrc, long long s
   auto warp_df = [&](float hi, float lo) {
     for (int o = 16; o > 0; o >>= 1) {
       const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
-      df_add(hi, lo, bh, bl);
+      df_add_sym(hi, lo, bh, bl);
     }
-    return make_float2(__shfl_sync(0xffffffffu, hi, 0), __shfl_sync(0xffffffffu, lo, 0));
+    return make_float2(hi, lo);
   };
   // b -= v conj(wk) + w conj(vk)
   auto rank2 = [](float4& b, float4 vt, float4 wt, float4 vk, float4 wk) {
@@ -430,10 +429,10 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(void* Hsrc, long long s
     const float4* vo = vb + (buf ^ 1) * n + 1;   // v_{j-1} at row j + 1
     const float4* wo = wb + 1;                   // w_{j-1} at row j + 1
     float4* p = pb + buf * n;
+    float2* kb = kbuf + buf * n;
     // own rows i > j, two per warp at a time: A <- A - v_{j-1} w^H - w v_{j-1}^H
-    // on columns > j, p_i = row . v_j, and this warp's share of K = v_j^H p
+    // on columns > j, p_i = row . v_j, and its term of K = v_j^H p
     const int l0 = ol + (oc > rank ? 1 : 0);   // first own row > j
-    float kh = 0.f, kl = 0.f;
     for (int li = l0 + warp; li < nloc; li += 2 * NW) {
       const bool two = li + NW < nloc;
       const int t = rank + li * CS - j - 1, t2 = t + NW * CS;
@@ -475,41 +474,32 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(void* Hsrc, long long s
           df_cmac<false>(acc, b, v[k]);
         }
       }
-      // both rows' sums in five steps: lanes 0-15 end with the first row's, 16-31 with the second's
+      // both rows' sums in five steps: lanes 0-15 end with the first row's, 16-31 with the second's, the
+      // same bits on each (every CTA gets them) and whichever place a row has
       const bool up = lane & 16;
       {
         const float4 give = up ? acc : acc2;
         acc = up ? acc2 : acc;
         const float bh = __shfl_xor_sync(0xffffffffu, give.x, 16), bl = __shfl_xor_sync(0xffffffffu, give.y, 16);
         const float ch = __shfl_xor_sync(0xffffffffu, give.z, 16), cl = __shfl_xor_sync(0xffffffffu, give.w, 16);
-        df_add(acc.x, acc.y, bh, bl);
-        df_add(acc.z, acc.w, ch, cl);
+        df_add_sym(acc.x, acc.y, bh, bl);
+        df_add_sym(acc.z, acc.w, ch, cl);
       }
       for (int o = 8; o > 0; o >>= 1) {
         const float bh = __shfl_xor_sync(0xffffffffu, acc.x, o), bl = __shfl_xor_sync(0xffffffffu, acc.y, o);
         const float ch = __shfl_xor_sync(0xffffffffu, acc.z, o), cl = __shfl_xor_sync(0xffffffffu, acc.w, o);
-        df_add(acc.x, acc.y, bh, bl);
-        df_add(acc.z, acc.w, ch, cl);
+        df_add_sym(acc.x, acc.y, bh, bl);
+        df_add_sym(acc.z, acc.w, ch, cl);
       }
-      if ((lane & 15) == 0 && (!up || two)) {
-        const float4 vt = v[up ? t2 : t];
+      if ((!up || two) && (lane & 15) < CS) {
+        const int tr = up ? t2 : t;
+        *cluster.map_shared_rank(p + tr, lane & 15) = acc;
+        const float4 vt = v[tr];
+        float kh = 0.f, kl = 0.f;
         df_mac(kh, kl, vt.x, vt.y, acc.x, acc.y);
         df_mac(kh, kl, vt.z, vt.w, acc.z, acc.w);
+        *cluster.map_shared_rank(kb + tr, lane & 15) = make_float2(kh, kl);
       }
-      // every CTA gets the same bits (the lanes' lo parts may differ by rounding)
-      const int src = lane & 16;
-      acc.x = __shfl_sync(0xffffffffu, acc.x, src);
-      acc.y = __shfl_sync(0xffffffffu, acc.y, src);
-      acc.z = __shfl_sync(0xffffffffu, acc.z, src);
-      acc.w = __shfl_sync(0xffffffffu, acc.w, src);
-      if ((!up || two) && (lane & 15) < CS) *cluster.map_shared_rank(p + (up ? t2 : t), lane & 15) = acc;
-    }
-    {
-      const float bh = __shfl_xor_sync(0xffffffffu, kh, 16), bl = __shfl_xor_sync(0xffffffffu, kl, 16);
-      df_add(kh, kl, bh, bl);
-      kh = __shfl_sync(0xffffffffu, kh, 0);
-      kl = __shfl_sync(0xffffffffu, kl, 0);
-      if (lane < CS) cluster.map_shared_rank(kbuf + ((size_t)buf * CS + rank) * NW, lane)[warp] = make_float2(kh, kl);
     }
     cluster.sync();
     // row j + 1 (its owner's last word on it), and K = v^H p by every warp
@@ -530,12 +520,32 @@ __global__ void __launch_bounds__(NT) tridiag_dfs_kernel(void* Hsrc, long long s
         }
       }
     }
-    float2 K = make_float2(0.f, 0.f);
-    {
-      const float2* kb = kbuf + (size_t)buf * CS * NW;
-      for (int q = lane; q < CS * NW; q += 32) df_add(K.x, K.y, kb[q].x, kb[q].y);
+    // (its terms in the order of the rows, not of their CTAs, whose number follows the batch)
+    float2 K;
+    if (ROWS == ROWS_GLOBAL) {
+      // up to 1023 terms: summed by every warp they took some 1000 cycles of issue slots, more than a barrier
+      K = tid < m ? kb[tid] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int q = 1; q < EPT; ++q)
+        if (tid + q * NT < m) df_add(K.x, K.y, kb[tid + q * NT].x, kb[tid + q * NT].y);
       K = warp_df(K.x, K.y);
-      if (ROWS == ROWS_GLOBAL && tid == 0) K_s = K;   // for the last column's update
+      if (lane == 0) redK[warp] = K;
+      __syncthreads();
+      K = warp_df(lane < NW ? redK[lane].x : 0.f, lane < NW ? redK[lane].y : 0.f);
+      if (tid == 0) K_s = K;   // for the last column's update
+    } else {
+      float2 part[4];   // four chains: the sum stands between the barrier and the next reflector
+#pragma unroll
+      for (int u = 0; u < 4; ++u) part[u] = lane + 32 * u < m ? kb[lane + 32 * u] : make_float2(0.f, 0.f);
+      for (int q = lane + 128; q < m; q += 128) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (q + 32 * u < m) df_add(part[u].x, part[u].y, kb[q + 32 * u].x, kb[q + 32 * u].y);
+      }
+      df_add(part[0].x, part[0].y, part[1].x, part[1].y);
+      df_add(part[2].x, part[2].y, part[3].x, part[3].y);
+      df_add(part[0].x, part[0].y, part[2].x, part[2].y);
+      K = warp_df(part[0].x, part[0].y);
     }
     const float k2h = -2.f * K.x, k2l = -2.f * K.y;
     auto wof = [&](float4 vt, float4 pt) {   // w = 2 p - 2 K v
@@ -647,12 +657,14 @@ constexpr size_t DFS_SMEM = 226 * 1024;   // dynamic shared memory per CTA (227 
 
 // CTAs per matrix: more of them shorten a column's pass over the matrix.  Sixteen is
 // the most a cluster holds, but only seven such clusters run at once on the GPU's GPCs
-// (one CTA per SM), of twelve eight: sixteen where that takes no more waves.  384 rows
-// of 12 CTAs fill their shared memory.  Measured, us, 12 and 16 CTAs: 161 rows 561 and
-// 554, 256 rows 1226 and 1120, 384 rows 2634 and 2425, 512 rows 5303 and 4245, 640 rows
-// 9096 and 7547 (five to seven matrices).  The kernels before: 256 rows, five matrices, 4.17 ms
-// (float64); 512 rows, eight, 9.9 and 640 rows 17.0 (lower triangle in L2, two barriers a column).
-constexpr int DFS_CS = 12, DFS_CS_FEW = 16, DFS_MAX = 384, DFS_GLOBAL_MAX = 1024;
+// (one CTA per SM), of twelve eight: sixteen where the launch's batch takes no more waves of
+// them (launches on other streams are not counted).  The result does not depend on the
+// number.  380 rows of 12 CTAs fill their shared memory.  Measured, us, five or six
+// matrices on 16 CTAs and eight on 12: 180 rows 625 and 629, 256 rows 1102 and 1203, 380 rows
+// 2349 and 2554, 512 rows 4224 and 5286; 640 rows, two and eight, 7561 and 9116.  The kernels
+// before: 256 rows, five matrices, 4.17 ms (float64); 512 rows, eight, 9.9 and 640 rows 17.0
+// (lower triangle in L2, two barriers a column).
+constexpr int DFS_CS = 12, DFS_CS_FEW = 16, DFS_MAX = 380, DFS_GLOBAL_MAX = 1024;
 
 // Clusters of `cs` CTAs that run at once, a CTA to an SM; cached per kernel, size and device.
 int dfs_active(const void* kernel, int cs, int threads) {
@@ -693,7 +705,7 @@ cudaError_t dfs_launch(cudaStream_t st, void* H, long long sH, int n0, int off, 
   const int few = dfs_active((const void*)kernel, DFS_CS_FEW, NT), many = dfs_active((const void*)kernel, DFS_CS, NT);
   const int cs = few > 0 && (many < 1 || (batch + few - 1) / few <= (batch + many - 1) / many) ? DFS_CS_FEW : DFS_CS;
   const int n = n0 - off, maxloc = (n + cs - 1) / cs;
-  const size_t smem = DfsLayout{n, cs, maxloc, NT / 32, ROWS == ROWS_GLOBAL}.bytes();
+  const size_t smem = DfsLayout{n, maxloc, ROWS == ROWS_GLOBAL}.bytes();
   if (n < 3 || n > NT * EPT || smem > DFS_SMEM) return cudaErrorInvalidValue;
   return launch_df(kernel, cs, batch, NT, smem, st, H, sH, n0, off, jend, d, e, ldde, Vh, sVh, pre, maxloc);
 }
