@@ -510,7 +510,7 @@ __global__ void re_d2f_pair_kernel(const double* a, const double* b, float* fa, 
 // the rounded tridiagonal brackets every eigenvalue to about eps_32 ||T||,
 // float64 bisection narrows the brackets.  scratch: batch x (2 n + r) floats.
 static cudaError_t bisect_f64(cudaStream_t st, const double* d, const double* e, int n, int r, float* scratch,
-                              double* lam, int batch) {
+                              double* lam, int batch, double width) {
   float* df = scratch;
   float* ef = df + (size_t)n * batch;
   float* lamf = ef + (size_t)n * batch;
@@ -522,7 +522,7 @@ static cudaError_t bisect_f64(cudaStream_t st, const double* d, const double* e,
     bisect_kernel<float><<<(total * 32 + 255) / 256, 256, 0, st>>>(df, ef, n, r, n, lamf, r, total);
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  return bisect64(st, d, e, n, r, lamf, lam, batch);
+  return bisect64(st, d, e, n, r, lamf, lam, batch, width);
 }
 
 EighWork eigh_workspace(int n, int r) {
@@ -584,7 +584,7 @@ cudaError_t eigh_top(cudaStream_t st, cx<R>* H, long long sH, int n, int r, cx<R
   const int total = batch * r;
   if constexpr (std::is_same<R, double>::value) {
     // the division-free float64 bisection (the inverse iteration's scratch is still free)
-    if ((ce = bisect_f64(st, d, eabs, n, r, reinterpret_cast<float*>(Ls), lam, batch)) != cudaSuccess) return ce;
+    if ((ce = bisect_f64(st, d, eabs, n, r, reinterpret_cast<float*>(Ls), lam, batch, BISECT_C128)) != cudaSuccess) return ce;
   } else {
     ProfScope ps(st, K_BISECT);
     bisect_kernel<R><<<(total * 32 + 255) / 256, 256, 0, st>>>(d, eabs, n, r, ldde, lam, r, total);
@@ -719,7 +719,7 @@ cudaError_t eigh_top_mixed(cudaStream_t st, cx<float>* H, long long sH, int n, i
     tridiag_phases_kernel<double><<<batch, 256, 0, st>>>(ed, n, n, eabs, phid);
   }
   if ((ce = cudaGetLastError()) != cudaSuccess) return ce;
-  if ((ce = bisect_f64(st, dd, eabs, n, r, df, lam, batch)) != cudaSuccess) return ce;
+  if ((ce = bisect_f64(st, dd, eabs, n, r, df, lam, batch, BISECT_C64)) != cudaSuccess) return ce;
   if ((ce = inviter64<float>(st, dd, eabs, n, r, lam, Zf, Z, Ls, U0, U1, U2, piv, batch)) != cudaSuccess) return ce;
   {
     ProfScope ps(st, K_ELEMWISE);

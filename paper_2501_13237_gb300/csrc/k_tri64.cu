@@ -100,7 +100,7 @@ __device__ __forceinline__ int sturm_minors(const double* ds, const double* b, i
 
 // Top r eigenvalues (descending) of the real tridiagonal (d, e).  L lanes per
 // eigenvalue count at L interior points of the bracket, which shrinks
-// (L + 1)-fold per round until it is 4 eps_64 ||T|| wide.  The bracket starts
+// (L + 1)-fold per round until it is width * eps_64 ||T|| wide.  The bracket starts
 // at lamf[t] -/+ 16 or 512 eps_32 ||T|| around the float32 eigenvalue of the
 // rounded tridiagonal when Sturm counts confirm that it holds the wanted
 // eigenvalue (the float32 counts are off by more than the former now and then,
@@ -109,7 +109,8 @@ constexpr int BIS64_THREADS = 64;
 
 template <int L>
 __global__ void __launch_bounds__(BIS64_THREADS) bisect64_kernel(const double* db, const double* eb, int n, int r,
-                                                                 int ldde, const float* lamfb, double* lamb, int ldl) {
+                                                                 int ldde, const float* lamfb, double* lamb, int ldl,
+                                                                 double width) {
   extern __shared__ double bis_smem[];
   double* ds = bis_smem;        // n: d scaled
   double* bs = bis_smem + n;    // n: e^2 scaled
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(BIS64_THREADS) bisect64_kernel(const double* d
   ghi = red[1][0] * sc;
   __syncthreads();
   const double tnorm = fmax(fabs(glo), fabs(ghi));
-  const double tol = 4 * DBL_EPSILON * tnorm + 0x1p-1000;
+  const double tol = width * DBL_EPSILON * tnorm + 0x1p-1000;
   glo -= 4 * DBL_EPSILON * tnorm;
   ghi += 4 * DBL_EPSILON * tnorm;
   const int sub = lane % L, g0 = lane - sub;
@@ -194,18 +195,18 @@ __global__ void __launch_bounds__(BIS64_THREADS) bisect64_kernel(const double* d
 }
 
 cudaError_t bisect64(cudaStream_t st, const double* d, const double* e, int n, int r, const float* lamf, double* lam,
-                     int batch) {
+                     int batch, double width) {
   ProfScope ps(st, K_BISECT64);
   const size_t bsm = 2 * sizeof(double) * (size_t)n;
   auto go = [&](auto kernel, int L) {
     const cudaError_t ce = ensure_kernel_smem((const void*)kernel, bsm, false);
     if (ce != cudaSuccess) return ce;
     const int per = BIS64_THREADS / L;   // eigenvalues per block
-    kernel<<<dim3((r + per - 1) / per, batch), BIS64_THREADS, bsm, st>>>(d, e, n, r, n, lamf, lam, r);
+    kernel<<<dim3((r + per - 1) / per, batch), BIS64_THREADS, bsm, st>>>(d, e, n, r, n, lamf, lam, r, width);
     return cudaGetLastError();
   };
-  // Rounds from the float32 bracket (32 bits): 14 with 4 lanes, 11 with 8, 8 with
-  // 16, 7 with 32; more lanes as long as a state's eigenvalues (up to 8 levels)
+  // Rounds from the float32 bracket (32 bits to width 4, 33 to 2): 14 or 15 with 4 lanes,
+  // 11 with 8, 8 or 9 with 16, 7 with 32; more lanes as long as a state's eigenvalues (up to 8 levels)
   // still find a sub-partition each.
   if (r <= 64) return go(bisect64_kernel<32>, 32);
   if (r <= 192) return go(bisect64_kernel<16>, 16);

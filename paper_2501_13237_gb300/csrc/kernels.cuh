@@ -107,9 +107,11 @@ cudaError_t gram_entropy(cudaStream_t st, cx<R>* H, long long sH, int n, void* c
                          double* S, long long sS);
 
 // ---- k_tri64.cu (float64 eigenpairs of real tridiagonals; d, e: batch x n)
-// Top r eigenvalues (descending) from float32 estimates lamf (batch x r each).
+// Top r eigenvalues (descending) from float32 estimates lamf (batch x r each), bracketed to width * eps_64 ||T||:
+// 2 for complex128 states; 4 for the problems of complex64 states, whose vectors are rounded to float32.
+constexpr double BISECT_C128 = 2, BISECT_C64 = 4;
 cudaError_t bisect64(cudaStream_t st, const double* d, const double* e, int n, int r, const float* lamf, double* lam,
-                     int batch);
+                     int batch, double width);
 // Their unit eigenvectors, columns of Z (n x r).  Y (may be Z), L, U0, U1, U2, piv: n x r scratch per matrix.
 template <typename OUT>
 cudaError_t inviter64(cudaStream_t st, const double* d, const double* e, int n, int r, const double* lam, OUT* Z,
