@@ -98,9 +98,10 @@ __device__ __forceinline__ float2 df_add2(float2 a, float2 b) {
   df_norm(a.x, a.y);
   return a;
 }
-// 1 / sqrt of a positive double-float.  y is the correctly rounded-ish float
-// estimate (relative error below 2^-22); with r = 1 - x y^2 formed in
-// double-float, y (1 + r / 2 + 3 r^2 / 8) is good to about 2^-46.
+// 1 / sqrt of a positive double-float (hi in [2^-100, 2^100]) from the hardware's float
+// estimate y (2 ulp): with r = 1 - x y^2 formed in double-float, the binomial series
+// y (1 + r / 2 + 3 r^2 / 8), whose first term left out is 2^-63; the float operations on r (below
+// 2^-21) leave a relative error of at most 2^-44.
 __device__ __forceinline__ float2 df_rsqrt(float2 x) {
   const float y = rsqrtf(x.x);
   const float2 y2 = df_mul(y, 0.f, y, 0.f);
@@ -110,6 +111,16 @@ __device__ __forceinline__ float2 df_rsqrt(float2 x) {
   const float c = y * fmaf(0.375f * r, r, 0.5f * r);
   const float h = __fadd_rn(y, c);
   return make_float2(h, __fsub_rn(c, __fsub_rn(h, y)));
+}
+// 1 / x of a double-float (hi in [1, 2)): one Newton step from the rounded 1 / hi, relative error at
+// most 2^-46.
+__device__ __forceinline__ float2 df_rcp(float2 x) {
+  const float y = __frcp_rn(x.x);
+  float rh = 1.f, rl = 0.f;
+  df_mac(rh, rl, -x.x, -x.y, y, 0.f);
+  float2 c = make_float2(y, y * (rh + rl));
+  df_norm(c.x, c.y);
+  return c;
 }
 
 }  // namespace nne

@@ -6,6 +6,7 @@
 #include <tuple>
 
 #include "kernels.cuh"
+#include "recip.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -217,17 +218,6 @@ __global__ void __launch_bounds__(KEEP_THREADS) tridiag_smem_kernel(const cx<dou
 // (the earlier two-barrier kernel in brackets), float64: n = 64:
 // 387 (515), 256: 3129 (4163); float32, n = 128: 234 (328).
 // Sums run in a fixed order.
-__device__ __forceinline__ float rsqrt_series(float x) {   // hardware estimate (2 ulp), one Newton step
-  const float y = rsqrtf(x);
-  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
-}
-// From a 20-bit estimate y with r = 1 - x y^2: y (1 + r/2 + 3 r^2/8 + 5 r^3 / 16), error r^4 = 2^-76 before rounding.
-__device__ __forceinline__ double rsqrt_series(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double r = fma(-x * y, y, 1.0);
-  return fma(y * r, fma(r, fma(r, 0.3125, 0.375), 0.5), y);
-}
 // Pivots smaller than SMALL are scaled by UP before they are squared (their squares
 // would be denormal and |x0| inaccurate, and the reflector not unitary).
 template <typename R> struct PivotScale;

@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "recip.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -610,11 +611,6 @@ __global__ void __launch_bounds__(QR_THREADS) qr_panel_reg_kernel(cx<R>* Ab, lon
 __device__ __forceinline__ void fused_pivot(double xn2, cx<double> x0, cx<double>* alpha, double* inv, double* tau) {
   hh_pivot<double>(xn2, x0, alpha, inv, tau);
 }
-// 1 / sqrt(x), x > 0: the hardware estimate (2 ulp) and one Newton step.
-__device__ __forceinline__ float rsqrt_newton(float x) {
-  const float y = rsqrtf(x);
-  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
-}
 // hh_pivot without divides and square roots on the column's chain (440 -> about
 // 150 cycles); |x0| below 2^-50 is scaled away from denormal squares.
 __device__ __forceinline__ void fused_pivot(float xn2, cx<float> x0, cx<float>* alpha, float* inv, float* tau) {
@@ -622,13 +618,13 @@ __device__ __forceinline__ void fused_pivot(float xn2, cx<float> x0, cx<float>* 
   const float up = s < 0x1p-50f ? 0x1p70f : 1.f, dn = s < 0x1p-50f ? 0x1p-70f : 1.f;
   const float a = x0.re * up, b = x0.im * up, q2 = fmaf(a, a, b * b);
   const bool nz = q2 > 0.f;
-  const float qi = nz ? rsqrt_newton(q2) : 0.f;
+  const float qi = nz ? rsqrt_series(q2) : 0.f;
   const float pr = nz ? a * qi : 1.f, pi = b * qi, ax0 = q2 * qi * dn;
   const bool live = xn2 > 0.f;
-  const float xn = live ? xn2 * rsqrt_newton(xn2) : 0.f;
+  const float xn = live ? xn2 * rsqrt_series(xn2) : 0.f;
   *alpha = mk<float>(-xn * pr, -xn * pi);
   const float un2 = 2.f * fmaf(xn, ax0, xn2);
-  *inv = live ? rsqrt_newton(un2) : 0.f;
+  *inv = live ? rsqrt_series(un2) : 0.f;
   *tau = live ? 2.f : 0.f;
 }
 template <typename R>

@@ -144,7 +144,7 @@ __device__ __forceinline__ cx<double> env_scale(cx<double> a, int e) {
   return mk<double>(a.re * h0 * h1, a.im * h0 * h1);
 }
 // The factor that brings the largest component to 1: 2^-e, and for double-floats the
-// reciprocal of the mantissa m left (one Newton step from the rounded 1 / m: 2^-47).
+// reciprocal of the mantissa m left.
 template <typename R> struct EnvNorm;
 template <> struct EnvNorm<float> {
   int e;
@@ -155,11 +155,7 @@ template <> struct EnvNorm<float> {
     e = key_exp<float>(__float_as_int(v.x));
     const float4 w = env_scale(make_float4(v.x, v.y, 0.f, 0.f), e);
     m = make_float2(w.x, w.y);
-    const float y = __frcp_rn(m.x);
-    float rh = 1.f, rl = 0.f;
-    df_mac(rh, rl, -m.x, -m.y, y, 0.f);
-    c = make_float2(y, y * (rh + rl));
-    df_norm(c.x, c.y);
+    c = df_rcp(m);
   }
   __device__ __forceinline__ float4 operator()(float4 a) const {
     a = env_scale(a, e);

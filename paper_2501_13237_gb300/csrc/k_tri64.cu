@@ -15,23 +15,13 @@
 #include <float.h>
 
 #include "kernels.cuh"
+#include "recip.cuh"
 
 namespace nne {
 
 namespace {
 
 __device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffLL; }
-
-// 1 / x from the hardware's 20-bit estimate y: with r = 1 - x y, 1 / x =
-// y (1 + r + r^2 + ...); cut after r^2 the error is r^3 = 2^-60 before
-// rounding (the third-order member of the Newton-Schulz family).  x normal
-// and finite.
-__device__ __forceinline__ double rcp_series(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double r = fma(-x, y, 1.0);
-  return fma(y, fma(r, r, r), y);
-}
 
 __device__ __forceinline__ unsigned long long splitmix64(unsigned long long x) {
   x += 0x9E3779B97F4A7C15ULL;
