@@ -189,7 +189,7 @@ nne_status nne_expect(nne_state* st, int n_obs, const uint8_t* paulis, double* r
 nne_status nne_entropy(nne_state* st, double* S_out);
 
 /* a8 -- noise extrapolation to lambda_star (Sec. 2.2.3 (B), App. B.2), FP64
- * on the device, one thread per observable.
+ * on the device: one thread per observable, a cluster of CTAs for those that need EXP3.
  *   lambdas host double[n_lambda]; values host double n_lambda x n_obs;
  *   log_fid host double[n_lambda] (log F per level) or NULL (= 0);
  *   y_zero  host double[n_obs] (lambda = 0 values, the sign reference of

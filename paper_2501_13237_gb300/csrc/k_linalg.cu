@@ -1,17 +1,18 @@
-// Dense linear algebra of the truncation step, written for GB300:
-//   * Householder reduction of a Hermitian matrix to real tridiagonal form,
-//     one thread-block cluster per matrix (hardware cluster barriers, matrix
-//     resident in L2), two cluster barriers per column;
+// The Hermitian eigensolver of the truncation step and the entropy, written for GB300:
+//   * Householder reduction to real tridiagonal form, one thread-block cluster
+//     per matrix: in the cluster's shared memory (k_eig_small.cu), double-float
+//     (k_tridiag_df.cu), or here, on the matrix in L2 with two cluster barriers per
+//     column;
 //   * eigenvalues of the tridiagonal by 32-way multisection with Sturm
-//     counts (one warp per wanted eigenvalue);
+//     counts (one warp per wanted eigenvalue; float64: k_tri64.cu narrows the
+//     float32 brackets);
 //   * eigenvectors by inverse iteration with a partially pivoted tridiagonal
-//     LU (one thread per eigenvector), back-transformed through the phase
-//     scaling and the Householder reflectors (one CTA per 32 columns);
-//   * Householder QR (one cluster per matrix, column blocks owned by CTAs,
-//     one cluster barrier per column) and explicit Q formation; used to
-//     orthonormalise the eigenvector block and for the centre moves.
-// Precision follows the state: float for complex64 states, double for
-// complex128.  The reductions are written in a fixed order, so results are
+//     LU (float32 here, one thread each; float64 in k_tri64.cu), back-transformed
+//     through the phase scaling and the Householder reflectors (k_eig_small.cu) and
+//     orthonormalised by the QR (k_qr.cu).
+// Precision follows the state: float for complex64 states (by default with the
+// reduction, eigenvalues and tridiagonal eigenvectors in float64 or double-float),
+// double for complex128.  The reductions are written in a fixed order, so results are
 // bitwise reproducible run to run.  The double-float and the L2-resident reductions do not
 // depend on what else is batched either; those in one cluster's shared memory (tridiag_smem,
 // _keep) sum K over as many CTAs as the batch lets run at once.

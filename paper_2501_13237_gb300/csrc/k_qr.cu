@@ -2,8 +2,8 @@
 //
 // Panels of 32 columns are factored by one thread-block cluster per matrix:
 // the panel rows are spread over the cluster's CTAs (cyclically) and kept in
-// shared memory; per column the cluster exchanges one round of partial sums
-// through distributed shared memory.  Each panel also yields the compact-WY
+// registers (shared memory where they do not fit); per column the cluster exchanges
+// one round of partial sums through distributed shared memory.  Each panel also yields the compact-WY
 // factor T (P_0 ... P_{b-1} = I - V T V^H).  Trailing updates and the explicit Q then apply each panel's
 // block reflector (wy_apply).  All reductions are in a fixed order (deterministic).
 #include <type_traits>
@@ -1011,8 +1011,8 @@ static cudaError_t panel_factor(cudaStream_t st, cx<R>* A, long long sA, int m, 
   if ((mp + csr - 1) / csr > 16 * QR_WARPS) csr = 16;
   const int nl = (mp + csr - 1) / csr;
   // The fused kernel is the faster at every size; complex64 matrices of up to
-  // QR_KEEP_MAX rows keep the other one so that small jobs' results stay as they
-  // were (see EIGH_F64_MAX).
+  // QR_KEEP_MAX rows (at most 64 to a CTA) keep the other one so that small jobs'
+  // results stay as they were (see EIGH_F64_MAX).
   const bool fused = std::is_same<R, double>::value || m > QR_KEEP_MAX;
   auto go = [&](auto kernel) {
     return launch_cluster_qr(kernel, csr, batch, fused ? FUSED_THREADS : QR_THREADS, 0, st, A, sA, n, m, pb, bw, V, sV, n, Tp, sT, zr);
@@ -1020,7 +1020,7 @@ static cudaError_t panel_factor(cudaStream_t st, cx<R>* A, long long sA, int m, 
 #define NNE_PANEL(RPW)                                                                       \
   if (nl <= RPW * QR_WARPS) {                                                                \
     if (fused) return go(qr_panel_fused_kernel<R, RPW>);                                     \
-    if constexpr (std::is_same<R, float>::value) return go(qr_panel_reg_kernel<R, RPW>);     \
+    if constexpr (std::is_same<R, float>::value && RPW <= 4) return go(qr_panel_reg_kernel<R, RPW>); \
   }
   NNE_PANEL(1)
   NNE_PANEL(2)

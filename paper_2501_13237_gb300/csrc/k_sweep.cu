@@ -66,7 +66,7 @@ __device__ __forceinline__ T block_max(T v, T* red) {
 namespace sweep {
 
 constexpr int THREADS = 256;
-constexpr int NB = 8;            // loads per thread and batch; also the float32 run length before a float64 fold
+constexpr int NB = 8;            // loads per thread and batch; also the length of a float32 sum before it is folded
 constexpr int RING_STAGES = 4;   // batches in flight per thread (cp.async ring in shared memory)
 
 // Elements of one 16-byte load: two complex64 or one complex128.
@@ -172,26 +172,6 @@ template <> struct EnvNorm<double> {
 };
 __device__ __forceinline__ cx<float> env_coef(float4 a) { return mk<float>(a.x, a.z); }
 __device__ __forceinline__ cx<double> env_coef(cx<double> a) { return a; }
-
-// Streaming loads (site tensors are read once per pass).
-template <typename R, int V>
-__device__ __forceinline__ void ldv(const cx<R>* p, cx<R>* o);
-template <>
-__device__ __forceinline__ void ldv<float, 2>(const cx<float>* p, cx<float>* o) {
-  const float4 v = __ldcs(reinterpret_cast<const float4*>(p));
-  o[0] = mk<float>(v.x, v.y);
-  o[1] = mk<float>(v.z, v.w);
-}
-template <>
-__device__ __forceinline__ void ldv<float, 1>(const cx<float>* p, cx<float>* o) {
-  const float2 v = __ldcs(reinterpret_cast<const float2*>(p));
-  o[0] = mk<float>(v.x, v.y);
-}
-template <>
-__device__ __forceinline__ void ldv<double, 1>(const cx<double>* p, cx<double>* o) {
-  const double2 v = __ldcs(reinterpret_cast<const double2*>(p));
-  o[0] = mk<double>(v.x, v.y);
-}
 
 // Asynchronous global -> shared copy of one load unit (16 bytes, or 8 for a
 // single complex64); bytes past `valid` are zero-filled.

@@ -227,13 +227,13 @@ __global__ void __launch_bounds__(512) tridiag_df_kernel(float4* Hb, long long s
 //   * one pass over the matrix per column: the rank-2 update of column j and
 //     the product with v_{j+1} read and write each entry once;
 //   * the pivot is formed by one warp (all warps doing so cost more issue slots
-//     than the broadcast; for K, and for gathering p to push it in one piece, the
-//     extra block barrier cost more than it saved);
+//     than the broadcast; for K of up to 380 rows, and for gathering p to push it in one
+//     piece, the extra block barrier cost more than it saved);
 //   * no float64: GB300 has two float64 lanes per SM.
 // The matrix is scaled by a power of two to a largest diagonal entry in
 // [1, 2); columns below norm 2^-50 then count as null (their squares would
 // leave float32's range, and an inaccurate norm makes a reflector that is not
-// unitary), a backward error below eps_64 ||H||.
+// unitary), a backward error of 2^-50 of that entry, below the arithmetic's 2^-46.
 //
 // ROWS_C64   rows in shared memory, from the complex64 matrix (lower triangle read);
 // ROWS_DF    rows in shared memory, from the double-float trailing block at
