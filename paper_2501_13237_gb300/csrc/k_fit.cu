@@ -329,6 +329,8 @@ struct Exp3Best {
   }
 };
 
+// ONE: one observable per cluster, whose levels are gathered before the first exchange.
+template <bool ONE>
 __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 8)
     exp3_kernel(int nl, const double* lam, const double* vals, int n_obs, double ls, const uint8_t* mask,
                 const double* fb, double* out, int* status, int per) {
@@ -345,31 +347,44 @@ __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 
   __shared__ double B_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   double *y = ys[NW], *lc = lams[NW];
+  auto levels = [&](int q) {   // of observable q of the list, by one thread
+    m_s = gather_levels(nl, lam, vals, nullptr, n_obs, list[q], mask, y, lc, nullptr);
+    double B = 0;
+    ok_s = exp3_range(m_s, lc, &B) ? 1 : 0;
+    B_s = B;
+  };
   for (long long o0 = (long long)cl * per; o0 < n_obs; o0 += (long long)ncl * per) {
-    // the marked observables, the same list in every CTA
-    const bool mine = tid < per && o0 + tid < n_obs && status[o0 + tid] == FIT_NEEDS_EXP3;
-    if (!__syncthreads_or(mine)) continue;
-    const unsigned votes = __ballot_sync(0xffffffffu, mine);
-    if (lane == 0) count[warp] = __popc(votes);
-    __syncthreads();
-    int n_fit = 0, before = 0;
-    for (int w = 0; w < NW; ++w) {
-      if (w < warp) before += count[w];
-      n_fit += count[w];
+    int n_fit = 1;
+    if (ONE) {
+      if (status[o0] != FIT_NEEDS_EXP3) return;
+      if (tid == 0) {
+        list[0] = (int)o0;
+        levels(0);
+      }
+    } else {
+      // the marked observables, the same list in every CTA
+      const bool mine = tid < per && o0 + tid < n_obs && status[o0 + tid] == FIT_NEEDS_EXP3;
+      if (!__syncthreads_or(mine)) continue;
+      const unsigned votes = __ballot_sync(0xffffffffu, mine);
+      if (lane == 0) count[warp] = __popc(votes);
+      __syncthreads();
+      n_fit = 0;
+      int before = 0;
+      for (int w = 0; w < NW; ++w) {
+        if (w < warp) before += count[w];
+        n_fit += count[w];
+      }
+      if (mine) list[before + __popc(votes & ((1u << lane) - 1))] = (int)(o0 + tid);
     }
-    if (mine) list[before + __popc(votes & ((1u << lane) - 1))] = (int)(o0 + tid);
     // also: every CTA runs, has read its statuses and is done with best_s
     cluster.sync();
-    const bool many = n_fit > EXP3_WARP;   // then a CTA for a grid
-    double step = 0;                       // of the last observable
+    const bool many = !ONE && n_fit > EXP3_WARP;   // then a CTA for a grid
+    double step = 0;                               // of the last observable
     for (int q = many ? rank : 0; q < n_fit; q += many ? EXP3_CS : 1) {
-      if (tid == 0) {
-        m_s = gather_levels(nl, lam, vals, nullptr, n_obs, list[q], mask, y, lc, nullptr);
-        double B = 0;
-        ok_s = exp3_range(m_s, lc, &B) ? 1 : 0;
-        B_s = B;
+      if (!ONE) {
+        if (tid == 0) levels(q);
+        __syncthreads();
       }
-      __syncthreads();
       const int m = m_s;
       const double B = B_s;
       if (ok_s) {
@@ -394,7 +409,7 @@ __global__ void __cluster_dims__(EXP3_CS, 1, 1) __launch_bounds__(EXP3_THREADS, 
           else *cluster.map_shared_rank(&best_s[q / EXP3_CS][rank], q % EXP3_CS) = best;
         }
       }
-      __syncthreads();   // y, lc, m_s are free
+      if (!ONE) __syncthreads();   // y, lc, m_s are free
     }
     cluster.sync();
     // observable q by CTA q % EXP3_CS
@@ -458,7 +473,8 @@ static cudaError_t launch_fit(cudaStream_t st, int nl, const double* lam, const 
   const long long passes = (n_obs - 1) / ((long long)EXP3_CLUSTERS * EXP3_MOST) + 1;
   const int per = (int)((n_obs - 1) / (passes * EXP3_CLUSTERS) + 1);
   const int clusters = std::min(EXP3_CLUSTERS, (n_obs - 1) / per + 1);
-  exp3_kernel<<<clusters * EXP3_CS, EXP3_THREADS, 0, st>>>(nl, lam, vals, n_obs, ls, mask, fb, out, status, per);
+  (per == 1 ? exp3_kernel<true> : exp3_kernel<false>)<<<clusters * EXP3_CS, EXP3_THREADS, 0, st>>>(
+      nl, lam, vals, n_obs, ls, mask, fb, out, status, per);
   return cudaGetLastError();
 }
 
